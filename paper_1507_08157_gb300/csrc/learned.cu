@@ -77,12 +77,42 @@ __global__ void row_weights_kernel(const float *__restrict__ s, long long per, f
         wi[r] = tot > 0.0 ? (float)((double)si[r] * si[r] / tot) : 0.0f;
 }
 
-// out[j] = sum_r D[r][j] (one thread per column, rows in order, float64 accumulation)
-__global__ void colsum_kernel(const float *__restrict__ D, long long n, int w, float *__restrict__ out) {
+// Column sums out[j] = sum_r D[r][j], the bias gradients. Bound by reading D once (67 MB for the
+// last layer at 16384 rows, 10 us at the HBM rate); one thread per column walking all rows kept 8
+// blocks busy and took 5.5 ms for the
+// three layers, this 0.1 ms. Blocks of 128 columns x 4 row phases over row
+// slices; each thread keeps a compensated float32 pair (Knuth's two-sum: the pair carries 48
+// bits, where float64 adds, scarce on this part, would bound the loop), the phases and slices are
+// added in float64 in a fixed order.
+constexpr int CS_COLS = 128, CS_PH = 4;
+__global__ void __launch_bounds__(CS_COLS * CS_PH) colsum_part_kernel(const float *__restrict__ D, long long n, int w,
+                                                                      long long per, double *__restrict__ part) {
+    __shared__ double red[CS_PH][CS_COLS];
+    const int j = blockIdx.x * CS_COLS + threadIdx.x;
+    const long long r0 = blockIdx.y * per, r1 = r0 + per < n ? r0 + per : n;
+    float s = 0.0f, c = 0.0f;
+    if (j < w) {
+#pragma unroll 8
+        for (long long r = r0 + threadIdx.y; r < r1; r += CS_PH) {
+            const float x = D[r * w + j];
+            const float t = s + x, z = t - s;
+            c += (s - (t - z)) + (x - z);
+            s = t;
+        }
+    }
+    red[threadIdx.y][threadIdx.x] = isfinite(s) ? (double)s + (double)c : (double)s;   // inf: its error term is NaN
+    __syncthreads();
+    if (threadIdx.y == 0 && j < w) {
+        double v = 0.0;
+        for (int q = 0; q < CS_PH; ++q) v += red[q][threadIdx.x];
+        part[(long long)blockIdx.y * w + j] = v;
+    }
+}
+__global__ void colsum_final_kernel(const double *__restrict__ part, int slices, int w, float *__restrict__ out) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= w) return;
     double s = 0.0;
-    for (long long r = 0; r < n; ++r) s += (double)D[r * w + j];
+    for (int q = 0; q < slices; ++q) s += part[(long long)q * w + j];
     out[j] = (float)s;
 }
 
@@ -334,6 +364,19 @@ void ensure_rows(tddft_mlp *m, long long rows) {
     B.rows = rows;
 }
 
+// out = column sums of D [n][w]; scratch (gram_scratch_doubles(64, 32) doubles) holds the slices' sums.
+// At least 64 rows per thread so that the partial sums stay a small part of the reads.
+void colsum(cudaStream_t st, const float *D, long long n, int w, float *out, double *scratch) {
+    const long long fit = gram_scratch_doubles(64, 32) / w;
+    const long long slices = std::max<long long>(1, std::min({(n + 64 * CS_PH - 1) / (64 * CS_PH), fit, 512LL}));
+    const long long per = (n + slices - 1) / slices;
+    const int used = (int)((n + per - 1) / per);
+    colsum_part_kernel<<<dim3((w + CS_COLS - 1) / CS_COLS, used), dim3(CS_COLS, CS_PH), 0, st>>>(D, n, w, per, scratch);
+    check_launch("colsum_part");
+    colsum_final_kernel<<<(w + 127) / 128, 128, 0, st>>>(scratch, used, w, out);
+    check_launch("colsum_final");
+}
+
 // vec(A) rows [n][nb^2] of the perceptron for feature rows F (row stride ldf); keeps H1, H2
 void perceptron(cudaStream_t st, tddft_mlp *m, const float *W, long long n, const float *F, int ldf, float *A) {
     const Offs o = offsets(m);
@@ -370,22 +413,19 @@ void loss_grad_rows(cudaStream_t st, tddft_mlp *m, long long n, const float *X, 
     float *g = m->g;
     // layer 3
     gemm<float>(st, true, false, w, nout, (int)n, 1.0f, B.H2, w, 0, B.dA, nout, 0, 0.0f, g + o.W3, nout, 0, 1);
-    colsum_kernel<<<(nout + 127) / 128, 128, 0, st>>>(B.dA, n, nout, g + o.b3);
-    check_launch("colsum");
+    colsum(st, B.dA, n, nout, g + o.b3, B.scr);
     gemm<float>(st, false, true, (int)n, w, nout, 1.0f, B.dA, nout, 0, m->W + o.W3, nout, 0, 0.0f, B.dH, w, 0, 1);
     relu_back_kernel<<<grid_of(n * w), 256, 0, st>>>(B.dH, B.H2, n * w);
     check_launch("relu_back");
     // layer 2 (dH holds dL/d(pre-activation 2))
     gemm<float>(st, true, false, w, w, (int)n, 1.0f, B.H1, w, 0, B.dH, w, 0, 0.0f, g + o.W2, w, 0, 1);
-    colsum_kernel<<<(w + 127) / 128, 128, 0, st>>>(B.dH, n, w, g + o.b2);
-    check_launch("colsum");
+    colsum(st, B.dH, n, w, g + o.b2, B.scr);
     gemm<float>(st, false, true, (int)n, w, w, 1.0f, B.dH, w, 0, m->W + o.W2, w, 0, 0.0f, B.H2, w, 0, 1);
     relu_back_kernel<<<grid_of(n * w), 256, 0, st>>>(B.H2, B.H1, n * w);
     check_launch("relu_back");
     // layer 1 (H2 now holds dL/d(pre-activation 1)); F = X + nb with row stride ld
     gemm<float>(st, true, false, nf, w, (int)n, 1.0f, X + nb, ld, 0, B.H2, w, 0, 0.0f, g + o.W1, w, 0, 1);
-    colsum_kernel<<<(w + 127) / 128, 128, 0, st>>>(B.H2, n, w, g + o.b1);
-    check_launch("colsum");
+    colsum(st, B.H2, n, w, g + o.b1, B.scr);
 }
 
 void adam(cudaStream_t st, tddft_mlp *m, float lr) {
