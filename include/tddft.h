@@ -255,8 +255,7 @@ tddft_status tddft_fxc(tddft_ctx *ctx, double *fxc);
  * TDDFT_MIXED context it times, on k trial states of the context's own system (deterministic
  * pseudo-random P and V), every candidate cut of the grid work into tensor-core units:
  *   response_density: the per-tile kernels (kind 0, when every tile fits them) and units of at
- *     most chi_chunk x phi_chunk functions of a tile (kind 1; chi 128..320 in steps of 64, phi 64
- *     or 128);
+ *     most chi_chunk x phi_chunk functions of a tile (kind 1; chi 128 or 256, phi 32 or 64);
  *   potential_integrals: units of at most chi_chunk (128, 256, 384) x phi_chunk (32, 64, 128).
  * Each candidate runs once to warm up and three times timed with CUDA events on the context's
  * stream (ms = the mean). The fastest of each stage is installed and kept by the context for all
@@ -485,20 +484,20 @@ tddft_status tddft_work(const tddft_ctx *ctx, double *pair_points, double *table
 
 /* Environment variables. Each selects an alternative code path of the same operation, for
  * comparisons and tests; none skips work. TDDFT_NO_TC is read once per process, the others at
- * every tddft_create (or, for TDDFT_NO_PERSISTENT_DENSITY, at the first density launch).
+ * every tddft_create.
  *   TDDFT_NO_TC=1                  matrix products on CUDA cores instead of tcgen05 (and with
  *                                  them the tensor-core grid kernels)
  *   TDDFT_NO_GRID_TC=1             response density and potential integrals on CUDA cores
  *   TDDFT_NO_PERSISTENT_DENSITY=1  the per-tile tensor-core density kernel instead of the
- *                                  persistent one
+ *                                  persistent density units, where it fits
  *   TDDFT_NO_QUAD_GATHER=1         gather the density's P block element by element instead of
  *                                  by aligned groups of four phi
  *   TDDFT_NO_REDUCED_PRECOND=1     the inner CG of the iterative preconditioner on the full
  *                                  N_chi x N_phi space instead of the conduction x valence
  *                                  subspace
- *   TDDFT_NO_DENSITY_UNITS=1       the CUDA-core density on systems whose tiles exceed the
- *                                  per-tile tensor-core kernels, instead of the density units
- *   TDDFT_DENSITY_UNITS=1          the density units even where the per-tile kernels fit
+ *   TDDFT_NO_DENSITY_UNITS=1       no density units: the per-tile tensor-core kernel, or the
+ *                                  CUDA-core density on systems whose tiles exceed it
+ *   TDDFT_DENSITY_UNITS=1          the density units even with TDDFT_NO_PERSISTENT_DENSITY=1
  *   TDDFT_INTEGRALS_CHUNK=nc,np    largest chi / phi slot counts of one tensor-core integrals
  *                                  unit (multiples of 128 up to 384, and of 16 up to 128;
  *                                  default 384,128); smaller values cut tiles that would fit,

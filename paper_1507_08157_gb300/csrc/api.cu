@@ -249,19 +249,15 @@ struct Impl {
     unsigned short *chi_fm16 = nullptr;   // function-major f16 chi tables [slot][512]
     unsigned short *phi_fm16 = nullptr;   // function-major f16 phi tables [slot][512]
     unsigned short *phi_pm = nullptr;     // point-major f16 phi tables [tile][512][NPmax], zero padded
-    // dense tiles: density units with chunked point-major f16 tables ([chunk][512][64] chi,
-    // [chunk][512][32] phi)
+    // density units with chunked point-major f16 tables ([chunk][512][64] chi, [chunk][512][32] phi)
     bool dens_units = false;              // the density runs on units (selected)
     bool units_ok = false;                // chunked tables built (every tile's phi in whole quads)
     unsigned short *chi_pmc = nullptr, *phi_pmc = nullptr;
     long long nchunks_chi = 0;
-    DUnit *dunits = nullptr;
-    int ndunits = 0;
-    int dens_cut[2] = {320, 128}, int_cut[2] = {384, 128};   // unit cuts in use (chi, phi)
+    DUnitList dunits;
     std::vector<int> coff_h, poff_h, cfirst_h, pfirst_h;    // host tile offsets, first chunks
     Mem umem_dens, umem_int;              // unit lists (replaced when the autotuner recuts)
-    int *live_tiles = nullptr;            // tiles with both chi and phi (the persistent density's items)
-    int nlive = 0;
+    unsigned short *P16 = nullptr;        // float16 copy of P for the units' gather (workspace)
     int CK = 0, NPmax = 0, nslots_chi = 0, nslots_phi = 0, maxc = 0;
     int NPint = 0;            // phi rows of the integrals' B stage (the largest unit's phi, to 16)
     bool grid_tc = false, integrals_tc = false;
@@ -349,14 +345,13 @@ void potential_integrals_tc(cudaStream_t st, const GridShape &g, const TileSet<f
 void response_density_tc(cudaStream_t st, const GridShape &g, const TileSet<float> &chi,
                          const TileSet<float> &phi, const unsigned short *chi_pm, int CK, int NPmax, int nphi,
                          const float *P, long long sP, int k, float *rho, unsigned *scratch_bits,
-                         float *scale, int *err, bool phi_quads, const unsigned short *phi_pm,
-                         const int *live_tiles, int nlive);
+                         float *scale, int *err, bool phi_quads, const unsigned short *phi_pm);
 long long build_chunked_pm(cudaStream_t st, Mem &mem, const TileSet<float> &ts, const std::vector<int> &off_h, int W,
                            unsigned short **out, std::vector<int> &first);
 void response_density_units(cudaStream_t st, const GridShape &g, const TileSet<float> &chi, const TileSet<float> &phi,
                             const unsigned short *chi_pmc, long long nchunks_chi, const unsigned short *phi_pmc,
-                            const DUnit *units, int nunits, int nphi, const float *P, long long sP, int k, float *rho,
-                            unsigned *scratch_bits, float *scale, int *err);
+                            const DUnitList &ul, int nchi, int nphi, const float *P, long long sP, int k, float *rho,
+                            unsigned short *P16, unsigned *bits, float *scale, int *err);
 int noalloc_max_states();
 void response_density_tc_noalloc(cudaStream_t st, const GridShape &g, const TileSet<float> &chi,
                                  const TileSet<float> &phi, const unsigned short *chi_pm, int CK, int NPmax,
@@ -674,12 +669,16 @@ void ensure_workspace(tddft_ctx *c, Impl<T> &I, int states) {
     I.stage = I.wmem.template alloc<double>(
         (size_t)std::max({states * len, states * n3, states * c->nnz_abi()}));
     I.tc_bits = I.wmem.template alloc<unsigned>((size_t)states);
-    I.tc_scale = I.wmem.template alloc<float>((size_t)states);
+    I.tc_scale = I.wmem.template alloc<float>((size_t)2 * states);
     if (c->sparse) {
         // the grid kernels address P and V densely; the tensor-core left products take their
         // right operand block-transposed
         I.dense = I.wmem.template alloc<T>((size_t)states * c->nc * c->nv);
         I.opT = I.wmem.template alloc<T>((size_t)states * len);
+        if (I.units_ok) I.P16 = I.wmem.template alloc<unsigned short>((size_t)(states + 1) / 2 * 2 * c->nc * c->nv);
+    } else {
+        // the potential matrix is free while a density is made, and holds the copy of its P
+        I.P16 = reinterpret_cast<unsigned short *>(I.Vmat);
     }
     I.cap = states;
 }
@@ -694,16 +693,15 @@ void density(tddft_ctx *c, Impl<T> &I, const T *P, int ns) {
     }
     if constexpr (sizeof(T) == 4) {
         if (I.dens_units) {
-            response_density_units(c->st, c->grid(), I.chi, I.phi, I.chi_pmc, I.nchunks_chi, I.phi_pmc, I.dunits,
-                                   I.ndunits, c->nv, P, (long long)c->nc * c->nv, ns, I.rho, I.tc_bits, I.tc_scale,
+            response_density_units(c->st, c->grid(), I.chi, I.phi, I.chi_pmc, I.nchunks_chi, I.phi_pmc, I.dunits, c->nc,
+                                   c->nv, P, (long long)c->nc * c->nv, ns, I.rho, I.P16, I.tc_bits, I.tc_scale,
                                    tc_error_word());
             return;
         }
         if (I.grid_tc) {
             response_density_tc(c->st, c->grid(), I.chi, I.phi, I.chi_pm, I.CK, I.NPmax, c->nv, P,
                                 (long long)c->nc * c->nv, ns,
-                                I.rho, I.tc_bits, I.tc_scale, tc_error_word(), I.phi_quads, I.phi_pm,
-                                I.live_tiles, I.nlive);
+                                I.rho, I.tc_bits, I.tc_scale, tc_error_word(), I.phi_quads, I.phi_pm);
             return;
         }
     }
@@ -996,27 +994,60 @@ bool build_density_chunks(tddft_ctx *c, Impl<float> &I) {
     return true;
 }
 
-// the density's units: chunks of at most cch chi (a multiple of 64, <= 320) and pch phi (a
-// multiple of 32, <= 128) of each tile
+// the density's items: whole tiles in chunks of at most 128 chi, or, for lists of 129 to cch chi (128 or
+// 256), two halves of the tile with all chi in one chunk, so that the sum over chi stays in one
+// accumulator; and at most pch phi (32 or 64; 32 in float32). Lists are cut evenly in whole table
+// chunks. Items in order of falling work: the persistent blocks take them in turn, so that they
+// finish together.
 void set_density_units(Impl<float> &I, int cch, int pch) {
     const int ntl = I.chi.ntiles;
     const std::vector<int> &coff = I.coff_h, &poff = I.poff_h;
+    DUnitList &L = I.dunits;
+    if (L.phi32) pch = 32;
+    std::vector<DItem> items;
+    std::vector<long long> work;
     std::vector<DUnit> us;
+    int live = 0;
     for (int t = 0; t < ntl; ++t) {
         const int nct = coff[t + 1] - coff[t], npt = poff[t + 1] - poff[t];
         if (nct == 0 || npt == 0) continue;
-        for (int cc = 0; cc < nct; cc += cch)
-            for (int pc = 0; pc < npt; pc += pch)
-                us.push_back(DUnit{t, coff[t] + cc, std::min(cch, nct - cc), poff[t] + pc, std::min(pch, npt - pc),
-                                   I.cfirst_h[t] + cc / 64, I.pfirst_h[t] + pc / 32, 0});
+        ++live;
+        const bool half = nct > 128 && nct <= cch;
+        const int nck = (nct + 63) / 64, npk = (npt + 31) / 32;
+        const int mc = half ? 1 : (nck + 1) / 2, mp = (npk * 32 + pch - 1) / pch;
+        const int u0 = (int)us.size();
+        for (int x = 0; x < mc; ++x)
+            for (int y = 0; y < mp; ++y) {
+                const int k0 = nck * x / mc, k1 = nck * (x + 1) / mc, q0 = npk * y / mp, q1 = npk * (y + 1) / mp;
+                us.push_back(DUnit{t, coff[t] + k0 * 64, std::min(k1 * 64, nct) - k0 * 64, poff[t] + q0 * 32,
+                                   std::min(q1 * 32, npt) - q0 * 32, I.cfirst_h[t] + k0, I.pfirst_h[t] + q0,
+                                   (y == 0 ? DUnit::FIRST : 0) | (y == mp - 1 ? DUnit::LAST : 0)});
+            }
+        // units that add to rho need not stay together: one item per chunk of chi, so that the densest
+        // tiles (forty times the mean work in a 200-atom cluster) do not hold one block up at the end
+        const int parts = L.adds ? mc : 1;
+        for (int h = 0; h < (half ? 2 : 1); ++h)
+            for (int x = 0; x < parts; ++x) {
+                items.push_back(DItem{t, h * 256, half ? 2 : 4, u0 + x * mp, parts > 1 ? u0 + (x + 1) * mp : (int)us.size()});
+                work.push_back((long long)nck * npk * (half ? 2 : 4) / parts);
+            }
     }
+    std::vector<int> order(items.size());
+    for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work[a] > work[b]; });
+    std::vector<DItem> sorted(items.size());
+    for (size_t i = 0; i < order.size(); ++i) sorted[i] = items[order[i]];
     I.umem_dens.release();
-    I.ndunits = (int)us.size();
-    I.dunits = I.umem_dens.alloc<DUnit>(std::max<size_t>(1, us.size()));
-    if (!us.empty())
-        check(cudaMemcpy(I.dunits, us.data(), us.size() * sizeof(DUnit), cudaMemcpyHostToDevice), "upload density units");
-    I.dens_cut[0] = cch;
-    I.dens_cut[1] = pch;
+    L.nitems = (int)sorted.size();
+    L.covers = live == ntl;
+    DUnit *du = I.umem_dens.alloc<DUnit>(us.size());
+    DItem *di = I.umem_dens.alloc<DItem>(sorted.size());
+    if (!us.empty()) {
+        check(cudaMemcpy(du, us.data(), us.size() * sizeof(DUnit), cudaMemcpyHostToDevice), "upload density units");
+        check(cudaMemcpy(di, sorted.data(), sorted.size() * sizeof(DItem), cudaMemcpyHostToDevice), "upload density items");
+    }
+    L.units = du;
+    L.items = di;
 }
 
 // the integrals' units: chunks of at most cch chi (a multiple of 128, <= 384) and pch phi (a
@@ -1051,8 +1082,6 @@ bool set_integrals_units(Impl<float> &I, int cch, int pch) {
               "upload integrals units");
     I.maxc = maxnc;
     I.NPint = NPi;
-    I.int_cut[0] = cch;
-    I.int_cut[1] = pch;
     return true;
 }
 
@@ -1110,16 +1139,6 @@ void build_impl(tddft_ctx *c, const tddft_system *s, const tddft_sparse_system *
                 check(cudaMemcpy(I->chi_pm, pm.data(), pm.size() * sizeof(unsigned short), cudaMemcpyHostToDevice),
                       "upload point-major chi");
                 I->CK = CK;
-                {
-                    std::vector<int> live;
-                    for (int t = 0; t < ntl; ++t)
-                        if (coff[t + 1] > coff[t] && poff[t + 1] > poff[t]) live.push_back(t);
-                    I->nlive = (int)live.size();
-                    I->live_tiles = I->mem.template alloc<int>(std::max<size_t>(1, live.size()));
-                    if (!live.empty())
-                        check(cudaMemcpy(I->live_tiles, live.data(), live.size() * sizeof(int), cudaMemcpyHostToDevice),
-                              "upload live tiles");
-                }
                 // point-major f16 phi tables for the density epilogue
                 if (NP % 32 == 0) {
                     std::vector<unsigned short> ppm((size_t)ntl * TILE_PTS * NP, 0);
@@ -1150,15 +1169,23 @@ void build_impl(tddft_ctx *c, const tddft_system *s, const tddft_sparse_system *
             }
             I->coff_h = coff;
             I->poff_h = poff;
-            // dense tiles: the density in units of <= 320 chi and <= 128 phi of a tile, when every
-            // tile's phi list is whole aligned atom quads (the P gather loads four phi at once);
-            // TDDFT_DENSITY_UNITS=1 takes them even where the per-tile kernels fit
+            // the density on units wherever every tile's phi list is whole aligned quads: faster
+            // there at every size measured (20 to 200 atoms, figures in density_units.cu);
+            // the per-tile kernel for other lists, and for TDDFT_NO_PERSISTENT_DENSITY=1 where it
+            // fits; TDDFT_NO_DENSITY_UNITS=1 takes the per-tile kernel, or the CUDA cores where that
+            // does not fit
             {
                 const char *nu = std::getenv("TDDFT_NO_DENSITY_UNITS");
                 const char *fu = std::getenv("TDDFT_DENSITY_UNITS");
-                const bool want = !I->grid_tc || (fu && fu[0] == '1');
-                if (want && !(nu && nu[0] == '1') && c->nv % 4 == 0 && build_density_chunks(c, *I)) {
-                    set_density_units(*I, 320, 128);
+                const char *np = std::getenv("TDDFT_NO_PERSISTENT_DENSITY");
+                const bool per_tile = I->grid_tc && np && np[0] == '1' && !(fu && fu[0] == '1');
+                // the arithmetic of the epilogue by the longest lists: phi in float32 where a tile's
+                // phi fill no whole float16 rows of 32, sums by 32 phi past the lists of 128 phi or 320 chi
+                I->dunits.adds = !I->grid_tc;
+                I->dunits.phi32 = I->grid_tc && NP % 32 != 0;
+                I->dunits.chunked = I->grid_tc && NP % 32 == 0 && (NP > 128 || CK > 320);
+                if (!per_tile && !(nu && nu[0] == '1') && c->nv % 4 == 0 && build_density_chunks(c, *I)) {
+                    set_density_units(*I, 256, 64);
                     I->dens_units = true;
                 }
             }
@@ -2688,7 +2715,7 @@ tddft_status tddft_autotune(tddft_ctx *c, int32_t k, tddft_tuning_entry *out, in
                 best_ms = rows.back().ms;
             }
             if (units_possible) {
-                const int cuts[][2] = {{320, 128}, {256, 128}, {192, 128}, {128, 128}, {320, 64}, {192, 64}, {128, 64}};
+                const int cuts[][2] = {{256, 64}, {128, 64}, {256, 32}, {128, 32}};
                 for (const auto &cut : cuts) {
                     set_density_units(I, cut[0], cut[1]);
                     I.dens_units = true;

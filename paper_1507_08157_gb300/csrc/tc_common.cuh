@@ -23,6 +23,10 @@ __device__ __forceinline__ void mbar_expect_tx(unsigned long long *b, unsigned b
                  : "memory");
 }
 
+__device__ __forceinline__ void mbar_arrive(unsigned long long *b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
+}
+
 __device__ __forceinline__ bool mbar_try_wait(unsigned long long *b, unsigned parity) {
     unsigned ok;
     asm volatile(
@@ -37,6 +41,7 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long *b, unsigned pa
 // already gave up
 __device__ __forceinline__ bool mbar_wait(unsigned long long *b, unsigned parity, volatile int *abort,
                                           long long limit) {
+    if (mbar_try_wait(b, parity)) return true;   // the usual case, without the clock
     const long long t0 = clock64();
     while (!mbar_try_wait(b, parity)) {
         if (*abort) return false;
@@ -76,6 +81,27 @@ __device__ __forceinline__ unsigned long long smem_desc(unsigned saddr) {
     return d;
 }
 
+// the same for an M/N-major operand: rows of 64 elements (128 bytes) along M/N, one row per K, 8-K
+// groups 1024 B apart; `blocks` bytes between consecutive blocks of 64 along M/N
+__device__ __forceinline__ unsigned long long smem_desc_mn(unsigned saddr, unsigned blocks) {
+    unsigned long long d = 0;
+    d |= (unsigned long long)((saddr & 0x3FFFF) >> 4);
+    d |= (unsigned long long)(blocks >> 4) << 16;
+    d |= (unsigned long long)(1024 >> 4) << 32;
+    d |= (unsigned long long)1 << 46;
+    d |= (unsigned long long)2 << 61;
+    return d;
+}
+
+// the low words of the two descriptors vary with the address alone, so that an issuing thread forms
+// a descriptor with one add: start address in 16-byte units, plus the block distance for M/N-major
+__device__ __forceinline__ unsigned desc_lo(unsigned saddr) { return ((saddr & 0x3FFFF) >> 4) | (1u << 16); }
+__device__ __forceinline__ unsigned desc_lo_mn(unsigned saddr, unsigned blocks) {
+    return ((saddr & 0x3FFFF) >> 4) | ((blocks >> 4) << 16);
+}
+constexpr unsigned DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);   // bits 32-63 of both
+__device__ __forceinline__ unsigned long long desc_of(unsigned lo) { return ((unsigned long long)DESC_HI << 32) | lo; }
+
 // instruction descriptor, kind::tf32: D f32, A/B tf32, both K-major
 __host__ __device__ constexpr unsigned idesc_tf32(int M, int N) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
@@ -100,6 +126,14 @@ __device__ __forceinline__ void mma_tf32(unsigned tmem_d, unsigned long long da,
         ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate));
 }
 
+// one lane of a converged warp; the compiler knows that a region under it has one thread, and keeps
+// what it computes for the tensor instructions in uniform registers
+__device__ __forceinline__ bool elect_one() {
+    unsigned p;
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void mma_commit(unsigned long long *bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
@@ -120,6 +154,20 @@ __device__ __forceinline__ void tmem_ld32(unsigned taddr, float *v) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+
+// 16 columns
+__device__ __forceinline__ void tmem_ld16(unsigned taddr, float *v) {
+    unsigned r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
+        "[%16];\n tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
 
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, unsigned long long *bar, int c0,
                                             int c1) {

@@ -91,16 +91,33 @@ struct VTile {
     int pad;
 };
 
-// One unit of the tensor-core density on dense tiles: a chunk of a tile's chi slots (at most five
-// blocks of 64) and of its phi slots (at most 128, in chunks of 32), with the indices of their first
-// 64-wide chi chunk and 32-wide phi chunk in the chunked point-major tables.
+// One unit of the tensor-core density: a chunk of a tile's chi slots (at most two blocks of 64 on a
+// whole tile, four on half a tile) and of its phi slots (at most 64, in chunks of 32), with the
+// indices of their first 64-wide chi chunk and 32-wide phi chunk in the chunked point-major tables.
 struct DUnit {
-    int t;        // grid tile
-    int c0, nc;   // first chi slot, count
-    int p0, np;   // first phi slot, count
-    int cch;      // first chi chunk
-    int pch;      // first phi chunk
-    int pad;
+    enum { FIRST = 1, LAST = 2 };
+    int t;         // grid tile
+    int c0, nc;    // first chi slot, count
+    int p0, np;    // first phi slot, count
+    int cch;       // first chi chunk
+    int pch;       // first phi chunk
+    int chi_use;   // FIRST / LAST unit of a run with the same chi chunk
+};
+
+// One item: 128 nmh points (nmh 4 or 2) of tile t from its point point0 on, and its units
+struct DItem {
+    int t, point0, nmh, u0, u1;
+};
+
+// the density's items and units (device arrays)
+struct DUnitList {
+    const DItem *items = nullptr;
+    const DUnit *units = nullptr;
+    int nitems = 0;
+    bool covers = false;      // every tile of the grid has both chi and phi
+    bool phi32 = false;       // phi in float32 instead of float16 (at most 32 per unit)
+    bool adds = false;        // units add to rho (float32 reductions, in their order) instead of carrying a sum
+    bool chunked = false;     // a point's sum over phi in dot products of 32, else one running sum
 };
 
 struct GridShape {
