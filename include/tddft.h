@@ -256,7 +256,9 @@ tddft_status tddft_fxc(tddft_ctx *ctx, double *fxc);
  * pseudo-random P and V), every candidate cut of the grid work into tensor-core units:
  *   response_density: the per-tile kernels (kind 0, when every tile fits them) and units of at
  *     most chi_chunk x phi_chunk functions of a tile (kind 1; chi 128 or 256, phi 32 or 64);
- *   potential_integrals: units of at most chi_chunk (128, 256, 384) x phi_chunk (32, 64, 128).
+ *   potential_integrals: chunks of at most 128 chi x phi_chunk (32, 48) where every tile's phi
+ *     list is whole aligned quads, else units of at most chi_chunk (128, 256, 384) x phi_chunk
+ *     (32, 64, 128).
  * Each candidate runs once to warm up and three times timed with CUDA events on the context's
  * stream (ms = the mean). The fastest of each stage is installed and kept by the context for all
  * later calls (chosen = 1). out receives up to cap entries, count the number of candidates.
@@ -500,8 +502,9 @@ tddft_status tddft_work(const tddft_ctx *ctx, double *pair_points, double *table
  *   TDDFT_DENSITY_UNITS=1          the density units even with TDDFT_NO_PERSISTENT_DENSITY=1
  *   TDDFT_INTEGRALS_CHUNK=nc,np    largest chi / phi slot counts of one tensor-core integrals
  *                                  unit (multiples of 128 up to 384, and of 16 up to 128;
- *                                  default 384,128); smaller values cut tiles that would fit,
- *                                  which tests the cut on small systems */
+ *                                  default 384,128; at most 128,48 are used where phi lists are
+ *                                  whole quads); smaller values cut tiles that would fit, which
+ *                                  tests the cut on small systems */
 
 #ifdef __cplusplus
 }

@@ -251,7 +251,8 @@ struct Impl {
     unsigned short *phi_pm = nullptr;     // point-major f16 phi tables [tile][512][NPmax], zero padded
     // density units with chunked point-major f16 tables ([chunk][512][64] chi, [chunk][512][32] phi)
     bool dens_units = false;              // the density runs on units (selected)
-    bool units_ok = false;                // chunked tables built (every tile's phi in whole quads)
+    bool quads_ok = false;                // every tile's phi in whole aligned quads
+    bool units_ok = false;                // chunked tables built
     unsigned short *chi_pmc = nullptr, *phi_pmc = nullptr;
     long long nchunks_chi = 0;
     DUnitList dunits;
@@ -265,6 +266,10 @@ struct Impl {
     // integrals launches: units (tiles, or chunks of dense tiles) grouped by 128-row chi blocks
     VTile *int_units = nullptr;
     int int_count[3] = {0, 0, 0};
+    // integrals on units (phi lists of whole aligned quads): items and most phi of a chunk
+    bool int_quads = false;
+    IItem *int_items = nullptr;
+    int nint_items = 0, int_pch = 48;
     unsigned *tc_bits = nullptr;
     float *tc_scale = nullptr;
     // operator workspace, sized for up to `cap` grid states
@@ -352,6 +357,10 @@ void response_density_units(cudaStream_t st, const GridShape &g, const TileSet<f
                             const unsigned short *chi_pmc, long long nchunks_chi, const unsigned short *phi_pmc,
                             const DUnitList &ul, int nchi, int nphi, const float *P, long long sP, int k, float *rho,
                             unsigned short *P16, unsigned *bits, float *scale, int *err);
+void potential_integrals_units(cudaStream_t st, const GridShape &g, const TileSet<float> &chi, const TileSet<float> &phi,
+                               const unsigned short *chi_fm16, int nslots, const unsigned short *phi_fm16,
+                               const IItem *list, int nlist, int pch, int nchi, int nphi, const float *V, int k,
+                               float *quads, float *out, unsigned *bits, int *err);
 int noalloc_max_states();
 void response_density_tc_noalloc(cudaStream_t st, const GridShape &g, const TileSet<float> &chi,
                                  const TileSet<float> &phi, const unsigned short *chi_pm, int CK, int NPmax,
@@ -712,9 +721,17 @@ template <typename T>
 void integrals(tddft_ctx *c, Impl<T> &I, int ns) {
     // sparse form: the dense integrals into the scratch, then T(V) into the cluster blocks
     T *out = c->sparse ? I.dense : I.Vmat;
-    bool done = false;
+    bool done = false, quads = false;
     if constexpr (sizeof(T) == 4) {
-        if (I.integrals_tc) {
+        if (I.int_quads) {
+            // summed in quads: into the sparse form's scratch, which its blocks are read from, or into the
+            // product buffer that is free here, and from there in row order
+            quads = c->sparse;
+            potential_integrals_units(c->st, c->grid(), I.chi, I.phi, I.chi_fm16, I.nslots_chi, I.phi_fm16, I.int_items,
+                                      I.nint_items, I.int_pch, c->nc, c->nv, I.V, ns, quads ? out : I.tmp,
+                                      quads ? nullptr : out, I.tc_bits, tc_error_word());
+            done = true;
+        } else if (I.integrals_tc) {
             potential_integrals_tc(c->st, c->grid(), I.chi, I.phi, I.chi_fm16, I.nslots_chi, I.phi_fm16, I.nslots_phi,
                                    I.NPint, I.maxc, c->nc,
                                    c->nv, I.V, ns, out, I.tc_bits, I.tc_scale, I.int_units, I.int_count,
@@ -723,7 +740,7 @@ void integrals(tddft_ctx *c, Impl<T> &I, int ns) {
         }
     }
     if (!done) potential_integrals<T>(c->st, c->grid(), I.chi, I.phi, c->nc, c->nv, I.V, ns, out);
-    if (c->sparse) cb_from_dense<T>(c->st, *c->sp, I.dense, I.Vmat, I.mask, ns);
+    if (c->sparse) cb_from_dense<T>(c->st, *c->sp, I.dense, I.Vmat, I.mask, ns, quads);
 }
 
 // ---- products with the constants -------------------------------------------------------------------
@@ -971,12 +988,10 @@ int projector_basis(cudaStream_t st, Mem &tmp, const double *Sh, const double *P
 }
 
 // ---- tensor-core units of the grid kernels (the cuts are what the autotuner varies) -------------
-// chunked point-major f16 tables of both sets for the density units; false unless every tile's
-// phi list is whole aligned atom quads
-bool build_density_chunks(tddft_ctx *c, Impl<float> &I) {
-    if (I.units_ok) return true;
-    const int ntl = I.chi.ntiles;
-    const std::vector<int> &coff = I.coff_h, &poff = I.poff_h;
+// every tile's phi list is whole aligned quads: four consecutive functions, the first a multiple of 4
+bool phi_lists_in_quads(const Impl<float> &I) {
+    const int ntl = I.phi.ntiles;
+    const std::vector<int> &poff = I.poff_h;
     std::vector<int> pids(poff[ntl]);
     if (!pids.empty())
         check(cudaMemcpy(pids.data(), I.phi.ids, pids.size() * sizeof(int), cudaMemcpyDeviceToHost), "D2H phi ids");
@@ -988,6 +1003,14 @@ bool build_density_chunks(tddft_ctx *c, Impl<float> &I) {
                   pids[p0 + q + 3] == pids[p0 + q] + 3))
                 return false;
     }
+    return true;
+}
+
+// chunked point-major f16 tables of both sets for the density units (phi lists in quads)
+bool build_density_chunks(tddft_ctx *c, Impl<float> &I) {
+    if (I.units_ok) return true;
+    if (!I.quads_ok) return false;
+    const std::vector<int> &coff = I.coff_h, &poff = I.poff_h;
     I.nchunks_chi = build_chunked_pm(c->st, I.mem, I.chi, coff, 64, &I.chi_pmc, I.cfirst_h);
     build_chunked_pm(c->st, I.mem, I.phi, poff, 32, &I.phi_pmc, I.pfirst_h);
     I.units_ok = true;
@@ -1048,6 +1071,29 @@ void set_density_units(Impl<float> &I, int cch, int pch) {
     }
     L.units = du;
     L.items = di;
+}
+
+// the integrals' items: each tile in chunks of 128 chi with all its phi, which the kernel takes in
+// chunks of at most pch (a multiple of 16, <= 48); in order of falling work, so that the persistent
+// blocks finish together
+void set_integrals_items(Impl<float> &I, int pch) {
+    const int ntl = I.chi.ntiles;
+    const std::vector<int> &coff = I.coff_h, &poff = I.poff_h;
+    std::vector<IItem> items;
+    for (int t = 0; t < ntl; ++t) {
+        const int nct = coff[t + 1] - coff[t], npt = poff[t + 1] - poff[t];
+        if (nct == 0 || npt == 0) continue;
+        for (int cc = 0; cc < nct; cc += 128)
+            items.push_back(IItem{t, coff[t] + cc, std::min(128, nct - cc), poff[t], npt});
+    }
+    std::stable_sort(items.begin(), items.end(), [](const IItem &a, const IItem &b) { return a.np > b.np; });
+    I.umem_int.release();
+    I.int_items = I.umem_int.alloc<IItem>(items.size());
+    if (!items.empty())
+        check(cudaMemcpy(I.int_items, items.data(), items.size() * sizeof(IItem), cudaMemcpyHostToDevice),
+              "upload integrals items");
+    I.nint_items = (int)items.size();
+    I.int_pch = pch;
 }
 
 // the integrals' units: chunks of at most cch chi (a multiple of 128, <= 384) and pch phi (a
@@ -1131,6 +1177,9 @@ void build_impl(tddft_ctx *c, const tddft_system *s, const tddft_sparse_system *
                           "D2H phi tables");
                 }
             };
+            I->coff_h = coff;
+            I->poff_h = poff;
+            I->quads_ok = c->nv % 4 == 0 && phi_lists_in_quads(*I);
             if (NP <= 256 && density_tc_group(CK / 64, NP, 1) >= 1) {
                 fetch_tables();
                 std::vector<unsigned short> pm((size_t)ntl * TILE_PTS * CK, 0);
@@ -1150,25 +1199,9 @@ void build_impl(tddft_ctx *c, const tddft_system *s, const tddft_sparse_system *
                 }
                 I->NPmax = NP;
                 I->grid_tc = true;
-                {
-                    // whole aligned phi quads in every tile (4 functions per atom, grouped by atom)
-                    std::vector<int> pids(poff[ntl]);
-                    check(cudaMemcpy(pids.data(), I->phi.ids, pids.size() * sizeof(int), cudaMemcpyDeviceToHost),
-                          "D2H phi ids");
-                    bool ok = c->nv % 4 == 0 && NP % 4 == 0;
-                    for (int t = 0; t < ntl && ok; ++t) {
-                        const int p0 = poff[t], np = poff[t + 1] - p0;
-                        if (np % 4) ok = false;
-                        for (int q = 0; q + 3 < np && ok; q += 4)
-                            ok = pids[p0 + q] % 4 == 0 && pids[p0 + q + 1] == pids[p0 + q] + 1 &&
-                                 pids[p0 + q + 2] == pids[p0 + q] + 2 && pids[p0 + q + 3] == pids[p0 + q] + 3;
-                    }
-                    const char *nq = std::getenv("TDDFT_NO_QUAD_GATHER");
-                    I->phi_quads = ok && !(nq && nq[0] == '1');
-                }
+                const char *nq = std::getenv("TDDFT_NO_QUAD_GATHER");
+                I->phi_quads = I->quads_ok && !(nq && nq[0] == '1');
             }
-            I->coff_h = coff;
-            I->poff_h = poff;
             // the density on units wherever every tile's phi list is whole aligned quads: faster
             // there at every size measured (20 to 200 atoms, figures in density_units.cu);
             // the per-tile kernel for other lists, and for TDDFT_NO_PERSISTENT_DENSITY=1 where it
@@ -1178,7 +1211,8 @@ void build_impl(tddft_ctx *c, const tddft_system *s, const tddft_sparse_system *
                 const char *nu = std::getenv("TDDFT_NO_DENSITY_UNITS");
                 const char *fu = std::getenv("TDDFT_DENSITY_UNITS");
                 const char *np = std::getenv("TDDFT_NO_PERSISTENT_DENSITY");
-                const bool per_tile = I->grid_tc && np && np[0] == '1' && !(fu && fu[0] == '1');
+                const char *eg = std::getenv("TDDFT_NO_QUAD_GATHER");
+                const bool per_tile = I->grid_tc && ((np && np[0] == '1') || (eg && eg[0] == '1')) && !(fu && fu[0] == '1');
                 // the arithmetic of the epilogue by the longest lists: phi in float32 where a tile's
                 // phi fill no whole float16 rows of 32, sums by 32 phi past the lists of 128 phi or 320 chi
                 I->dunits.adds = !I->grid_tc;
@@ -1202,7 +1236,13 @@ void build_impl(tddft_ctx *c, const tddft_system *s, const tddft_sparse_system *
                         pch = b;
                     }
                 }
-                if (set_integrals_units(*I, cch, pch)) {
+                // lists in quads take the items kernel (faster at every size measured, figures in
+                // integrals_units.cu), other lists the units
+                if (I->quads_ok) {
+                    set_integrals_items(*I, std::min(pch, 48));
+                    I->int_quads = true;
+                }
+                if (I->int_quads || set_integrals_units(*I, cch, pch)) {
                     // function-major f16 copies of both tables, rounded on the device (the f16 phi
                     // rows are the integrals' B operand, TMA-loaded and scaled by V in place)
                     const long long nch = (long long)coff[ntl] * TILE_PTS, nph = (long long)poff[ntl] * TILE_PTS;
@@ -2741,8 +2781,18 @@ tddft_status tddft_autotune(tddft_ctx *c, int32_t k, tddft_tuning_entry *out, in
             const int cuts[][2] = {{384, 128}, {256, 128}, {128, 128}, {384, 64}, {256, 64}, {128, 64}, {384, 32}};
             int best = -1;
             double best_ms = 1e300;
+            if (I.int_quads) {
+                for (const int pch : {48, 32}) {
+                    set_integrals_items(I, pch);
+                    add("potential_integrals", 1, 128, pch, time_it([&]() { integrals(c, I, k); }));
+                    if (rows.back().ms < best_ms) {
+                        best_ms = rows.back().ms;
+                        best = (int)rows.size() - 1;
+                    }
+                }
+            }
             for (const auto &cut : cuts) {
-                if (!set_integrals_units(I, cut[0], cut[1])) continue;
+                if (I.int_quads || !set_integrals_units(I, cut[0], cut[1])) continue;
                 add("potential_integrals", 1, cut[0], cut[1], time_it([&]() { integrals(c, I, k); }));
                 if (rows.back().ms < best_ms) {
                     best_ms = rows.back().ms;
@@ -2751,7 +2801,8 @@ tddft_status tddft_autotune(tddft_ctx *c, int32_t k, tddft_tuning_entry *out, in
             }
             if (best >= 0) {
                 rows[best].chosen = 1;
-                set_integrals_units(I, rows[best].chi_chunk, rows[best].phi_chunk);
+                if (I.int_quads) set_integrals_items(I, rows[best].phi_chunk);
+                else set_integrals_units(I, rows[best].chi_chunk, rows[best].phi_chunk);
             }
         }
         check_tc_error(c);

@@ -196,14 +196,15 @@ __global__ void cb_to_dense_kernel(LayoutView v, const T *__restrict__ src, T *_
 
 template <typename T>
 __global__ void cb_from_dense_kernel(LayoutView v, const T *__restrict__ src, T *__restrict__ dst,
-                                     const T *__restrict__ mask, int k) {
+                                     const T *__restrict__ mask, int k, bool quads) {
     const long long tot = v.len * k;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
         const long long b = e / v.len, q = e - b * v.len;
         const long long blk = q / CB_SIZE;
         const int w = (int)(q - blk * CB_SIZE), r = w / CB_C, c = w - r * CB_C;
         const int f = v.rowfun[v.blk_row[blk] * CB_R + r], g = v.colfun[v.blk_col[blk] * CB_C + c];
-        dst[e] = (f >= 0 && g >= 0) ? mask[q] * src[b * (long long)v.nc * v.nv + (long long)f * v.nv + g] : T(0);
+        const long long at = quads ? ((long long)(g >> 2) * v.nc + f) * 4 + (g & 3) : (long long)f * v.nv + g;
+        dst[e] = (f >= 0 && g >= 0) ? mask[q] * src[b * (long long)v.nc * v.nv + at] : T(0);
     }
 }
 
@@ -504,8 +505,8 @@ void cb_to_dense(cudaStream_t st, const SparseLayout &L, const T *src, T *dst, i
     check_launch("cb_to_dense_kernel");
 }
 template <typename T>
-void cb_from_dense(cudaStream_t st, const SparseLayout &L, const T *src, T *dst, const T *mask, int k) {
-    cb_from_dense_kernel<T><<<grid_for(L.len() * k), 256, 0, st>>>(view(L), src, dst, mask, k);
+void cb_from_dense(cudaStream_t st, const SparseLayout &L, const T *src, T *dst, const T *mask, int k, bool quads) {
+    cb_from_dense_kernel<T><<<grid_for(L.len() * k), 256, 0, st>>>(view(L), src, dst, mask, k, quads);
     check_launch("cb_from_dense_kernel");
 }
 template <typename T>
@@ -521,7 +522,7 @@ void cb_mask(cudaStream_t st, const SparseLayout &L, T *mask) {
     template void cb_from_abi<T>(cudaStream_t, const SparseLayout &, const double *, T *, int);                  \
     template void cb_to_abi<T>(cudaStream_t, const SparseLayout &, const T *, double *, int);                    \
     template void cb_to_dense<T>(cudaStream_t, const SparseLayout &, const T *, T *, int);                       \
-    template void cb_from_dense<T>(cudaStream_t, const SparseLayout &, const T *, T *, const T *, int);          \
+    template void cb_from_dense<T>(cudaStream_t, const SparseLayout &, const T *, T *, const T *, int, bool);    \
     template void cb_mask<T>(cudaStream_t, const SparseLayout &, T *);
 INST(float)
 INST(double)

@@ -109,8 +109,10 @@ template <typename T>
 void cb_to_abi(cudaStream_t st, const SparseLayout &L, const T *src, double *dst, int k);
 template <typename T>
 void cb_to_dense(cudaStream_t st, const SparseLayout &L, const T *src, T *dst, int k);
+// quads: src is laid out [k][nv / 4][nc][4] instead of [k][nc][nv]
 template <typename T>
-void cb_from_dense(cudaStream_t st, const SparseLayout &L, const T *src, T *dst, const T *mask, int k);
+void cb_from_dense(cudaStream_t st, const SparseLayout &L, const T *src, T *dst, const T *mask, int k,
+                   bool quads = false);
 // the 0/1 kernel-pattern mask in the cluster-block layout
 template <typename T>
 void cb_mask(cudaStream_t st, const SparseLayout &L, T *mask);

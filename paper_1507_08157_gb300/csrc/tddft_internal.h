@@ -120,6 +120,11 @@ struct DUnitList {
     bool chunked = false;     // a point's sum over phi in dot products of 32, else one running sum
 };
 
+// One item of the tensor-core integrals on units: at most 128 chi slots of a tile, all its phi slots
+struct IItem {
+    int t, c0, nc, p0, np;
+};
+
 struct GridShape {
     int n;          // points per side
     int nt;         // tiles per side = ceil(n / 8)
