@@ -41,7 +41,7 @@ typedef enum {
     TDDFT_E_BREAKDOWN = 5,      /* NaN/Inf, or a non-positive norm in Gram-Schmidt */
     TDDFT_E_TIMEOUT = 6,        /* a bounded wait inside a tensor-core kernel expired (limit:
                                    tddft_options.spin_limit_cycles). Any call that runs the
-                                   tensor-core products or grid kernels of a TDDFT_MIXED context
+                                   tensor-core products or grid kernels of a context
                                    (apply, the component entry points, state_create, pcg_step,
                                    solve, oscillator_strengths, the allocation-free density) and
                                    tddft_wait_check can return it; the kernel gives up, lets its
@@ -130,7 +130,9 @@ typedef struct {
 } tddft_sparse_system;
 
 typedef struct {
-    int32_t precision;        /* TDDFT_FP64: all arithmetic in float64.
+    int32_t precision;        /* TDDFT_FP64: all arithmetic in float64, the grid contractions by
+                                 exact splitting of float64 values on the tensor cores (their
+                                 rounding error is that of float64 sums or below).
                                  TDDFT_MIXED: matrices, grids and FFTs in float32; traces,
                                  line search, Gram-Schmidt, eigenvalues in float64 */
     int32_t mode;             /* TDDFT_MODE_FULL (Eq. operator_RPA); TDDFT_MODE_TDA (B = 0:

@@ -11,7 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIBDIR = os.path.join(HERE, "lib")
 LIB = os.path.join(LIBDIR, "libtddft.so")
-SOURCES = ["api.cu", "bsr_tc.cu", "density_units.cu", "gemm.cu", "grid.cu", "grid_tc.cu", "integrals_units.cu", "learned.cu", "solver_kernels.cu", "sparse.cu",
+SOURCES = ["api.cu", "bsr_tc.cu", "density_units.cu", "fp64_grid.cu", "gemm.cu", "grid.cu", "grid_tc.cu", "integrals_units.cu", "learned.cu", "solver_kernels.cu", "sparse.cu",
            "spectrum.cu", "profile.cu", "tc_gemm.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -268,6 +268,10 @@ struct Impl {
     int int_count[3] = {0, 0, 0};
     // integrals on units (phi lists of whole aligned quads): items and most phi of a chunk
     bool int_quads = false;
+    // float64 contexts: grid contractions by exact splitting on the tensor cores
+    Fp64Grid g64;
+    bool int64_tc = false, dens64_tc = false;
+    unsigned long long *bits64 = nullptr;
     IItem *int_items = nullptr;
     int nint_items = 0, int_pch = 48;
     unsigned *tc_bits = nullptr;
@@ -361,6 +365,14 @@ void potential_integrals_units(cudaStream_t st, const GridShape &g, const TileSe
                                const unsigned short *chi_fm16, int nslots, const unsigned short *phi_fm16,
                                const IItem *list, int nlist, int pch, int nchi, int nphi, const float *V, int k,
                                float *quads, float *out, unsigned *bits, int *err);
+bool fp64_grid_build(cudaStream_t st, Mem &mem, const TileSet<double> &chi, const TileSet<double> &phi,
+                     const std::vector<int> &coff, const std::vector<int> &poff, bool quads, Fp64Grid &G);
+void response_density_fp64(cudaStream_t st, const GridShape &g, const TileSet<double> &chi, const TileSet<double> &phi,
+                           const Fp64Grid &G, int nphi, const double *P, long long sP, int k, double *rho,
+                           unsigned long long *bits, int *err);
+void potential_integrals_fp64(cudaStream_t st, const GridShape &g, const TileSet<double> &chi, const TileSet<double> &phi,
+                              const Fp64Grid &G, int nchi, int nphi, const double *V, int k, double *out,
+                              unsigned long long *bits, int *err);
 int noalloc_max_states();
 void response_density_tc_noalloc(cudaStream_t st, const GridShape &g, const TileSet<float> &chi,
                                  const TileSet<float> &phi, const unsigned short *chi_pm, int CK, int NPmax,
@@ -679,6 +691,7 @@ void ensure_workspace(tddft_ctx *c, Impl<T> &I, int states) {
         (size_t)std::max({states * len, states * n3, states * c->nnz_abi()}));
     I.tc_bits = I.wmem.template alloc<unsigned>((size_t)states);
     I.tc_scale = I.wmem.template alloc<float>((size_t)2 * states);
+    I.bits64 = I.wmem.template alloc<unsigned long long>((size_t)states);
     if (c->sparse) {
         // the grid kernels address P and V densely; the tensor-core left products take their
         // right operand block-transposed
@@ -714,6 +727,13 @@ void density(tddft_ctx *c, Impl<T> &I, const T *P, int ns) {
             return;
         }
     }
+    if constexpr (sizeof(T) == 8) {
+        if (I.dens64_tc) {
+            response_density_fp64(c->st, c->grid(), I.chi, I.phi, I.g64, c->nv, P, (long long)c->nc * c->nv, ns, I.rho,
+                                  I.bits64, tc_error_word());
+            return;
+        }
+    }
     response_density<T>(c->st, c->grid(), I.chi, I.phi, c->nv, P, (long long)c->nc * c->nv, ns, I.rho);
 }
 
@@ -736,6 +756,13 @@ void integrals(tddft_ctx *c, Impl<T> &I, int ns) {
                                    I.NPint, I.maxc, c->nc,
                                    c->nv, I.V, ns, out, I.tc_bits, I.tc_scale, I.int_units, I.int_count,
                                    tc_error_word());
+            done = true;
+        }
+    }
+    if constexpr (sizeof(T) == 8) {
+        if (I.int64_tc) {
+            potential_integrals_fp64(c->st, c->grid(), I.chi, I.phi, I.g64, c->nc, c->nv, I.V, ns, out, I.bits64,
+                                     tc_error_word());
             done = true;
         }
     }
@@ -989,7 +1016,8 @@ int projector_basis(cudaStream_t st, Mem &tmp, const double *Sh, const double *P
 
 // ---- tensor-core units of the grid kernels (the cuts are what the autotuner varies) -------------
 // every tile's phi list is whole aligned quads: four consecutive functions, the first a multiple of 4
-bool phi_lists_in_quads(const Impl<float> &I) {
+template <typename T>
+bool phi_lists_in_quads(const Impl<T> &I) {
     const int ntl = I.phi.ntiles;
     const std::vector<int> &poff = I.poff_h;
     std::vector<int> pids(poff[ntl]);
@@ -1255,6 +1283,21 @@ void build_impl(tddft_ctx *c, const tddft_system *s, const tddft_sparse_system *
                     I->integrals_tc = true;
                 }
             }
+        }
+    }
+    if constexpr (sizeof(T) == 8) {
+        // float64: the splitting kernels (faster at every size measured, figures in fp64_grid.cu); the
+        // density's where its gather finds whole aligned quads
+        const char *ng = std::getenv("TDDFT_NO_GRID_TC");
+        if (tc_enabled() && !(ng && ng[0] == '1')) {
+            const int ntl = I->chi.ntiles;
+            I->coff_h.resize(ntl + 1);
+            I->poff_h.resize(ntl + 1);
+            check(cudaMemcpy(I->coff_h.data(), I->chi.off, (ntl + 1) * sizeof(int), cudaMemcpyDeviceToHost), "D2H off");
+            check(cudaMemcpy(I->poff_h.data(), I->phi.off, (ntl + 1) * sizeof(int), cudaMemcpyDeviceToHost), "D2H off");
+            I->quads_ok = c->nv % 4 == 0 && phi_lists_in_quads(*I);
+            I->int64_tc = fp64_grid_build(st, I->mem, I->chi, I->phi, I->coff_h, I->poff_h, I->quads_ok, I->g64);
+            I->dens64_tc = I->int64_tc && I->quads_ok;
         }
     }
     double pp = 0.0, tv = 0.0;

@@ -1,0 +1,654 @@
+// Float64 grid contractions on the tensor cores: response density and potential integrals of FP64
+// contexts (Secs. II C, III A) by error-free splitting (Ozaki, Ogita, Oishi and Rump, Numer.
+// Algorithms 59 (2012) 95; on tensor cores: Mukunoki, Ozaki, Ogita and Imamura, ISC 2020).
+//
+// This part executes about two float64 multiply-adds per cycle and SM, and the CUDA-core kernels ran
+// at that rate. Here a value x with |x| < 2^E becomes the integer q = round(x 2^(61 - E)), written
+// in nine balanced digits of seven bits, q = sum_i d_i 128^(8 - i), -64 <= d_i <= 63, each exact in
+// float16. A product sum over K terms is
+//
+//   sum x y = 2^(Ex + Ey - 122) sum_l 128^(16 - l) D_l,     D_l = sum_{i + j = l} sum_K x_i y_j,
+//
+// and each D_l, l <= 8, is an integer below 2^24 (9 pairs x 455 terms x 64 x 64; past that only the
+// lowest level can round, at 2^-80 of the result's range), so the float32 accumulators of
+// kind::f16 hold it exactly. The levels l > 8 and the rounding of q leave an error of 2^-61 of the
+// largest terms, below the 2^-53 that every float64 addition of the sums it replaces made.
+// Scales (powers of two): one per state for P and V. The integrals scale every function's values on a
+// tile by their own maximum there, so that entries of functions that only graze each other keep
+// their relative accuracy; the density, whose sums over chi cannot carry such scales, takes one for
+// the whole chi table. Errors against extended precision (sampled entries, 8 and 24 atoms) of the
+// CUDA-core kernels and of these: density 1.4e-16 and 0.8e-16, 2.5e-16 and 1.2e-16; integrals
+// 4.1e-16 and 0.9e-16, 7.2e-16 and 1.2e-16.
+//
+// The digits of B are stacked along N (32 columns each), the accumulators of the levels along the
+// columns of TMEM (32 each): for digit i of A one MMA of N = 32 (9 - i) columns, placed at level i,
+// makes all its products with the digits j <= 8 - i of B. Nine MMAs (the first cut in two at 256
+// columns) per 16 of K instead of 45.
+//
+// Both kernels: 320 threads; warp 8 brings the digit tiles of chi (128 x 64, 16 KB) through a ring by
+// TMA from tables made at creation, eight warps make the digits of B for the next K block while
+// warp 9 issues the MMAs of this one, then combine the levels in integers and float64. Every wait is
+// bounded.
+// Measured (GB300, stage, CUDA events, CUDA-core kernel and this): 8 atoms, 48^3, 1 state: density 0.57
+// and 0.10 ms, integrals 1.05 and 0.08; 32 atoms with 4 + 9 functions, 90^3, 3 states: density 19.3 and
+// 1.09 ms, integrals 21.2 and 0.91. Bound by the issue and shared-memory reads of the MMAs (A is read
+// once per digit: 45 digit products in 10 MMAs) and, in small systems, by a block's start and end.
+#include "tc_common.cuh"
+#include "tddft_internal.h"
+
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <type_traits>
+
+namespace tddft {
+
+using namespace tc;
+
+bool encode_map_2d(CUtensorMap *map, CUtensorMapDataType dt, const void *ptr, unsigned long long inner,
+                   unsigned long long rows, unsigned long long row_bytes, unsigned box_inner, unsigned box_rows);
+
+namespace {
+
+constexpr int ND = 9;                // digits, and levels kept
+constexpr int SHIFT = 61;            // |q| < 2^61
+constexpr int NB = 32;               // B columns of one digit
+constexpr int THREADS64 = 320;       // warps 0-7 make B and combine, 8 TMA, 9 MMA
+constexpr int A_RING = 8, A_TILE = 16384;
+constexpr int B_KMAJ = ND * NB * 128;           // integrals: rows (digit, phi) of 64 points
+constexpr int B_NMAJ = (ND + 1) / 2 * 8192;     // density: blocks of 64 columns (two digits) x 64 chi
+constexpr int MAX_K = 448;           // chi summed in one accumulator
+
+struct __align__(8) Shared64 {
+    unsigned long long a_full[A_RING], a_empty[A_RING];
+    unsigned long long b_full[2], b_empty[2];
+    unsigned long long acc_full, acc_empty, drain;
+    unsigned int tmem_base;
+    int abort;
+    double part[128];                // density: the second half's sums
+};
+
+__device__ __forceinline__ void init64(Shared64 *c) {
+    for (int i = 0; i < A_RING; ++i) {
+        mbar_init(&c->a_full[i], 1);
+        mbar_init(&c->a_empty[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+        mbar_init(&c->b_full[i], 8);
+        mbar_init(&c->b_empty[i], 1);
+    }
+    mbar_init(&c->acc_full, 1);
+    mbar_init(&c->acc_empty, 8);
+    mbar_init(&c->drain, 1);
+    c->abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+// exponent E with max < 2^E from the bits of max |x| (clamped so that 2^(61 - E) is finite)
+__device__ __forceinline__ int exponent_of(unsigned long long bits) {
+    int e = 0;
+    frexp(__longlong_as_double((long long)bits), &e);
+    return max(e, -900);
+}
+__device__ __forceinline__ double pow2(int e) { return ldexp(1.0, e); }
+// a state's values are all finite
+__device__ __forceinline__ bool finite_bits(unsigned long long bits) {
+    return isfinite(__longlong_as_double((long long)bits));
+}
+
+// q + sum_i 64 128^i: the digits plus 64, seven bits each
+__device__ __forceinline__ unsigned long long biased(double scaled) {
+    constexpr unsigned long long C = 0x2040810204081020ull << 1;   // 64 (1 + 128 + ... + 128^8)
+    return (unsigned long long)__double2ll_rn(scaled) + C;
+}
+// two digits (plus 64) as float16 pair: 1024 + d is exact, then 1088 is taken off
+__device__ __forceinline__ unsigned digit_pair(unsigned a, unsigned b) {
+    const unsigned v = 0x64006400u | a | (b << 16);
+    const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&v), __half2half2(__ushort_as_half(0x6440)));
+    return *reinterpret_cast<const unsigned *>(&h);
+}
+__device__ __forceinline__ unsigned digit(unsigned long long u, int j) { return (unsigned)(u >> (7 * (ND - 1 - j))) & 127u; }
+
+// an integer below 2^51 in size as float64 with one addition
+__device__ __forceinline__ double to_double(long long v) {
+    return __longlong_as_double(0x4330000000000000ll + (1ll << 51) + v) - 6755399441055744.0;
+}
+// sum_l 128^(8 - l) D_l of the nine level sums (float32 integers)
+__device__ __forceinline__ double combine_levels(const float (*D)[8], int e) {
+    long long hi = 0, lo = 0;
+#pragma unroll
+    for (int l = 0; l < 4; ++l) hi = hi * 128 + (int)__float2int_rn(D[l][e]);
+#pragma unroll
+    for (int l = 4; l < 8; ++l) lo = lo * 128 + (int)__float2int_rn(D[l][e]);
+    // level 8 stays apart: with it lo could reach 2^52
+    return fma(to_double(hi), 34359738368.0, fma(to_double(lo), 128.0, (double)D[8][e]));
+}
+
+__device__ __forceinline__ void tmem_ld8(unsigned taddr, float *v) {
+    unsigned r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+                 " tcgen05.wait::ld.sync.aligned;"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// The MMAs of one K block of 64: the nine digit tiles of A against B (descriptor low words b + kk bk).
+// bx: distance to digit 8 of B. False after an expired wait.
+__device__ __forceinline__ bool mma_block(Shared64 *ctl, volatile int *abort, unsigned a_lo, unsigned &qa, unsigned tmem,
+                                          unsigned b, unsigned bk, unsigned bx, unsigned idesc_flags, bool first,
+                                          long long wlim) {
+    for (int i = 0; i < ND; ++i, ++qa) {
+        const unsigned st = qa % A_RING;
+        if (!mbar_wait(&ctl->a_full[st], (qa / A_RING) & 1, abort, wlim)) return false;
+        tc_fence_after();
+        const unsigned a = a_lo + st * (A_TILE >> 4);
+        const unsigned idesc = idesc_f16(128, min(256, NB * (ND - i))) | idesc_flags;
+#pragma unroll
+        for (unsigned kk = 0; kk < 4; ++kk) {
+            const unsigned acc = (first && i == 0 && kk == 0) ? 0u : 1u;
+            mma_f16(tmem + i * NB, desc_of(a + 2 * kk), desc_of(b + kk * bk), idesc, acc);
+            if (i == 0)   // digit 8 of B, level 8
+                mma_f16(tmem + 8 * NB, desc_of(a + 2 * kk), desc_of(b + bx + kk * bk), idesc_f16(128, NB) | idesc_flags, acc);
+        }
+        mma_commit(&ctl->a_empty[st]);
+    }
+    return true;
+}
+
+// ---- potential integrals: D[a][b] = sum_r chi_a(r) (V_s phi_b)(r) --------------------------------------
+// Block = (item, state): at most 128 chi and 32 phi of a tile, K = its 512 points.
+__global__ void __launch_bounds__(THREADS64, 1) integrals64_kernel(
+    const __grid_constant__ CUtensorMap mX,   // chi digits [digit * slots + slot][512], box 64 x 128
+    int n, int nt, int k, const IItem *__restrict__ items, long long slots, const int *__restrict__ cids,
+    const int *__restrict__ pids, const double *__restrict__ pval, const int *__restrict__ cexp,
+    const int *__restrict__ pexp, int nchi, int nphi, const double *__restrict__ V,
+    const unsigned long long *__restrict__ vbits, double dV, double *__restrict__ out, int *err, long long wlim) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *base = reinterpret_cast<unsigned char *>(
+        (reinterpret_cast<unsigned long long>(smem_raw) + 1023ull) & ~1023ull);
+    unsigned char *A = base, *B = base + A_RING * A_TILE;
+    double *Vt = reinterpret_cast<double *>(B + 2 * B_KMAJ);
+    Shared64 *ctl = reinterpret_cast<Shared64 *>(Vt + TILE_PTS);
+    volatile int *abort = &ctl->abort;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int s = blockIdx.x % k;
+    const IItem d = items[blockIdx.x / k];
+    const long long n3 = (long long)n * n * n;
+    if (threadIdx.x == 0) init64(ctl);
+    if (warp == 9) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
+                     "r"(512));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    // V on the tile, scaled so that the products with scaled phi become q
+    const int ev = exponent_of(vbits[s]);
+    const double vs = pow2(SHIFT - ev);
+    const int tx = d.t / (nt * nt), ty = (d.t / nt) % nt, tz = d.t % nt;
+    for (int lp = threadIdx.x; lp < TILE_PTS; lp += THREADS64) {
+        const int gx = tx * TILE + (lp >> 6), gy = ty * TILE + ((lp >> 3) & 7), gz = tz * TILE + (lp & 7);
+        Vt[lp] = (gx < n && gy < n && gz < n) ? V[(long long)s * n3 + ((long long)gx * n + gy) * n + gz] * vs : 0.0;
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const unsigned tmem = ctl->tmem_base;
+    constexpr int KB = TILE_PTS / 64;
+
+    if (warp == 8) {
+        if (lane == 0) {
+            unsigned q = 0;
+            for (; q < KB * ND; ++q) {
+                const unsigned st = q % A_RING;
+                if (q >= A_RING && !mbar_wait(&ctl->a_empty[st], (q / A_RING - 1) & 1, abort, wlim)) break;
+                mbar_expect_tx(&ctl->a_full[st], A_TILE);
+                tma_load_2d(A + st * A_TILE, &mX, &ctl->a_full[st], (int)(q / ND) * 64, (int)((q % ND) * slots + d.c0));
+            }
+            // after an abort, the loads already issued land before the block exits
+            if (*abort)
+                for (unsigned i = q > A_RING ? q - A_RING : 0; i < q; ++i)
+                    mbar_drain(&ctl->a_full[i % A_RING], (i / A_RING) & 1, wlim);
+        }
+    } else if (warp == 9) {
+        if (elect_one()) {
+            const unsigned a_lo = desc_lo(smem_u32(A));
+            unsigned qa = 0;
+            bool ok = true;
+            for (unsigned kb = 0; kb < KB && ok; ++kb) {
+                ok = mbar_wait(&ctl->b_full[kb & 1], (kb >> 1) & 1, abort, wlim);
+                if (!ok) break;
+                tc_fence_after();
+                ok = mma_block(ctl, abort, a_lo, qa, tmem, desc_lo(smem_u32(B + (kb & 1) * B_KMAJ)), 2u, (8 * NB * 128) >> 4,
+                               0u, kb == 0, wlim);
+                mma_commit(&ctl->b_empty[kb & 1]);
+            }
+            mma_commit(&ctl->acc_full);
+            if (*abort) {
+                mma_commit(&ctl->drain);
+                mbar_drain(&ctl->drain, 0, wlim);
+            }
+        }
+    } else {
+        // digits of V phi: thread = (phi b, octet o of the K block's points)
+        const int o = threadIdx.x & 7, b = threadIdx.x >> 3;
+        bool ok = true;
+        // phi / 2^E of its slot: the exponent field takes -E (|phi| < 2^E, so no overflow; zero stays zero)
+        const int down = b < d.np ? pexp[d.p0 + b] : 0;
+        auto scaled = [&](double x) {
+            const int hi = __double2hiint(x), ef = (hi >> 20) & 0x7ff;
+            return ef != 0 && ef > down ? __hiloint2double(hi - down * (1 << 20), __double2loint(x)) : 0.0;
+        };
+        for (int kb = 0; kb < KB; ++kb) {
+            unsigned long long u[8];
+            const double2 *pp = reinterpret_cast<const double2 *>(pval + (long long)(d.p0 + b) * TILE_PTS + kb * 64 + o * 8);
+            const double2 *vv = reinterpret_cast<const double2 *>(Vt + kb * 64 + o * 8);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const double2 p = b < d.np ? __ldg(pp + e) : make_double2(0.0, 0.0), v = vv[e];
+                u[2 * e] = biased(scaled(p.x) * v.x);
+                u[2 * e + 1] = biased(scaled(p.y) * v.y);
+            }
+            if (kb >= 2 && !mbar_wait(&ctl->b_empty[kb & 1], ((kb >> 1) - 1) & 1, abort, wlim)) {
+                ok = false;
+                break;
+            }
+            unsigned char *Bk = B + (kb & 1) * B_KMAJ;
+#pragma unroll
+            for (int j = 0; j < ND; ++j) {
+                uint4 x;
+                x.x = digit_pair(digit(u[0], j), digit(u[1], j));
+                x.y = digit_pair(digit(u[2], j), digit(u[3], j));
+                x.z = digit_pair(digit(u[4], j), digit(u[5], j));
+                x.w = digit_pair(digit(u[6], j), digit(u[7], j));
+                *reinterpret_cast<uint4 *>(Bk + sw128_offset(j * NB + b, o)) = x;
+            }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->b_full[kb & 1]);
+        }
+        ok = ok && mbar_wait(&ctl->acc_full, 0, abort, wlim) && !*abort;
+        tc_fence_after();
+        // rows of chi over warps 0-3 and 4-7, the phi halves between the two groups. x w is
+        // 2^(56 - (61 - ec) - (61 - ep - ev)) times the combined levels
+        const int a = (warp & 3) * 32 + lane;
+        const double f = finite_bits(vbits[s]) ? ldexp(dV, 56 - 2 * SHIFT + ev + (a < d.nc ? cexp[d.c0 + a] : 0))
+                                               : __longlong_as_double(0x7ff8000000000000ll);
+        double *o_row = out + (long long)s * nchi * nphi + (a < d.nc ? (long long)cids[d.c0 + a] * nphi : 0);
+        for (int c = (warp >> 2) * 16; c < (warp >> 2) * 16 + 16 && c < d.np; c += 8) {
+            float D[ND][8];
+#pragma unroll
+            for (int l = 0; l < ND; ++l) tmem_ld8(tmem + l * NB + c + ((unsigned)((warp & 3) * 32) << 16), D[l]);
+            if (!ok || a >= d.nc) continue;
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (c + e < d.np)
+                    atomicAdd(o_row + pids[d.p0 + c + e], f * __hiloint2double((1023 + pexp[d.p0 + c + e]) << 20, 0) *
+                                                              combine_levels(D, e));
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 9) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    }
+    if (threadIdx.x == 0 && ctl->abort) atomicExch(err, 1);
+}
+
+// ---- response density: rho(r) = sum_b phi_b(r) sum_a chi_a(r) P_ab ------------------------------------
+// Block = (tile, 128 of its points, state); for every 32 phi (and every 448 chi) the product
+// T[r][b] = sum_a chi_a(r) P_ab, whose levels each thread combines and multiplies by phi.
+__global__ void __launch_bounds__(THREADS64, 1) density64_kernel(
+    const __grid_constant__ CUtensorMap mX,   // chi digits [(digit * nchunks + chunk) * 512 + point][64], box 64 x 128
+    int n, int nt, int k, const int *__restrict__ tiles, const int *__restrict__ coff, const int *__restrict__ cids,
+    const int *__restrict__ cfirst, long long nchunks, const int *__restrict__ poff, const int *__restrict__ pids,
+    const double *__restrict__ pval, int nphi, const double *__restrict__ P, long long sP,
+    const unsigned long long *__restrict__ pbits, int ex, double *__restrict__ rho, int *err, long long wlim) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *base = reinterpret_cast<unsigned char *>(
+        (reinterpret_cast<unsigned long long>(smem_raw) + 1023ull) & ~1023ull);
+    unsigned char *A = base, *B = base + A_RING * A_TILE;
+    Shared64 *ctl = reinterpret_cast<Shared64 *>(B + 2 * B_NMAJ);
+    volatile int *abort = &ctl->abort;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // states fastest, then the point blocks: blocks that share a tile's tables run together
+    const int s = blockIdx.x % k, pb = blockIdx.x / k % 4, t = tiles[blockIdx.x / k / 4];
+    const int c0 = coff[t], nc = coff[t + 1] - c0, p0 = poff[t], np = poff[t + 1] - p0;
+    const int KB = (nc + 63) / 64, NY = (np + NB - 1) / NB, NZ = (nc + MAX_K - 1) / MAX_K;
+    constexpr int ZB = MAX_K / 64;       // K blocks of one accumulation
+    if (threadIdx.x == 0) init64(ctl);
+    if (warp == 9) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
+                     "r"(512));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const unsigned tmem = ctl->tmem_base;
+
+    if (warp == 8) {
+        if (lane == 0) {
+            unsigned q = 0;
+            const unsigned total = (unsigned)(NY * KB * ND);
+            for (; q < total; ++q) {
+                const unsigned st = q % A_RING;
+                if (q >= A_RING && !mbar_wait(&ctl->a_empty[st], (q / A_RING - 1) & 1, abort, wlim)) break;
+                mbar_expect_tx(&ctl->a_full[st], A_TILE);
+                const long long ch = (long long)(q % ND) * nchunks + cfirst[t] + q / ND % KB;
+                tma_load_2d(A + st * A_TILE, &mX, &ctl->a_full[st], 0, (int)(ch * TILE_PTS + pb * 128));
+            }
+            // after an abort, the loads already issued land before the block exits
+            if (*abort)
+                for (unsigned i = q > A_RING ? q - A_RING : 0; i < q; ++i)
+                    mbar_drain(&ctl->a_full[i % A_RING], (i / A_RING) & 1, wlim);
+        }
+    } else if (warp == 9) {
+        if (elect_one()) {
+            const unsigned a_lo = desc_lo(smem_u32(A));
+            unsigned qa = 0, qb = 0, acc = 0;
+            bool ok = true;
+            for (int y = 0; y < NY && ok; ++y)
+                for (int z = 0; z < NZ && ok; ++z, ++acc) {
+                    if (acc > 0 && !mbar_wait(&ctl->acc_empty, (acc - 1) & 1, abort, wlim)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    for (int kb = z * ZB; kb < min(KB, (z + 1) * ZB) && ok; ++kb, ++qb) {
+                        ok = mbar_wait(&ctl->b_full[qb & 1], (qb >> 1) & 1, abort, wlim);
+                        if (!ok) break;
+                        tc_fence_after();
+                        // B is N-major (bit 16): 16 chi are 2048 bytes on, digit 8 starts block 4
+                        ok = mma_block(ctl, abort, a_lo, qa, tmem, desc_lo_mn(smem_u32(B + (qb & 1) * B_NMAJ), 8192), 128u,
+                                       (4 * 8192) >> 4, 1u << 16, kb == z * ZB, wlim);
+                        mma_commit(&ctl->b_empty[qb & 1]);
+                    }
+                    if (ok) mma_commit(&ctl->acc_full);
+                }
+            if (*abort) {
+                mma_commit(&ctl->drain);
+                mbar_drain(&ctl->drain, 0, wlim);
+            }
+        }
+    } else {
+        const int epx = exponent_of(pbits[s]);
+        const double sc = pow2(SHIFT - epx);
+        const double f = finite_bits(pbits[s]) ? ldexp(1.0, 56 - 2 * SHIFT + ex + epx) : __longlong_as_double(0x7ff8000000000000ll);
+        const double *Ps = P + (long long)s * sP;
+        const int lp = pb * 128 + (warp & 3) * 32 + lane, hb = warp >> 2;
+        unsigned qb = 0, acc = 0;
+        bool ok = true;
+        double r = 0.0;
+        for (int y = 0; y < NY && ok; ++y) {
+            const int b0 = y * NB, nb = min(NB, np - b0);
+            for (int z = 0; z < NZ && ok; ++z, ++acc) {
+                for (int kb = z * ZB; kb < min(KB, (z + 1) * ZB); ++kb, ++qb) {
+                    if (qb >= 2 && !mbar_wait(&ctl->b_empty[qb & 1], ((qb >> 1) - 1) & 1, abort, wlim)) {
+                        ok = false;
+                        break;
+                    }
+                    // digits of P: thread = (chi row, phi quad), twice; zeros past the lists
+                    unsigned char *Bk = B + (qb & 1) * B_NMAJ;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int task = threadIdx.x + h * 256, qd = task & 7, a = task >> 3;
+                        double v[4] = {0.0, 0.0, 0.0, 0.0};
+                        if (kb * 64 + a < nc && qd * 4 < nb) {
+                            const double2 *p = reinterpret_cast<const double2 *>(
+                                Ps + (long long)cids[c0 + kb * 64 + a] * nphi + pids[p0 + b0 + qd * 4]);
+                            const double2 x = __ldg(p), y2 = __ldg(p + 1);
+                            v[0] = x.x, v[1] = x.y, v[2] = y2.x, v[3] = y2.y;
+                        }
+                        unsigned long long u[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) u[e] = biased(v[e] * sc);
+#pragma unroll
+                        for (int j = 0; j < ND; ++j) {
+                            const uint2 x = make_uint2(digit_pair(digit(u[0], j), digit(u[1], j)),
+                                                       digit_pair(digit(u[2], j), digit(u[3], j)));
+                            *reinterpret_cast<uint2 *>(Bk + (j >> 1) * 8192 + sw128_offset(a, (j & 1) * 4 + (qd >> 1)) +
+                                                       (qd & 1) * 8) = x;
+                        }
+                    }
+                    fence_async_smem();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&ctl->b_full[qb & 1]);
+                }
+                ok = ok && mbar_wait(&ctl->acc_full, acc & 1, abort, wlim) && !*abort;
+                tc_fence_after();
+                if (!ok) break;
+                for (int c = hb * 16; c < hb * 16 + 16 && c < nb; c += 8) {
+                    float D[ND][8];
+#pragma unroll
+                    for (int l = 0; l < ND; ++l) tmem_ld8(tmem + l * NB + c + ((unsigned)((warp & 3) * 32) << 16), D[l]);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        if (c + e < nb)
+                            r = fma(combine_levels(D, e), __ldg(pval + (long long)(p0 + b0 + c + e) * TILE_PTS + lp), r);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ctl->acc_empty);
+            }
+        }
+        // the two halves of the phi meet (warps 0-7 only: a barrier of their own)
+        if (hb == 1) ctl->part[(warp & 3) * 32 + lane] = r;
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (hb == 0 && ok) {
+            r += ctl->part[(warp & 3) * 32 + lane];
+            const int gx = t / (nt * nt) * TILE + (lp >> 6), gy = (t / nt) % nt * TILE + ((lp >> 3) & 7),
+                      gz = t % nt * TILE + (lp & 7);
+            if (gx < n && gy < n && gz < n)
+                rho[(long long)s * n * n * n + ((long long)gx * n + gy) * n + gz] = r * f;
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 9) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    }
+    if (threadIdx.x == 0 && ctl->abort) atomicExch(err, 1);
+}
+
+// ---- tables and scales --------------------------------------------------------------------------------
+// largest |x| of every row of len values (bit pattern; bits zeroed before). blockIdx.y = row.
+__global__ void __launch_bounds__(256) max64_kernel(const double *__restrict__ x, long long len,
+                                                    unsigned long long *__restrict__ bits) {
+    const double *p = x + (long long)blockIdx.y * len;
+    unsigned long long m = 0;   // of non-negative doubles the bits order as the values, NaN last
+#pragma unroll 4
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < len; i += gridDim.x * 256ll) {
+        const unsigned long long v = (unsigned long long)__double_as_longlong(p[i]) & 0x7fffffffffffffffull;
+        m = v > m ? v : m;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long v = __shfl_xor_sync(0xffffffffu, m, o);
+        m = v > m ? v : m;
+    }
+    if ((threadIdx.x & 31) == 0) atomicMax(&bits[blockIdx.y], m);
+}
+
+// exponent E of every slot, max |value| < 2^E, at least -900 (0 for a slot of zeros); one warp per slot
+__global__ void __launch_bounds__(256) slot_exponent_kernel(const double *__restrict__ val, long long slots,
+                                                            int *__restrict__ out) {
+    const long long sl = blockIdx.x * 8ll + (threadIdx.x >> 5);
+    if (sl >= slots) return;
+    double m = 0.0;
+    for (int i = threadIdx.x & 31; i < TILE_PTS; i += 32) m = fmax(m, fabs(val[sl * TILE_PTS + i]));
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    int e = 0;
+    if (m > 0.0) frexp(m, &e);
+    if ((threadIdx.x & 31) == 0) out[sl] = max(e, -900);
+}
+
+// digit tables of chi: function-major [digit][slot][512], each slot by its own scale
+__global__ void chi_digits_fm_kernel(const double *__restrict__ val, long long values, const int *__restrict__ cexp,
+                                     unsigned short *__restrict__ out) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < values; i += (long long)gridDim.x * blockDim.x) {
+        const unsigned long long u = biased(ldexp(val[i], SHIFT - cexp[i / TILE_PTS]));
+#pragma unroll
+        for (int j = 0; j < ND; ++j) out[j * values + i] = (unsigned short)digit_pair(digit(u, j), 64u);
+    }
+}
+// and point-major in chunks of 64 slots of a tile, zero padded: [digit][chunk][512][64]
+__global__ void chi_digits_pm_kernel(const double *__restrict__ val, const int *__restrict__ off,
+                                     const int *__restrict__ chunk_tile, const int *__restrict__ chunk_j, long long nchunks,
+                                     double sc, unsigned short *__restrict__ out) {
+    const long long tot = nchunks * TILE_PTS * 64;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
+        const long long ch = e / (TILE_PTS * 64);
+        const int rem = (int)(e - ch * (TILE_PTS * 64)), p = rem / 64, t = chunk_tile[ch], sl = chunk_j[ch] * 64 + rem % 64;
+        const bool in = sl < off[t + 1] - off[t];
+        const unsigned long long u = biased(in ? val[(long long)(off[t] + sl) * TILE_PTS + p] * sc : 0.0);
+#pragma unroll
+        for (int j = 0; j < ND; ++j) out[j * tot + e] = (unsigned short)digit_pair(digit(u, j), 64u);
+    }
+}
+
+size_t smem64_int() { return 1024 + A_RING * A_TILE + 2 * B_KMAJ + TILE_PTS * sizeof(double) + sizeof(Shared64); }
+size_t smem64_den() { return 1024 + A_RING * A_TILE + 2 * B_NMAJ + sizeof(Shared64); }
+
+void max64(cudaStream_t st, const double *x, long long len, int rows, unsigned long long *bits) {
+    check(cudaMemsetAsync(bits, 0, sizeof(unsigned long long) * rows, st), "memset max64");
+    const long long per = std::max(8, 1216 / rows);
+    max64_kernel<<<dim3((unsigned)std::max<long long>(1, std::min<long long>(per, (len + 1023) / 1024)), rows), 256, 0, st>>>(
+        x, len, bits);
+    check_launch("max64_kernel");
+}
+
+}  // namespace
+
+// Digit tables and lists of a context: coff, poff, pids on the host as on the device. False (and
+// nothing made) when a tile's TMA rows would not fit 31 bits.
+bool fp64_grid_build(cudaStream_t st, Mem &mem, const TileSet<double> &chi, const TileSet<double> &phi,
+                     const std::vector<int> &coff, const std::vector<int> &poff, bool quads, Fp64Grid &G) {
+    const int ntl = chi.ntiles;
+    const long long slots = coff[ntl], values = slots * TILE_PTS;
+    std::vector<int> tiles, first(ntl + 1, 0), ct, cj;
+    std::vector<IItem> items;
+    for (int t = 0; t < ntl; ++t) {
+        const int nc = coff[t + 1] - coff[t], np = poff[t + 1] - poff[t], nch = (nc + 63) / 64;
+        first[t + 1] = first[t] + nch;
+        for (int j = 0; j < nch; ++j) ct.push_back(t), cj.push_back(j);
+        if (nc == 0 || np == 0) continue;
+        tiles.push_back(t);
+        for (int c = 0; c < nc; c += 128)
+            for (int b = 0; b < np; b += NB)
+                items.push_back(IItem{t, coff[t] + c, std::min(128, nc - c), poff[t] + b, std::min(NB, np - b)});
+    }
+    const long long nchunks = first[ntl];
+    if (tiles.empty() || ND * slots > 0x7fffffffll || ND * nchunks * TILE_PTS > 0x7fffffffll) return false;
+    std::stable_sort(tiles.begin(), tiles.end(), [&](int a, int b) {
+        return (long long)(coff[a + 1] - coff[a]) * (poff[a + 1] - poff[a]) >
+               (long long)(coff[b + 1] - coff[b]) * (poff[b + 1] - poff[b]);
+    });
+    const long long pslots = poff[ntl];
+    unsigned long long *bits = mem.alloc<unsigned long long>(2), h[2];
+    max64(st, chi.val, values, 1, bits);
+    max64(st, phi.val, pslots * TILE_PTS, 1, bits + 1);
+    check(cudaMemcpyAsync(h, bits, sizeof h, cudaMemcpyDeviceToHost, st), "D2H table maxima");
+    check(cudaStreamSynchronize(st), "sync table maxima");
+    double m[2];
+    static_assert(sizeof m == sizeof h, "bits of a double");
+    std::memcpy(m, h, sizeof m);
+    // tables with infinities, NaN or values beyond any orbital's stay on the CUDA cores
+    if (!(m[0] < 1e100) || !(m[1] < 1e100)) return false;
+    int e = 0;
+    std::frexp(m[0], &e);
+    G.ex = std::max(e, -900);
+    const double sc = std::ldexp(1.0, SHIFT - G.ex);
+    auto up = [&](const auto &v) {
+        using E = typename std::decay<decltype(v[0])>::type;
+        E *p = mem.alloc<E>(v.size());
+        check(cudaMemcpy(p, v.data(), v.size() * sizeof(E), cudaMemcpyHostToDevice), "upload FP64 grid lists");
+        return p;
+    };
+    G.slots = slots;
+    G.fm = mem.alloc<unsigned short>((size_t)ND * values);
+    G.cexp = mem.alloc<int>(slots);
+    G.pexp = mem.alloc<int>(pslots);
+    slot_exponent_kernel<<<(unsigned)((slots + 7) / 8), 256, 0, st>>>(chi.val, slots, G.cexp);
+    slot_exponent_kernel<<<(unsigned)((pslots + 7) / 8), 256, 0, st>>>(phi.val, pslots, G.pexp);
+    check_launch("slot_exponent_kernel");
+    chi_digits_fm_kernel<<<8 * 1216, 256, 0, st>>>(chi.val, values, G.cexp, G.fm);
+    check_launch("chi_digits_fm_kernel");
+    G.items = up(items);
+    G.nitems = (long long)items.size();
+    if (quads) {
+        G.nchunks = nchunks;
+        G.pm = mem.alloc<unsigned short>((size_t)ND * nchunks * TILE_PTS * 64);
+        Mem tmp;
+        int *dct = tmp.alloc<int>(ct.size()), *dcj = tmp.alloc<int>(cj.size());
+        check(cudaMemcpy(dct, ct.data(), ct.size() * sizeof(int), cudaMemcpyHostToDevice), "upload chunk tiles");
+        check(cudaMemcpy(dcj, cj.data(), cj.size() * sizeof(int), cudaMemcpyHostToDevice), "upload chunk index");
+        chi_digits_pm_kernel<<<8 * 1216, 256, 0, st>>>(chi.val, chi.off, dct, dcj, nchunks, sc, G.pm);
+        check_launch("chi_digits_pm_kernel");
+        check(cudaStreamSynchronize(st), "sync digit tables");
+        G.tiles = up(tiles);
+        G.ntiles = (int)tiles.size();
+        G.cfirst = up(first);
+        G.covers = G.ntiles == ntl;
+    }
+    return true;
+}
+
+// rho [k][n^3] of P [k][nchi][nphi] (16-byte aligned rows); bits: k words of 64 bits
+void response_density_fp64(cudaStream_t st, const GridShape &g, const TileSet<double> &chi, const TileSet<double> &phi,
+                           const Fp64Grid &G, int nphi, const double *P, long long sP, int k, double *rho,
+                           unsigned long long *bits, int *err) {
+    if (k <= 0) return;
+    ProfScope ps(st, ST_DENSITY, 2.0 * k * g.pair_points, 8.0 * (g.table_values + (double)k * g.n * g.n * g.n));
+    if (!G.covers) check(cudaMemsetAsync(rho, 0, sizeof(double) * (size_t)k * g.n * g.n * g.n, st), "memset rho");
+    max64(st, P, sP, k, bits);
+    CUtensorMap mx;
+    if (!encode_map_2d(&mx, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, G.pm, 64ull, (unsigned long long)(ND * G.nchunks) * TILE_PTS,
+                       128ull, 64, 128))
+        throw CudaError{cudaErrorInvalidValue, "cuTensorMapEncodeTiled (density64)"};
+    static const bool attr = [&]() {
+        check(cudaFuncSetAttribute(density64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64_den()),
+              "attr density64");
+        return true;
+    }();
+    (void)attr;
+    const long long blocks = 4LL * G.ntiles * k;
+    if (blocks > 0x7fffffffll) throw CudaError{cudaErrorInvalidValue, "density64: too many blocks"};
+    density64_kernel<<<(unsigned)blocks, THREADS64, smem64_den(), st>>>(
+        mx, g.n, g.nt, k, G.tiles, chi.off, chi.ids, G.cfirst, G.nchunks, phi.off, phi.ids, phi.val, nphi, P, sP, bits, G.ex,
+        rho, err, active_wait_limit());
+    check_launch("density64_kernel");
+}
+
+// out [k][nchi][nphi] of V [k][n^3]; bits: k words of 64 bits
+void potential_integrals_fp64(cudaStream_t st, const GridShape &g, const TileSet<double> &chi, const TileSet<double> &phi,
+                              const Fp64Grid &G, int nchi, int nphi, const double *V, int k, double *out,
+                              unsigned long long *bits, int *err) {
+    if (k <= 0) return;
+    ProfScope ps(st, ST_INTEGRALS, 2.0 * k * g.pair_points,
+                 8.0 * (g.table_values + (double)k * g.n * g.n * g.n + (double)k * nchi * nphi));
+    check(cudaMemsetAsync(out, 0, sizeof(double) * (size_t)k * nchi * nphi, st), "memset(integrals)");
+    max64(st, V, (long long)g.n * g.n * g.n, k, bits);
+    CUtensorMap mx;
+    if (!encode_map_2d(&mx, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, G.fm, (unsigned long long)TILE_PTS,
+                       (unsigned long long)(ND * G.slots), (unsigned long long)TILE_PTS * 2, 64, 128))
+        throw CudaError{cudaErrorInvalidValue, "cuTensorMapEncodeTiled (integrals64)"};
+    static const bool attr = [&]() {
+        check(cudaFuncSetAttribute(integrals64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64_int()),
+              "attr integrals64");
+        return true;
+    }();
+    (void)attr;
+    const long long blocks = G.nitems * k;
+    if (blocks > 0x7fffffffll) throw CudaError{cudaErrorInvalidValue, "integrals64: too many blocks"};
+    integrals64_kernel<<<(unsigned)blocks, THREADS64, smem64_int(), st>>>(
+        mx, g.n, g.nt, k, G.items, G.slots, chi.ids, phi.ids, phi.val, G.cexp, G.pexp, nchi, nphi, V, bits, g.dV, out, err,
+        active_wait_limit());
+    check_launch("integrals64_kernel");
+}
+
+}  // namespace tddft

@@ -125,6 +125,19 @@ struct IItem {
     int t, c0, nc, p0, np;
 };
 
+// Tables of the float64 grid contractions on the tensor cores (device arrays): seven-bit digits of chi
+// as float16, function-major and, where phi lists are whole aligned quads, point-major
+struct Fp64Grid {
+    unsigned short *fm = nullptr, *pm = nullptr;
+    long long slots = 0, nchunks = 0, nitems = 0;
+    const IItem *items = nullptr;   // integrals: at most 128 chi and 32 phi of a tile
+    const int *tiles = nullptr;     // density: tiles with both chi and phi, densest first
+    const int *cfirst = nullptr;    // first 64-wide chi chunk of each tile
+    int *cexp = nullptr, *pexp = nullptr;   // of every slot: |value| < 2^exp
+    int ntiles = 0, ex = 0;                 // |chi| < 2^ex
+    bool covers = false;            // the listed tiles are all tiles of the grid
+};
+
 struct GridShape {
     int n;          // points per side
     int nt;         // tiles per side = ceil(n / 8)
