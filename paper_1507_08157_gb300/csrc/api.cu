@@ -1501,6 +1501,7 @@ struct tddft_state {
     int it = 0;
     int fallbacks = 0;             // learned steps that took the CG solve instead
     long long inner_iters = 0;     // inner CG iterations over all steps
+    bool inner_pending = false;    // the last solve's count is on its way to host[2k] (second int)
     bool evaluated = false;
     bool have_prev_omega = false;
     std::vector<double> omega, resid, omega_prev;
@@ -1587,11 +1588,23 @@ void sandwich(tddft_ctx *c, int nb, const T *Lm, const T *X, const T *Rm, T *out
     gemm<T>(c->st, false, false, nb * nc, nv, nv, T(1), tmp, nv, 0, Rm, nv, 0, T(0), out, nv, 0, 1, approx);
 }
 
+// take the pending inner-CG count (waits for the stream where one is pending)
+void settle_inner(tddft_ctx *c, tddft_state *S) {
+    if (!S->inner_pending) return;
+    check(ctx_sync(c), "sync inner count");
+    S->inner_iters += reinterpret_cast<const int *>(S->host + 2 * S->k)[1];
+    S->inner_pending = false;
+}
+
 void sync_status(tddft_ctx *c, tddft_state *S, const int *dstatus) {
     check(cudaMemcpyAsync(reinterpret_cast<int *>(S->host + 2 * S->k), dstatus, sizeof(int),
                           cudaMemcpyDeviceToHost, c->st),
           "D2H status");
     check_tc_error(c);   // waits for the status copy too
+    if (S->inner_pending) {
+        S->inner_iters += reinterpret_cast<const int *>(S->host + 2 * S->k)[1];
+        S->inner_pending = false;
+    }
     const int stv = *reinterpret_cast<int *>(S->host + 2 * S->k);
     if (stv == DEV_BREAKDOWN) throw Breakdown{"non-positive norm in Gram-Schmidt (dependent trial pairs)"};
     if (stv == DEV_NAN) throw Breakdown{"NaN or Inf in the trial pairs"};
@@ -1757,12 +1770,20 @@ void precondition(tddft_ctx *c, tddft_state *S, const T *h, T *z) {
         T *r = B.qr, *p = B.qp, *Lp = B.qL, *zh = B.qz;
         gemm<T>(st, false, false, rc, nv, nc, T(1), I.Wc, nc, 0, h, nv, len, T(0), B.tmp, nv, (long long)rc * nv, k2);
         gemm<T>(st, false, false, k2 * rc, rv, nv, T(1), B.tmp, nv, 0, I.Wv, rv, 0, T(0), r, rv, 0, 1);
-        check(cudaMemsetAsync(zh, 0, k2 * lr * sizeof(T), st), "memset z");
-        check(cudaMemcpyAsync(p, r, k2 * lr * sizeof(T), cudaMemcpyDeviceToDevice, st), "copy p");
-        dots<T>(st, r, lr, r, lr, k2, lr, B.dvec2, B.gscr);
-        cg_init(st, k2, ptol, B.dvec2, B.cg_rr, B.cg_r0, B.cg_active, B.cg_nactive);
         int *hn = reinterpret_cast<int *>(S->host + 2 * S->k) + 1;
-        for (int it = 0; it < c->opt.precond_maxit; ++it) {
+        const bool one_block = cg_reduced<T>(st, rc, rv, I.Mch, I.Mvh, r, zh, k2, ptol, c->opt.precond_maxit, B.cg_nactive);
+        if (one_block) {
+            // the count is read with the next wait for the stream (settle_inner)
+            settle_inner(c, S);
+            check(cudaMemcpyAsync(hn, B.cg_nactive, sizeof(int), cudaMemcpyDeviceToHost, st), "D2H cg iterations");
+            S->inner_pending = true;
+        } else {
+            check(cudaMemsetAsync(zh, 0, k2 * lr * sizeof(T), st), "memset z");
+            check(cudaMemcpyAsync(p, r, k2 * lr * sizeof(T), cudaMemcpyDeviceToDevice, st), "copy p");
+            dots<T>(st, r, lr, r, lr, k2, lr, B.dvec2, B.gscr);
+            cg_init(st, k2, ptol, B.dvec2, B.cg_rr, B.cg_r0, B.cg_active, B.cg_nactive);
+        }
+        for (int it = 0; !one_block && it < c->opt.precond_maxit; ++it) {
             check(cudaMemcpyAsync(hn, B.cg_nactive, sizeof(int), cudaMemcpyDeviceToHost, st), "D2H n_active");
             check(ctx_sync(c), "sync cg");
             if (*hn == 0) break;
@@ -2905,6 +2926,7 @@ tddft_status tddft_samples(tddft_ctx *c, tddft_state *S, int64_t cap, float *X, 
             learned_features<T>(c->st, h, k, na, c->nca, c->nva, c->nc, c->nv, I.lfc, I.lfv, I.ldist, X, I.ls);
             learned_targets<T>(c->st, B.z, h, I.ls, k, na, c->nca, c->nva, c->nc, c->nv, Tg, Wt);
             check(ctx_sync(c), "sync samples");
+            settle_inner(c, S);
             return TDDFT_OK;
         })());
     });

@@ -389,6 +389,36 @@ __global__ void __launch_bounds__(256) gram_rows_kernel(const T *__restrict__ X,
         }
 }
 
+// Trace products of short vectors: one warp per pair, runs of eight products added to a compensated
+// sum per lane, the lanes in float64. The row kernel above keeps 4 x 4 pairs per thread, so that a
+// few short rows leave it a handful of threads (float64, 1024 elements, 2 x 8 rows: 180 us there,
+// 6 us here).
+template <typename T>
+__global__ void __launch_bounds__(128) gram_short_kernel(const T *__restrict__ X, long long sx, int nx, const YSet<T> ys,
+                                                         long long sy, int ny, long long len, GOut out) {
+    const int p = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (p >= nx * ny) return;
+    const int i = p / ny, j = p - i * ny, q = j / ys.per;
+    const T *x = X + i * sx;
+    const T *set = q == 0 ? ys.p[0] : q == 1 ? ys.p[1] : q == 2 ? ys.p[2] : ys.p[3];
+    const T *y = set + (long long)(j - q * ys.per) * sy;
+    T tot = T(0), cmp = T(0);
+    for (long long e0 = lane; e0 < len; e0 += 256) {
+        T run = T(0);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const long long e = e0 + 32 * u;
+            if (e < len) run = fma(x[e], y[e], run);
+        }
+        const T v = run - cmp, s = tot + v;
+        cmp = (s - tot) - v;
+        tot = s;
+    }
+    double d = (double)tot - (double)cmp;
+    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    if (lane == 0) out.g[q][i * ys.per + (j - q * ys.per)] = d;
+}
+
 // Batched element-wise kernels: blockIdx.y = matrix b of nb, blockIdx.x strides over the len
 // entries of one matrix (in 16-byte vectors when len allows), so the per-matrix coefficient is
 // read once per thread and no index division runs per element.
@@ -996,6 +1026,80 @@ __global__ void cg_scalars_kernel(int n, int phase, double tol, const double *pL
     if (phase == 1 && i == 0) *n_active = cnt;
 }
 
+// The whole inner CG of one system on the reduced space in one block: L p = Mc p - p Mv on rc x rv
+// coordinates, from z = 0 and r given, with the decisions of the kernels above (a system is
+// independent of the others, so each stops by itself). Everything stays in shared memory: an
+// iteration otherwise takes eleven launches and a host wait (about 45 us whatever the size, 13
+// iterations a step at 8 atoms). iters: the most iterations of any system (zeroed before).
+constexpr int CG_THREADS = 512;
+__device__ double block_sum(double v, double *red) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();                 // the last call's readers are done
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double s = 0.0;
+    for (int w = 0; w < CG_THREADS / 32; ++w) s += red[w];
+    return s;
+}
+template <typename T>
+__global__ void __launch_bounds__(CG_THREADS) cg_reduced_kernel(int rc, int rv, const T *__restrict__ Mc,
+                                                                const T *__restrict__ Mv, const T *__restrict__ rin,
+                                                                T *__restrict__ zout, double tol, int maxit, int *iters) {
+    extern __shared__ __align__(16) unsigned char cg_smem[];
+    __shared__ double red[CG_THREADS / 32];
+    const int n = rc * rv, t = threadIdx.x;
+    T *mc = reinterpret_cast<T *>(cg_smem), *mv = mc + rc * rc, *p = mv + rv * rv, *r = p + n, *z = r + n, *Lp = z + n;
+    const long long base = (long long)blockIdx.x * n;
+    for (int i = t; i < rc * rc; i += CG_THREADS) mc[i] = Mc[i];
+    for (int i = t; i < rv * rv; i += CG_THREADS) mv[i] = Mv[i];
+    double s = 0.0;
+    for (int i = t; i < n; i += CG_THREADS) {
+        const T x = rin[base + i];
+        r[i] = x;
+        p[i] = x;
+        z[i] = T(0);
+        s += (double)x * (double)x;
+    }
+    double rr = block_sum(s, red);
+    const double r0 = sqrt(rr > 0.0 ? rr : 0.0);
+    bool active = r0 > 0.0 && isfinite(r0);
+    int it = 0;
+    for (; it < maxit && active; ++it) {
+        __syncthreads();             // p is whole
+        s = 0.0;
+        for (int e = t; e < n; e += CG_THREADS) {
+            const int i = e / rv, j = e - i * rv;
+            T a = T(0), b = T(0);
+            for (int q = 0; q < rc; ++q) a = fma(mc[i * rc + q], p[q * rv + j], a);
+            for (int q = 0; q < rv; ++q) b = fma(p[i * rv + q], mv[q * rv + j], b);
+            const T l = a - b;
+            Lp[e] = l;
+            s += (double)p[e] * (double)l;
+        }
+        const double pLp = block_sum(s, red);
+        if (!(pLp > 0.0 && isfinite(pLp))) {
+            active = false;
+            continue;
+        }
+        const double alpha = rr / pLp;
+        const T ap = T(alpha), am = T(-alpha);
+        s = 0.0;
+        for (int e = t; e < n; e += CG_THREADS) {
+            z[e] = fma(ap, p[e], z[e]);
+            const T x = fma(am, Lp[e], r[e]);
+            r[e] = x;
+            s += (double)x * (double)x;
+        }
+        const double rrn = block_sum(s, red);
+        const T beta = T(rr != 0.0 ? rrn / rr : 0.0);
+        rr = rrn;
+        if (!(sqrt(rrn > 0.0 ? rrn : 0.0) > tol * r0)) active = false;
+        for (int e = t; e < n; e += CG_THREADS) p[e] = fma(beta, p[e], r[e]);
+    }
+    for (int i = t; i < n; i += CG_THREADS) zout[base + i] = z[i];
+    if (t == 0) atomicMax(iters, it);
+}
+
 __global__ void cg_init_kernel(int n, double tol, const double *rr0, double *rr, double *r0,
                                int *active, int *n_active) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
@@ -1166,6 +1270,14 @@ void gram_multi(cudaStream_t st, const T *X, long long sx, int nx, int nset, con
         go.g[q] = q < nset ? G[q] : G[0];
     }
     ys.per = per;
+    // float64 rows of at most 8192 elements: a warp walks 256 elements a step, so its share stays short
+    // of the row kernel's (1024 elements: 180 us and 6 us for 16 pairs; 8192 elements, 64 pairs: the
+    // warps read the rows about as fast as the row kernel's few blocks)
+    if (sizeof(T) == 8 && len > 0 && len <= 8192) {
+        gram_short_kernel<T><<<(pairs + 3) / 4, 128, 0, st>>>(X, sx, nx, ys, sy, ny, len, go);
+        check_launch("gram_short_kernel");
+        return;
+    }
     constexpr int VW = sizeof(T) == 4 ? 4 : 2;   // 16-byte loads
     bool vec = len % VW == 0 && sx % VW == 0 && sy % VW == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0;
     for (int q = 0; q < nset; ++q) vec = vec && reinterpret_cast<uintptr_t>(Y[q]) % 16 == 0;
@@ -1313,6 +1425,30 @@ void cg_init(cudaStream_t st, int n, double tol, const double *rr0, double *rr, 
     cg_init_kernel<<<1, 1, 0, st>>>(n, tol, rr0, rr, r0, active, n_active);
     check_launch("cg_init_kernel");
 }
+// the one-block form for nb systems: false (nothing done) where it does not apply. In float64 up to
+// rc rv (rc + rv) = 131072 multiply-adds an iteration, 35 us at the two per cycle of one SM, what the
+// launches of the other form take; float32 products keep their own kernels.
+template <typename T>
+bool cg_reduced(cudaStream_t st, int rc, int rv, const T *Mc, const T *Mv, const T *r, T *z, int nb, double tol, int maxit,
+                int *iters) {
+    const size_t sm = sizeof(T) * ((size_t)rc * rc + (size_t)rv * rv + 4 * (size_t)rc * rv);
+    if (sizeof(T) != 8 || nb < 1 || (long long)rc * rv * (rc + rv) > 131072 || sm > 200 * 1024) return false;
+    ProfScope ps(st, ST_SMALL, 0.0, 0.0);
+    static const bool attr = []() {   // once per process, thread-safe
+        check(cudaFuncSetAttribute(cg_reduced_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024),
+              "attr cg_reduced");
+        return true;
+    }();
+    (void)attr;
+    check(cudaMemsetAsync(iters, 0, sizeof(int), st), "memset cg iterations");
+    cg_reduced_kernel<T><<<nb, CG_THREADS, sm, st>>>(rc, rv, Mc, Mv, r, z, tol, maxit, iters);
+    check_launch("cg_reduced_kernel");
+    return true;
+}
+template bool cg_reduced<float>(cudaStream_t, int, int, const float *, const float *, const float *, float *, int, double,
+                                int, int *);
+template bool cg_reduced<double>(cudaStream_t, int, int, const double *, const double *, const double *, double *, int,
+                                 double, int, int *);
 void cg_scalars(cudaStream_t st, int n, int phase, double tol, const double *pLp, const double *rr_new,
                 double *rr, const double *r0, double *alpha, double *beta, int *active, int *n_active) {
     ProfScope ps(st, ST_SMALL, 0.0, 0.0);

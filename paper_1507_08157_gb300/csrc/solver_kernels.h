@@ -28,6 +28,9 @@ void line_gs(cudaStream_t st, int k, const double *A, const double *BDf, const d
 void init_gs(cudaStream_t st, int k, const double *PP, double *Cp, double *Cq, int *status);
 void cg_init(cudaStream_t st, int n, double tol, const double *rr0, double *rr, double *r0,
              int *active, int *n_active);
+template <typename T>
+bool cg_reduced(cudaStream_t st, int rc, int rv, const T *Mc, const T *Mv, const T *r, T *z, int nb, double tol, int maxit,
+                int *iters);
 void cg_scalars(cudaStream_t st, int n, int phase, double tol, const double *pLp,
                 const double *rr_new, double *rr, const double *r0, double *alpha, double *beta,
                 int *active, int *n_active);
