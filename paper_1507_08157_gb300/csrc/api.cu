@@ -244,6 +244,7 @@ struct Impl {
     bool exact = false;
     T *Dn = nullptr;
     double *fxc64 = nullptr;
+    T *fft_tw = nullptr;      // FFT twiddles of the grid size
     // tensor-core grid path (float32 contexts): point-major f16 chi tables [tile][512][CK]
     unsigned short *chi_pm = nullptr;
     unsigned short *chi_fm16 = nullptr;   // function-major f16 chi tables [slot][512]
@@ -857,7 +858,7 @@ void apply_impl(tddft_ctx *c, Impl<T> &I, int k, const T *P, T *f, bool mirror =
         lprod<T>(c, I, SP_M, P, f, k, T(1), T(0));
         rprod<T>(c, I, P, SP_M, f, k, T(-1), T(1));
         density(c, I, P, k);
-        hartree_fxc<T>(st, c->grid(), I.rho, I.fxc, k, I.V, I.fft);
+        hartree_fxc<T>(st, c->grid(), I.rho, I.fxc, k, I.V, I.fft, I.fft_tw);
         integrals(c, I, k);
         lprod<T>(c, I, SP_P, I.Vmat, I.tmp, k, T(1), T(0));
         rprod<T>(c, I, I.tmp, SP_P, f, k, T(1), T(1));
@@ -878,7 +879,7 @@ void apply_impl(tddft_ctx *c, Impl<T> &I, int k, const T *P, T *f, bool mirror =
     const T alpha = tda ? T(1) : T(2);
     const GridShape g = c->grid();
     density(c, I, Ps, ns);
-    hartree_fxc<T>(st, g, I.rho, I.fxc, ns, I.V, I.fft);
+    hartree_fxc<T>(st, g, I.rho, I.fxc, ns, I.V, I.fft, I.fft_tw);
     integrals(c, I, ns);
     // coupling: f_q += 2 P^c V_SCF P^v
     lprod<T>(c, I, SP_P, I.Vmat, I.tmp, ns, T(1), T(0));
@@ -1320,6 +1321,8 @@ void build_impl(tddft_ctx *c, const tddft_system *s, const tddft_sparse_system *
     };
     if (s) build_dense_matrices<T>(c, I.get(), s, tmpm);
     else build_sparse_matrices<T>(c, I.get());
+    I->fft_tw = I->mem.template alloc<T>(2 * (size_t)n);
+    fft_twiddles<T>(st, n, I->fft_tw);
     // f_xc[n0], float64, once per system
     const long long n3 = c->n3();
     I->fxc64 = I->mem.template alloc<double>(n3);
@@ -2447,7 +2450,7 @@ tddft_status tddft_response_potential(tddft_ctx *c, int32_t k, const double *rho
             Impl<T> &I = impl<T>(c);
             ensure_workspace(c, I, k);
             upload<T>(c, I, rho, I.rho, (long long)k * c->n3());
-            hartree_fxc<T>(c->st, c->grid(), I.rho, I.fxc, k, I.V, I.fft);
+            hartree_fxc<T>(c->st, c->grid(), I.rho, I.fxc, k, I.V, I.fft, I.fft_tw);
             download<T>(c, I, I.V, V, (long long)k * c->n3());
             check(ctx_sync(c), "sync potential");
             return TDDFT_OK;

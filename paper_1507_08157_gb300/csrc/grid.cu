@@ -267,220 +267,294 @@ __device__ __forceinline__ void small_dft(int R, V *v) {
     }
 }
 
-// Per-CTA tables of a plan, built once before the transforms: the stage twiddles
-// tw[off_s + kk (R - 1) + r - 1] = exp(-2 pi i kk r / (Ns R)) (forward sign; the inverse takes the
-// conjugate) and kk = j mod Ns for every butterfly index j of every stage. The transforms then
-// look these up instead of evaluating sines and dividing per element.
-constexpr int FFT_KK_BYTES = 2048;      // sum over stages of n / R (n <= 256)
-
+// Stage twiddles of a plan, tw[off_s + kk (R - 1) + r - 1] = exp(-2 pi i kk r / (Ns R)) (forward sign;
+// the inverse takes the conjugate), made once per context; n - 1 values
 template <typename T>
-__device__ void fft_tables(const Plan &pl, typename C2<T>::t *tw, unsigned char *kkt) {
-    const int n = pl.n;
-    int Ns = 1, toff = 0, koff = 0;
+__global__ void fft_twiddles_kernel(Plan pl, typename C2<T>::t *__restrict__ tw) {
+    int Ns = 1, toff = 0;
     for (int st = 0; st < pl.nst; ++st) {
-        const int R = pl.radix[st], nb = n / R;
+        const int R = pl.radix[st];
         for (int i = threadIdx.x; i < Ns * (R - 1); i += blockDim.x) {
             const int kk = i / (R - 1), r = i - kk * (R - 1) + 1;
             T sn, cs;
             sincospi_t<T>(T(-2) * T(kk * r) / T(Ns * R), &sn, &cs);
             tw[toff + i] = {cs, sn};
         }
-        for (int jj = threadIdx.x; jj < nb; jj += blockDim.x) kkt[koff + jj] = (unsigned char)(jj % Ns);
         toff += Ns * (R - 1);
-        koff += nb;
         Ns *= R;
     }
 }
 
-// One Stockham stage of radix R (a compile-time constant, so that the R values of a butterfly
-// stay in registers) on one line: butterflies j = t0, t0 + tpl, ... < nb = n / R.
-template <typename T, int SG, int R>
-__device__ __forceinline__ void fft_stage(const typename C2<T>::t *src, typename C2<T>::t *dst, int nb, int Ns,
-                                          int t0, int tpl, const typename C2<T>::t *tws,
-                                          const unsigned char *kks) {
+// The five passes over the grid move ~10 words of global memory a point; what bounds them is the trip
+// of a block's lines through shared memory between its load and its store, with few blocks resident.
+// Hence stages in pairs (float32), twiddles from a table of the context instead of sines per block, and
+// registers capped so that four blocks of 256 threads fit (float32). float32, Hartree and f_xc, before
+// and after: 90^3, 5 states 0.085 and 0.062 ms; 135^3, 10 states 0.71 and 0.53; 144^3, 8 states 0.67 and
+// 0.43; 180^3, 5 states 0.76 and 0.44. float64: 90^3, 3 states 0.92 and 0.79.
+
+// shared-memory place of point i of a line, and the distance of lines. PAD: one element per 16, so that
+// the outputs of a first pair of stages whose product is 8 or 16 fall into different banks (144^3, 8
+// states 0.57 and 0.43 ms); other sizes lose by it (135^3, 10 states: 0.53 and 0.68).
+template <bool PAD> __device__ __forceinline__ int fft_at(int i) { return PAD ? i + (i >> 4) : i; }
+template <bool PAD> __host__ __device__ constexpr int fft_ld(int n) { return PAD ? n + (n >> 4) + 1 : n + 1; }
+
+// Two Stockham stages of radix R1, then R2 (1: only the first), in registers on one line. The group of
+// points j + m n / (R1 R2), m < R1 R2, is closed under both stages: the first takes the points m = r2 +
+// R2 r1 to position (j - kk) R1 + kk + r1 Ns + r2 n / R2, kk = j mod Ns, which is the second's input
+// r2 of its butterfly kk + r1 Ns. One trip through shared memory per two stages instead of two, and
+// every value is computed as by single stages.
+template <typename T, bool PAD, int SG, int R1, int R2>
+__device__ __forceinline__ void fft_step(const typename C2<T>::t *src, typename C2<T>::t *dst, int n, int Ns, int t0,
+                                         int tpl, const typename C2<T>::t *tw1, const typename C2<T>::t *tw2) {
     using V = typename C2<T>::t;
+    constexpr int RR = R1 * R2;
+    const int nb = n / RR;
     for (int j = t0; j < nb; j += tpl) {
-        V v[R];
+        V v[RR];
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = src[j + r * nb];
-        const int kk = kks[j];
-        if (Ns > 1) {
-            const V *w = tws + kk * (R - 1) - 1;
+        for (int m = 0; m < RR; ++m) v[m] = src[fft_at<PAD>(j + m * nb)];
+        const int kk = Ns == 1 ? 0 : j % Ns;
 #pragma unroll
-            for (int r = 1; r < R; ++r) v[r] = cmul(v[r], w[r].x, SG < 0 ? w[r].y : -w[r].y);
+        for (int r2 = 0; r2 < R2; ++r2) {
+            V u[R1];
+#pragma unroll
+            for (int r = 0; r < R1; ++r) u[r] = v[r2 + R2 * r];
+            if (Ns > 1) {
+                const V *w = tw1 + kk * (R1 - 1) - 1;
+#pragma unroll
+                for (int r = 1; r < R1; ++r) u[r] = cmul(u[r], w[r].x, SG < 0 ? w[r].y : -w[r].y);
+            }
+            small_dft<T, SG>(R1, u);
+#pragma unroll
+            for (int r = 0; r < R1; ++r) v[r2 + R2 * r] = u[r];
         }
-        small_dft<T, SG>(R, v);
-        const int base = (j - kk) * R + kk;
+        const int base = (j - kk) * RR + kk;
 #pragma unroll
-        for (int r = 0; r < R; ++r) dst[base + r * Ns] = v[r];
+        for (int r = 0; r < R1; ++r) {
+            V u[R2];
+#pragma unroll
+            for (int r2 = 0; r2 < R2; ++r2) u[r2] = v[r2 + R2 * r];
+            if (R2 > 1) {
+                const V *w = tw2 + (kk + r * Ns) * (R2 - 1) - 1;
+#pragma unroll
+                for (int r2 = 1; r2 < R2; ++r2) u[r2] = cmul(u[r2], w[r2].x, SG < 0 ? w[r2].y : -w[r2].y);
+                small_dft<T, SG>(R2, u);
+            }
+#pragma unroll
+            for (int r2 = 0; r2 < R2; ++r2) dst[fft_at<PAD>(base + r * Ns + r2 * Ns * R1)] = u[r2];
+        }
     }
 }
 
-// FFT of `lines` lines of length n held at buf0 (line-major, lines ld >= n apart); returns the
-// buffer with the result. blockDim.x / lines threads work on each line (lines divides blockDim.x).
-template <typename T, int SG>
-__device__ typename C2<T>::t *fft_lines(typename C2<T>::t *buf0, typename C2<T>::t *buf1, int lines, int ld,
-                                        const Plan &pl, const typename C2<T>::t *tw, const unsigned char *kkt) {
+// FFT of the block's lines held at buf0 (line-major, ld apart, point i at fft_at<PAD>(i)); returns the
+// buffer with the result. tpl threads work on each line. In float32 stages are taken in pairs where their product is at
+// most 16 (32 registers of data a thread); in float64, where the arithmetic bounds the passes, twice
+// the threads take single stages (pairs left most of them idle: 90^3, 3 states 1.09 ms against 0.92).
+template <typename T> __host__ __device__ constexpr int fft_tpl() { return sizeof(T) == 8 ? 32 : 16; }
+template <typename T> __host__ __device__ constexpr int fft_pair_max() { return sizeof(T) == 8 ? 1 : 16; }
+template <typename T, bool PAD, int SG>
+__device__ typename C2<T>::t *fft_lines(typename C2<T>::t *buf0, typename C2<T>::t *buf1, int ld, const Plan &pl,
+                                        const typename C2<T>::t *tw) {
     using V = typename C2<T>::t;
     V *in = buf0, *out = buf1;
     const int n = pl.n;
-    const int tpl = blockDim.x / lines;
+    constexpr int tpl = fft_tpl<T>();
     const int line = threadIdx.x / tpl, t0 = threadIdx.x - line * tpl;
-    int Ns = 1, toff = 0, koff = 0;
-    for (int st = 0; st < pl.nst; ++st) {
-        const int R = pl.radix[st];
-        const int nb = n / R;
-        if (line < lines) {
-            const V *src = in + line * ld;
-            V *dst = out + line * ld;
-            switch (R) {
-                case 2: fft_stage<T, SG, 2>(src, dst, nb, Ns, t0, tpl, tw + toff, kkt + koff); break;
-                case 3: fft_stage<T, SG, 3>(src, dst, nb, Ns, t0, tpl, tw + toff, kkt + koff); break;
-                case 4: fft_stage<T, SG, 4>(src, dst, nb, Ns, t0, tpl, tw + toff, kkt + koff); break;
-                default: fft_stage<T, SG, 5>(src, dst, nb, Ns, t0, tpl, tw + toff, kkt + koff); break;
+    int Ns = 1, toff = 0;
+    for (int st = 0; st < pl.nst;) {
+        const int R1 = pl.radix[st], R2 = st + 1 < pl.nst && R1 * pl.radix[st + 1] <= fft_pair_max<T>() ? pl.radix[st + 1] : 1;
+        const V *src = in + line * ld, *w1 = tw + toff, *w2 = w1 + Ns * (R1 - 1);
+        V *dst = out + line * ld;
+        bool done = false;
+        if constexpr (fft_pair_max<T>() > 1) {
+            done = true;
+            switch (R1 * 8 + R2) {
+                case 4 * 8 + 4: fft_step<T, PAD, SG, 4, 4>(src, dst, n, Ns, t0, tpl, w1, w2); break;
+                case 4 * 8 + 2: fft_step<T, PAD, SG, 4, 2>(src, dst, n, Ns, t0, tpl, w1, w2); break;
+                case 4 * 8 + 3: fft_step<T, PAD, SG, 4, 3>(src, dst, n, Ns, t0, tpl, w1, w2); break;
+                case 2 * 8 + 3: fft_step<T, PAD, SG, 2, 3>(src, dst, n, Ns, t0, tpl, w1, w2); break;
+                case 2 * 8 + 5: fft_step<T, PAD, SG, 2, 5>(src, dst, n, Ns, t0, tpl, w1, w2); break;
+                case 3 * 8 + 3: fft_step<T, PAD, SG, 3, 3>(src, dst, n, Ns, t0, tpl, w1, w2); break;
+                case 3 * 8 + 5: fft_step<T, PAD, SG, 3, 5>(src, dst, n, Ns, t0, tpl, w1, w2); break;
+                default: done = false;
+            }
+        }
+        if (!done) {
+            switch (R1) {
+                case 2: fft_step<T, PAD, SG, 2, 1>(src, dst, n, Ns, t0, tpl, w1, w2); break;
+                case 3: fft_step<T, PAD, SG, 3, 1>(src, dst, n, Ns, t0, tpl, w1, w2); break;
+                case 4: fft_step<T, PAD, SG, 4, 1>(src, dst, n, Ns, t0, tpl, w1, w2); break;
+                default: fft_step<T, PAD, SG, 5, 1>(src, dst, n, Ns, t0, tpl, w1, w2); break;
             }
         }
         __syncthreads();
         V *tmp = in;
         in = out;
         out = tmp;
-        toff += Ns * (R - 1);
-        koff += nb;
-        Ns *= R;
+        toff += Ns * (R1 - 1) + Ns * R1 * (R2 - 1);
+        Ns *= R1 * R2;
+        st += R2 > 1 ? 2 : 1;
     }
     return in;
 }
 
+// lines of a block: 128 bytes of a grid row in the strided passes
 template <typename T> __host__ __device__ constexpr int lines_per_cta() { return sizeof(T) == 8 ? 8 : 16; }
+template <typename T> __host__ __device__ constexpr int fft_threads() { return lines_per_cta<T>() * fft_tpl<T>(); }
+template <typename T> __host__ __device__ constexpr int fft_blocks() { return sizeof(T) == 8 ? 3 : 4; }
+
+template <typename T>
+__device__ __forceinline__ void load_twiddles(const typename C2<T>::t *g, typename C2<T>::t *tw, int n) {
+    for (int i = threadIdx.x; i < n - 1; i += blockDim.x) tw[i] = g[i];
+}
 
 // forward transform along z of (rho_a + i rho_b); lines = n*n per pair
-template <typename T>
-__global__ void __launch_bounds__(256) fft_z_forward_real(Plan pl, const T *__restrict__ rho, int k,
-                                                          typename C2<T>::t *__restrict__ work) {
+template <typename T, bool PAD>
+__global__ void __launch_bounds__(fft_threads<T>(), fft_blocks<T>())
+fft_z_forward_real(Plan pl, const typename C2<T>::t *__restrict__ twg, const T *__restrict__ rho, int k,
+                   typename C2<T>::t *__restrict__ work) {
     using V = typename C2<T>::t;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = pl.n, L = lines_per_cta<T>();
-    V *b0 = reinterpret_cast<V *>(smem_raw), *b1 = b0 + L * n, *tw = b1 + L * n;
-    unsigned char *kkt = reinterpret_cast<unsigned char *>(tw + n);
-    fft_tables<T>(pl, tw, kkt);
+    const int ld = PAD ? fft_ld<PAD>(n) : n;
+    V *b0 = reinterpret_cast<V *>(smem_raw), *b1 = b0 + L * ld, *tw = b1 + L * ld;
+    load_twiddles<T>(twg, tw, n);
     const long long n3 = (long long)n * n * n;
     const int pair = blockIdx.y;
-    const long long line0 = (long long)blockIdx.x * L;
-    const long long nlines = (long long)n * n;
-    const T *ra = rho + (2LL * pair) * n3;
+    const long long line0 = (long long)blockIdx.x * L, nlines = (long long)n * n, g0 = line0 * n;
     const bool has_b = 2 * pair + 1 < k;
-    const T *rb = rho + (2LL * pair + 1) * n3;
-    for (int i = threadIdx.x; i < L * n; i += blockDim.x) {
-        const int l = i / n, j = i - l * n;
+    const T *ra = rho + (2LL * pair) * n3 + g0, *rb = ra + n3;
+    V *w = work + (long long)pair * n3 + g0;
+    // a block's lines are one run of the grid: packed in shared memory the block takes consecutive points
+    // of the run, padded fft_tpl threads take a line
+    const int cnt = (int)(nlines - line0 < L ? (nlines - line0) * n : (long long)L * n);
+    auto load = [&](int i) {
         V v = {T(0), T(0)};
-        if (line0 + l < nlines) {
-            const long long gi = (line0 + l) * n + j;
-            v.x = ra[gi];
-            v.y = has_b ? rb[gi] : T(0);
+        if (i < cnt) {
+            v.x = ra[i];
+            v.y = has_b ? rb[i] : T(0);
         }
-        b0[i] = v;
+        return v;
+    };
+    const int row = threadIdx.x / fft_tpl<T>(), t0 = threadIdx.x % fft_tpl<T>();
+    if constexpr (PAD) {
+#pragma unroll 8
+        for (int j = t0; j < n; j += fft_tpl<T>()) b0[row * ld + fft_at<PAD>(j)] = load(row * n + j);
+    } else {
+#pragma unroll 4
+        for (int i = threadIdx.x; i < L * n; i += fft_threads<T>()) b0[i] = load(i);
     }
     __syncthreads();
-    V *res = fft_lines<T, -1>(b0, b1, L, n, pl, tw, kkt);
-    V *w = work + (long long)pair * n3;
-    for (int i = threadIdx.x; i < L * n; i += blockDim.x) {
-        const int l = i / n, j = i - l * n;
-        if (line0 + l < nlines) w[(line0 + l) * n + j] = res[i];
+    V *res = fft_lines<T, PAD, -1>(b0, b1, ld, pl, tw);
+    if constexpr (PAD) {
+        if (row * n < cnt)
+#pragma unroll 8
+            for (int j = t0; j < n; j += fft_tpl<T>()) w[row * n + j] = res[row * ld + fft_at<PAD>(j)];
+    } else {
+#pragma unroll 4
+        for (int i = threadIdx.x; i < cnt; i += fft_threads<T>()) w[i] = res[i];
     }
 }
 
 // inverse transform along z, then V = Re/Im + fxc * rho
-template <typename T>
-__global__ void __launch_bounds__(256) fft_z_inverse_real(Plan pl, const typename C2<T>::t *__restrict__ work,
-                                                          const T *__restrict__ rho,
-                                                          const T *__restrict__ fxc, int k,
-                                                          T *__restrict__ V) {
+template <typename T, bool PAD>
+__global__ void __launch_bounds__(fft_threads<T>(), fft_blocks<T>())
+fft_z_inverse_real(Plan pl, const typename C2<T>::t *__restrict__ twg, const typename C2<T>::t *__restrict__ work,
+                   const T *__restrict__ rho, const T *__restrict__ fxc, int k, T *__restrict__ V) {
     using Vc = typename C2<T>::t;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = pl.n, L = lines_per_cta<T>();
-    Vc *b0 = reinterpret_cast<Vc *>(smem_raw), *b1 = b0 + L * n, *tw = b1 + L * n;
-    unsigned char *kkt = reinterpret_cast<unsigned char *>(tw + n);
-    fft_tables<T>(pl, tw, kkt);
+    const int ld = PAD ? fft_ld<PAD>(n) : n;
+    Vc *b0 = reinterpret_cast<Vc *>(smem_raw), *b1 = b0 + L * ld, *tw = b1 + L * ld;
+    load_twiddles<T>(twg, tw, n);
     const long long n3 = (long long)n * n * n;
     const int pair = blockIdx.y;
-    const long long line0 = (long long)blockIdx.x * L;
-    const long long nlines = (long long)n * n;
-    const Vc *w = work + (long long)pair * n3;
-    for (int i = threadIdx.x; i < L * n; i += blockDim.x) {
-        const int l = i / n, j = i - l * n;
-        b0[i] = (line0 + l < nlines) ? w[(line0 + l) * n + j] : Vc{T(0), T(0)};
+    const long long line0 = (long long)blockIdx.x * L, nlines = (long long)n * n, g0 = line0 * n;
+    const bool has_b = 2 * pair + 1 < k;
+    const int cnt = (int)(nlines - line0 < L ? (nlines - line0) * n : (long long)L * n);
+    const Vc *w = work + (long long)pair * n3 + g0;
+    const int row = threadIdx.x / fft_tpl<T>(), t0 = threadIdx.x % fft_tpl<T>();
+    if constexpr (PAD) {
+#pragma unroll 8
+        for (int j = t0; j < n; j += fft_tpl<T>())
+            b0[row * ld + fft_at<PAD>(j)] = row * n + j < cnt ? w[row * n + j] : Vc{T(0), T(0)};
+    } else {
+#pragma unroll 4
+        for (int i = threadIdx.x; i < L * n; i += fft_threads<T>()) b0[i] = i < cnt ? w[i] : Vc{T(0), T(0)};
     }
     __syncthreads();
-    Vc *res = fft_lines<T, +1>(b0, b1, L, n, pl, tw, kkt);
-    const bool has_b = 2 * pair + 1 < k;
-    for (int i = threadIdx.x; i < L * n; i += blockDim.x) {
-        const int l = i / n, j = i - l * n;
-        if (line0 + l >= nlines) continue;
-        const long long gi = (line0 + l) * n + j;
-        const T f = fxc ? fxc[gi] : T(0);
-        const long long ia = (2LL * pair) * n3 + gi;
-        V[ia] = res[i].x + f * rho[ia];
-        if (has_b) {
-            const long long ib = (2LL * pair + 1) * n3 + gi;
-            V[ib] = res[i].y + f * rho[ib];
-        }
+    const Vc *res = fft_lines<T, PAD, +1>(b0, b1, ld, pl, tw);
+    const long long ia = (2LL * pair) * n3 + g0;
+    auto store = [&](int i, Vc r) {
+        const T f = fxc ? fxc[g0 + i] : T(0);
+        V[ia + i] = r.x + f * rho[ia + i];
+        if (has_b) V[ia + n3 + i] = r.y + f * rho[ia + n3 + i];
+    };
+    if constexpr (PAD) {
+        if (row * n < cnt)
+#pragma unroll 4
+            for (int j = t0; j < n; j += fft_tpl<T>()) store(row * n + j, res[row * ld + fft_at<PAD>(j)]);
+    } else {
+#pragma unroll 4
+        for (int i = threadIdx.x; i < cnt; i += fft_threads<T>()) store(i, res[i]);
     }
 }
 
 // transform along a strided axis (stride s: n for y, n*n for x) for a block of W consecutive
 // z columns; AXIS 1 = y, 0 = x. For the x axis the forward transform, the Poisson kernel
 // 4 pi / |G|^2 / n^3 (G = 0 -> 0) and the inverse transform are fused.
-template <typename T, int AXIS, int SG, bool POISSON>
-__global__ void __launch_bounds__(256) fft_strided(Plan pl, typename C2<T>::t *__restrict__ work,
-                                                   T two_pi_over_L) {
+template <typename T, bool PAD, int AXIS, int SG, bool POISSON>
+__global__ void __launch_bounds__(fft_threads<T>(), fft_blocks<T>())
+fft_strided(Plan pl, const typename C2<T>::t *__restrict__ twg, typename C2<T>::t *__restrict__ work, T two_pi_over_L) {
     using V = typename C2<T>::t;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int n = pl.n, W = lines_per_cta<T>();
-    // lines n + 1 apart: the transposing loads and stores (consecutive threads, consecutive
-    // lines) then hit distinct banks
-    const int ld = n + 1;
+    const int n = pl.n;
+    constexpr int W = lines_per_cta<T>();
+    const int ld = fft_ld<PAD>(n);
     V *b0 = reinterpret_cast<V *>(smem_raw), *b1 = b0 + W * ld, *tw = b1 + W * ld;
-    unsigned char *kkt = reinterpret_cast<unsigned char *>(tw + n);
-    fft_tables<T>(pl, tw, kkt);
+    load_twiddles<T>(twg, tw, n);
     const long long n3 = (long long)n * n * n;
     const int pair = blockIdx.z;
     const int o = blockIdx.y;            // x index (AXIS 1) or y index (AXIS 0)
     const int w0 = blockIdx.x * W;       // first z column
     const long long s = AXIS == 1 ? n : (long long)n * n;
     const long long base = (long long)pair * n3 + (AXIS == 1 ? (long long)o * n * n : (long long)o * n);
-    V *data = work + base;
-    for (int i = threadIdx.x; i < W * n; i += blockDim.x) {
-        const int j = i / W, w = i - j * W;    // consecutive threads -> consecutive z
+    // consecutive threads take consecutive z: column cw of every tpl-th point
+    const int cw = threadIdx.x % W, j0 = threadIdx.x / W;
+    const bool in = w0 + cw < n;
+    V *data = work + base + w0 + cw;
+#pragma unroll 8
+    for (int j = j0; j < n; j += fft_tpl<T>()) {
         V v = {T(0), T(0)};
-        if (w0 + w < n) v = data[(long long)j * s + w0 + w];
-        b0[w * ld + j] = v;
+        if (in) v = data[(long long)j * s];
+        b0[cw * ld + fft_at<PAD>(j)] = v;
     }
     __syncthreads();
     V *res;
     if (!POISSON) {
-        res = fft_lines<T, SG>(b0, b1, W, ld, pl, tw, kkt);
+        res = fft_lines<T, PAD, SG>(b0, b1, ld, pl, tw);
     } else {
-        res = fft_lines<T, -1>(b0, b1, W, ld, pl, tw, kkt);
+        res = fft_lines<T, PAD, -1>(b0, b1, ld, pl, tw);
         const T inv_n3 = T(1) / T(n3);
-        for (int i = threadIdx.x; i < W * n; i += blockDim.x) {
-            const int w = i / n, j = i - w * n;
+        const int w = threadIdx.x / fft_tpl<T>();
+        const int my = o <= n / 2 ? o : o - n;
+        const int zz = w0 + w;
+        const int mz = zz <= n / 2 ? zz : zz - n;
+        for (int j = threadIdx.x % fft_tpl<T>(); j < n; j += fft_tpl<T>()) {
             const int mx = j <= n / 2 ? j : j - n;
-            const int my = o <= n / 2 ? o : o - n;
-            const int zz = w0 + w;
-            const int mz = zz <= n / 2 ? zz : zz - n;
             const T g2 = two_pi_over_L * two_pi_over_L * T(mx * mx + my * my + mz * mz);
             const T kern = (mx == 0 && my == 0 && mz == 0) ? T(0) : T(4.0 * 3.14159265358979323846) / g2 * inv_n3;
-            res[w * ld + j].x *= kern;
-            res[w * ld + j].y *= kern;
+            V &x = res[w * ld + fft_at<PAD>(j)];
+            x.x *= kern;
+            x.y *= kern;
         }
         __syncthreads();
         V *other = (res == b0) ? b1 : b0;
-        res = fft_lines<T, +1>(res, other, W, ld, pl, tw, kkt);
+        res = fft_lines<T, PAD, +1>(res, other, ld, pl, tw);
     }
-    for (int i = threadIdx.x; i < W * n; i += blockDim.x) {
-        const int j = i / W, w = i - j * W;
-        if (w0 + w < n) data[(long long)j * s + w0 + w] = res[w * ld + j];
-    }
+#pragma unroll 8
+    for (int j = j0; j < n; j += fft_tpl<T>())
+        if (in) data[(long long)j * s] = res[cw * ld + fft_at<PAD>(j)];
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -560,42 +634,65 @@ void potential_integrals(cudaStream_t st, const GridShape &g, const TileSet<T> &
 }
 
 template <typename T>
-void hartree_fxc(cudaStream_t st, const GridShape &g, const T *rho, const T *fxc, int k, T *V,
-                 void *work) {
-    if (k <= 0) return;
-    using Vc = typename C2<T>::t;
+void fft_twiddles(cudaStream_t st, int n, T *tw) {
     Plan pl;
-    if (!make_plan(g.n, pl)) throw CudaError{cudaErrorInvalidValue, "FFT size not 2/3/5-smooth"};
-    const int n = g.n, L = lines_per_cta<T>();
-    const int pairs = (k + 1) / 2;
-    const double n3d = (double)n * n * n;
-    ProfScope ps(st, ST_FFT, pairs * 2.0 * 5.0 * n3d * std::log2(n3d), sizeof(T) * (2.0 * k + 1.0) * n3d);
-    const size_t sm = (2 * (size_t)L * (n + 1) + n) * sizeof(Vc) + FFT_KK_BYTES;
+    if (!make_plan(n, pl)) throw CudaError{cudaErrorInvalidValue, "FFT size not 2/3/5-smooth"};
+    fft_twiddles_kernel<T><<<1, 256, 0, st>>>(pl, reinterpret_cast<typename C2<T>::t *>(tw));
+    check_launch("fft_twiddles_kernel");
+}
+template void fft_twiddles<float>(cudaStream_t, int, float *);
+template void fft_twiddles<double>(cudaStream_t, int, double *);
+
+namespace {
+template <typename T, bool PAD>
+void poisson(cudaStream_t st, const GridShape &g, const Plan &pl, const T *rho, const T *fxc, int k, T *V,
+             typename C2<T>::t *w, const typename C2<T>::t *tw) {
+    using Vc = typename C2<T>::t;
+    const int n = g.n, L = lines_per_cta<T>(), pairs = (k + 1) / 2;
+    constexpr int NT = fft_threads<T>();
+    const size_t sm = (2 * (size_t)L * fft_ld<PAD>(n) + n) * sizeof(Vc);
     static const bool attr = [&]() {   // once per process, thread-safe
-        const int mx = (2 * L * 257 + 256) * (int)sizeof(Vc) + FFT_KK_BYTES;
-        check(cudaFuncSetAttribute(fft_z_forward_real<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr fz");
-        check(cudaFuncSetAttribute(fft_z_inverse_real<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr iz");
-        check(cudaFuncSetAttribute(fft_strided<T, 1, -1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr fy");
-        check(cudaFuncSetAttribute(fft_strided<T, 1, +1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr iy");
-        check(cudaFuncSetAttribute(fft_strided<T, 0, -1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr x");
+        const int mx = (2 * L * fft_ld<PAD>(256) + 256) * (int)sizeof(Vc);
+        check(cudaFuncSetAttribute(fft_z_forward_real<T, PAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr fz");
+        check(cudaFuncSetAttribute(fft_z_inverse_real<T, PAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr iz");
+        check(cudaFuncSetAttribute(fft_strided<T, PAD, 1, -1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr fy");
+        check(cudaFuncSetAttribute(fft_strided<T, PAD, 1, +1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr iy");
+        check(cudaFuncSetAttribute(fft_strided<T, PAD, 0, -1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr x");
         return true;
     }();
     (void)attr;
-    Vc *w = reinterpret_cast<Vc *>(work);
     const long long nlines = (long long)n * n;
     dim3 gz((unsigned)((nlines + L - 1) / L), pairs);
     dim3 gs((n + L - 1) / L, n, pairs);
     const T tpl = T(2.0 * 3.14159265358979323846 / g.cell);
-    fft_z_forward_real<T><<<gz, 256, sm, st>>>(pl, rho, k, w);
+    fft_z_forward_real<T, PAD><<<gz, NT, sm, st>>>(pl, tw, rho, k, w);
     check_launch("fft_z_forward_real");
-    fft_strided<T, 1, -1, false><<<gs, 256, sm, st>>>(pl, w, tpl);
+    fft_strided<T, PAD, 1, -1, false><<<gs, NT, sm, st>>>(pl, tw, w, tpl);
     check_launch("fft_y_forward");
-    fft_strided<T, 0, -1, true><<<gs, 256, sm, st>>>(pl, w, tpl);
+    fft_strided<T, PAD, 0, -1, true><<<gs, NT, sm, st>>>(pl, tw, w, tpl);
     check_launch("fft_x_poisson");
-    fft_strided<T, 1, +1, false><<<gs, 256, sm, st>>>(pl, w, tpl);
+    fft_strided<T, PAD, 1, +1, false><<<gs, NT, sm, st>>>(pl, tw, w, tpl);
     check_launch("fft_y_inverse");
-    fft_z_inverse_real<T><<<gz, 256, sm, st>>>(pl, w, rho, fxc, k, V);
+    fft_z_inverse_real<T, PAD><<<gz, NT, sm, st>>>(pl, tw, w, rho, fxc, k, V);
     check_launch("fft_z_inverse_real");
+}
+}  // namespace
+
+template <typename T>
+void hartree_fxc(cudaStream_t st, const GridShape &g, const T *rho, const T *fxc, int k, T *V,
+                 void *work, const T *tw) {
+    if (k <= 0) return;
+    using Vc = typename C2<T>::t;
+    Plan pl;
+    if (!make_plan(g.n, pl)) throw CudaError{cudaErrorInvalidValue, "FFT size not 2/3/5-smooth"};
+    const int pairs = (k + 1) / 2;
+    const double n3d = (double)g.n * g.n * g.n;
+    ProfScope ps(st, ST_FFT, pairs * 2.0 * 5.0 * n3d * std::log2(n3d), sizeof(T) * (2.0 * k + 1.0) * n3d);
+    Vc *w = reinterpret_cast<Vc *>(work);
+    const Vc *twv = reinterpret_cast<const Vc *>(tw);
+    // the first pair of stages: 4 x 4 or 4 x 2 where n is a multiple of 8
+    if (sizeof(T) == 4 && g.n % 8 == 0) poisson<T, true>(st, g, pl, rho, fxc, k, V, w, twv);
+    else poisson<T, false>(st, g, pl, rho, fxc, k, V, w, twv);
 }
 
 void fxc_lda(cudaStream_t st, const double *n0, double *fxc, long long npts) {
@@ -616,8 +713,8 @@ template void potential_integrals<double>(cudaStream_t, const GridShape &, const
                                           const TileSet<double> &, int, int, const double *, int,
                                           double *);
 template void hartree_fxc<float>(cudaStream_t, const GridShape &, const float *, const float *, int,
-                                 float *, void *);
+                                 float *, void *, const float *);
 template void hartree_fxc<double>(cudaStream_t, const GridShape &, const double *, const double *,
-                                  int, double *, void *);
+                                  int, double *, void *, const double *);
 
 }  // namespace tddft

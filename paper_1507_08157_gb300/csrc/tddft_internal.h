@@ -171,10 +171,13 @@ template <typename T>
 void potential_integrals(cudaStream_t st, const GridShape &g, const TileSet<T> &chi,
                          const TileSet<T> &phi, int nchi, int nphi, const T *V, int k, T *out);
 
-// V_s = v_H[rho_s] + fxc * rho_s for k states; work: complex buffer of ceil(k/2) * n^3
+// V_s = v_H[rho_s] + fxc * rho_s for k states; work: complex buffer of ceil(k/2) * n^3; tw: the grid
+// size's twiddles from fft_twiddles (2 n values of T)
 template <typename T>
 void hartree_fxc(cudaStream_t st, const GridShape &g, const T *rho, const T *fxc, int k, T *V,
-                 void *work);
+                 void *work, const T *tw);
+template <typename T>
+void fft_twiddles(cudaStream_t st, int n, T *tw);
 
 void fxc_lda(cudaStream_t st, const double *n0, double *fxc, long long npts);
 
