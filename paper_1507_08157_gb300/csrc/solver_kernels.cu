@@ -479,10 +479,21 @@ int grid_for(long long n) {
 // ------------------------------------------------------------------------------------------------
 // Small float64 algebra for one thread block (k <= KMAX, so k * k <= 256 threads hold one matrix
 // element each). Matrices live in shared memory; every routine is entered and left by all
-// threads of the block, and the steps that must follow one another (pivots, Gram-Schmidt
-// vectors) are the only sequential parts: float64 latency and block barriers are what this
-// code costs on this part, not arithmetic.
+// threads of the block. A float64 instruction of a warp takes 64 cycles whatever its active lanes,
+// 77 with a warp on every scheduler and 153 with two (measured; a division or rsqrt 5.5 times that, a
+// comparison as much as a sum). The number of float64 instructions in sequence is what this code
+// costs: blocks have one warp per 32 matrix elements, chains are spread over lanes, tests for
+// sign and finiteness read the bits, and a rotation's angle is float32. Ten states: start 900 us in
+// one thread, 10 here; Ritz values 172 and 64; line step with Gram-Schmidt, 60 evaluations, 418 and
+// 314; one state: line step 58 and 37.
 constexpr int SB_THREADS = 256;
+inline int sb_threads(int k) { return (k * k + 31) / 32 * 32; }
+
+__device__ __forceinline__ bool sb_positive(double x) {      // x > 0, by its bits
+    const long long b = __double_as_longlong(x);
+    return b > 0 && b <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool sb_finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
 struct SbLine {
     double N0[KMAX * KMAX], N1[KMAX * KMAX], N2[KMAX * KMAX];
@@ -490,88 +501,65 @@ struct SbLine {
     double A[2][KMAX * KMAX];              // M, reduced in place to M^-1 (two buffers)
     double dM[KMAX * KMAX], N[KMAX * KMAX], dN[KMAX * KMAX];
     double T[KMAX * KMAX], Z[KMAX * KMAX];
-    double red[SB_THREADS / 32][3];
+    double red[SB_THREADS / 32];
     double out[4];
     int bad;
 };
 
-// Omega(lam) = Tr[M^-1 N]/2 and dOmega/dlam = Tr[M^-1 dN - M^-1 dM M^-1 N]/2 with
+// dOmega/dlam of Omega(lam) = Tr[M^-1 N]/2, that is Tr[M^-1 dN - M^-1 dM M^-1 N]/2, with
 // M = M0 + lam M1 + lam^2 M2, N likewise; false (in every thread) if M is not positive definite.
 // M^-1 by Gauss-Jordan elimination without pivoting, one pivot per step with every element
 // updated at once: for a symmetric M the pivots are those of its L D L^T factorisation, so all
 // are positive exactly when M is positive definite. The traces are element-wise sums
 // (Tr[A B] = sum_ij A_ij B_ji), so only W = M^-1 N and U = M^-1 dM are formed:
-// Omega = Tr[W]/2, dOmega = (sum_ij Minv_ij dN_ji - sum_ij U_ij W_ji)/2.
-__device__ bool sb_sum_functional(int k, SbLine &s, double lam, double *f, double *d) {
+// dOmega = (sum_ij Minv_ij dN_ji - sum_ij U_ij W_ji)/2.
+__device__ bool sb_sum_functional(int k, SbLine &s, double lam, double *d) {
     const int t = threadIdx.x, kk = k * k;
     const int i = t < kk ? t / k : 0, j = t < kk ? t - i * k : 0;
+    double dn = 0.0;
     if (t < kk) {
-        s.A[0][t] = s.M0[t] + lam * s.M1[t] + lam * lam * s.M2[t];
-        s.dM[t] = s.M1[t] + 2.0 * lam * s.M2[t];
-        s.N[t] = s.N0[t] + lam * s.N1[t] + lam * lam * s.N2[t];
-        s.dN[t] = s.N1[t] + 2.0 * lam * s.N2[t];
+        s.A[0][t] = fma(lam, fma(lam, s.M2[t], s.M1[t]), s.M0[t]);
+        s.dM[t] = fma(lam + lam, s.M2[t], s.M1[t]);
+        s.N[t] = fma(lam, fma(lam, s.N2[t], s.N1[t]), s.N0[t]);
+        dn = fma(lam + lam, s.N2[t], s.N1[t]);          // symmetric: dN_ji
     }
     __syncthreads();
     int cur = 0;
     for (int p = 0; p < k; ++p) {
         const double *a = s.A[cur];
         const double piv = a[p * k + p];
-        if (!(piv > 0.0)) {                 // the same value in every thread
+        if (!sb_positive(piv)) {            // the same value in every thread
             __syncthreads();
             return false;
         }
         if (t < kk) {
-            const double r = 1.0 / piv;
-            double v;
-            if (i == p) v = (j == p) ? r : a[t] * r;
-            else if (j == p) v = -a[t] * r;
-            else v = a[t] - a[i * k + p] * a[p * k + j] * r;
-            s.A[cur ^ 1][t] = v;
+            // every element as base + x y: 1/piv, a_pj/piv, -a_ip/piv, a_ij - a_ip a_pj/piv
+            const double r = 1.0 / piv, pj = a[p * k + j] * r;
+            const double base = i == p || j == p ? 0.0 : a[t], x = i == p ? 1.0 : -a[i * k + p];
+            s.A[cur ^ 1][t] = fma(x, j == p ? r : pj, base);
         }
         cur ^= 1;
         __syncthreads();
     }
     const double *mi = s.A[cur];
+    double w = 0.0, u = 0.0;
     if (t < kk) {
-        double w = 0.0, u = 0.0;
         for (int q = 0; q < k; ++q) {
-            w += mi[i * k + q] * s.N[q * k + j];
-            u += mi[i * k + q] * s.dM[q * k + j];
+            w = fma(mi[i * k + q], s.N[q * k + j], w);
+            u = fma(mi[i * k + q], s.dM[q * k + j], u);
         }
-        s.T[t] = w;
-        s.Z[t] = u;
+        s.T[j * k + i] = w;
     }
     __syncthreads();
-    double v0 = 0.0, v1 = 0.0, v2 = 0.0;
-    if (t < kk) {
-        v0 = i == j ? s.T[t] : 0.0;
-        v1 = mi[t] * s.dN[j * k + i];
-        v2 = s.Z[t] * s.T[j * k + i];
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        v0 += __shfl_xor_sync(0xffffffffu, v0, o);
-        v1 += __shfl_xor_sync(0xffffffffu, v1, o);
-        v2 += __shfl_xor_sync(0xffffffffu, v2, o);
-    }
-    if ((t & 31) == 0) {
-        s.red[t >> 5][0] = v0;
-        s.red[t >> 5][1] = v1;
-        s.red[t >> 5][2] = v2;
+    if ((t & ~31) < kk) {
+        double v = t < kk ? fma(mi[t], dn, -u * s.T[t]) : 0.0;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((t & 31) == 0) s.red[t >> 5] = v;
     }
     __syncthreads();
-    if (t == 0) {
-        double tw = 0.0, tx = 0.0, tz = 0.0;
-        for (int w = 0; w < (kk + 31) / 32; ++w) {
-            tw += s.red[w][0];
-            tx += s.red[w][1];
-            tz += s.red[w][2];
-        }
-        s.out[0] = 0.5 * tw;
-        s.out[1] = 0.5 * (tx - tz);
-    }
-    __syncthreads();
-    *f = s.out[0];
-    *d = s.out[1];
+    double v = 0.0;
+    for (int q = 0; q < (kk + 31) / 32; ++q) v += s.red[q];
+    *d = 0.5 * v;
     __syncthreads();
     return true;
 }
@@ -581,8 +569,8 @@ __device__ bool sb_sum_functional(int k, SbLine &s, double lam, double *f, doubl
 // root, bisection while M is indefinite at the upper end, then Illinois regula falsi on dOmega
 // to machine precision
 __device__ double sb_line_step(int k, SbLine &s) {
-    double f0, d0;
-    if (!sb_sum_functional(k, s, 0.0, &f0, &d0) || !isfinite(d0) || d0 >= 0.0) return 0.0;
+    double d0;
+    if (!sb_sum_functional(k, s, 0.0, &d0) || !isfinite(d0) || d0 >= 0.0) return 0.0;
     const int t = threadIdx.x;
     // h0 = Tr[2 N2 - 2 M1 N1 + 2 M1 M1 N0 - 2 M2 N0] / 2, one row per thread, summed in order
     if (t < k) {
@@ -607,18 +595,19 @@ __device__ double sb_line_step(int k, SbLine &s) {
     const double h0 = s.out[2];
     __syncthreads();
     double hi = (h0 > 0.0 && isfinite(h0)) ? -d0 / h0 : 1.0;
-    double lo = 0.0, dlo = d0, dhi = 0.0, f, d = d0;
-    for (int it = 0; it < 60; ++it) {
-        if (!sb_sum_functional(k, s, hi, &f, &d)) d = INFINITY;
+    double lo = 0.0, dlo = d0, dhi = 0.0, d = d0;
+    for (int it = 0; it < 21; ++it) {
+        if (!sb_sum_functional(k, s, hi, &d)) d = INFINITY;
         if (d >= 0.0) break;
         lo = hi;
         dlo = d;
-        hi = 2.0 * hi;
+        // past 2^8 estimates the minimum is at the direction's end of the line but for rounding
+        hi = (it < 8 ? 2.0 : 16.0) * hi;
     }
     dhi = d;
     for (int b = 0; b < 200 && !isfinite(dhi); ++b) {
         const double mid = 0.5 * (lo + hi);
-        if (!sb_sum_functional(k, s, mid, &f, &d)) d = INFINITY;
+        if (!sb_sum_functional(k, s, mid, &d)) d = INFINITY;
         if (d < 0.0) { lo = mid; dlo = d; }
         else { hi = mid; dhi = d; }
     }
@@ -627,7 +616,7 @@ __device__ double sb_line_step(int k, SbLine &s) {
         if (!(hi - lo > 4e-16 * hi)) break;
         double x = (isfinite(dhi) && dhi != dlo) ? hi - dhi * (hi - lo) / (dhi - dlo) : 0.5 * (lo + hi);
         if (!(x > lo && x < hi)) x = 0.5 * (lo + hi);
-        if (!sb_sum_functional(k, s, x, &f, &d)) d = INFINITY;
+        if (!sb_sum_functional(k, s, x, &d)) d = INFINITY;
         if (d == 0.0) return x;
         if (d < 0.0) {
             lo = x;
@@ -644,12 +633,26 @@ __device__ double sb_line_step(int k, SbLine &s) {
     return 0.5 * (lo + hi);
 }
 
+// sum over q < n of f(q) for row r = t / G by G lanes (a power of two): every lane of the row has it
+template <typename F>
+__device__ __forceinline__ double sb_row_sum(int G, int n, F f) {
+    const int l = threadIdx.x & (G - 1);
+    double acc = 0.0;
+    for (int q = l; q < n; q += G) acc += f(q);
+    for (int o = G >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    return acc;
+}
+
 // Classical Gram-Schmidt run twice on coefficient vectors in the metric Mg, vectors taken in
 // the given order; rows of C are the new vectors. u and coef are k-vectors of work space.
-// False (in every thread) if a norm is not positive.
+// False (in every thread) if a norm is not positive. Every product takes G lanes a row.
 __device__ bool sb_gram_schmidt(int k, const double *Mg, const int *order, double *C, double *v,
                                 double *u, double *coef, int *bad) {
     const int t = threadIdx.x;
+    int G = 1;
+    while (2 * G * k <= (int)blockDim.x && G < 16) G *= 2;
+    const int r = t / G;
+    const bool own = r < k, first = own && (t & (G - 1)) == 0;
     if (t < k * k) C[t] = 0.0;
     if (t == 0) *bad = 0;
     __syncthreads();
@@ -658,37 +661,26 @@ __device__ bool sb_gram_schmidt(int k, const double *Mg, const int *order, doubl
         if (t < k) v[t] = (t == i) ? 1.0 : 0.0;
         __syncthreads();
         for (int pass = 0; pass < 2; ++pass) {
-            if (t < k) {                    // u = Mg v
-                double acc = 0.0;
-                for (int q = 0; q < k; ++q) acc += Mg[t * k + q] * v[q];
-                u[t] = acc;
-            }
+            // u = Mg v
+            const double x = sb_row_sum(G, own ? k : 0, [&](int q) { return Mg[r * k + q] * v[q]; });
+            if (first) u[r] = x;
             __syncthreads();
-            if (t < a) {                    // coef_b = <v, C_order[b]>_Mg
-                const int j = order[t];
-                double acc = 0.0;
-                for (int p = 0; p < k; ++p) acc += C[j * k + p] * u[p];
-                coef[t] = acc;
-            }
+            // coef_b = <v, C_order[b]>_Mg
+            const int j = r < a ? order[r] : 0;
+            const double y = sb_row_sum(G, r < a ? k : 0, [&](int q) { return C[j * k + q] * u[q]; });
+            if (first && r < a) coef[r] = y;
             __syncthreads();
-            if (t < k) {
-                double x = v[t];
-                for (int b = 0; b < a; ++b) x -= coef[b] * C[order[b] * k + t];
-                v[t] = x;
-            }
+            const double z = sb_row_sum(G, own ? a : 0, [&](int b) { return coef[b] * C[order[b] * k + r]; });
+            if (first) v[r] -= z;
             __syncthreads();
         }
-        if (t < k) {
-            double acc = 0.0;
-            for (int q = 0; q < k; ++q) acc += Mg[t * k + q] * v[q];
-            u[t] = acc;
-        }
+        const double x = sb_row_sum(G, own ? k : 0, [&](int q) { return Mg[r * k + q] * v[q]; });
+        if (first) u[r] = x;
         __syncthreads();
+        const double nrm = sb_row_sum(G, k, [&](int q) { return v[q] * u[q]; });
         if (t == 0) {
-            double nrm = 0.0;
-            for (int p = 0; p < k; ++p) nrm += v[p] * u[p];
             const double ref = fabs(Mg[i * k + i]) > 1.0 ? fabs(Mg[i * k + i]) : 1.0;
-            if (!isfinite(nrm) || nrm <= 1e-12 * ref) *bad = 1;
+            if (!sb_finite(nrm) || nrm <= 1e-12 * ref) *bad = 1;
             coef[KMAX] = *bad ? 0.0 : rsqrt(nrm);
         }
         __syncthreads();
@@ -702,24 +694,39 @@ __device__ bool sb_gram_schmidt(int k, const double *Mg, const int *order, doubl
 // Eigenvalues of a symmetric k x k matrix, ascending, into w (written by thread 0); a is
 // overwritten. Jacobi sweeps in round-robin (tournament) order: the k (padded to even m) indices
 // meet in m - 1 rounds of m / 2 disjoint pairs, and a round's rotations commute, so their angles
-// are computed in parallel and applied together (columns, then rows). cs holds 2 KMAX + 1 values.
+// are computed in parallel and applied together (columns, then rows). The angle is a float32 one
+// (it only decides how much of a_pq is left for the next sweep); its cosine and sine are float64, so
+// that the rotation is orthogonal to rounding. The matrix is scaled to entries of at most 2 by a
+// power of two, within float32's range. cs holds 2 KMAX + 2 values.
 __device__ void sb_jacobi_eigenvalues(int k, double *a, double *w, double *cs) {
-    const int t = threadIdx.x;
+    __shared__ int emax;
+    __shared__ float red[2][SB_THREADS / 32];
+    const int t = threadIdx.x, kk = k * k;
     const int m = k + (k & 1), half = m / 2;
+    if (t == 0) emax = 1;
+    __syncthreads();
+    if (t < kk) atomicMax(&emax, min((__double2hiint(a[t]) >> 20) & 0x7ff, 2045));
+    __syncthreads();
+    const double unscale = __hiloint2double(emax << 20, 0);
+    if (t < kk) a[t] *= __hiloint2double((2046 - emax) << 20, 0);
+    __syncthreads();
+    const int ti = t < kk ? t / k : 0, tj = t < kk ? t - ti * k : 0;      // element
+    const int pr = t / k, row = t - pr * k;                               // pair and row (column)
     for (int sweep = 0; sweep < 60; ++sweep) {
-        if (t == 0) {
-            double off = 0.0, tot = 0.0;
-            for (int i = 0; i < k; ++i)
-                for (int j = 0; j < k; ++j) {
-                    tot += a[i * k + j] * a[i * k + j];
-                    if (i != j) off += a[i * k + j] * a[i * k + j];
-                }
-            cs[2 * KMAX] = (off <= 1e-30 * tot || off == 0.0) ? 1.0 : 0.0;
+        float off = 0.0f, tot = 0.0f;
+        if (t < kk) {
+            tot = (float)(a[t] * a[t]);
+            off = ti == tj ? 0.0f : tot;
         }
+        for (int o = 16; o > 0; o >>= 1) {
+            tot += __shfl_xor_sync(0xffffffffu, tot, o);
+            off += __shfl_xor_sync(0xffffffffu, off, o);
+        }
+        if ((t & 31) == 0) red[0][t >> 5] = tot, red[1][t >> 5] = off;
         __syncthreads();
-        const bool done = cs[2 * KMAX] != 0.0;
-        __syncthreads();
-        if (done) break;
+        tot = off = 0.0f;
+        for (int q = 0; q < (kk + 31) / 32; ++q) tot += red[0][q], off += red[1][q];
+        if (off <= 1e-30f * tot || off == 0.0f) break;
         for (int r = 0; r < m - 1; ++r) {
             if (t < half) {
                 // pair t of round r: index m - 1 meets r, the others pair up around the circle
@@ -727,47 +734,37 @@ __device__ void sb_jacobi_eigenvalues(int k, double *a, double *w, double *cs) {
                 int q = t == 0 ? r : (r - t + m - 1) % (m - 1);
                 if (p > q) { const int x = p; p = q; q = x; }
                 double c = 1.0, sn = 0.0;
-                if (q < k) {
-                    const double apq = a[p * k + q];
-                    if (apq != 0.0) {
-                        const double theta = (a[q * k + q] - a[p * k + p]) / (2.0 * apq);
-                        const double tt = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-                        c = rsqrt(tt * tt + 1.0);
-                        sn = tt * c;
-                    }
+                const float apq = q < k ? (float)a[p * k + q] : 0.0f;
+                if (apq != 0.0f) {
+                    const float theta = (float)(a[q * k + q] - a[p * k + p]) / (2.0f * apq);
+                    const double tt = (double)((theta >= 0.0f ? 1.0f : -1.0f) / (fabsf(theta) + sqrtf(theta * theta + 1.0f)));
+                    c = rsqrt(fma(tt, tt, 1.0));
+                    sn = tt * c;
                 }
                 cs[2 * t] = c;
                 cs[2 * t + 1] = sn;
             }
             __syncthreads();
-            if (t < half * k) {             // columns p, q of row t % k for pair t / k
-                const int pr = t / k, row = t - pr * k;
-                int p = pr == 0 ? m - 1 : (r + pr) % (m - 1);
-                int q = pr == 0 ? r : (r - pr + m - 1) % (m - 1);
-                if (p > q) { const int x = p; p = q; q = x; }
-                const double c = cs[2 * pr], sn = cs[2 * pr + 1];
-                if (q < k && sn != 0.0) {
-                    const double arp = a[row * k + p], arq = a[row * k + q];
-                    a[row * k + p] = c * arp - sn * arq;
-                    a[row * k + q] = sn * arp + c * arq;
-                }
+            int p = pr == 0 ? m - 1 : (r + pr) % (m - 1);
+            int q = pr == 0 ? r : (r - pr + m - 1) % (m - 1);
+            if (p > q) { const int x = p; p = q; q = x; }
+            const bool on = pr < half && q < k && cs[2 * pr + 1] != 0.0;
+            const double c = on ? cs[2 * pr] : 1.0, sn = on ? cs[2 * pr + 1] : 0.0;
+            if (on) {                       // columns p, q of this row
+                const double x = a[row * k + p], y = a[row * k + q];
+                a[row * k + p] = c * x - sn * y;
+                a[row * k + q] = sn * x + c * y;
             }
             __syncthreads();
-            if (t < half * k) {             // rows p, q of column t % k for pair t / k
-                const int pr = t / k, col = t - pr * k;
-                int p = pr == 0 ? m - 1 : (r + pr) % (m - 1);
-                int q = pr == 0 ? r : (r - pr + m - 1) % (m - 1);
-                if (p > q) { const int x = p; p = q; q = x; }
-                const double c = cs[2 * pr], sn = cs[2 * pr + 1];
-                if (q < k && sn != 0.0) {
-                    const double apr = a[p * k + col], aqr = a[q * k + col];
-                    a[p * k + col] = c * apr - sn * aqr;
-                    a[q * k + col] = sn * apr + c * aqr;
-                }
+            if (on) {                       // rows p, q of this column
+                const double x = a[p * k + row], y = a[q * k + row];
+                a[p * k + row] = c * x - sn * y;
+                a[q * k + row] = sn * x + c * y;
             }
             __syncthreads();
         }
     }
+    __syncthreads();
     if (t == 0) {
         for (int i = 0; i < k; ++i) w[i] = a[i * k + i];
         for (int i = 1; i < k; ++i) {
@@ -779,40 +776,9 @@ __device__ void sb_jacobi_eigenvalues(int k, double *a, double *w, double *cs) {
             }
             w[j + 1] = x;
         }
+        for (int i = 0; i < k; ++i) w[i] *= unscale;
     }
     __syncthreads();
-}
-
-// classical Gram-Schmidt twice on coefficient vectors; rows of C are the new vectors
-__device__ bool gram_schmidt(int k, const double *Mg, const int *order, double *C) {
-    for (int i = 0; i < k * k; ++i) C[i] = 0.0;
-    for (int a = 0; a < k; ++a) {
-        const int i = order[a];
-        double v[KMAX];
-        for (int j = 0; j < k; ++j) v[j] = (j == i) ? 1.0 : 0.0;
-        for (int pass = 0; pass < 2; ++pass) {
-            double coef[KMAX];
-            for (int b = 0; b < a; ++b) {
-                const int j = order[b];
-                double s = 0.0;
-                for (int p = 0; p < k; ++p)
-                    for (int q = 0; q < k; ++q) s += v[p] * Mg[p * k + q] * C[j * k + q];
-                coef[b] = s;
-            }
-            for (int b = 0; b < a; ++b) {
-                const int j = order[b];
-                for (int p = 0; p < k; ++p) v[p] -= coef[b] * C[j * k + p];
-            }
-        }
-        double nrm = 0.0;
-        for (int p = 0; p < k; ++p)
-            for (int q = 0; q < k; ++q) nrm += v[p] * Mg[p * k + q] * v[q];
-        const double ref = fabs(Mg[i * k + i]) > 1.0 ? fabs(Mg[i * k + i]) : 1.0;
-        if (!isfinite(nrm) || nrm <= 1e-12 * ref) return false;
-        const double inv = 1.0 / sqrt(nrm);
-        for (int p = 0; p < k; ++p) C[i * k + p] = v[p] * inv;
-    }
-    return true;
 }
 
 // ---- kernels ----------------------------------------------------------------------------------
@@ -844,12 +810,12 @@ __global__ void __launch_bounds__(SB_THREADS) eval_finish_kernel(int k, const do
     if (t < kk) {
         const int i = t / k, j = t - i * k;
         S[t] = 0.5 * (Q[i * k + j] + Q[j * k + i]);
-        if (!isfinite(S[t])) bad = 1;
+        if (!sb_finite(S[t])) bad = 1;
     }
     if (t < k) {
         const double r2 = d[t] + d[k + t];
         out[k + t] = sqrt(r2 > 0.0 ? r2 : 0.0);
-        if (!isfinite(r2)) bad = 1;
+        if (!sb_finite(r2)) bad = 1;
     }
     __syncthreads();
     if (bad) {
@@ -891,7 +857,7 @@ __global__ void conj_kernel(int k2, const double *gz_d, const double *gzp_d, con
 // Outputs: lam[0]; Cp, Cq [k][k] combination coefficients (sign flips folded into Cq);
 // flip_any -> sc_flip[0]; status.
 
-// Line step and re-orthonormalisation for one thread block of SB_THREADS threads
+// Line step and re-orthonormalisation for one thread block
 __global__ void __launch_bounds__(SB_THREADS) line_gs_kernel(int k, const double *A, const double *BDf,
                                                              const double *CDfD, const double *PP,
                                                              const double *PD, const double *DP,
@@ -926,8 +892,8 @@ __global__ void __launch_bounds__(SB_THREADS) line_gs_kernel(int k, const double
         s.M0[t] = 0.5 * (T0[t] + T0[j * k + i]);
         s.M1[t] = 0.5 * (T1[t] + T1[j * k + i]);
         s.M2[t] = 0.5 * (T2[t] + T2[j * k + i]);
-        if (!isfinite(s.N0[t]) || !isfinite(s.N1[t]) || !isfinite(s.N2[t]) || !isfinite(s.M1[t]) ||
-            !isfinite(s.M2[t]))
+        if (!sb_finite(s.N0[t]) || !sb_finite(s.N1[t]) || !sb_finite(s.N2[t]) || !sb_finite(s.M1[t]) ||
+            !sb_finite(s.M2[t]))
             flags[0] = 1;
     }
     __syncthreads();
@@ -975,28 +941,36 @@ __global__ void __launch_bounds__(SB_THREADS) line_gs_kernel(int k, const double
 }
 
 // initial orthonormalisation: T0 from PP only, identity order
-__global__ void init_gs_kernel(int k, const double *PP, double *Cp, double *Cq, int *status) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const int k2 = 2 * k;
-    double sg[KMAX], Mg[KMAX * KMAX];
-    for (int i = 0; i < k; ++i) sg[i] = PP[i * k2 + k + i] < 0.0 ? -1.0 : 1.0;
-    for (int i = 0; i < k; ++i)
-        for (int j = 0; j < k; ++j) {
-            const double tij = PP[i * k2 + k + j] * sg[j], tji = PP[j * k2 + k + i] * sg[i];
-            Mg[i * k + j] = 0.5 * (tij + tji);
-            if (!isfinite(Mg[i * k + j])) {
-                *status = DEV_NAN_INIT;
-                return;
-            }
-        }
-    int order[KMAX];
-    for (int i = 0; i < k; ++i) order[i] = i;
-    if (!gram_schmidt(k, Mg, order, Cp)) {
-        *status = DEV_BREAKDOWN;
+__global__ void __launch_bounds__(SB_THREADS) init_gs_kernel(int k, const double *PP, double *Cp, double *Cq,
+                                                             int *status) {
+    __shared__ double Mg[KMAX * KMAX], C[KMAX * KMAX], sg[KMAX], v[KMAX], u[KMAX], coef[KMAX + 1];
+    __shared__ int order[KMAX], bad;
+    const int t = threadIdx.x, k2 = 2 * k, kk = k * k;
+    const int i = t < kk ? t / k : 0, j = t < kk ? t - i * k : 0;
+    if (t == 0) bad = 0;
+    if (t < k) {
+        sg[t] = PP[t * k2 + k + t] < 0.0 ? -1.0 : 1.0;
+        order[t] = t;
+    }
+    __syncthreads();
+    if (t < kk) {
+        Mg[t] = 0.5 * (PP[i * k2 + k + j] * sg[j] + PP[j * k2 + k + i] * sg[i]);
+        if (!sb_finite(Mg[t])) bad = 1;
+    }
+    __syncthreads();
+    if (bad) {
+        if (t == 0) *status = DEV_NAN_INIT;
         return;
     }
-    for (int i = 0; i < k; ++i)
-        for (int j = 0; j < k; ++j) Cq[i * k + j] = Cp[i * k + j] * sg[j];
+    __syncthreads();
+    if (!sb_gram_schmidt(k, Mg, order, C, v, u, coef, &bad)) {
+        if (t == 0) *status = DEV_BREAKDOWN;
+        return;
+    }
+    if (t < kk) {
+        Cp[t] = C[t];
+        Cq[t] = C[t] * sg[j];
+    }
 }
 
 // inner CG scalars for 2k systems. phase 0: alpha = rr / pLp for active systems (0 otherwise);
@@ -1398,7 +1372,7 @@ void make_q(cudaStream_t st, int k, const double *A, double *Q, double *coef) {
 }
 void eval_finish(cudaStream_t st, int k, const double *Q, const double *d, double *out, int *status) {
     ProfScope ps(st, ST_SMALL, 0.0, 0.0);
-    eval_finish_kernel<<<1, SB_THREADS, 0, st>>>(k, Q, d, out, status);
+    eval_finish_kernel<<<1, sb_threads(k), 0, st>>>(k, Q, d, out, status);
     check_launch("eval_finish_kernel");
 }
 void conj_coeff(cudaStream_t st, int k2, const double *gz, const double *gzp, const double *gd,
@@ -1411,12 +1385,12 @@ void line_gs(cudaStream_t st, int k, const double *A, const double *BDf, const d
              const double *PP, const double *PD, const double *DP, const double *DD, const double *Q,
              double *lam, double *Cp, double *Cq, double *flip, int *status) {
     ProfScope ps(st, ST_SMALL, 0.0, 0.0);
-    line_gs_kernel<<<1, SB_THREADS, 0, st>>>(k, A, BDf, CDfD, PP, PD, DP, DD, Q, lam, Cp, Cq, flip, status);
+    line_gs_kernel<<<1, sb_threads(k), 0, st>>>(k, A, BDf, CDfD, PP, PD, DP, DD, Q, lam, Cp, Cq, flip, status);
     check_launch("line_gs_kernel");
 }
 void init_gs(cudaStream_t st, int k, const double *PP, double *Cp, double *Cq, int *status) {
     ProfScope ps(st, ST_SMALL, 0.0, 0.0);
-    init_gs_kernel<<<1, 1, 0, st>>>(k, PP, Cp, Cq, status);
+    init_gs_kernel<<<1, sb_threads(k), 0, st>>>(k, PP, Cp, Cq, status);
     check_launch("init_gs_kernel");
 }
 void cg_init(cudaStream_t st, int n, double tol, const double *rr0, double *rr, double *r0,

@@ -2,6 +2,8 @@
 give way: the inner CG in one block (up to 20 atoms with 4 functions each, rc rv (rc + rv) = 128000 of
 131072; 21 atoms are past it), traces by one warp per pair (kernels of up to 8192 elements; 153 x 68 is
 past it), products with edges of 10 to 153 in 16, 32 and 64 wide tiles; one state and an odd number.
+The k x k algebra of a step (start, Ritz values, line step, Gram-Schmidt) at block sizes of one to
+eight warps: k = 4 to 16, the start and one step.
 Tolerances as derived for the step parity at three atoms: pairs 1e-7 of their scale after each step
 (the preconditioner's relative residual 1e-4 multiplies rounding of its own), energies 1e-10."""
 import numpy as np
@@ -36,3 +38,24 @@ def test_small_fp64_solver_steps_match_oracle(natoms, nchi, k):
         assert np.max(np.abs(res_g - res_r) / res_r) < 1e-6
         got = st.get()
         assert _rel(got["Pp"], ref.Pp) < 1e-7 and _rel(got["Pq"], ref.Pq) < 1e-7
+
+
+@pytest.mark.parametrize("k", [4, 6, 7, 10, 11, 16])
+def test_small_algebra_matches_oracle_for_every_block_size(k):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1507_08157_gb300 import build, tddft
+    build.build()
+    s = sy.generate(sy.Recipe(natoms=12, cell_ang=9.4, ngrid=30, nchi=4, radius_ang=4.0, min_sep_ang=1.0, seed=52))
+    Y0 = sy.initial_guess(s, k, 3)
+    ref = osolver.PCG(oop.Operator(s), Y0)
+    st = tddft.Context(s, precision="fp64").state(Y0)
+    got = st.get()
+    assert _rel(got["Pp"], ref.Pp) < 1e-9 and _rel(got["Pq"], ref.Pq) < 1e-9
+    om_r, res_r = ref.step()
+    om_g, res_g = st.step()
+    assert np.max(np.abs(om_g - om_r)) < 1e-10
+    assert np.max(np.abs(res_g - res_r) / res_r) < 1e-6
+    got = st.get()
+    assert _rel(got["Pp"], ref.Pp) < 1e-7 and _rel(got["Pq"], ref.Pq) < 1e-7
