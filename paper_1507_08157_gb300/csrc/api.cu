@@ -1493,7 +1493,7 @@ struct StateBufs {
     double *A, *BDf, *CDfD, *PP, *PD, *DP, *DD, *Q, *coef, *Cp, *Cq, *lam, *sc, *flip;
     double *dvec, *dvec2, *dvec3, *evout;
     double *cg_pLp, *cg_rr, *cg_rrn, *cg_r0, *cg_alpha, *cg_beta, *gscr;
-    int *status, *cg_active, *cg_nactive;
+    int *status, *cg_active, *cg_nactive, *cg_count;
 };
 
 }  // namespace
@@ -1557,6 +1557,8 @@ void alloc_state(tddft_ctx *c, tddft_state *S) {
     B->status = B->mem.template alloc<int>(1);
     B->cg_active = B->mem.template alloc<int>(k2);
     B->cg_nactive = B->mem.template alloc<int>(1);
+    B->cg_count = B->mem.template alloc<int>(k2 + 1);
+    check(cudaMemsetAsync(B->cg_count, 0, (k2 + 1) * sizeof(int), c->st), "memset cg counts");
     check(cudaMemsetAsync(B->sc, 0, 4 * sizeof(double), c->st), "memset sc");
     check(cudaMemsetAsync(B->flip, 0, sizeof(double), c->st), "memset flip");
     check(cudaMemsetAsync(B->status, 0, sizeof(int), c->st), "memset status");
@@ -1616,17 +1618,13 @@ void sync_status(tddft_ctx *c, tddft_state *S, const int *dstatus) {
     if (stv == DEV_NAN_INIT) throw Breakdown{"NaN or Inf in the starting trial pairs"};
 }
 
-// recombine Y, P, f and cov(P) with the Gram-Schmidt coefficients (sign flips folded into Cq);
-// cov is linear, so cov(P) follows the same combinations as P
+// Y, P, f and cov(P), each plus lam times its direction (lam not NULL), recombined with the Gram-Schmidt
+// coefficients (sign flips folded into Cq); cov is linear, so cov(P) follows the same combinations as P
 template <typename T>
-void recombine(tddft_ctx *c, StateBufs<T> &B, int k) {
-    const long long len = c->len();
-    T *arrs[] = {B.Y, B.P, B.f, B.covP};
-    for (T *X : arrs) {
-        check(cudaMemcpyAsync(B.tmp, X, 2 * k * len * sizeof(T), cudaMemcpyDeviceToDevice, c->st), "copy recombine");
-        combine<T>(c->st, B.Cp, k, k, k, B.tmp, len, X, len, len, false);
-        combine<T>(c->st, B.Cq, k, k, k, B.tmp + k * len, len, X + k * len, len, len, false);
-    }
+void recombine(tddft_ctx *c, StateBufs<T> &B, int k, const double *lam) {
+    T *const X[] = {B.Y, B.P, B.f, B.covP};
+    const T *const D[] = {B.dir, B.D, B.fD, B.covD};
+    step_combine<T>(c->st, k, B.Cp, B.Cq, lam, X, D, 4, c->len());
 }
 
 template <typename T>
@@ -1643,11 +1641,13 @@ void state_init(tddft_ctx *c, tddft_state *S, const double *Y0) {
     // P = P^c S^chi L S^phi P^v (Eq. auxiliary)
     sandwich_x<T>(c, I, 2 * k, SP_R, B.Y, B.P, B.tmp);
     covariant<T>(c, I, 2 * k, B.P, B.covP, B.tmp);
-    gram<T>(c->st, B.covP, len, 2 * k, B.P, len, 2 * k, len, B.PP, B.gscr);
+    // <p_i, q_j>, the block of PP that is read
+    const GramBlock<T> pq{B.covP, 1, {B.P + k * len}, {B.PP + k}};
+    gram_blocks<T>(c->st, k, 1, &pq, 2 * k, len, B.gscr);
     init_gs(c->st, k, B.PP, B.Cp, B.Cq, B.status);
     sync_status(c, S, B.status);
     check(cudaMemsetAsync(B.f, 0, 2 * k * len * sizeof(T), c->st), "memset f");
-    recombine<T>(c, B, k);
+    recombine<T>(c, B, k, nullptr);
     apply_impl<T>(c, I, k, B.P, B.f, true);
     check(ctx_sync(c), "sync init");
 }
@@ -1661,11 +1661,13 @@ void evaluate(tddft_ctx *c, tddft_state *S) {
     const long long len = c->len();
     cudaStream_t st = c->st;
     // cov(P) is carried along with P (state creation, line step, recombination, re-application)
-    gram<T>(st, B.covP, len, 2 * k, B.f, len, 2 * k, len, B.A, B.gscr);   // A[x][y] = <P_x, f_y>
+    // A[x][y] = <P_x, f_y>, x and y both p or both q
+    const GramBlock<T> pf[2] = {{B.covP, 1, {B.f}, {B.A}},
+                                {B.covP + k * len, 1, {B.f + k * len}, {B.A + (2 * k + 1) * k}}};
+    gram_blocks<T>(st, k, 2, pf, 2 * k, len, B.gscr);
     make_q(st, k, B.A, B.Q, B.coef);
     // g = f - swap(P) Q^T
-    check(cudaMemcpyAsync(B.g, B.f, 2 * k * len * sizeof(T), cudaMemcpyDeviceToDevice, st), "copy g");
-    combine<T>(st, B.coef, 2 * k, 2 * k, 2 * k, B.P, len, B.g, len, len, true);
+    combine<T>(st, B.coef, 2 * k, 2 * k, 2 * k, B.P, B.f, B.g, len);
     if (c->sparse) {
         // truncated form: G_L is the exact gradient of the sum functional with respect to L
         // through the truncated map P = T(T(R_c L) R_v): its adjoint applied to the Frobenius
@@ -1726,7 +1728,7 @@ void precondition(tddft_ctx *c, tddft_state *S, const T *h, T *z) {
         check(cudaMemcpyAsync(p, h, tot * sizeof(T), cudaMemcpyDeviceToDevice, st), "copy p");
         covariant<T>(c, I, k2, r, cv, B.tmp);
         dots<T>(st, cv, len, r, len, k2, len, B.dvec2, B.gscr);
-        cg_init(st, k2, ptol, B.dvec2, B.cg_rr, B.cg_r0, B.cg_active, B.cg_nactive);
+        cg_init(st, k2, B.dvec2, B.cg_rr, B.cg_r0, B.cg_active, B.cg_nactive);
         int *hn = reinterpret_cast<int *>(S->host + 2 * S->k) + 1;
         for (int it = 0; it < c->opt.precond_maxit; ++it) {
             check(cudaMemcpyAsync(hn, B.cg_nactive, sizeof(int), cudaMemcpyDeviceToHost, st), "D2H n_active");
@@ -1784,7 +1786,7 @@ void precondition(tddft_ctx *c, tddft_state *S, const T *h, T *z) {
             check(cudaMemsetAsync(zh, 0, k2 * lr * sizeof(T), st), "memset z");
             check(cudaMemcpyAsync(p, r, k2 * lr * sizeof(T), cudaMemcpyDeviceToDevice, st), "copy p");
             dots<T>(st, r, lr, r, lr, k2, lr, B.dvec2, B.gscr);
-            cg_init(st, k2, ptol, B.dvec2, B.cg_rr, B.cg_r0, B.cg_active, B.cg_nactive);
+            cg_init(st, k2, B.dvec2, B.cg_rr, B.cg_r0, B.cg_active, B.cg_nactive);
         }
         for (int it = 0; !one_block && it < c->opt.precond_maxit; ++it) {
             check(cudaMemcpyAsync(hn, B.cg_nactive, sizeof(int), cudaMemcpyDeviceToHost, st), "D2H n_active");
@@ -1793,14 +1795,8 @@ void precondition(tddft_ctx *c, tddft_state *S, const T *h, T *z) {
             S->inner_iters += 1;
             gemm<T>(st, false, false, rc, rv, rc, T(1), I.Mch, rc, 0, p, rv, lr, T(0), Lp, rv, lr, k2);
             gemm<T>(st, false, false, k2 * rc, rv, rv, T(-1), p, rv, 0, I.Mvh, rv, 0, T(1), Lp, rv, 0, 1);
-            dots<T>(st, p, lr, Lp, lr, k2, lr, B.cg_pLp, B.gscr);
-            cg_scalars(st, k2, 0, ptol, B.cg_pLp, B.cg_rrn, B.cg_rr, B.cg_r0, B.cg_alpha, B.cg_beta, B.cg_active,
-                       B.cg_nactive);
-            axpy_dev<T>(st, B.cg_alpha, 1, 1.0, zh, p, lr, k2);
-            axpy_dev<T>(st, B.cg_alpha, 1, -1.0, r, Lp, lr, k2);
-            dots<T>(st, r, lr, r, lr, k2, lr, B.cg_rrn, B.gscr);
-            cg_scalars(st, k2, 1, ptol, B.cg_pLp, B.cg_rrn, B.cg_rr, B.cg_r0, B.cg_alpha, B.cg_beta, B.cg_active,
-                       B.cg_nactive);
+            cg_step<T>(st, p, Lp, zh, r, lr, k2, ptol, B.gscr, B.cg_count, B.cg_pLp, B.cg_rr, B.cg_r0, B.cg_alpha,
+                       B.cg_beta, B.cg_active, B.cg_nactive);
             cg_dir<T>(st, p, r, B.cg_beta, lr, k2);
         }
         gemm<T>(st, false, false, nc, rv, rc, T(1), I.Vc, rc, 0, zh, rv, lr, T(0), B.tmp, rv, (long long)nc * rv, k2);
@@ -1812,7 +1808,7 @@ void precondition(tddft_ctx *c, tddft_state *S, const T *h, T *z) {
     sandwich<T>(c, k2, I.Sch, h, I.Svh, r, B.tmp);           // r~ = h~
     check(cudaMemcpyAsync(p, r, tot * sizeof(T), cudaMemcpyDeviceToDevice, st), "copy p");
     dots<T>(st, r, len, r, len, k2, len, B.dvec2, B.gscr);
-    cg_init(st, k2, ptol, B.dvec2, B.cg_rr, B.cg_r0, B.cg_active, B.cg_nactive);
+    cg_init(st, k2, B.dvec2, B.cg_rr, B.cg_r0, B.cg_active, B.cg_nactive);
     int *hn = reinterpret_cast<int *>(S->host + 2 * S->k) + 1;
     for (int it = 0; it < c->opt.precond_maxit; ++it) {
         check(cudaMemcpyAsync(hn, B.cg_nactive, sizeof(int), cudaMemcpyDeviceToHost, st), "D2H n_active");
@@ -1821,13 +1817,7 @@ void precondition(tddft_ctx *c, tddft_state *S, const T *h, T *z) {
         S->inner_iters += 1;
         gemm<T>(st, false, false, nc, nv, nc, T(1), I.Mct, nc, 0, p, nv, len, T(0), Lp, nv, len, k2);
         gemm<T>(st, false, false, k2 * nc, nv, nv, T(-1), p, nv, 0, I.Mvt, nv, 0, T(1), Lp, nv, 0, 1);
-        dots<T>(st, p, len, Lp, len, k2, len, B.cg_pLp, B.gscr);
-        cg_scalars(st, k2, 0, ptol, B.cg_pLp, B.cg_rrn, B.cg_rr, B.cg_r0, B.cg_alpha,
-                   B.cg_beta, B.cg_active, B.cg_nactive);
-        axpy_dev<T>(st, B.cg_alpha, 1, 1.0, zt, p, len, k2);
-        axpy_dev<T>(st, B.cg_alpha, 1, -1.0, r, Lp, len, k2);
-        dots<T>(st, r, len, r, len, k2, len, B.cg_rrn, B.gscr);
-        cg_scalars(st, k2, 1, ptol, B.cg_pLp, B.cg_rrn, B.cg_rr, B.cg_r0, B.cg_alpha,
+        cg_step<T>(st, p, Lp, zt, r, len, k2, ptol, B.gscr, B.cg_count, B.cg_pLp, B.cg_rr, B.cg_r0, B.cg_alpha,
                    B.cg_beta, B.cg_active, B.cg_nactive);
         cg_dir<T>(st, p, r, B.cg_beta, len, k2);
     }
@@ -1956,21 +1946,17 @@ void update(tddft_ctx *c, tddft_state *S) {
     apply_impl<T>(c, I, k, B.D, B.fD, true);
     covariant<T>(c, I, k2, B.D, B.covD, B.tmp);
     {
-        // the six traces of the line step in two passes (cov(D) and cov(P) read once each)
-        const T *yd[4] = {B.f, B.fD, B.P, B.D};
-        double *gd[4] = {B.BDf, B.CDfD, B.DP, B.DD};
-        gram_multi<T>(st, B.covD, len, k2, 4, yd, len, k2, len, gd, B.gscr);
-        const T *yp[2] = {B.P, B.D};
-        double *gp[2] = {B.PP, B.PD};
-        gram_multi<T>(st, B.covP, len, k2, 2, yp, len, k2, len, gp, B.gscr);
+        // the six traces of the line step, of each the blocks that are read: cov(D) and cov(P) once
+        const long long q = k * len;
+        const GramBlock<T> job[3] = {
+            {B.covD, 4, {B.f, B.fD, B.P + q, B.D + q}, {B.BDf, B.CDfD, B.DP + k, B.DD + k}},
+            {B.covD + q, 2, {B.f + q, B.fD + q}, {B.BDf + (2 * k + 1) * k, B.CDfD + (2 * k + 1) * k}},
+            {B.covP, 2, {B.P + q, B.D + q}, {B.PP + k, B.PD + k}}};
+        gram_blocks<T>(st, k, 3, job, 2 * k, len, B.gscr);
     }
     line_gs(st, k, B.A, B.BDf, B.CDfD, B.PP, B.PD, B.DP, B.DD, B.Q, B.lam, B.Cp, B.Cq, B.flip,
             B.status);
-    axpy_dev<T>(st, B.lam, 0, 1.0, B.Y, B.dir, tot, 1);
-    axpy_dev<T>(st, B.lam, 0, 1.0, B.P, B.D, tot, 1);
-    axpy_dev<T>(st, B.lam, 0, 1.0, B.f, B.fD, tot, 1);
-    axpy_dev<T>(st, B.lam, 0, 1.0, B.covP, B.covD, tot, 1);
-    recombine<T>(c, B, k);
+    recombine<T>(c, B, k, B.lam);
     check(cudaMemcpyAsync(S->host + 2 * k + 1, B.lam, sizeof(double), cudaMemcpyDeviceToHost, st), "D2H lam");
     sync_status(c, S, B.status);
     S->it += 1;

@@ -28,30 +28,31 @@ __global__ void gram_final(const double *__restrict__ partial, int nblocks, int 
     if (lane == 0) G[p] = s;
 }
 
-// up to four Gram matrices of one X against several Y sets, [nx][per] each
-struct GOut {
+// Trace products of a launch: job m takes the k rows of x against the k rows of each of its nset sets y
+// (rows len apart) into k x k blocks g (rows ldg apart); its pairs start at pair `first` of the launch
+struct GramJob {
+    const void *x, *y[4];
     double *g[4];
+    int nset, first;
 };
-__global__ void gram_final_multi(const double *__restrict__ partial, int nblocks, int pairs, int ny, int per,
-                                 GOut out) {
+struct GramJobs {
+    GramJob j[GRAM_JOBS];
+    int n, k, ldg, pairs;
+};
+__global__ void gram_final_jobs(const double *__restrict__ partial, int nblocks, const GramJobs js) {
     const int lane = threadIdx.x & 31;
     const int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (p >= pairs) return;
+    if (p >= js.pairs) return;
     double s = 0.0;
-    for (int b = lane; b < nblocks; b += 32) s += partial[(long long)b * pairs + p];
+    for (int b = lane; b < nblocks; b += 32) s += partial[(long long)b * js.pairs + p];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
-        const int i = p / ny, j = p - i * ny, q = j / per;
-        out.g[q][i * per + (j - q * per)] = s;
+        int m = 0;
+        while (m + 1 < js.n && p >= js.j[m + 1].first) ++m;
+        const int ny = js.j[m].nset * js.k, i = (p - js.j[m].first) / ny, j = p - js.j[m].first - i * ny, q = j / js.k;
+        js.j[m].g[q][i * js.ldg + (j - q * js.k)] = s;
     }
 }
-
-// the Y rows of a trace product: row j is row (j % per) of set j / per
-template <typename T>
-struct YSet {
-    const T *p[4];
-    int per;
-};
 
 // ------------------------------------------------------------------------------------------------
 // Register-tiled trace products. Block (x, y): pair tile x of TI x TJ (i, j), element slice y
@@ -69,11 +70,15 @@ constexpr int TI = 4;   // pair tile: TI x TJ (TJ = 8 for scalar loads, 4 for pa
 template <typename T, int VEC> struct VecLd;
 template <typename T> struct VecLd<T, 1> {
     static __device__ __forceinline__ void ld(const T *p, long long e, T *o) { o[0] = p[e]; }
+    static __device__ __forceinline__ void st(T *p, long long e, const T *o) { p[e] = o[0]; }
 };
 template <> struct VecLd<float, 2> {
     static __device__ __forceinline__ void ld(const float *p, long long e, float *o) {
         const float2 v = reinterpret_cast<const float2 *>(p)[e];
         o[0] = v.x, o[1] = v.y;
+    }
+    static __device__ __forceinline__ void st(float *p, long long e, const float *o) {
+        reinterpret_cast<float2 *>(p)[e] = make_float2(o[0], o[1]);
     }
 };
 template <> struct VecLd<float, 4> {
@@ -90,18 +95,20 @@ template <> struct VecLd<double, 2> {
 };
 
 template <typename T, int VEC, int TJ>
-__global__ void __launch_bounds__(256, 2) gram_tiled(const T *__restrict__ X, long long sx, int nx,
-                                                     const YSet<T> ys, long long sy, int ny,
-                                                     long long len, int tiles_j, double *__restrict__ partial,
-                                                     int pairs) {
+__global__ void __launch_bounds__(256, 2) gram_tiled(const GramJobs js, long long len, int tiles_j,
+                                                     double *__restrict__ partial) {
     __shared__ double red[TI][TJ][8];
+    const GramJob &jb = js.j[blockIdx.z];
+    const T *X = static_cast<const T *>(jb.x);
+    const int nx = js.k, ny = jb.nset * js.k;
     const int ti = blockIdx.x / tiles_j, tj = blockIdx.x - ti * tiles_j;
     const int i0 = ti * TI, j0 = tj * TJ;
+    if (j0 >= ny) return;                 // a job with fewer sets than the launch's widest
     const T *yr[TJ];
 #pragma unroll
     for (int b = 0; b < TJ; ++b) {
-        const int j = j0 + b < ny ? j0 + b : 0, q = j / ys.per;
-        yr[b] = ys.p[q] + (long long)(j - q * ys.per) * sy;
+        const int j = j0 + b < ny ? j0 + b : 0, q = j / js.k;
+        yr[b] = static_cast<const T *>(jb.y[q]) + (j - q * js.k) * len;
     }
     T tot[TI][TJ], run[TI][TJ];
 #pragma unroll
@@ -115,7 +122,7 @@ __global__ void __launch_bounds__(256, 2) gram_tiled(const T *__restrict__ X, lo
         T xv[TI][VEC], yv[TJ][VEC];
 #pragma unroll
         for (int a = 0; a < TI; ++a) {
-            if (i0 + a < nx) VecLd<T, VEC>::ld(X + (i0 + a) * sx, e, xv[a]);
+            if (i0 + a < nx) VecLd<T, VEC>::ld(X + (i0 + a) * len, e, xv[a]);
             else
 #pragma unroll
                 for (int u = 0; u < VEC; ++u) xv[a][u] = T(0);
@@ -156,46 +163,65 @@ __global__ void __launch_bounds__(256, 2) gram_tiled(const T *__restrict__ X, lo
         double v = 0.0;
         for (int w = 0; w < 8; ++w) v += red[a][b][w];
         const int i = i0 + a, j = j0 + b;
-        if (i < nx && j < ny) partial[(long long)blockIdx.y * pairs + i * ny + j] = v;
+        if (i < nx && j < ny) partial[(long long)blockIdx.y * js.pairs + jb.first + i * ny + j] = v;
     }
 }
 
-// d_i = sum_e X_i[e] Y_i[e]: one row per blockIdx.y, the same two-level runs and reductions
+// the block's sum of the threads' v, by a butterfly per warp in T and in float64 over the eight
+// warps; thread 0 has it
 template <typename T>
-__global__ void __launch_bounds__(256) dots_kernel(const T *__restrict__ X, long long sx, const T *__restrict__ Y,
-                                                   long long sy, long long len, int n, double *__restrict__ partial) {
+__device__ double dots_reduce(T v) {
     __shared__ double red[8];
-    const int i = blockIdx.y;
-    const T *x = X + i * sx;
-    const T *y = Y + i * sy;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (double)v;
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < 8; ++w) s += red[w];
+    return s;
+}
+// the block's share of sum_e x[e] y[e] in thread 0, the same two-level runs; eight elements of both
+// rows are on their way before the first product
+template <typename T>
+__device__ double dots_block(const T *__restrict__ x, const T *__restrict__ y, long long len) {
     T tot = T(0), run = T(0);
     int cnt = 0;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < len; e += stride) {
-        run = fma(x[e], y[e], run);
-        if (++cnt == RUN) {
+    for (long long e0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; e0 < len; e0 += 8 * stride) {
+        T a[8], b[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const long long e = e0 + u * stride;
+            a[u] = e < len ? x[e] : T(0);
+            b[u] = e < len ? y[e] : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) run = fma(a[u], b[u], run);
+        if (++cnt == RUN / 8) {
             tot += run;
             run = T(0);
             cnt = 0;
         }
     }
-    T v = tot + run;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = (double)v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < 8; ++w) s += red[w];
-        partial[(long long)blockIdx.x * n + i] = s;
-    }
+    return dots_reduce<T>(tot + run);
+}
+
+// d_i = sum_e X_i[e] Y_i[e]: one row per blockIdx.y (140 atoms, 20 rows of 705600: 40 us with one
+// element on its way per thread, 26 with eight)
+template <typename T>
+__global__ void __launch_bounds__(256) dots_kernel(const T *__restrict__ X, long long sx, const T *__restrict__ Y,
+                                                   long long sy, long long len, int n, double *__restrict__ partial) {
+    const int i = blockIdx.y;
+    const double s = dots_block<T>(X + i * sx, Y + i * sy, len);
+    if (threadIdx.x == 0) partial[(long long)blockIdx.x * n + i] = s;
 }
 
 // ------------------------------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256) combine_kernel(const double *__restrict__ C, int ldc, int nout,
                                                       int nin, const T *__restrict__ in,
-                                                      long long sin, T *__restrict__ out,
-                                                      long long sout, long long len, bool accumulate) {
+                                                      const T *__restrict__ base, T *__restrict__ out,
+                                                      long long len) {
     __shared__ T Cs[32 * 32];
     // every slot the product loop reads is written (zero past nin): stale shared memory from an
     // earlier kernel may hold NaN patterns, and NaN * 0 is NaN
@@ -208,12 +234,66 @@ __global__ void __launch_bounds__(256) combine_kernel(const double *__restrict__
          e += (long long)gridDim.x * blockDim.x) {
         T x[32];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) x[j] = j < nin ? in[j * sin + e] : T(0);
-        for (int i = 0; i < nout; ++i) {
-            T s = accumulate ? out[i * sout + e] : T(0);
+        for (int j = 0; j < 32; ++j) x[j] = j < nin ? in[j * len + e] : T(0);
+#pragma unroll 5
+        for (int i = 0; i < nout; ++i) {     // unrolled, so that several loads of base are on their way
+            T s = base[i * len + e];
 #pragma unroll
             for (int j = 0; j < 32; ++j) s = fma(Cs[i * 32 + j], x[j], s);
-            out[i * sout + e] = s;
+            out[i * len + e] = s;
+        }
+    }
+}
+
+// Rows X_i <- sum_j C_ij (X_j + lam D_j) of up to four arrays X in place (blockIdx.z), p half with Cp and
+// q half with Cq (blockIdx.y); without lam X_i <- sum_j C_ij X_j. Every element is read once and written
+// once: bound by memory. 140 atoms, 10 states, four arrays: 0.40 ms as an update, a copy and two
+// combinations each, 0.10 here. KP >= k rows are held in registers.
+struct CombArrays {
+    void *x[4];
+    const void *d[4];
+};
+template <typename T, int VEC, int KP>
+__global__ void __launch_bounds__(256) step_combine_kernel(const double *__restrict__ Cp, const double *__restrict__ Cq,
+                                                           const double *__restrict__ lam, int k, const CombArrays ar,
+                                                           long long len) {
+    __shared__ T Cs[KP * KP];
+    const double *C = blockIdx.y ? Cq : Cp;
+    for (int i = threadIdx.x; i < KP * KP; i += blockDim.x) {
+        const int r = i / KP, c = i - r * KP;
+        Cs[i] = r < k && c < k ? T(C[r * k + c]) : T(0);
+    }
+    const T l = lam ? T(*lam) : T(0);
+    __syncthreads();
+    T *X = static_cast<T *>(ar.x[blockIdx.z]) + blockIdx.y * k * len;
+    const T *D = static_cast<const T *>(ar.d[blockIdx.z]) + blockIdx.y * k * len;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < len / VEC; e += (long long)gridDim.x * blockDim.x) {
+        T x[KP][VEC];
+#pragma unroll
+        for (int j = 0; j < KP; ++j) {
+#pragma unroll
+            for (int u = 0; u < VEC; ++u) x[j][u] = T(0);
+            if (j < k) VecLd<T, VEC>::ld(X + j * len, e, x[j]);
+        }
+        if (lam) {
+#pragma unroll
+            for (int j = 0; j < KP; ++j)
+                if (j < k) {
+                    T d[VEC];
+                    VecLd<T, VEC>::ld(D + j * len, e, d);
+#pragma unroll
+                    for (int u = 0; u < VEC; ++u) x[j][u] = fma(l, d[u], x[j][u]);
+                }
+        }
+        for (int i = 0; i < k; ++i) {
+            T s[VEC];
+#pragma unroll
+            for (int u = 0; u < VEC; ++u) s[u] = T(0);
+#pragma unroll
+            for (int j = 0; j < KP; ++j)
+#pragma unroll
+                for (int u = 0; u < VEC; ++u) s[u] = fma(Cs[i * KP + j], x[j][u], s[u]);
+            VecLd<T, VEC>::st(X + i * len, e, s);
         }
     }
 }
@@ -252,10 +332,9 @@ template <> struct Vec16<double> {
 // distinct bank groups. The pair grid (at most 128 threads) is held twice: the two halves of
 // the block take the two halves of every chunk. Products are summed in T over a half chunk,
 // those sums in a compensated (Kahan) sum in T; the halves meet in shared memory at the end and
-// partial[s][pair] is written in float64, summed over the slices by gram_final_multi.
+// partial[s][pair] is written in float64, summed over the slices by gram_final_jobs.
 template <typename T> __host__ __device__ constexpr int gram_chunk() { return 256 / (int)sizeof(T); }
 template <typename T> __host__ __device__ constexpr int gram_row() { return 272 / (int)sizeof(T); }
-constexpr int GQ = 4;           // pair tile edge
 constexpr int GST = 4;          // ring stages
 constexpr int GMAXT = 10;       // 16-byte copies per thread and chunk: nx + ny <= 160
 
@@ -266,11 +345,12 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, bool full
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <typename T>
-__global__ void __launch_bounds__(256) gram_rows_kernel(const T *__restrict__ X, long long sx, int nx,
-                                                        const YSet<T> ys, long long sy, int ny, long long len,
-                                                        long long per_slice, int RX, int RY,
-                                                        double *__restrict__ partial, int pairs) {
+template <typename T, int GQ>
+__global__ void __launch_bounds__(256) gram_rows_kernel(const GramJobs js, long long len, long long per_slice, int RX,
+                                                        int RY, double *__restrict__ partial) {
+    const GramJob &jb = js.j[blockIdx.y];
+    const T *X = static_cast<const T *>(jb.x);
+    const int nx = js.k, ny = jb.nset * js.k;
     extern __shared__ __align__(16) unsigned char gram_smem[];
     constexpr int VW = Vec16<T>::n;
     constexpr int GC = gram_chunk<T>();      // elements per staged chunk of a row
@@ -299,12 +379,11 @@ __global__ void __launch_bounds__(256) gram_rows_kernel(const T *__restrict__ X,
                     const T *src;
                     int srow;
                     if (row < nx) {
-                        src = X + row * sx;
+                        src = X + row * len;
                         srow = row;
                     } else {
-                        const int j = row - nx, s = j / ys.per;
-                        const T *set = s == 0 ? ys.p[0] : s == 1 ? ys.p[1] : s == 2 ? ys.p[2] : ys.p[3];
-                        src = set + (long long)(j - s * ys.per) * sy;
+                        const int j = row - nx, s = j / js.k;
+                        src = static_cast<const T *>(jb.y[s]) + (j - s * js.k) * len;
                         srow = RX + j;
                     }
                     const bool in = e < e1;
@@ -384,7 +463,7 @@ __global__ void __launch_bounds__(256) gram_rows_kernel(const T *__restrict__ X,
         for (int b = 0; b < GQ; ++b) {
             const int i = ta + a * gx, j = tb + b * gy;
             if (i < nx && j < ny)
-                partial[(long long)blockIdx.x * pairs + i * ny + j] =
+                partial[(long long)blockIdx.x * js.pairs + jb.first + i * ny + j] =
                     ((double)tot[a][b] - (double)cmp[a][b]) + hand[(a * GQ + b) * 128 + tl];
         }
 }
@@ -394,14 +473,15 @@ __global__ void __launch_bounds__(256) gram_rows_kernel(const T *__restrict__ X,
 // few short rows leave it a handful of threads (float64, 1024 elements, 2 x 8 rows: 180 us there,
 // 6 us here).
 template <typename T>
-__global__ void __launch_bounds__(128) gram_short_kernel(const T *__restrict__ X, long long sx, int nx, const YSet<T> ys,
-                                                         long long sy, int ny, long long len, GOut out) {
+__global__ void __launch_bounds__(128) gram_short_kernel(const GramJobs js, long long len) {
     const int p = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (p >= nx * ny) return;
-    const int i = p / ny, j = p - i * ny, q = j / ys.per;
-    const T *x = X + i * sx;
-    const T *set = q == 0 ? ys.p[0] : q == 1 ? ys.p[1] : q == 2 ? ys.p[2] : ys.p[3];
-    const T *y = set + (long long)(j - q * ys.per) * sy;
+    if (p >= js.pairs) return;
+    int m = 0;
+    while (m + 1 < js.n && p >= js.j[m + 1].first) ++m;
+    const GramJob &jb = js.j[m];
+    const int ny = jb.nset * js.k, i = (p - jb.first) / ny, j = p - jb.first - i * ny, q = j / js.k;
+    const T *x = static_cast<const T *>(jb.x) + i * len;
+    const T *y = static_cast<const T *>(jb.y[q]) + (j - q * js.k) * len;
     T tot = T(0), cmp = T(0);
     for (long long e0 = lane; e0 < len; e0 += 256) {
         T run = T(0);
@@ -416,7 +496,7 @@ __global__ void __launch_bounds__(128) gram_short_kernel(const T *__restrict__ X
     }
     double d = (double)tot - (double)cmp;
     for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-    if (lane == 0) out.g[q][i * ys.per + (j - q * ys.per)] = d;
+    if (lane == 0) jb.g[q][i * js.ldg + (j - q * js.k)] = d;
 }
 
 // Batched element-wise kernels: blockIdx.y = matrix b of nb, blockIdx.x strides over the len
@@ -1000,91 +1080,198 @@ __global__ void cg_scalars_kernel(int n, int phase, double tol, const double *pL
     if (phase == 1 && i == 0) *n_active = cnt;
 }
 
+// The slices' sums of system i by the block that finishes last (count[i], left at zero): true in the
+// first warp of that block, *out the sum in the order of gram_final. `partial` is this launch's.
+__device__ bool cg_last_sum(double v, int i, int n, double *partial, int *count, double *out) {
+    __shared__ int last;
+    if (threadIdx.x == 0) {
+        partial[(long long)blockIdx.x * n + i] = v;
+        __threadfence();
+        last = atomicAdd(count + i, 1) == (int)gridDim.x - 1;
+        if (last) count[i] = 0;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return false;
+    __threadfence();
+    double s = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) s += __ldcg(partial + (long long)b * n + i);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    *out = s;
+    return true;
+}
+
+// Inner CG of n systems (blockIdx.y): pLp = <p, Lp> and alpha. The sum is the one of dots.
+template <typename T>
+__global__ void __launch_bounds__(256) cg_curvature_kernel(const T *__restrict__ p, const T *__restrict__ Lp, long long len,
+                                                           int n, double *partial, int *count, double *pLp,
+                                                           const double *__restrict__ rr, double *alpha, int *active) {
+    const int i = blockIdx.y;
+    const double v = dots_block<T>(p + i * len, Lp + i * len, len);
+    double s;
+    if (cg_last_sum(v, i, n, partial, count, &s) && threadIdx.x == 0) {
+        const bool go = active[i] && s > 0.0 && isfinite(s);
+        if (!go) active[i] = 0;
+        pLp[i] = s;
+        alpha[i] = go ? rr[i] / s : 0.0;
+    }
+}
+
+// z += alpha p, r -= alpha Lp, then <r, r>, beta and which systems go on; count has n + 1 entries
+template <typename T>
+__global__ void __launch_bounds__(256) cg_move_kernel(const T *__restrict__ p, const T *__restrict__ Lp, T *__restrict__ z,
+                                                      T *__restrict__ r, long long len, int n, double tol, double *partial,
+                                                      int *count, const double *__restrict__ alpha, double *rr,
+                                                      const double *__restrict__ r0, double *beta, int *active,
+                                                      int *n_active) {
+    const int i = blockIdx.y;
+    const T ap = T(alpha[i]), am = T(-alpha[i]);
+    const T *pi = p + i * len, *li = Lp + i * len;
+    T *zi = z + i * len, *ri = r + i * len;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    T tot = T(0), run = T(0);
+    int cnt = 0;
+    for (long long e0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; e0 < len; e0 += 4 * stride) {
+        T a[4], l[4], x[4], y[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const long long e = e0 + u * stride;
+            const bool in = e < len;
+            a[u] = in ? pi[e] : T(0);
+            l[u] = in ? li[e] : T(0);
+            x[u] = in ? ri[e] : T(0);
+            y[u] = in ? zi[e] : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const long long e = e0 + u * stride;
+            if (e < len) {
+                zi[e] = fma(ap, a[u], y[u]);
+                x[u] = fma(am, l[u], x[u]);
+                ri[e] = x[u];
+                run = fma(x[u], x[u], run);
+            }
+        }
+        if (++cnt == RUN / 4) {
+            tot += run;
+            run = T(0);
+            cnt = 0;
+        }
+    }
+    const double v = dots_reduce<T>(tot + run);
+    double s;
+    if (cg_last_sum(v, i, n, partial, count, &s) && threadIdx.x == 0) {
+        const bool on = active[i] != 0;
+        beta[i] = on && rr[i] != 0.0 ? s / rr[i] : 0.0;
+        if (on) {
+            rr[i] = s;
+            if (!(sqrt(s > 0.0 ? s : 0.0) > tol * r0[i])) active[i] = 0;
+        }
+        __threadfence();
+        if (atomicAdd(count + n, 1) == n - 1) {          // the last system: how many go on
+            count[n] = 0;
+            __threadfence();
+            int c = 0;
+            for (int q = 0; q < n; ++q) c += __ldcg(active + q);
+            *n_active = c;
+        }
+    }
+}
+
 // The whole inner CG of one system on the reduced space in one block: L p = Mc p - p Mv on rc x rv
 // coordinates, from z = 0 and r given, with the decisions of the kernels above (a system is
 // independent of the others, so each stops by itself). Everything stays in shared memory: an
-// iteration otherwise takes eleven launches and a host wait (about 45 us whatever the size, 13
-// iterations a step at 8 atoms). iters: the most iterations of any system (zeroed before).
+// iteration otherwise takes five launches and a host wait (25 us and more whatever the size; 5 here at
+// 8 atoms, 13 iterations a step). Bound by float64 instructions in sequence: a thread per element up
+// to CG_THREADS, sums finished by one warp. iters: the most iterations of any system (zeroed before).
 constexpr int CG_THREADS = 512;
-__device__ double block_sum(double v, double *red) {
+// the sum over the block, and f of it, by the first warp (float64 instructions of other warps of its
+// scheduler would wait for one another)
+template <typename F>
+__device__ __forceinline__ void block_sum(double v, double *red, F f) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();                 // the last call's readers are done
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
-    double s = 0.0;
-    for (int w = 0; w < CG_THREADS / 32; ++w) s += red[w];
-    return s;
+    if (threadIdx.x < 32) {
+        double s = threadIdx.x < blockDim.x / 32 ? red[threadIdx.x] : 0.0;
+        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) f(s);
+    }
+    __syncthreads();
 }
 template <typename T>
 __global__ void __launch_bounds__(CG_THREADS) cg_reduced_kernel(int rc, int rv, const T *__restrict__ Mc,
                                                                 const T *__restrict__ Mv, const T *__restrict__ rin,
                                                                 T *__restrict__ zout, double tol, int maxit, int *iters) {
     extern __shared__ __align__(16) unsigned char cg_smem[];
-    __shared__ double red[CG_THREADS / 32];
-    const int n = rc * rv, t = threadIdx.x;
+    __shared__ double red[CG_THREADS / 32], sc[4];       // sc: rr, r0, alpha, beta
+    __shared__ int active;
+    const int n = rc * rv, t = threadIdx.x, nt = blockDim.x;
     T *mc = reinterpret_cast<T *>(cg_smem), *mv = mc + rc * rc, *p = mv + rv * rv, *r = p + n, *z = r + n, *Lp = z + n;
     const long long base = (long long)blockIdx.x * n;
-    for (int i = t; i < rc * rc; i += CG_THREADS) mc[i] = Mc[i];
-    for (int i = t; i < rv * rv; i += CG_THREADS) mv[i] = Mv[i];
+    for (int i = t; i < rc * rc; i += nt) mc[i] = Mc[i];
+    for (int i = t; i < rv * rv; i += nt) mv[i] = Mv[i];
     double s = 0.0;
-    for (int i = t; i < n; i += CG_THREADS) {
+    for (int i = t; i < n; i += nt) {
         const T x = rin[base + i];
         r[i] = x;
         p[i] = x;
         z[i] = T(0);
-        s += (double)x * (double)x;
+        s = fma((double)x, (double)x, s);
     }
-    double rr = block_sum(s, red);
-    const double r0 = sqrt(rr > 0.0 ? rr : 0.0);
-    bool active = r0 > 0.0 && isfinite(r0);
+    block_sum(s, red, [&](double rr) {
+        sc[0] = rr;
+        sc[1] = sqrt(rr > 0.0 ? rr : 0.0);
+        active = sc[1] > 0.0 && isfinite(sc[1]);
+    });
     int it = 0;
     for (; it < maxit && active; ++it) {
-        __syncthreads();             // p is whole
         s = 0.0;
-        for (int e = t; e < n; e += CG_THREADS) {
+        for (int e = t; e < n; e += nt) {
             const int i = e / rv, j = e - i * rv;
             T a = T(0), b = T(0);
             for (int q = 0; q < rc; ++q) a = fma(mc[i * rc + q], p[q * rv + j], a);
             for (int q = 0; q < rv; ++q) b = fma(p[i * rv + q], mv[q * rv + j], b);
             const T l = a - b;
             Lp[e] = l;
-            s += (double)p[e] * (double)l;
+            s = fma((double)p[e], (double)l, s);
         }
-        const double pLp = block_sum(s, red);
-        if (!(pLp > 0.0 && isfinite(pLp))) {
-            active = false;
-            continue;
-        }
-        const double alpha = rr / pLp;
-        const T ap = T(alpha), am = T(-alpha);
+        block_sum(s, red, [&](double pLp) {
+            active = pLp > 0.0 && isfinite(pLp);
+            sc[2] = sc[0] / pLp;
+        });
+        if (!active) continue;
+        const T ap = T(sc[2]), am = -ap;
         s = 0.0;
-        for (int e = t; e < n; e += CG_THREADS) {
+        for (int e = t; e < n; e += nt) {
             z[e] = fma(ap, p[e], z[e]);
             const T x = fma(am, Lp[e], r[e]);
             r[e] = x;
-            s += (double)x * (double)x;
+            s = fma((double)x, (double)x, s);
         }
-        const double rrn = block_sum(s, red);
-        const T beta = T(rr != 0.0 ? rrn / rr : 0.0);
-        rr = rrn;
-        if (!(sqrt(rrn > 0.0 ? rrn : 0.0) > tol * r0)) active = false;
-        for (int e = t; e < n; e += CG_THREADS) p[e] = fma(beta, p[e], r[e]);
+        block_sum(s, red, [&](double rrn) {
+            sc[3] = sc[0] != 0.0 ? rrn / sc[0] : 0.0;
+            sc[0] = rrn;
+            active = sqrt(rrn > 0.0 ? rrn : 0.0) > tol * sc[1];
+        });
+        const T beta = T(sc[3]);
+        for (int e = t; e < n; e += nt) p[e] = fma(beta, p[e], r[e]);
+        __syncthreads();             // p is whole
     }
-    for (int i = t; i < n; i += CG_THREADS) zout[base + i] = z[i];
+    for (int i = t; i < n; i += nt) zout[base + i] = z[i];
     if (t == 0) atomicMax(iters, it);
 }
 
-__global__ void cg_init_kernel(int n, double tol, const double *rr0, double *rr, double *r0,
-                               int *active, int *n_active) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    int cnt = 0;
-    for (int i = 0; i < n; ++i) {
+__global__ void cg_init_kernel(int n, const double *rr0, double *rr, double *r0, int *active, int *n_active) {
+    const int i = threadIdx.x;       // one thread per system
+    int act = 0;
+    if (i < n) {
         rr[i] = rr0[i];
         r0[i] = sqrt(rr0[i] > 0.0 ? rr0[i] : 0.0);
-        active[i] = (r0[i] > 0.0 && isfinite(r0[i])) ? 1 : 0;
-        cnt += active[i];
+        act = r0[i] > 0.0 && isfinite(r0[i]);
+        active[i] = act;
     }
-    *n_active = cnt;
+    const int cnt = __syncthreads_count(act);
+    if (i == 0) *n_active = cnt;
 }
 
 // X_b *= mask (blockIdx.y = b)
@@ -1218,80 +1405,80 @@ int trace_slices(long long len, int want, int cap) {
 }
 
 template <typename T>
-void gram(cudaStream_t st, const T *X, long long sx, int nx, const T *Y, long long sy, int ny,
-          long long len, double *G, double *scratch) {
-    gram_multi<T>(st, X, sx, nx, 1, &Y, sy, ny, len, &G, scratch);
-}
-
-template <typename T>
-void gram_multi(cudaStream_t st, const T *X, long long sx, int nx, int nset, const T *const *Y, long long sy,
-                int per, long long len, double *const *G, double *scratch) {
-    if (nx <= 0 || per <= 0 || nset < 1) return;
-    if (nset > 4 || nx * per > 64 * 32) throw CudaError{cudaErrorInvalidValue, "gram: too many matrices"};
-    if (nx * per * nset > 64 * 32) {
-        // the partial sums of all pairs must fit the scratch: split the sets
-        const int h = nset / 2;
-        gram_multi<T>(st, X, sx, nx, h, Y, sy, per, len, G, scratch);
-        gram_multi<T>(st, X, sx, nx, nset - h, Y + h, sy, per, len, G + h, scratch);
-        return;
+void gram_blocks(cudaStream_t st, int k, int njob, const GramBlock<T> *job, int ldg, long long len, double *scratch) {
+    if (k <= 0 || njob <= 0 || len <= 0) return;
+    constexpr int VW = sizeof(T) == 4 ? 4 : 2;   // 16-byte loads
+    bool vec = len % VW == 0;
+    GramJobs js{};
+    js.n = njob, js.k = k, js.ldg = ldg;
+    int most = 0, sets = 0;
+    for (int m = 0; m < njob; ++m) {
+        GramJob &o = js.j[m];
+        o.x = job[m].x, o.nset = job[m].nset, o.first = js.pairs;
+        vec = vec && reinterpret_cast<uintptr_t>(o.x) % 16 == 0;
+        for (int q = 0; q < o.nset; ++q) {
+            o.y[q] = job[m].y[q], o.g[q] = job[m].g[q];
+            vec = vec && reinterpret_cast<uintptr_t>(o.y[q]) % 16 == 0;
+        }
+        js.pairs += o.nset * k * k;
+        sets += 1 + o.nset;
+        most = std::max(most, o.nset);
     }
-    const int ny = nset * per, pairs = nx * ny;
-    ProfScope ps(st, ST_TRACE, 2.0 * pairs * (double)len, sizeof(T) * (double)(nx + ny) * len);
-    YSet<T> ys{};
-    GOut go{};
-    for (int q = 0; q < 4; ++q) {
-        ys.p[q] = q < nset ? Y[q] : Y[0];
-        go.g[q] = q < nset ? G[q] : G[0];
-    }
-    ys.per = per;
+    if (njob > GRAM_JOBS || most > 4 || js.pairs > 64 * 32) throw CudaError{cudaErrorInvalidValue, "gram: too many matrices"};
+    ProfScope ps(st, ST_TRACE, 2.0 * js.pairs * (double)len, sizeof(T) * (double)sets * k * len);
     // float64 rows of at most 8192 elements: a warp walks 256 elements a step, so its share stays short
     // of the row kernel's (1024 elements: 180 us and 6 us for 16 pairs; 8192 elements, 64 pairs: the
     // warps read the rows about as fast as the row kernel's few blocks)
-    if (sizeof(T) == 8 && len > 0 && len <= 8192) {
-        gram_short_kernel<T><<<(pairs + 3) / 4, 128, 0, st>>>(X, sx, nx, ys, sy, ny, len, go);
+    if (sizeof(T) == 8 && len <= 8192) {
+        gram_short_kernel<T><<<(js.pairs + 3) / 4, 128, 0, st>>>(js, len);
         check_launch("gram_short_kernel");
         return;
     }
-    constexpr int VW = sizeof(T) == 4 ? 4 : 2;   // 16-byte loads
-    bool vec = len % VW == 0 && sx % VW == 0 && sy % VW == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0;
-    for (int q = 0; q < nset; ++q) vec = vec && reinterpret_cast<uintptr_t>(Y[q]) % 16 == 0;
-    const int gx = (nx + GQ - 1) / GQ, gy = (ny + GQ - 1) / GQ;
-    if (vec && len > 0 && nx + ny <= 256 * GMAXT / 16 && gx * gy <= 128) {
-        // every row read once (all pairs of a slice in one block)
+    const int ny = most * k;
+    auto grid_of = [&](int q) { return ((k + q - 1) / q) * ((ny + q - 1) / q); };
+    if (vec && k + ny <= 256 * GMAXT / 16 && grid_of(4) <= 128) {
+        // every row read once (all pairs of a slice in one block). Pair tiles of 2 x 2 where 128 threads
+        // hold them: the block waits for its slowest warp, and a warp's share of a chunk is a
+        // quarter of that of 4 x 4 tiles (10 x 10 pairs of 705600 elements: 64 and 45 us; the
+        // line step's three jobs at 140 atoms 206 and 136)
         constexpr int GC = gram_chunk<T>();
         const long long chunks = (len + GC - 1) / GC;
         const long long want = std::max<long long>(1, std::min<long long>(2 * TRACE_SLICES, (chunks + 15) / 16));
         const long long per_slice = (chunks + want - 1) / want * GC;
         const int slices = (int)((len + per_slice - 1) / per_slice);
-        const int RX = GQ * gx, RY = GQ * gy;
+        const int q = grid_of(2) <= 128 ? 2 : 4;
+        const int RX = (k + q - 1) / q * q, RY = (ny + q - 1) / q * q;
         const size_t smem = std::max((size_t)GST * (RX + RY) * gram_row<T>() * sizeof(T),
-                                     (size_t)GQ * GQ * 128 * sizeof(double));
+                                     (size_t)q * q * 128 * sizeof(double));
         // the attribute is set once, to the most any launch asks for: contexts on other host
         // threads launch this kernel concurrently, and a per-launch value would race with them
         static const bool attr = []() {
-            check(cudaFuncSetAttribute(gram_rows_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024),
+            check(cudaFuncSetAttribute(gram_rows_kernel<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024),
+                  "gram_rows smem");
+            check(cudaFuncSetAttribute(gram_rows_kernel<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024),
                   "gram_rows smem");
             return true;
         }();
         (void)attr;
-        gram_rows_kernel<T><<<slices, 256, smem, st>>>(X, sx, nx, ys, sy, ny, len, per_slice, RX, RY, scratch, pairs);
+        if (q == 2) gram_rows_kernel<T, 2><<<dim3(slices, njob), 256, smem, st>>>(js, len, per_slice, RX, RY, scratch);
+        else gram_rows_kernel<T, 4><<<dim3(slices, njob), 256, smem, st>>>(js, len, per_slice, RX, RY, scratch);
         check_launch("gram_rows_kernel");
-        gram_final_multi<<<(pairs + 7) / 8, 256, 0, st>>>(scratch, slices, pairs, ny, per, go);
-        check_launch("gram_final");
+        gram_final_jobs<<<(js.pairs + 7) / 8, 256, 0, st>>>(scratch, slices, js);
+        check_launch("gram_final_jobs");
         return;
     }
     const int slices = trace_slices(len, TRACE_SLICES, 2 * TRACE_SLICES);
-    const int ti = (nx + TI - 1) / TI;
+    const int ti = (k + TI - 1) / TI;
     if (vec) {
         const int tj = (ny + 3) / 4;
-        gram_tiled<T, VW, 4><<<dim3(ti * tj, slices), 256, 0, st>>>(X, sx, nx, ys, sy, ny, len, tj, scratch, pairs);
+        gram_tiled<T, VW, 4><<<dim3(ti * tj, slices, njob), 256, 0, st>>>(js, len, tj, scratch);
     } else {
         const int tj = (ny + 7) / 8;
-        gram_tiled<T, 1, 8><<<dim3(ti * tj, slices), 256, 0, st>>>(X, sx, nx, ys, sy, ny, len, tj, scratch, pairs);
+        gram_tiled<T, 1, 8><<<dim3(ti * tj, slices, njob), 256, 0, st>>>(js, len, tj, scratch);
     }
     check_launch("gram_tiled");
-    gram_final_multi<<<(pairs + 7) / 8, 256, 0, st>>>(scratch, slices, pairs, ny, per, go);
-    check_launch("gram_final");
+    gram_final_jobs<<<(js.pairs + 7) / 8, 256, 0, st>>>(scratch, slices, js);
+    check_launch("gram_final_jobs");
 }
 
 template <typename T>
@@ -1307,13 +1494,38 @@ void dots(cudaStream_t st, const T *X, long long sx, const T *Y, long long sy, i
 }
 
 template <typename T>
-void combine(cudaStream_t st, const double *C, int ldc, int nout, int nin, const T *in, long long sin,
-             T *out, long long sout, long long len, bool accumulate) {
+void step_combine(cudaStream_t st, int k, const double *Cp, const double *Cq, const double *lam, T *const *X,
+                  const T *const *D, int narr, long long len) {
+    if (k <= 0 || narr <= 0) return;
+    if (k > KMAX || narr > 4) throw CudaError{cudaErrorInvalidValue, "step_combine: too many rows"};
+    ProfScope ps(st, ST_VECTOR, 4.0 * narr * k * k * (double)len, sizeof(T) * (lam ? 6.0 : 4.0) * narr * k * (double)len);
+    CombArrays ar{};
+    constexpr int VW = sizeof(T) == 4 ? 2 : 1;   // elements a thread: 16 rows of them stay in registers
+    bool v = len % VW == 0;
+    for (int a = 0; a < narr; ++a) {
+        ar.x[a] = X[a];
+        ar.d[a] = lam ? D[a] : X[a];
+        v = v && reinterpret_cast<uintptr_t>(ar.x[a]) % 16 == 0 && reinterpret_cast<uintptr_t>(ar.d[a]) % 16 == 0;
+    }
+    const long long units = v ? len / VW : len;
+    const dim3 g((unsigned)std::max<long long>(1, std::min<long long>((units + 255) / 256, 152)), 2, narr);
+    if (v) {
+        if (k <= 4) step_combine_kernel<T, VW, 4><<<g, 256, 0, st>>>(Cp, Cq, lam, k, ar, len);
+        else if (k <= 8) step_combine_kernel<T, VW, 8><<<g, 256, 0, st>>>(Cp, Cq, lam, k, ar, len);
+        else if (k <= 12) step_combine_kernel<T, VW, 12><<<g, 256, 0, st>>>(Cp, Cq, lam, k, ar, len);
+        else step_combine_kernel<T, VW, 16><<<g, 256, 0, st>>>(Cp, Cq, lam, k, ar, len);
+    } else {
+        step_combine_kernel<T, 1, 16><<<g, 256, 0, st>>>(Cp, Cq, lam, k, ar, len);
+    }
+    check_launch("step_combine_kernel");
+}
+
+template <typename T>
+void combine(cudaStream_t st, const double *C, int ldc, int nout, int nin, const T *in, const T *base, T *out,
+             long long len) {
     if (nout > 32 || nin > 32) throw CudaError{cudaErrorInvalidValue, "combine: too many states"};
-    ProfScope ps(st, ST_VECTOR, 2.0 * nout * nin * (double)len,
-                 sizeof(T) * (double)(nin + nout * (accumulate ? 2 : 1)) * len);
-    combine_kernel<T><<<grid_for(len), 256, 0, st>>>(C, ldc, nout, nin, in, sin, out, sout, len,
-                                                      accumulate);
+    ProfScope ps(st, ST_VECTOR, 2.0 * nout * nin * (double)len, sizeof(T) * (double)(nin + nout * 2) * len);
+    combine_kernel<T><<<grid_for(len), 256, 0, st>>>(C, ldc, nout, nin, in, base, out, len);
     check_launch("combine_kernel");
 }
 
@@ -1393,11 +1605,27 @@ void init_gs(cudaStream_t st, int k, const double *PP, double *Cp, double *Cq, i
     init_gs_kernel<<<1, sb_threads(k), 0, st>>>(k, PP, Cp, Cq, status);
     check_launch("init_gs_kernel");
 }
-void cg_init(cudaStream_t st, int n, double tol, const double *rr0, double *rr, double *r0,
+void cg_init(cudaStream_t st, int n, const double *rr0, double *rr, double *r0,
              int *active, int *n_active) {
     ProfScope ps(st, ST_SMALL, 0.0, 0.0);
-    cg_init_kernel<<<1, 1, 0, st>>>(n, tol, rr0, rr, r0, active, n_active);
+    cg_init_kernel<<<1, 32, 0, st>>>(n, rr0, rr, r0, active, n_active);
     check_launch("cg_init_kernel");
+}
+// alpha from <p, Lp>, then z, r, <r, r>, beta and n_active: one launch each (dots, sums, scalars and
+// updates took eight launches of 3 to 4 us; 14400 elements, 10 systems: 7 and 10 us). partial as for dots; count: n + 1 zeros
+template <typename T>
+void cg_step(cudaStream_t st, const T *p, const T *Lp, T *z, T *r, long long len, int n, double tol, double *partial,
+             int *count, double *pLp, double *rr, const double *r0, double *alpha, double *beta, int *active, int *n_active) {
+    if (n <= 0) return;
+    const dim3 g(trace_slices(len, 2 * TRACE_SLICES, 2 * TRACE_SLICES), n);
+    {
+        ProfScope ps(st, ST_TRACE, 2.0 * n * (double)len, sizeof(T) * 2.0 * n * len);
+        cg_curvature_kernel<T><<<g, 256, 0, st>>>(p, Lp, len, n, partial, count, pLp, rr, alpha, active);
+        check_launch("cg_curvature_kernel");
+    }
+    ProfScope ps(st, ST_VECTOR, 6.0 * n * (double)len, sizeof(T) * 6.0 * n * len);
+    cg_move_kernel<T><<<g, 256, 0, st>>>(p, Lp, z, r, len, n, tol, partial, count, alpha, rr, r0, beta, active, n_active);
+    check_launch("cg_move_kernel");
 }
 // the one-block form for nb systems: false (nothing done) where it does not apply. In float64 up to
 // rc rv (rc + rv) = 131072 multiply-adds an iteration, 35 us at the two per cycle of one SM, what the
@@ -1415,7 +1643,7 @@ bool cg_reduced(cudaStream_t st, int rc, int rv, const T *Mc, const T *Mv, const
     }();
     (void)attr;
     check(cudaMemsetAsync(iters, 0, sizeof(int), st), "memset cg iterations");
-    cg_reduced_kernel<T><<<nb, CG_THREADS, sm, st>>>(rc, rv, Mc, Mv, r, z, tol, maxit, iters);
+    cg_reduced_kernel<T><<<nb, std::min(CG_THREADS, (rc * rv + 127) / 128 * 128), sm, st>>>(rc, rv, Mc, Mv, r, z, tol, maxit, iters);
     check_launch("cg_reduced_kernel");
     return true;
 }
@@ -1437,18 +1665,18 @@ void subspace(cudaStream_t st, int k, const double *A, double *omega, double *pa
 }
 
 #define INST(T)                                                                                   \
-    template void gram<T>(cudaStream_t, const T *, long long, int, const T *, long long, int,      \
-                          long long, double *, double *);                                         \
-    template void gram_multi<T>(cudaStream_t, const T *, long long, int, int, const T *const *,     \
-                                long long, int, long long, double *const *, double *);            \
+    template void gram_blocks<T>(cudaStream_t, int, int, const GramBlock<T> *, int, long long, double *); \
+    template void step_combine<T>(cudaStream_t, int, const double *, const double *, const double *, T *const *, \
+                                  const T *const *, int, long long);                              \
     template void dots<T>(cudaStream_t, const T *, long long, const T *, long long, int, long long, \
                           double *, double *);                                                    \
-    template void combine<T>(cudaStream_t, const double *, int, int, int, const T *, long long,    \
-                             T *, long long, long long, bool);                                    \
+    template void combine<T>(cudaStream_t, const double *, int, int, int, const T *, const T *, T *, long long); \
     template void mask_mul<T>(cudaStream_t, T *, const T *, long long, int);                      \
     template void axpy_dev<T>(cudaStream_t, const double *, int, double, T *, const T *, long long, \
                               int);                                                               \
     template void direction<T>(cudaStream_t, T *, const T *, const T *, const double *, long long); \
+    template void cg_step<T>(cudaStream_t, const T *, const T *, T *, T *, long long, int, double, double *, int *, double *, \
+                             double *, const double *, double *, double *, int *, int *);          \
     template void cg_dir<T>(cudaStream_t, T *, const T *, const double *, long long, int);
 INST(float)
 INST(double)

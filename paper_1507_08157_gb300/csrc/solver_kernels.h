@@ -26,8 +26,11 @@ void line_gs(cudaStream_t st, int k, const double *A, const double *BDf, const d
              const double *PP, const double *PD, const double *DP, const double *DD, const double *Q,
              double *lam, double *Cp, double *Cq, double *flip, int *status);
 void init_gs(cudaStream_t st, int k, const double *PP, double *Cp, double *Cq, int *status);
-void cg_init(cudaStream_t st, int n, double tol, const double *rr0, double *rr, double *r0,
-             int *active, int *n_active);
+void cg_init(cudaStream_t st, int n, const double *rr0, double *rr, double *r0, int *active, int *n_active);
+// one iteration's alpha, z, r, beta and n_active from p and L p of n systems; count: n + 1 zeros, left zero
+template <typename T>
+void cg_step(cudaStream_t st, const T *p, const T *Lp, T *z, T *r, long long len, int n, double tol, double *partial,
+             int *count, double *pLp, double *rr, const double *r0, double *alpha, double *beta, int *active, int *n_active);
 template <typename T>
 bool cg_reduced(cudaStream_t st, int rc, int rv, const T *Mc, const T *Mv, const T *r, T *z, int nb, double tol, int maxit,
                 int *iters);

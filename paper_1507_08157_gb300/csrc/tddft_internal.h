@@ -185,22 +185,31 @@ bool fft_size_ok(int n);
 
 // ---------------------------------------------------------------------------------------------
 // solver primitives
-// G[i][j] = sum_e X_i[e] * Y_j[e], i < nx, j < ny (float64 result; fixed reduction order).
-// X_i = X + i*sx, Y_j = Y + j*sy. scratch: >= gram_scratch_doubles(nx, ny) doubles.
+// Trace products of blocks of k rows (rows len apart): for every job and q < nset <= 4,
+// g[q][i * ldg + j] = sum_e x_i[e] y[q]_j[e], i, j < k (float64 result; fixed reduction order). A job's x
+// is read once for all its sets. scratch: >= gram_scratch_doubles(64, 32) doubles.
+constexpr int GRAM_JOBS = 3;
+template <typename T>
+struct GramBlock {
+    const T *x;
+    int nset;
+    const T *y[4];
+    double *g[4];
+};
 long long gram_scratch_doubles(int nx, int ny);
 template <typename T>
-void gram(cudaStream_t st, const T *X, long long sx, int nx, const T *Y, long long sy, int ny,
-          long long len, double *G, double *scratch);
-// several Gram matrices of one X at once: Y[q] (q < nset <= 4) holds `per` rows of stride sy and
-// G[q] receives [nx][per]; X is read once for all of them
-template <typename T>
-void gram_multi(cudaStream_t st, const T *X, long long sx, int nx, int nset, const T *const *Y, long long sy,
-                int per, long long len, double *const *G, double *scratch);
+void gram_blocks(cudaStream_t st, int k, int njob, const GramBlock<T> *job, int ldg, long long len, double *scratch);
 
-// out_i = beta * out_i + sum_j C[i*ldc + j] * in_j (C float64 on the device), out != in.
+// out_i = base_i + sum_j C[i*ldc + j] * in_j (C float64 on the device), out != in, rows len apart.
 template <typename T>
-void combine(cudaStream_t st, const double *C, int ldc, int nout, int nin, const T *in,
-             long long sin, T *out, long long sout, long long len, bool accumulate);
+void combine(cudaStream_t st, const double *C, int ldc, int nout, int nin, const T *in, const T *base, T *out,
+             long long len);
+
+// X_i <- sum_j C_ij (X_j + lam D_j) for narr <= 4 arrays of k p rows (C = Cp) and k q rows (Cq), in place;
+// lam a device scalar, or NULL: X_i <- sum_j C_ij X_j (D is not read)
+template <typename T>
+void step_combine(cudaStream_t st, int k, const double *Cp, const double *Cq, const double *lam, T *const *X,
+                  const T *const *D, int narr, long long len);
 
 // X_b[e] *= mask[e % len] for b < nb
 template <typename T>
