@@ -18,7 +18,9 @@
 #include <cstring>
 #include <initializer_list>
 #include <memory>
+#include <mutex>
 #include <new>
+#include <set>
 #include <stdexcept>
 #include <string>
 #include <thread>
@@ -302,8 +304,148 @@ struct Impl {
 
 using namespace tddft;
 
+namespace tddft {
+// The device memory of a context's states: one allocation per state, of which a context keeps the last
+// one given back for its next state (a state of 140 atoms and 10 states is 1.5 GB in 50 pieces, whose
+// allocation and release took 3 ms). Kept memory is bounded over all contexts (SLAB_KEEP), is only
+// reused by states of its own context (its stream orders the uses), and is freed with the
+// context, or when an allocation of any context fails. States share ownership of the pool: one may
+// outlive its context.
+class SlabPool {
+  public:
+    SlabPool() {
+        std::lock_guard<std::mutex> l(registry_mutex());
+        registry().insert(this);
+    }
+    ~SlabPool() {
+        {
+            std::lock_guard<std::mutex> l(registry_mutex());
+            registry().erase(this);
+        }
+        drop();
+        if (host_) cudaFreeHost(host_);
+    }
+    void *take(size_t bytes, size_t *got) {
+        {
+            std::lock_guard<std::mutex> l(m_);
+            if (p_ && size_ >= bytes && size_ / 2 <= bytes) {
+                void *p = p_;
+                *got = size_;
+                kept() -= size_;
+                p_ = nullptr;
+                return p;
+            }
+        }
+        drop();
+        void *p = nullptr;
+        cudaError_t e = cudaMalloc(&p, bytes);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            if (release_spare_slabs()) e = cudaMalloc(&p, bytes);
+        }
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            throw std::bad_alloc();
+        }
+        *got = bytes;
+        return p;
+    }
+    void give(void *p, size_t size) {
+        {
+            std::lock_guard<std::mutex> l(m_);
+            if (open_ && !p_) {
+                if (kept().fetch_add(size) + size <= SLAB_KEEP) {
+                    p_ = p;
+                    size_ = size;
+                    return;
+                }
+                kept() -= size;
+            }
+        }
+        cudaFree(p);
+    }
+    double *take_host() {      // pinned, HOST_DOUBLES
+        {
+            std::lock_guard<std::mutex> l(m_);
+            if (host_) {
+                double *h = host_;
+                host_ = nullptr;
+                return h;
+            }
+        }
+        double *h = nullptr;
+        check(cudaMallocHost(reinterpret_cast<void **>(&h), HOST_DOUBLES * sizeof(double)), "cudaMallocHost");
+        return h;
+    }
+    void give_host(double *h) {
+        {
+            std::lock_guard<std::mutex> l(m_);
+            if (open_ && !host_) {
+                host_ = h;
+                return;
+            }
+        }
+        cudaFreeHost(h);
+    }
+    bool drop() {              // frees the kept memory
+        void *p = nullptr;
+        {
+            std::lock_guard<std::mutex> l(m_);
+            if (p_) kept() -= size_;
+            std::swap(p, p_);
+        }
+        if (p) cudaFree(p);
+        return p != nullptr;
+    }
+    void close() {             // the context is gone: keep nothing from now on
+        {
+            std::lock_guard<std::mutex> l(m_);
+            open_ = false;
+        }
+        drop();
+    }
+    // never destroyed: pools may go after the process's other statics
+    static std::mutex &registry_mutex() { static auto *m = new std::mutex; return *m; }
+    static std::set<SlabPool *> &registry() { static auto *s = new std::set<SlabPool *>; return *s; }
+
+  private:
+    static constexpr size_t SLAB_KEEP = 4ull << 30;
+    static constexpr int HOST_DOUBLES = 4 * KMAX + 16;
+    static std::atomic<size_t> &kept() { static auto *k = new std::atomic<size_t>{0}; return *k; }
+    std::mutex m_;
+    void *p_ = nullptr;
+    size_t size_ = 0;
+    double *host_ = nullptr;
+    bool open_ = true;
+};
+
+bool release_spare_slabs() {
+    std::lock_guard<std::mutex> l(SlabPool::registry_mutex());
+    bool any = false;
+    for (SlabPool *p : SlabPool::registry()) any = p->drop() || any;
+    return any;
+}
+
+// pieces of one allocation: a first pass with no memory adds up the sizes
+struct Slab {
+    std::shared_ptr<SlabPool> pool;
+    char *base = nullptr;
+    size_t used = 0, size = 0;
+    template <typename U>
+    U *piece(size_t n) {
+        char *p = base ? base + used : nullptr;
+        used += (std::max<size_t>(n, 1) * sizeof(U) + 255) / 256 * 256;
+        return reinterpret_cast<U *>(p);
+    }
+    ~Slab() {
+        if (base) pool->give(base, size);
+    }
+};
+}  // namespace tddft
+
 struct tddft_ctx {
     cudaStream_t st = nullptr;
+    std::shared_ptr<SlabPool> slabs = std::make_shared<SlabPool>();
     tddft_options opt{};
     int prec = TDDFT_FP64;
     int n = 0, nt = 0, natoms = 0, nc = 0, nv = 0;
@@ -399,6 +541,7 @@ void register_constants(Impl<double> &) {}
 
 tddft_ctx::~tddft_ctx() {
     if (own_stream && st) cudaStreamSynchronize(st);
+    slabs->close();
     if (prof) profiler_delete(prof);
     if (d32) {
         Impl<float> &I = *d32;
@@ -1485,10 +1628,10 @@ namespace {
 
 template <typename T>
 struct StateBufs {
-    Mem mem;
+    Slab mem;
     T *Y, *P, *f, *g, *G1, *h, *z, *Z, *dir, *D, *fD, *covP, *covD;
     T *pdir, *pD, *pz, *pZ, *tmp;
-    T *cr, *cp, *cLp, *cLpp, *cpv, *cLv;   // inner CG
+    T *cr, *cp, *cLp, *cLpp;   // inner CG
     T *qr = nullptr, *qp = nullptr, *qL = nullptr, *qz = nullptr;   // inner CG on the reduced space
     double *A, *BDf, *CDfD, *PP, *PD, *DP, *DD, *Q, *coef, *Cp, *Cq, *lam, *sc, *flip;
     double *dvec, *dvec2, *dvec3, *evout;
@@ -1510,10 +1653,11 @@ struct tddft_state {
     std::vector<double> omega, resid, omega_prev;
     std::unique_ptr<StateBufs<double>> s64;
     std::unique_ptr<StateBufs<float>> s32;
+    std::shared_ptr<SlabPool> slabs;
     double *host = nullptr;   // pinned, 4k + 16 doubles: [omega k][resid k][status, n_active][lam]
                               // (tddft_subspace uses [omega k][pairing 2k])
     ~tddft_state() {
-        if (host) cudaFreeHost(host);
+        if (host) slabs->give_host(host);
     }
 };
 
@@ -1525,39 +1669,44 @@ template <> StateBufs<float> &bufs<float>(tddft_state *s) { return *s->s32; }
 
 template <typename T>
 void alloc_state(tddft_ctx *c, tddft_state *S) {
+    S->slabs = c->slabs;
+    S->host = c->slabs->take_host();
     auto B = std::make_unique<StateBufs<T>>();
+    Impl<T> &I = impl<T>(c);
     const size_t n2 = (size_t)2 * S->k * c->len();
-    T **mats[] = {&B->Y, &B->P, &B->f, &B->g, &B->G1, &B->h, &B->z, &B->Z, &B->dir, &B->D,
-                  &B->fD, &B->covP, &B->covD, &B->pdir, &B->pD, &B->pz, &B->pZ, &B->tmp,
-                  &B->cr, &B->cp, &B->cLp, &B->cLpp, &B->cpv, &B->cLv};
-    for (T **m : mats) *m = B->mem.template alloc<T>(n2);
     const size_t k2 = 2 * S->k, kk4 = k2 * k2, kk = (size_t)S->k * S->k;
-    double **sm[] = {&B->A, &B->BDf, &B->CDfD, &B->PP, &B->PD, &B->DP, &B->DD, &B->coef};
-    for (double **m : sm) *m = B->mem.template alloc<double>(kk4);
-    B->Q = B->mem.template alloc<double>(kk);
-    B->Cp = B->mem.template alloc<double>(kk);
-    B->Cq = B->mem.template alloc<double>(kk);
-    B->lam = B->mem.template alloc<double>(1);
-    B->sc = B->mem.template alloc<double>(4);
-    B->flip = B->mem.template alloc<double>(1);
-    double **vv[] = {&B->dvec, &B->dvec2, &B->dvec3, &B->evout, &B->cg_pLp, &B->cg_rr, &B->cg_rrn,
-                     &B->cg_r0, &B->cg_alpha, &B->cg_beta};
-    for (double **m : vv) *m = B->mem.template alloc<double>(k2);
-    B->gscr = B->mem.template alloc<double>((size_t)gram_scratch_doubles(64, 32));
-    {
-        Impl<T> &I = impl<T>(c);
+    auto place = [&]() {
+        Slab &m = B->mem;
+        T **mats[] = {&B->Y, &B->P, &B->f, &B->g, &B->G1, &B->h, &B->z, &B->Z, &B->dir, &B->D,
+                      &B->fD, &B->covP, &B->covD, &B->pdir, &B->pD, &B->pz, &B->pZ, &B->tmp,
+                      &B->cr, &B->cp, &B->cLp, &B->cLpp};
+        for (T **x : mats) *x = m.piece<T>(n2);
+        double **sm[] = {&B->A, &B->BDf, &B->CDfD, &B->PP, &B->PD, &B->DP, &B->DD, &B->coef};
+        for (double **x : sm) *x = m.piece<double>(kk4);
+        double **sq[] = {&B->Q, &B->Cp, &B->Cq};
+        for (double **x : sq) *x = m.piece<double>(kk);
+        B->lam = m.piece<double>(1);
+        B->sc = m.piece<double>(4);
+        B->flip = m.piece<double>(1);
+        double **vv[] = {&B->dvec, &B->dvec2, &B->dvec3, &B->evout, &B->cg_pLp, &B->cg_rr, &B->cg_rrn,
+                         &B->cg_r0, &B->cg_alpha, &B->cg_beta};
+        for (double **x : vv) *x = m.piece<double>(k2);
+        B->gscr = m.piece<double>((size_t)gram_scratch_doubles(64, 32));
         if (I.rc) {
-            const size_t nq = (size_t)2 * S->k * I.rc * I.rv;
-            B->qr = B->mem.template alloc<T>(nq);
-            B->qp = B->mem.template alloc<T>(nq);
-            B->qL = B->mem.template alloc<T>(nq);
-            B->qz = B->mem.template alloc<T>(nq);
+            T **qs[] = {&B->qr, &B->qp, &B->qL, &B->qz};
+            for (T **x : qs) *x = m.piece<T>((size_t)2 * S->k * I.rc * I.rv);
         }
-    }
-    B->status = B->mem.template alloc<int>(1);
-    B->cg_active = B->mem.template alloc<int>(k2);
-    B->cg_nactive = B->mem.template alloc<int>(1);
-    B->cg_count = B->mem.template alloc<int>(k2 + 1);
+        B->status = m.piece<int>(1);
+        B->cg_active = m.piece<int>(k2);
+        B->cg_nactive = m.piece<int>(1);
+        B->cg_count = m.piece<int>(k2 + 1);
+    };
+    place();
+    const size_t need = B->mem.used;
+    B->mem.pool = c->slabs;
+    B->mem.base = static_cast<char *>(c->slabs->take(need, &B->mem.size));
+    B->mem.used = 0;
+    place();
     check(cudaMemsetAsync(B->cg_count, 0, (k2 + 1) * sizeof(int), c->st), "memset cg counts");
     check(cudaMemsetAsync(B->sc, 0, 4 * sizeof(double), c->st), "memset sc");
     check(cudaMemsetAsync(B->flip, 0, sizeof(double), c->st), "memset flip");
@@ -2478,7 +2627,6 @@ tddft_status tddft_state_create(tddft_ctx *c, int32_t k, const double *Y0, tddft
         if (k <= 0 || k > KMAX || !Y0) throw InvalidArg{"tddft_state_create: need 1 <= k <= 16 and Y0"};
         S->ctx = c;
         S->k = k;
-        check(cudaMallocHost(reinterpret_cast<void **>(&S->host), (4 * k + 16) * sizeof(double)), "cudaMallocHost");
         return DISPATCH(c, ([&]() {
             alloc_state<T>(c, S.get());
             state_init<T>(c, S.get(), Y0);
@@ -2605,8 +2753,6 @@ tddft_status tddft_state_import(tddft_ctx *c, const void *buf, size_t len, tddft
         S->fallbacks = h.fallbacks;
         S->inner_iters = h.inner_iters;
         S->have_prev_omega = h.have_prev_omega != 0;
-        check(cudaMallocHost(reinterpret_cast<void **>(&S->host), (4 * S->k + 16) * sizeof(double)),
-              "cudaMallocHost");
         return DISPATCH(c, ([&]() {
             Impl<T> &I = impl<T>(c);
             alloc_state<T>(c, S.get());

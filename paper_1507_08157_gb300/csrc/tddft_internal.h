@@ -19,6 +19,8 @@ struct CudaError {
 };
 
 // owning list of device allocations (freed on release or destruction)
+bool release_spare_slabs();   // frees the memory that contexts keep of destroyed states; true if there was any
+
 struct Mem {
     std::vector<void *> ptrs;
     template <typename T>
@@ -26,6 +28,10 @@ struct Mem {
         void *p = nullptr;
         if (n == 0) n = 1;
         cudaError_t e = cudaMalloc(&p, n * sizeof(T));
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            if (release_spare_slabs()) e = cudaMalloc(&p, n * sizeof(T));
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             throw std::bad_alloc();
