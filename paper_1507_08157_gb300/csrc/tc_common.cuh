@@ -126,6 +126,14 @@ __device__ __forceinline__ void mma_tf32(unsigned tmem_d, unsigned long long da,
         ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate));
 }
 
+// the same with the A operand in TMEM: row i in lane i, one 32-bit column per element of K
+__device__ __forceinline__ void mma_tf32_ta(unsigned tmem_d, unsigned tmem_a, unsigned long long db, unsigned idesc,
+                                            unsigned accumulate) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n"
+        ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(accumulate));
+}
+
 // one lane of a converged warp; the compiler knows that a region under it has one thread, and keeps
 // what it computes for the tensor instructions in uniform registers
 __device__ __forceinline__ bool elect_one() {
@@ -154,6 +162,17 @@ __device__ __forceinline__ void tmem_ld32(unsigned taddr, float *v) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+
+// 16 columns of the warp's lanes into TMEM; visible to MMAs after tmem_st_wait, a fence and a barrier
+__device__ __forceinline__ void tmem_st16(unsigned taddr, const float *v) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15};" ::"f"(v[0]),
+        "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]), "f"(v[10]),
+        "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]), "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // 16 columns
 __device__ __forceinline__ void tmem_ld16(unsigned taddr, float *v) {

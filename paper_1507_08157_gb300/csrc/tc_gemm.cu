@@ -278,6 +278,303 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(
     if (threadIdx.x == 0 && ctl->abort) atomicExch(err, 1);
 }
 
+// ---- variable times constant -------------------------------------------------------------------
+// C[b] = alpha W X[b] + beta C[b] (LEFT: W M x K constant, X K x N) or C = alpha X W^T + beta C (X M x K
+// variable, W N x K constant), three-term split (SPLIT) or
+// plain TF32, with the variable operand in TMEM as the MMA's A.
+// What bounds the kernel above at 128 x 128 tiles is shared memory: per K slice of 32 the TMA's writes,
+// the splits and the reads of three MMAs are 196 KB or more, 1500 cycles at 128 bytes a cycle, against 830
+// of tensor work. Here X never returns to shared memory after its split (it goes to TMEM) and the
+// MMAs read only W there: 144 KB a slice, of which 32 KB come through L2 (X and W unsplit;
+// 44 to 60 KB above). LEFT computes C^T tiles (lanes along N), so that X is read as it lies, without a
+// transposed copy, and a warp's stores of one row of C are 128 consecutive bytes. The products
+// of an element are added in the order of the kernel above (the same results bit by bit). 140 atoms,
+// 1260 x 560: 20 and 10 systems from the left and right 0.57 ms with the kernel above and its transposed
+// copies, 0.42 here; one-term products of 20 systems 70 us with and 45 without copies.
+// 14 warps: 0-3 read the accumulators and write C, 4-7 split X into TMEM (warp w owns lanes
+// 32 (w % 4) on), 8-11 split W in place, 12 loads by TMA, 13 issues the MMAs. TMEM: two accumulators of
+// 128 columns and four stages of 64 (hi and lo of 32 K).
+// cvt.rna.tf32 by the bits (half a unit of the 13 dropped bits added to the magnitude): the conversion
+// runs at a fraction of the integer rate (5 % of the kernel). A NaN may lose its mark in hi but keeps
+// it in x - hi.
+__device__ __forceinline__ float tf32_bits(float x) {
+    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
+}
+constexpr int XS = 4;                                       // stages
+constexpr int X_STAGE_BYTES = 3 * TILE_BYTES;               // X, W (hi in place), W lo
+constexpr int XGEMM_THREADS = 14 * 32;
+struct __align__(8) XShared {
+    unsigned long long full[XS], ready[XS], empty[XS], acc_full[2], acc_empty[2], drain;
+    unsigned int tmem_base;
+    int abort;
+};
+constexpr size_t XGEMM_SMEM = (size_t)XS * X_STAGE_BYTES + STAGE_FLOATS * sizeof(float) + sizeof(XShared) + 1024;
+
+template <bool LEFT, int TN, bool SPLIT>
+__global__ void __launch_bounds__(XGEMM_THREADS, 1) tc_gemm_x_kernel(
+    const __grid_constant__ CUtensorMap mX, const __grid_constant__ CUtensorMap mW, int M, int N, int K, int batch,
+    float alpha, float beta, float *__restrict__ C, int ldc, long long sC, int *err, long long wlim) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *tiles = reinterpret_cast<unsigned char *>(
+        (reinterpret_cast<unsigned long long>(smem_raw) + 1023ull) & ~1023ull);
+    float *staging = reinterpret_cast<float *>(tiles + (size_t)XS * X_STAGE_BYTES);
+    XShared *ctl = reinterpret_cast<XShared *>(staging + STAGE_FLOATS);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // tiles: 128 lanes along N (LEFT) or M, TN columns along the other, the lanes' index fastest
+    const int tl = ((LEFT ? N : M) + 127) / 128, tc = ((LEFT ? M : N) + TN - 1) / TN;
+    const int ntiles = tl * tc * batch, nk = (K + TBK - 1) / TBK;
+    auto tile = [&](int t, int &l0, int &c0, int &b) {
+        // the columns' tiles of one stretch of X follow one another (LEFT: X is the larger operand too)
+        c0 = (t % tc) * TN;
+        l0 = ((t / tc) % tl) * 128;
+        b = t / (tc * tl);
+    };
+    volatile int *abort = &ctl->abort;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < XS; ++s) {
+            mbar_init(&ctl->full[s], 1);
+            mbar_init(&ctl->ready[s], SPLIT ? 256 : 128);
+            mbar_init(&ctl->empty[s], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&ctl->acc_full[i], 1);
+            mbar_init(&ctl->acc_empty[i], 128);
+        }
+        mbar_init(&ctl->drain, 1);
+        ctl->abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 13) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
+                     "r"(512));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const unsigned tmem = ctl->tmem_base, tmem_x = tmem + 256;
+
+    if (warp == 12) {
+        if (lane == 0) {
+            long long it = 0;
+            bool go = true;
+            for (int t = blockIdx.x; t < ntiles && go; t += gridDim.x) {
+                int l0, c0, b;
+                tile(t, l0, c0, b);
+                for (int kb = 0; kb < nk; ++kb, ++it) {
+                    const int s = (int)(it % XS);
+                    if (!mbar_wait(&ctl->empty[s], (unsigned)(((it / XS) & 1) ^ 1), abort, wlim)) {
+                        go = false;
+                        break;
+                    }
+                    unsigned char *st = tiles + (size_t)s * X_STAGE_BYTES;
+                    mbar_expect_tx(&ctl->full[s], TILE_BYTES + TN * TBK * 4);
+                    if (LEFT) tma_load_3d(st, &mX, &ctl->full[s], l0, kb * TBK, b);
+                    else tma_load_3d(st, &mX, &ctl->full[s], kb * TBK, l0, b);
+                    tma_load_3d(st + TILE_BYTES, &mW, &ctl->full[s], kb * TBK, c0, 0);
+                }
+            }
+            if (*abort)      // the loads already issued land before the block exits
+                for (long long j = it > XS ? it - XS : 0; j < it; ++j)
+                    mbar_drain(&ctl->full[j % XS], (unsigned)((j / XS) & 1), wlim);
+        }
+    } else if (warp == 13) {
+        constexpr unsigned idesc = idesc_tf32(128, TN);
+        long long it = 0;
+        int tcount = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tcount) {
+            const int buf = tcount & 1, use = tcount >> 1;
+            // the whole warp goes on or none of it
+            if (!__all_sync(0xffffffffu, mbar_wait(&ctl->acc_empty[buf], (unsigned)((use & 1) ^ 1), abort, wlim))) break;
+            const unsigned acc_t = tmem + (unsigned)(buf * 128);
+            for (int kb = 0; kb < nk; ++kb, ++it) {
+                const int s = (int)(it % XS);
+                // (one term: W is used as it landed)
+                ok = __all_sync(0xffffffffu, (SPLIT || mbar_wait(&ctl->full[s], (unsigned)((it / XS) & 1), abort, wlim)) &&
+                                                 mbar_wait(&ctl->ready[s], (unsigned)((it / XS) & 1), abort, wlim));
+                if (!ok) break;
+                tc_fence_after();
+                if (elect_one()) {
+                    const unsigned w = desc_lo(smem_u32(tiles + (size_t)s * X_STAGE_BYTES + TILE_BYTES));
+                    const unsigned xh = tmem_x + (unsigned)(s * 64), xl = xh + 32;
+#pragma unroll
+                    for (int kk = 0; kk < TBK / 8; ++kk) {
+                        // 8 K: 8 columns of X, 32 bytes inside the swizzle rows of W
+                        const unsigned long long wh = desc_of(w + kk * 2), wl = desc_of(w + kk * 2 + TILE_BYTES / 16);
+                        mma_tf32_ta(acc_t, xh + kk * 8, wh, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+                        if (SPLIT) {
+                            mma_tf32_ta(acc_t, LEFT ? xl + kk * 8 : xh + kk * 8, LEFT ? wh : wl, idesc, 1u);
+                            mma_tf32_ta(acc_t, LEFT ? xh + kk * 8 : xl + kk * 8, LEFT ? wl : wh, idesc, 1u);
+                        }
+                    }
+                    mma_commit(&ctl->empty[s]);
+                }
+                __syncwarp();
+            }
+            if (!ok) break;
+            if (elect_one()) mma_commit(&ctl->acc_full[buf]);
+            __syncwarp();
+        }
+        if (*abort) {        // the MMAs already issued finish before TMEM is freed
+            if (elect_one()) {
+                mma_commit(&ctl->drain);
+                mbar_drain(&ctl->drain, 0, wlim);
+            }
+            __syncwarp();
+        }
+    } else if (warp >= 8) {
+        const int ts = threadIdx.x - 256;
+        long long it = 0;
+        bool go = true;
+        for (int t = blockIdx.x; SPLIT && t < ntiles && go; t += gridDim.x)
+            for (int kb = 0; kb < nk; ++kb, ++it) {
+                const int s = (int)(it % XS);
+                if (!mbar_wait(&ctl->full[s], (unsigned)((it / XS) & 1), abort, wlim)) {
+                    go = false;
+                    break;
+                }
+                float4 *hi = reinterpret_cast<float4 *>(tiles + (size_t)s * X_STAGE_BYTES + TILE_BYTES);
+                float4 *lo = hi + TILE_BYTES / 16;
+                // element-wise, so that the swizzled layout carries over
+#pragma unroll
+                for (int i = 0; i < TN * TBK / 4 / 128; ++i) {
+                    const float4 x = hi[ts + 128 * i];
+                    float4 h, l;
+                    h.x = tf32_bits(x.x);
+                    h.y = tf32_bits(x.y);
+                    h.z = tf32_bits(x.z);
+                    h.w = tf32_bits(x.w);
+                    l.x = x.x - h.x;
+                    l.y = x.y - h.y;
+                    l.z = x.z - h.z;
+                    l.w = x.w - h.w;
+                    hi[ts + 128 * i] = h;
+                    lo[ts + 128 * i] = l;
+                }
+                fence_async_smem();
+                mbar_arrive(&ctl->ready[s]);
+            }
+    } else if (warp >= 4) {
+        const int row = (warp - 4) * 32 + lane;              // this thread's lane of TMEM
+        const unsigned tq = tmem_x + ((unsigned)((warp - 4) * 32) << 16);
+        long long it = 0;
+        bool go = true;
+        for (int t = blockIdx.x; t < ntiles && go; t += gridDim.x)
+            for (int kb = 0; kb < nk; ++kb, ++it) {
+                const int s = (int)(it % XS);
+                go = mbar_wait(&ctl->full[s], (unsigned)((it / XS) & 1), abort, wlim);
+                if (!__all_sync(0xffffffffu, go)) {          // the stores below are for the whole warp
+                    go = false;
+                    break;
+                }
+                const unsigned char *st = tiles + (size_t)s * X_STAGE_BYTES;
+                tc_fence_after();      // the stage's last MMAs are done: their completion came before the load
+#pragma unroll
+                for (int k0 = 0; k0 < 32; k0 += 16) {
+                    float h[16], l[16];
+                    if (LEFT) {
+                        const float *x = reinterpret_cast<const float *>(st) + row;  // [k][128 lanes]
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) l[k] = x[(k0 + k) * 128];
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {                                // 16 bytes of a swizzled row
+                            const float4 x = *reinterpret_cast<const float4 *>(st + sw128_offset(row, k0 / 4 + c));
+                            l[4 * c] = x.x, l[4 * c + 1] = x.y, l[4 * c + 2] = x.z, l[4 * c + 3] = x.w;
+                        }
+                    }
+                    if (SPLIT) {
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) {
+                            h[k] = tf32_bits(l[k]);
+                            l[k] = l[k] - h[k];
+                        }
+                        tmem_st16(tq + (unsigned)(s * 64 + k0), h);
+                        tmem_st16(tq + (unsigned)(s * 64 + 32 + k0), l);
+                    } else {
+                        tmem_st16(tq + (unsigned)(s * 64 + k0), l);
+                    }
+                }
+                tmem_st_wait();
+                tc_fence_before();
+                mbar_arrive(&ctl->ready[s]);
+            }
+    } else {
+        float *stg = staging + warp * 32 * 33;
+        int tcount = 0;
+        for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++tcount) {
+            const int buf = tcount & 1, use = tcount >> 1;
+            const bool full = mbar_wait(&ctl->acc_full[buf], (unsigned)(use & 1), abort, wlim);
+            if (!__all_sync(0xffffffffu, full)) break;
+            tc_fence_after();
+            int l0, c0, b;
+            tile(t, l0, c0, b);
+            const unsigned ta = tmem + (unsigned)(buf * 128) + ((unsigned)(warp * 32) << 16);
+            l0 += warp * 32;
+            if (LEFT) {
+                float *cw = C + (long long)b * sC + (long long)c0 * ldc + l0 + lane;     // lane = column of C
+                const bool on = l0 + lane < N;
+                for (int j0 = 0; j0 < TN; j0 += 16) {
+                    const int nrow = min(16, M - (c0 + j0));
+                    float v[16], old[16];
+                    float *cj = cw + (long long)j0 * ldc;
+                    if (beta != 0.0f) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) old[j] = (j < nrow && on) ? cj[(long long)j * ldc] : 0.0f;
+                    }
+                    tmem_ld16(ta + (unsigned)j0, v);
+                    if (beta == 0.0f) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (j < nrow && on) cj[(long long)j * ldc] = alpha * v[j];
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (j < nrow && on) cj[(long long)j * ldc] = fmaf(alpha, v[j], beta * old[j]);
+                    }
+                }
+            } else {
+                const int nrow = min(32, M - l0);                                        // rows of this warp inside C
+                for (int j0 = 0; j0 < TN; j0 += 32) {
+                    const int col = c0 + j0 + lane;
+                    const bool on = j0 + lane < TN && col < N;
+                    float *cw = C + (long long)b * sC + (long long)l0 * ldc + col;
+                    float old[32];
+                    if (beta != 0.0f) {
+#pragma unroll
+                        for (int r = 0; r < 32; ++r) old[r] = (r < nrow && on) ? cw[(long long)r * ldc] : 0.0f;
+                    }
+                    float v[32];
+                    tmem_ld32(ta + (unsigned)j0, v);
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) stg[lane * 33 + j] = v[j];
+                    __syncwarp();
+                    if (beta == 0.0f) {
+#pragma unroll 8
+                        for (int r = 0; r < 32; ++r)
+                            if (r < nrow && on) cw[(long long)r * ldc] = alpha * stg[r * 33 + lane];
+                    } else {
+#pragma unroll
+                        for (int r = 0; r < 32; ++r)
+                            if (r < nrow && on) cw[(long long)r * ldc] = fmaf(alpha, stg[r * 33 + lane], beta * old[r]);
+                    }
+                    __syncwarp();
+                }
+            }
+            tc_fence_before();
+            mbar_arrive(&ctl->acc_empty[buf]);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 13) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    }
+    if (threadIdx.x == 0 && ctl->abort) atomicExch(err, 1);
+}
+
 // ---- host side ---------------------------------------------------------------------------------
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -337,6 +634,68 @@ int *error_word() {
 }  // namespace
 
 bool tc_gemm_available() { return encode_fn() != nullptr; }
+
+namespace {
+// X [batch][K][N] (LEFT) or [batch][M][K] with row stride ldx and batch stride sx, W rows K-contiguous
+template <bool LEFT, int TN, bool SPLIT>
+void launch_x(cudaStream_t st, int M, int N, int K, float alpha, const float *X, int ldx, long long sx, const float *W,
+              int ldw, float beta, float *C, int ldc, long long sC, int batch) {
+    CUtensorMap mx, mw;
+    bool ok = make_map(&mw, W, K, LEFT ? M : N, ldw, 0, 1, TN);
+    if (LEFT) {
+        // box 128 (N) x 32 (K), rows of the box 512 bytes apart in shared memory, zero fill outside
+        auto fn = encode_fn();
+        cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)K, (cuuint64_t)batch};
+        cuuint64_t strides[2] = {(cuuint64_t)ldx * 4, (cuuint64_t)(batch > 1 ? sx * 4 : (long long)ldx * K * 4)};
+        cuuint32_t box[3] = {128, TBK, 1}, estr[3] = {1, 1, 1};
+        ok = ok && fn(&mx, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(X), dims, strides, box, estr,
+                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    } else {
+        ok = ok && make_map(&mx, X, K, M, ldx, sx, batch, 128);
+    }
+    if (!ok) throw CudaError{cudaErrorInvalidValue, "cuTensorMapEncodeTiled (variable times constant)"};
+    static const bool attr = []() {   // once per process, thread-safe
+        check(cudaFuncSetAttribute(tc_gemm_x_kernel<LEFT, TN, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)XGEMM_SMEM), "attr tc_gemm_x");
+        return true;
+    }();
+    (void)attr;
+    const long long ntiles = (long long)(((LEFT ? N : M) + 127) / 128) * (((LEFT ? M : N) + TN - 1) / TN) * batch;
+    const int grid = (int)std::min<long long>(ntiles, sm_count());
+    tc_gemm_x_kernel<LEFT, TN, SPLIT><<<grid, XGEMM_THREADS, XGEMM_SMEM, st>>>(mx, mw, M, N, K, batch, alpha, beta, C, ldc, sC,
+                                                                        error_word(), active_wait_limit());
+    check_launch("tc_gemm_x_kernel");
+}
+
+// The width of the tiles: a slice costs about 256 + 7 TN cycles of shared memory (X is written and read
+// once; W written, split and read three times) and the busiest SM does ceil(tiles / SMs) tiles, so that
+// products of few tiles take narrower ones (60 atoms, 150 products of 120 to 240 wide matrices of 10
+// systems: 2.02 ms all in 128 wide tiles, 1.51 by this rule).
+template <bool LEFT, bool SPLIT>
+void gemm_x_tiles(cudaStream_t st, int M, int N, int K, float alpha, const float *X, int ldx, long long sx, const float *W,
+            int ldw, float beta, float *C, int ldc, long long sC, int batch) {
+    const int lanes = LEFT ? N : M, cols = LEFT ? M : N;
+    auto cost = [&](int tn) {
+        const long long tiles = (long long)((lanes + 127) / 128) * ((cols + tn - 1) / tn) * batch;
+        return (tiles + sm_count() - 1) / sm_count() * (256 + 7 * tn);
+    };
+    int best = cols % 112 == 0 ? 112 : 128;
+    for (int tn : {64, 32})
+        if (cost(tn) < cost(best)) best = tn;
+    auto go = [&](auto launch) { launch(st, M, N, K, alpha, X, ldx, sx, W, ldw, beta, C, ldc, sC, batch); };
+    if (best == 128) go(launch_x<LEFT, 128, SPLIT>);
+    else if (best == 112) go(launch_x<LEFT, 112, SPLIT>);
+    else if (best == 64) go(launch_x<LEFT, 64, SPLIT>);
+    else go(launch_x<LEFT, 32, SPLIT>);
+}
+template <bool LEFT>
+void gemm_x(bool split, cudaStream_t st, int M, int N, int K, float alpha, const float *X, int ldx, long long sx,
+            const float *W, int ldw, float beta, float *C, int ldc, long long sC, int batch) {
+    if (split) gemm_x_tiles<LEFT, true>(st, M, N, K, alpha, X, ldx, sx, W, ldw, beta, C, ldc, sC, batch);
+    else gemm_x_tiles<LEFT, false>(st, M, N, K, alpha, X, ldx, sx, W, ldw, beta, C, ldc, sC, batch);
+}
+}  // namespace
 
 // 3-D tiled float32 map, 128-byte swizzle, zero fill outside: dims d0 (contiguous) x d1 x d2,
 // strides of dims 1 and 2 in bytes, box b0 x b1 x 1
@@ -530,21 +889,21 @@ std::vector<SplitCopy> *const_entry(const float *p) {
     return nullptr;
 }
 
-// hi/lo K-major copy of a constant operand: rows x K out of a (rows x K, !trans) or (K x rows,
-// trans) matrix with leading dimension ld
-bool const_split(cudaStream_t st, const float *p, bool trans, int rows, int K, int ld, SplitCopy *out) {
+// K-major copy of a constant operand, hi/lo or (raw) as it is: rows x K out of a (rows x K, !trans) or
+// (K x rows, trans) matrix with leading dimension ld
+bool const_split(cudaStream_t st, const float *p, bool trans, int rows, int K, int ld, SplitCopy *out, bool raw = false) {
     std::lock_guard<std::mutex> lock(g_const_mu);
     std::vector<SplitCopy> *v = const_entry(p);
     if (!v) return false;
     for (const SplitCopy &c : *v)
-        if (c.trans == trans && c.rows == rows && c.cols == K && c.ld == ld) {
+        if (c.trans == trans && c.rows == rows && c.cols == K && c.ld == ld && raw == !c.lo) {
             *out = c;
             return true;
         }
     SplitCopy c{trans, rows, K, ld, nullptr, nullptr, (K + 3) / 4 * 4};
     const size_t n = (size_t)rows * c.kp;
     check(cudaMalloc(&c.hi, n * sizeof(float)), "cudaMalloc constant split");
-    check(cudaMalloc(&c.lo, n * sizeof(float)), "cudaMalloc constant split");
+    if (!raw) check(cudaMalloc(&c.lo, n * sizeof(float)), "cudaMalloc constant split");
     if (!trans) {
         split_kernel<<<grid1((long long)n), 256, 0, st>>>(p, rows, K, ld, 0, c.hi, c.lo, c.kp, 0, 1);
     } else {
@@ -577,8 +936,9 @@ void tc_unregister_constant(const float *p) {
 }
 
 // Dispatch of a row-major C[b] = alpha op(A[b]) op(B[b]) + beta C[b] onto the tensor cores. The
-// kernel wants both operands K-contiguous with 16-byte row starts. A registered constant operand
-// comes from its cached hi/lo copy; a K-contiguous variable operand goes in as it lies and is
+// kernels want 16-byte row starts. A registered constant times a variable operand that lies as a tensor
+// map can read it goes to the kernel for that form, the constant from a cached K-major copy. Else both
+// operands are K-contiguous: a registered constant comes from its cached hi/lo copy; a K-contiguous variable operand goes in as it lies and is
 // split inside the kernel; any other operand gets a hi/lo K-major copy in scratch.
 void tc_gemm(cudaStream_t st, bool ta, bool tb, int M, int N, int K, float alpha, const float *A, int lda,
              long long sA, const float *B, int ldb, long long sB, float beta, float *C, int ldc, long long sC,
@@ -588,6 +948,18 @@ void tc_gemm(cudaStream_t st, bool ta, bool tb, int M, int N, int K, float alpha
         return reinterpret_cast<unsigned long long>(p) % 16 == 0 && ld % 4 == 0 && s % 4 == 0;
     };
     SplitCopy cav{}, cbv{};
+    if (!ta) {
+        // a constant operand times a variable one that lies as a tensor map can read it
+        if (!tb && bA == 1 && (bB == batch || batch == 1) && direct(B, ldb, sB) &&
+            const_split(st, A, false, M, K, lda, &cav, true)) {
+            gemm_x<true>(split, st, M, N, K, alpha, B, ldb, sB, cav.hi, cav.kp, beta, C, ldc, sC, batch);
+            return;
+        }
+        if (bB == 1 && direct(A, lda, sA) && (bA == batch || batch == 1) && const_split(st, B, !tb, N, K, ldb, &cbv, true)) {
+            gemm_x<false>(split, st, M, N, K, alpha, A, lda, sA, cbv.hi, cbv.kp, beta, C, ldc, sC, batch);
+            return;
+        }
+    }
     const SplitCopy *ca = (split && bA == 1 && const_split(st, A, ta, M, K, lda, &cav)) ? &cav : nullptr;
     const SplitCopy *cb = (split && bB == 1 && const_split(st, B, !tb, N, K, ldb, &cbv)) ? &cbv : nullptr;
     const bool a_direct = !ca && !ta && direct(A, lda, sA), b_direct = !cb && tb && direct(B, ldb, sB);
