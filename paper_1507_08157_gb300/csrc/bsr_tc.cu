@@ -50,10 +50,9 @@ struct __align__(8) BtShared {
     int abort;
 };
 
+// x rounded to tf32, ties away (cvt.rna.tf32 by the bits, at the integer rate)
 __device__ __forceinline__ float tf32_hi(float x) {
-    unsigned r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
+    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
 }
 
 template <int NSPLIT>

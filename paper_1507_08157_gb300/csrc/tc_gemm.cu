@@ -55,10 +55,11 @@ constexpr int STAGE_FLOATS = 4 * 32 * 33;      // epilogue staging: one 32 x 33 
 
 using namespace tc;
 
-__device__ __forceinline__ float tf32_rna_dev(float x) {
-    unsigned r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
+// cvt.rna.tf32 by the bits (half a unit of the 13 dropped bits added to the magnitude): the conversion
+// runs at a fraction of the integer rate (5 % of a split product). A NaN may lose its mark in hi but
+// keeps it in x - hi.
+__device__ __forceinline__ float tf32_bits(float x) {
+    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
 }
 
 // NSPLIT = 1: plain TF32 on the raw tiles; 3: three-term split, hi/lo made in shared memory
@@ -209,10 +210,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(
                         for (int i = ts; i < nvec; i += 128) {
                             const float4 x = hi[i];
                             float4 h, l;
-                            h.x = tf32_rna_dev(x.x);
-                            h.y = tf32_rna_dev(x.y);
-                            h.z = tf32_rna_dev(x.z);
-                            h.w = tf32_rna_dev(x.w);
+                            h.x = tf32_bits(x.x);
+                            h.y = tf32_bits(x.y);
+                            h.z = tf32_bits(x.z);
+                            h.w = tf32_bits(x.w);
                             l.x = x.x - h.x;
                             l.y = x.y - h.y;
                             l.z = x.z - h.z;
@@ -291,29 +292,32 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(
 // of an element are added in the order of the kernel above (the same results bit by bit). 140 atoms,
 // 1260 x 560: 20 and 10 systems from the left and right 0.57 ms with the kernel above and its transposed
 // copies, 0.42 here; one-term products of 20 systems 70 us with and 45 without copies.
-// 14 warps: 0-3 read the accumulators and write C, 4-7 split X into TMEM (warp w owns lanes
-// 32 (w % 4) on), 8-11 split W in place, 12 loads by TMA, 13 issues the MMAs. TMEM: two accumulators of
-// 128 columns and four stages of 64 (hi and lo of 32 K).
-// cvt.rna.tf32 by the bits (half a unit of the 13 dropped bits added to the magnitude): the conversion
-// runs at a fraction of the integer rate (5 % of the kernel). A NaN may lose its mark in hi but keeps
-// it in x - hi.
-__device__ __forceinline__ float tf32_bits(float x) {
-    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
-}
-constexpr int XS = 4;                                       // stages
-constexpr int X_STAGE_BYTES = 3 * TILE_BYTES;               // X, W (hi in place), W lo
+// 14 warps: 0-3 read the accumulators and write C, 4-7 and 8-11 take alternate slices and split X into
+// TMEM (warp w owns lanes 32 (w % 4) on) and W in place, 12 loads by TMA, 13 issues the MMAs. TMEM: two
+// accumulators and stages of 64 columns (hi and lo of 32 K).
+__host__ __device__ constexpr int x_acc(int TN) { return TN <= 64 ? 64 : 128; }             // columns of an accumulator
+// stages, even so that a stage always belongs to the same warps; narrow tiles have room for two more.
+// (16384 long sums on 6 to 64 blocks: 185 us with four, 175 with six, 304 in 128 wide tiles; then
+// bound by the chain of 6144 accumulations of each element, about 54 cycles each)
+__host__ __device__ constexpr int x_stages(int TN) { return TN <= 64 ? 6 : 4; }
+__host__ __device__ constexpr int x_wbytes(int TN) { return TN * TBK * 4; }
+__host__ __device__ constexpr int x_stage_bytes(int TN) { return TILE_BYTES + 2 * x_wbytes(TN); }    // X, W (hi in place), W lo
 constexpr int XGEMM_THREADS = 14 * 32;
 struct __align__(8) XShared {
-    unsigned long long full[XS], ready[XS], empty[XS], acc_full[2], acc_empty[2], drain;
+    unsigned long long full[6], ready[6], empty[6], acc_full[2], acc_empty[2], drain;
     unsigned int tmem_base;
     int abort;
 };
-constexpr size_t XGEMM_SMEM = (size_t)XS * X_STAGE_BYTES + STAGE_FLOATS * sizeof(float) + sizeof(XShared) + 1024;
+constexpr size_t x_smem(int TN) {
+    return (size_t)x_stages(TN) * x_stage_bytes(TN) + STAGE_FLOATS * sizeof(float) + sizeof(XShared) + 1024;
+}
 
 template <bool LEFT, int TN, bool SPLIT>
 __global__ void __launch_bounds__(XGEMM_THREADS, 1) tc_gemm_x_kernel(
     const __grid_constant__ CUtensorMap mX, const __grid_constant__ CUtensorMap mW, int M, int N, int K, int batch,
     float alpha, float beta, float *__restrict__ C, int ldc, long long sC, int *err, long long wlim) {
+    constexpr int XS = x_stages(TN), ACC = x_acc(TN), WB = x_wbytes(TN), X_STAGE_BYTES = x_stage_bytes(TN);
+    static_assert(2 * ACC + 64 * XS <= 512 && XS % 2 == 0 && X_STAGE_BYTES % 1024 == 0 && WB % 1024 == 0, "stages");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *tiles = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<unsigned long long>(smem_raw) + 1023ull) & ~1023ull);
@@ -333,7 +337,7 @@ __global__ void __launch_bounds__(XGEMM_THREADS, 1) tc_gemm_x_kernel(
     if (threadIdx.x == 0) {
         for (int s = 0; s < XS; ++s) {
             mbar_init(&ctl->full[s], 1);
-            mbar_init(&ctl->ready[s], SPLIT ? 256 : 128);
+            mbar_init(&ctl->ready[s], 128);
             mbar_init(&ctl->empty[s], 1);
         }
         for (int i = 0; i < 2; ++i) {
@@ -352,7 +356,7 @@ __global__ void __launch_bounds__(XGEMM_THREADS, 1) tc_gemm_x_kernel(
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const unsigned tmem = ctl->tmem_base, tmem_x = tmem + 256;
+    const unsigned tmem = ctl->tmem_base, tmem_x = tmem + 2 * ACC;
 
     if (warp == 12) {
         if (lane == 0) {
@@ -368,7 +372,7 @@ __global__ void __launch_bounds__(XGEMM_THREADS, 1) tc_gemm_x_kernel(
                         break;
                     }
                     unsigned char *st = tiles + (size_t)s * X_STAGE_BYTES;
-                    mbar_expect_tx(&ctl->full[s], TILE_BYTES + TN * TBK * 4);
+                    mbar_expect_tx(&ctl->full[s], TILE_BYTES + WB);
                     if (LEFT) tma_load_3d(st, &mX, &ctl->full[s], l0, kb * TBK, b);
                     else tma_load_3d(st, &mX, &ctl->full[s], kb * TBK, l0, b);
                     tma_load_3d(st + TILE_BYTES, &mW, &ctl->full[s], kb * TBK, c0, 0);
@@ -387,7 +391,7 @@ __global__ void __launch_bounds__(XGEMM_THREADS, 1) tc_gemm_x_kernel(
             const int buf = tcount & 1, use = tcount >> 1;
             // the whole warp goes on or none of it
             if (!__all_sync(0xffffffffu, mbar_wait(&ctl->acc_empty[buf], (unsigned)((use & 1) ^ 1), abort, wlim))) break;
-            const unsigned acc_t = tmem + (unsigned)(buf * 128);
+            const unsigned acc_t = tmem + (unsigned)(buf * ACC);
             for (int kb = 0; kb < nk; ++kb, ++it) {
                 const int s = (int)(it % XS);
                 // (one term: W is used as it landed)
@@ -401,7 +405,7 @@ __global__ void __launch_bounds__(XGEMM_THREADS, 1) tc_gemm_x_kernel(
 #pragma unroll
                     for (int kk = 0; kk < TBK / 8; ++kk) {
                         // 8 K: 8 columns of X, 32 bytes inside the swizzle rows of W
-                        const unsigned long long wh = desc_of(w + kk * 2), wl = desc_of(w + kk * 2 + TILE_BYTES / 16);
+                        const unsigned long long wh = desc_of(w + kk * 2), wl = desc_of(w + kk * 2 + WB / 16);
                         mma_tf32_ta(acc_t, xh + kk * 8, wh, idesc, (kb > 0 || kk > 0) ? 1u : 0u);
                         if (SPLIT) {
                             mma_tf32_ta(acc_t, LEFT ? xl + kk * 8 : xh + kk * 8, LEFT ? wh : wl, idesc, 1u);
@@ -423,52 +427,19 @@ __global__ void __launch_bounds__(XGEMM_THREADS, 1) tc_gemm_x_kernel(
             }
             __syncwarp();
         }
-    } else if (warp >= 8) {
-        const int ts = threadIdx.x - 256;
-        long long it = 0;
-        bool go = true;
-        for (int t = blockIdx.x; SPLIT && t < ntiles && go; t += gridDim.x)
-            for (int kb = 0; kb < nk; ++kb, ++it) {
-                const int s = (int)(it % XS);
-                if (!mbar_wait(&ctl->full[s], (unsigned)((it / XS) & 1), abort, wlim)) {
-                    go = false;
-                    break;
-                }
-                float4 *hi = reinterpret_cast<float4 *>(tiles + (size_t)s * X_STAGE_BYTES + TILE_BYTES);
-                float4 *lo = hi + TILE_BYTES / 16;
-                // element-wise, so that the swizzled layout carries over
-#pragma unroll
-                for (int i = 0; i < TN * TBK / 4 / 128; ++i) {
-                    const float4 x = hi[ts + 128 * i];
-                    float4 h, l;
-                    h.x = tf32_bits(x.x);
-                    h.y = tf32_bits(x.y);
-                    h.z = tf32_bits(x.z);
-                    h.w = tf32_bits(x.w);
-                    l.x = x.x - h.x;
-                    l.y = x.y - h.y;
-                    l.z = x.z - h.z;
-                    l.w = x.w - h.w;
-                    hi[ts + 128 * i] = h;
-                    lo[ts + 128 * i] = l;
-                }
-                fence_async_smem();
-                mbar_arrive(&ctl->ready[s]);
-            }
     } else if (warp >= 4) {
-        const int row = (warp - 4) * 32 + lane;              // this thread's lane of TMEM
-        const unsigned tq = tmem_x + ((unsigned)((warp - 4) * 32) << 16);
+        const int row = (warp & 3) * 32 + lane, group = (warp - 4) >> 2;      // this thread's lane of TMEM
+        const unsigned tq = tmem_x + ((unsigned)((warp & 3) * 32) << 16);
         long long it = 0;
         bool go = true;
         for (int t = blockIdx.x; t < ntiles && go; t += gridDim.x)
             for (int kb = 0; kb < nk; ++kb, ++it) {
+                if ((int)(it & 1) != group) continue;
                 const int s = (int)(it % XS);
-                go = mbar_wait(&ctl->full[s], (unsigned)((it / XS) & 1), abort, wlim);
-                if (!__all_sync(0xffffffffu, go)) {          // the stores below are for the whole warp
-                    go = false;
-                    break;
-                }
-                const unsigned char *st = tiles + (size_t)s * X_STAGE_BYTES;
+                // the stores into TMEM are for the whole warp: it goes on or none of it
+                go = __all_sync(0xffffffffu, mbar_wait(&ctl->full[s], (unsigned)((it / XS) & 1), abort, wlim));
+                if (!go) break;
+                unsigned char *st = tiles + (size_t)s * X_STAGE_BYTES;
                 tc_fence_after();      // the stage's last MMAs are done: their completion came before the load
 #pragma unroll
                 for (int k0 = 0; k0 < 32; k0 += 16) {
@@ -496,6 +467,27 @@ __global__ void __launch_bounds__(XGEMM_THREADS, 1) tc_gemm_x_kernel(
                         tmem_st16(tq + (unsigned)(s * 64 + k0), l);
                     }
                 }
+                if (SPLIT) {
+                    // W, element-wise, so that the swizzled layout carries over
+                    float4 *hi = reinterpret_cast<float4 *>(st + TILE_BYTES) + row;
+                    float4 *lo = hi + WB / 16;
+#pragma unroll
+                    for (int i = 0; i < TN * TBK / 4 / 128; ++i) {
+                        const float4 x = hi[128 * i];
+                        float4 h, l;
+                        h.x = tf32_bits(x.x);
+                        h.y = tf32_bits(x.y);
+                        h.z = tf32_bits(x.z);
+                        h.w = tf32_bits(x.w);
+                        l.x = x.x - h.x;
+                        l.y = x.y - h.y;
+                        l.z = x.z - h.z;
+                        l.w = x.w - h.w;
+                        hi[128 * i] = h;
+                        lo[128 * i] = l;
+                    }
+                    fence_async_smem();
+                }
                 tmem_st_wait();
                 tc_fence_before();
                 mbar_arrive(&ctl->ready[s]);
@@ -510,7 +502,7 @@ __global__ void __launch_bounds__(XGEMM_THREADS, 1) tc_gemm_x_kernel(
             tc_fence_after();
             int l0, c0, b;
             tile(t, l0, c0, b);
-            const unsigned ta = tmem + (unsigned)(buf * 128) + ((unsigned)(warp * 32) << 16);
+            const unsigned ta = tmem + (unsigned)(buf * ACC) + ((unsigned)(warp * 32) << 16);
             l0 += warp * 32;
             if (LEFT) {
                 float *cw = C + (long long)b * sC + (long long)c0 * ldc + l0 + lane;     // lane = column of C
@@ -657,13 +649,13 @@ void launch_x(cudaStream_t st, int M, int N, int K, float alpha, const float *X,
     if (!ok) throw CudaError{cudaErrorInvalidValue, "cuTensorMapEncodeTiled (variable times constant)"};
     static const bool attr = []() {   // once per process, thread-safe
         check(cudaFuncSetAttribute(tc_gemm_x_kernel<LEFT, TN, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)XGEMM_SMEM), "attr tc_gemm_x");
+                                   (int)x_smem(TN)), "attr tc_gemm_x");
         return true;
     }();
     (void)attr;
     const long long ntiles = (long long)(((LEFT ? N : M) + 127) / 128) * (((LEFT ? M : N) + TN - 1) / TN) * batch;
     const int grid = (int)std::min<long long>(ntiles, sm_count());
-    tc_gemm_x_kernel<LEFT, TN, SPLIT><<<grid, XGEMM_THREADS, XGEMM_SMEM, st>>>(mx, mw, M, N, K, batch, alpha, beta, C, ldc, sC,
+    tc_gemm_x_kernel<LEFT, TN, SPLIT><<<grid, XGEMM_THREADS, x_smem(TN), st>>>(mx, mw, M, N, K, batch, alpha, beta, C, ldc, sC,
                                                                         error_word(), active_wait_limit());
     check_launch("tc_gemm_x_kernel");
 }
@@ -948,17 +940,40 @@ void tc_gemm(cudaStream_t st, bool ta, bool tb, int M, int N, int K, float alpha
         return reinterpret_cast<unsigned long long>(p) % 16 == 0 && ld % 4 == 0 && s % 4 == 0;
     };
     SplitCopy cav{}, cbv{};
-    if (!ta) {
-        // a constant operand times a variable one that lies as a tensor map can read it
-        if (!tb && bA == 1 && (bB == batch || batch == 1) && direct(B, ldb, sB) &&
-            const_split(st, A, false, M, K, lda, &cav, true)) {
-            gemm_x<true>(split, st, M, N, K, alpha, B, ldb, sB, cav.hi, cav.kp, beta, C, ldc, sC, batch);
-            return;
-        }
-        if (bB == 1 && direct(A, lda, sA) && (bA == batch || batch == 1) && const_split(st, B, !tb, N, K, ldb, &cbv, true)) {
-            gemm_x<false>(split, st, M, N, K, alpha, A, lda, sA, cbv.hi, cbv.kp, beta, C, ldc, sC, batch);
-            return;
-        }
+    // variable times shared operand: B as it lies and A K-contiguous (left), or A as it lies and B^T
+    // K-contiguous (right). The shared one is a registered constant's copy, the operand itself, or a
+    // copy in scratch, in this order of preference.
+    const bool left = !tb && bA == 1 && (bB == batch || batch == 1) && direct(B, ldb, sB);
+    const bool right = !ta && bB == 1 && (bA == batch || batch == 1) && direct(A, lda, sA);
+    if (left && const_split(st, A, ta, M, K, lda, &cav, true)) {
+        gemm_x<true>(split, st, M, N, K, alpha, B, ldb, sB, cav.hi, cav.kp, beta, C, ldc, sC, batch);
+        return;
+    }
+    if (right && const_split(st, B, !tb, N, K, ldb, &cbv, true)) {
+        gemm_x<false>(split, st, M, N, K, alpha, A, lda, sA, cbv.hi, cbv.kp, beta, C, ldc, sC, batch);
+        return;
+    }
+    if (left && !ta && direct(A, lda, 0)) {
+        gemm_x<true>(split, st, M, N, K, alpha, B, ldb, sB, A, lda, beta, C, ldc, sC, batch);
+        return;
+    }
+    if (right && tb && direct(B, ldb, 0)) {
+        gemm_x<false>(split, st, M, N, K, alpha, A, lda, sA, B, ldb, beta, C, ldc, sC, batch);
+        return;
+    }
+    if (left || right) {
+        const float *W = left ? A : B;
+        const int rows = left ? M : N, ldw = left ? lda : ldb, kp = (K + 3) / 4 * 4;
+        float *Wk = scratch(st).get((size_t)rows * kp);
+        if (left ? !ta : tb)
+            split_kernel<<<grid1((long long)rows * kp), 256, 0, st>>>(W, rows, K, ldw, 0, Wk, nullptr, kp, 0, 1);
+        else
+            transpose_split_kernel<<<dim3((rows + 31) / 32, (kp + 31) / 32, 1), dim3(32, 8), 0, st>>>(W, K, rows, ldw, 0, Wk,
+                                                                                                  nullptr, kp, 0);
+        check_launch("tc copy W");
+        if (left) gemm_x<true>(split, st, M, N, K, alpha, B, ldb, sB, Wk, kp, beta, C, ldc, sC, batch);
+        else gemm_x<false>(split, st, M, N, K, alpha, A, lda, sA, Wk, kp, beta, C, ldc, sC, batch);
+        return;
     }
     const SplitCopy *ca = (split && bA == 1 && const_split(st, A, ta, M, K, lda, &cav)) ? &cav : nullptr;
     const SplitCopy *cb = (split && bB == 1 && const_split(st, B, !tb, N, K, ldb, &cbv)) ? &cbv : nullptr;
