@@ -260,7 +260,7 @@ struct Impl {
     long long nchunks_chi = 0;
     DUnitList dunits;
     std::vector<int> coff_h, poff_h, cfirst_h, pfirst_h;    // host tile offsets, first chunks
-    Mem umem_dens, umem_int;              // unit lists (replaced when the autotuner recuts)
+    Mem umem_dens, umem_int, umem_iu;              // unit lists (replaced when the autotuner recuts)
     unsigned short *P16 = nullptr;        // float16 copy of P for the units' gather (workspace)
     int CK = 0, NPmax = 0, nslots_chi = 0, nslots_phi = 0, maxc = 0;
     int NPint = 0;            // phi rows of the integrals' B stage (the largest unit's phi, to 16)
@@ -271,6 +271,7 @@ struct Impl {
     int int_count[3] = {0, 0, 0};
     // integrals on units (phi lists of whole aligned quads): items and most phi of a chunk
     bool int_quads = false;
+    bool int_single = false;  // one state takes the units though the lists are in quads
     // float64 contexts: grid contractions by exact splitting on the tensor cores
     Fp64Grid g64;
     bool int64_tc = false, dens64_tc = false;
@@ -887,7 +888,7 @@ void integrals(tddft_ctx *c, Impl<T> &I, int ns) {
     T *out = c->sparse ? I.dense : I.Vmat;
     bool done = false, quads = false;
     if constexpr (sizeof(T) == 4) {
-        if (I.int_quads) {
+        if (I.int_quads && !(ns == 1 && I.int_single)) {
             // summed in quads: into the sparse form's scratch, which its blocks are read from, or into the
             // product buffer that is free here, and from there in row order
             quads = c->sparse;
@@ -1293,8 +1294,8 @@ bool set_integrals_units(Impl<float> &I, int cch, int pch) {
         I.int_count[q] = (int)by[q].size();
         all.insert(all.end(), by[q].begin(), by[q].end());
     }
-    I.umem_int.release();
-    I.int_units = I.umem_int.alloc<VTile>(std::max<size_t>(1, all.size()));
+    I.umem_iu.release();
+    I.int_units = I.umem_iu.alloc<VTile>(std::max<size_t>(1, all.size()));
     if (!all.empty())
         check(cudaMemcpy(I.int_units, all.data(), all.size() * sizeof(VTile), cudaMemcpyHostToDevice),
               "upload integrals units");
@@ -1408,11 +1409,16 @@ void build_impl(tddft_ctx *c, const tddft_system *s, const tddft_sparse_system *
                         pch = b;
                     }
                 }
-                // lists in quads take the items kernel (faster at every size measured, figures in
-                // integrals_units.cu), other lists the units
+                // lists in quads take the items kernel (faster at every size measured with two states or
+                // more, figures in integrals_units.cu), other lists the units
                 if (I->quads_ok) {
                     set_integrals_items(*I, std::min(pch, 48));
                     I->int_quads = true;
+                    // one state uses an item's chi once, and the item kernel waits for each 128 KB of it,
+                    // where the units keep two or three blocks on an SM: on many tiles they win (17^3 tiles,
+                    // 140 atoms with 4 + 9 and 4 + 4 functions 245 and 184 us against 276 and 226; 15^3,
+                    // 200 atoms 327 and 347, 110 atoms 172 and 166; 12^3, 60 atoms 113 and 89)
+                    I->int_single = I->chi.ntiles > 2048 && set_integrals_units(*I, cch, pch);
                 }
                 if (I->int_quads || set_integrals_units(*I, cch, pch)) {
                     // function-major f16 copies of both tables, rounded on the device (the f16 phi

@@ -10,7 +10,7 @@
 //   A  [512 or 256 points][chi] float16, K-major, brought once by TMA from a chunked point-major
 //      table and kept for all phi chunks and states (128 KB);
 //   B  [chi][phi quad][2 states][4] float16, N-major, gathered by five warps into a ring of stages of
-//      32 chi (8 KB);
+//      32 chi (8 KB); of a last state without a partner [chi][phi], half as wide;
 //   D  one accumulator of up to 128 columns per 128 points, four in TMEM (512 columns); two groups
 //      of four warps multiply each by phi, which they keep in registers across the states.
 //
@@ -27,11 +27,14 @@
 // 0.59; one that streamed chi from L2 for every state and converted float32 P in the gather
 // took 1.55 ms (140 atoms, 10 states, 135^3, GB300).
 // Measured (GB300, whole stage, CUDA events, before and after): 140 atoms, 4 + 9 functions each, 135^3,
-// 10 states 1.59 and 0.59 ms; 200 atoms, 4 + 4, 0.1 per A^3, 120^3, 5 states 0.80 and 0.61; the same at
-// 60 atoms, 90^3 3.08 and 0.13, at 20 atoms with 2 states 0.35 and 0.036 (those two took the per-tile
+// 10 states 1.59 and 0.59 ms; 200 atoms, 4 + 4, 0.1 per A^3, 120^3, 5 states 0.80 and 0.51; the same at
+// 60 atoms, 90^3 3.08 and 0.12, at 20 atoms with 2 states 0.35 and 0.036 (those two took the per-tile
 // kernel); 200 atoms, 4 + 9, 180^3, 4 states 1.87 and 1.26. Not bound by HBM (0.17 ms of tables at 140
 // atoms): 5400 MMAs, 9900 warp loads of the gather and 710 accumulators per SM share 1.1 M cycles,
 // and the epilogue's path per accumulator (TMEM loads and dependent multiply-adds) is the longest.
+// A state without a partner takes half a pair's gather, MMAs and epilogue (three states of the 200
+// atoms 0.43 and 0.36 ms). One state alone uses each 128 KB of chi once and waits for it: there the
+// chi streaming kernel was faster on dense clusters (200 atoms 0.21 and 0.23, 140 atoms 0.25 and 0.21).
 #include "tc_common.cuh"
 #include "tddft_internal.h"
 
@@ -176,9 +179,11 @@ __global__ void __launch_bounds__(DU_THREADS, 1) density_units_kernel(
                     const DUnit u = units[ui];
                     const int KS = (u.nc + DU_ROWS - 1) / DU_ROWS;
                     const int tail = u.nc - (KS - 1) * DU_ROWS;   // chi of the last stage
-                    const unsigned idesc = idesc_f16(128, (u.np + 15) / 16 * 32) | (1u << 16);   // B is N-major
+                    const unsigned idesc2 = idesc_f16(128, (u.np + 15) / 16 * 32) | (1u << 16);   // B is N-major
+                    const unsigned idesc1 = idesc_f16(128, (u.np + 15) / 16 * 16) | (1u << 16);
                     if (u.chi_use & DUnit::FIRST) ++loads;
                     for (int q = q0; q < q1 && ok; ++q) {
+                        const unsigned idesc = 2 * q + 1 < k ? idesc2 : idesc1;
                         for (int mh = par; mh < d.nmh; mh += 2) {
                             const int acc = acc_of(d.nmh, q, mh);
                             const unsigned d0 = tmem + acc * 128, au = acc >> 1 ? uses[1]++ : uses[0]++;
@@ -250,6 +255,22 @@ __global__ void __launch_bounds__(DU_THREADS, 1) density_units_kernel(
                         // rows past the list up to a multiple of 16 are read too: zeros
                         unsigned char *b = B + bi * B_STAGE + lane * 128;
                         const unsigned x = (lane & 7) << 4;
+                        if (2 * q + 1 == k) {     // a state without a partner: pieces of two quads
+                            const uint2 *Pl = reinterpret_cast<const uint2 *>(Ps);
+                            uint4 v[8];
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                const int r0 = __shfl_sync(0xffffffffu, qr, 2 * j), r1 = __shfl_sync(0xffffffffu, qr, 2 * j + 1);
+                                const uint2 y0 = (id >= 0 && r0 >= 0) ? __ldg(Pl + (r0 + id)) : make_uint2(0u, 0u);
+                                const uint2 y1 = (id >= 0 && r1 >= 0) ? __ldg(Pl + (r1 + id)) : make_uint2(0u, 0u);
+                                v[j] = make_uint4(y0.x, y0.y, y1.x, y1.y);
+                            }
+                            if (buse > 0) ok = mbar_wait(&ctl->b_empty[bi], (buse - 1) & 1, abort, wlim);
+                            if (ok)
+#pragma unroll
+                                for (int j = 0; j < 8; ++j)
+                                    if (2 * j < nq) *reinterpret_cast<uint4 *>(b + ((j << 4) ^ x)) = v[j];
+                        } else
                         for (int h = 0; h * 8 < nq; ++h) {
                             uint4 v[8];
 #pragma unroll
@@ -335,6 +356,30 @@ __global__ void __launch_bounds__(DU_THREADS, 1) density_units_kernel(
                     if (!ok) break;
                     float r0 = chunked ? 0.0f : t0, r1 = chunked ? 0.0f : t1;
                     const unsigned ta = tmem + grp * 128 + ((unsigned)((warp & 3) * 32) << 16);
+                    if (s1 == s0) {
+                        // a state without a partner: column b is phi b
+#pragma unroll
+                        for (int c = 0; c < (PHI32 ? 2 : 4); ++c)
+                            if (c * 32 < ncol) {
+                                float v[16];
+                                tmem_ld16(ta + c * 16, v);
+#pragma unroll
+                                for (int e = 0; e < 16; e += 2) {
+                                    if (PHI32) {
+                                        r0 = __fadd_rn(r0, __fmul_rn(v[e], __uint_as_float(ph[(c * 16 + e) & 31])));
+                                        r0 = __fadd_rn(r0, __fmul_rn(v[e + 1], __uint_as_float(ph[(c * 16 + e + 1) & 31])));
+                                    } else {
+                                        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&ph[c * 8 + e / 2]));
+                                        r0 = fmaf(v[e], f.x, r0);
+                                        r0 = fmaf(v[e + 1], f.y, r0);
+                                    }
+                                }
+                                if (!PHI32 && chunked && ((c & 1) || (c + 1) * 32 >= ncol)) {
+                                    t0 += r0;
+                                    r0 = 0.0f;
+                                }
+                            }
+                    } else
 #pragma unroll
                     for (int c = 0; c < (PHI32 ? 4 : 8); ++c)
                         if (c * 16 < ncol) {
@@ -404,8 +449,8 @@ __global__ void __launch_bounds__(256) max_bits_kernel(const float *__restrict__
     if ((threadIdx.x & 31) == 0) atomicMax(&bits[blockIdx.y], __float_as_uint(m));
 }
 
-// P16[s / 2][q][a][s % 2][4] = float16(P[s][a][4q .. 4q+3] * scale_s), zeros for the missing state of
-// an odd count: 32 x 32 (chi, quad) tiles of a state pair through shared memory, both sides in rows
+// P16[s / 2][q][a][s % 2][4] = float16(P[s][a][4q .. 4q+3] * scale_s), the last state of an odd count
+// [q][a][4]: 32 x 32 (chi, quad) tiles of a state pair through shared memory, both sides in rows
 // of 16-byte pieces. scale [k] and its inverse [k] are left for the kernel.
 __global__ void __launch_bounds__(256) pack_quads_kernel(const float *__restrict__ P, long long sP, int nchi, int nphi,
                                                          int k, const unsigned *__restrict__ bits,
@@ -442,7 +487,12 @@ __global__ void __launch_bounds__(256) pack_quads_kernel(const float *__restrict
     __syncthreads();
     for (int i = threadIdx.y; i < 32; i += 8) {
         const int q = q0 + i, a = a0 + threadIdx.x;
-        if (a < nchi && q < nq) out[(long long)sp * sout + (long long)q * nchi + a] = t[threadIdx.x][i];
+        if (a < nchi && q < nq) {
+            const uint4 x = t[threadIdx.x][i];
+            const long long o = (long long)q * nchi + a;
+            if (two) out[(long long)sp * sout + o] = x;
+            else reinterpret_cast<uint2 *>(out + (long long)sp * sout)[o] = make_uint2(x.x, x.y);
+        }
     }
 }
 

@@ -81,18 +81,8 @@ __device__ __forceinline__ unsigned long long smem_desc(unsigned saddr) {
     return d;
 }
 
-// the same for an M/N-major operand: rows of 64 elements (128 bytes) along M/N, one row per K, 8-K
-// groups 1024 B apart; `blocks` bytes between consecutive blocks of 64 along M/N
-__device__ __forceinline__ unsigned long long smem_desc_mn(unsigned saddr, unsigned blocks) {
-    unsigned long long d = 0;
-    d |= (unsigned long long)((saddr & 0x3FFFF) >> 4);
-    d |= (unsigned long long)(blocks >> 4) << 16;
-    d |= (unsigned long long)(1024 >> 4) << 32;
-    d |= (unsigned long long)1 << 46;
-    d |= (unsigned long long)2 << 61;
-    return d;
-}
-
+// For an M/N-major operand: rows of 64 elements (128 bytes) along M/N, one row per K, 8-K groups 1024 B
+// apart, the leading byte offset the distance of consecutive blocks of 64 along M/N.
 // the low words of the two descriptors vary with the address alone, so that an issuing thread forms
 // a descriptor with one add: start address in 16-byte units, plus the block distance for M/N-major
 __device__ __forceinline__ unsigned desc_lo(unsigned saddr) { return ((saddr & 0x3FFFF) >> 4) | (1u << 16); }

@@ -30,3 +30,19 @@ def test_integrals_match_oracle_at_list_edges(natoms, nchi, nphi, k):
     ref = ogrid.potential_integrals(ogrid.BoxedSet(s.chi, s.n), ogrid.BoxedSet(s.phi, s.n), V, s.dV)
     for q in range(k):
         assert np.max(np.abs(got[q] - ref[q])) <= 2e-3 * np.max(np.abs(ref[q])), q
+
+
+@pytest.mark.parametrize("ngrid,k", [(96, 1), (108, 1), (108, 2)])
+def test_single_state_on_few_and_many_tiles(ngrid, k):
+    # one state takes the kernel by units from 2049 tiles on (13^3 at 108), the item kernel below
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1507_08157_gb300 import build, tddft
+    build.build()
+    s = sy.generate(sy.Recipe(natoms=10, cell_ang=ngrid / 4.0, ngrid=ngrid, nchi=9, radius_ang=3.0, min_sep_ang=1.0, seed=3))
+    ctx = tddft.Context(s, precision="mixed", precond="none")
+    V = np.random.default_rng(k).standard_normal((k, s.n, s.n, s.n))
+    got = ctx.potential_integrals(V)
+    ref = ogrid.potential_integrals(ogrid.BoxedSet(s.chi, s.n), ogrid.BoxedSet(s.phi, s.n), V, s.dV)
+    assert np.max(np.abs(got - ref)) <= 2e-3 * np.max(np.abs(ref))
