@@ -380,12 +380,11 @@ def learned_vs_plain(tddft, sy, torch, stream, k=10, train_atoms=16, eval_atoms=
             "max_domega_learned_vs_plain_Ha": dw, "train_s": train_s, "train_loss": [l0, l1]}
 
 
-# DRAM bytes (read + write) per tc_gemm_kernel launch in a timed PCG step of the default workload,
-# mean over the step's 16 launches, from one capture of this build:
+# DRAM bytes (read + write) per tc_gemm_x_kernel launch in a PCG step of the default workload, mean
+# over the step's 16 launches, from one capture of the same products (profiles/operator_chromophore140.md):
 #   ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum --clock-control none
-#       -k regex:tc_gemm_kernel --csv python bench.py --steps 1 --warmup 1 --no-cpu-baseline
-#       --no-time-to-k --no-iter-line --no-autotune
-GEMM_TRAFFIC_PER_LAUNCH = 82.0e6
+#       -k regex:tc_gemm_x --csv
+GEMM_TRAFFIC_PER_LAUNCH = 63.4e6
 
 
 def stage_rooflines(prof, peaks, args):
@@ -551,8 +550,8 @@ def run_ours(args):
     stage_roofs, summed = stage_rooflines(prof, peaks, args)
     if roof.get("kernel") == "gemm" and roof.get("bound") == "tensor":
         roof["traffic"] = GEMM_TRAFFIC_PER_LAUNCH
-        roof["traffic_note"] = ("dram__bytes_read.sum + dram__bytes_write.sum per tc_gemm_kernel launch, mean "
-                                "over the 16 launches of one timed PCG step (one ncu capture of this build)")
+        roof["traffic_note"] = ("dram__bytes_read.sum + dram__bytes_write.sum per tc_gemm_x_kernel launch, mean "
+                                "over the 16 launches of one PCG step (one ncu capture of this build)")
 
     # the same PCG steps with the paper's preconditioner (inner CG on Eq. precond to 1e-4), when
     # the timed steps used another one: both are reported
