@@ -842,7 +842,9 @@ void ensure_workspace(tddft_ctx *c, Impl<T> &I, int states) {
         // right operand block-transposed
         I.dense = I.wmem.template alloc<T>((size_t)states * c->nc * c->nv);
         I.opT = I.wmem.template alloc<T>((size_t)states * len);
-        if (I.units_ok) I.P16 = I.wmem.template alloc<unsigned short>((size_t)(states + 1) / 2 * 2 * c->nc * c->nv);
+        // for the density units, which the autotuner may select after this
+        if (sizeof(T) == 4 && I.quads_ok)
+            I.P16 = I.wmem.template alloc<unsigned short>((size_t)(states + 1) / 2 * 2 * c->nc * c->nv);
     } else {
         // the potential matrix is free while a density is made, and holds the copy of its P
         I.P16 = reinterpret_cast<unsigned short *>(I.Vmat);

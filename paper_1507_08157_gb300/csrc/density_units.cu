@@ -507,6 +507,7 @@ void response_density_units(cudaStream_t st, const GridShape &g, const TileSet<f
                             const DUnitList &ul, int nchi, int nphi, const float *P, long long sP, int k, float *rho,
                             unsigned short *P16, unsigned *bits, float *scale, int *err) {
     if (k <= 0) return;
+    if (!P16) throw CudaError{cudaErrorInvalidValue, "density units: no scratch for the packed kernels"};
     ProfScope ps(st, ST_DENSITY, 2.0 * k * g.pair_points, 2.0 * g.table_values + 4.0 * k * g.n * g.n * g.n);
     const long long n3 = (long long)g.n * g.n * g.n;
     if (!ul.covers || ul.adds) check(cudaMemsetAsync(rho, 0, sizeof(float) * (size_t)k * n3, st), "memset rho");
