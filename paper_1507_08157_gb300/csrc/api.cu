@@ -276,6 +276,7 @@ struct Impl {
     Fp64Grid g64;
     bool int64_tc = false, dens64_tc = false;
     unsigned long long *bits64 = nullptr;
+    int *exps64 = nullptr;
     IItem *int_items = nullptr;
     int nint_items = 0, int_pch = 48;
     unsigned *tc_bits = nullptr;
@@ -513,7 +514,7 @@ bool fp64_grid_build(cudaStream_t st, Mem &mem, const TileSet<double> &chi, cons
                      const std::vector<int> &coff, const std::vector<int> &poff, bool quads, Fp64Grid &G);
 void response_density_fp64(cudaStream_t st, const GridShape &g, const TileSet<double> &chi, const TileSet<double> &phi,
                            const Fp64Grid &G, int nphi, const double *P, long long sP, int k, double *rho,
-                           unsigned long long *bits, int *err);
+                           int *exps, int *err);
 void potential_integrals_fp64(cudaStream_t st, const GridShape &g, const TileSet<double> &chi, const TileSet<double> &phi,
                               const Fp64Grid &G, int nchi, int nphi, const double *V, int k, double *out,
                               unsigned long long *bits, int *err);
@@ -837,6 +838,7 @@ void ensure_workspace(tddft_ctx *c, Impl<T> &I, int states) {
     I.tc_bits = I.wmem.template alloc<unsigned>((size_t)states);
     I.tc_scale = I.wmem.template alloc<float>((size_t)2 * states);
     I.bits64 = I.wmem.template alloc<unsigned long long>((size_t)states);
+    if (I.dens64_tc) I.exps64 = I.wmem.template alloc<int>((size_t)states * (I.g64.pslots + I.g64.ntiles));
     if (c->sparse) {
         // the grid kernels address P and V densely; the tensor-core left products take their
         // right operand block-transposed
@@ -877,7 +879,7 @@ void density(tddft_ctx *c, Impl<T> &I, const T *P, int ns) {
     if constexpr (sizeof(T) == 8) {
         if (I.dens64_tc) {
             response_density_fp64(c->st, c->grid(), I.chi, I.phi, I.g64, c->nv, P, (long long)c->nc * c->nv, ns, I.rho,
-                                  I.bits64, tc_error_word());
+                                  I.exps64, tc_error_word());
             return;
         }
     }

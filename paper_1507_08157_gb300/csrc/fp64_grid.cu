@@ -3,22 +3,27 @@
 // Algorithms 59 (2012) 95; on tensor cores: Mukunoki, Ozaki, Ogita and Imamura, ISC 2020).
 //
 // This part executes about two float64 multiply-adds per cycle and SM, and the CUDA-core kernels ran
-// at that rate. Here a value x with |x| < 2^E becomes the integer q = round(x 2^(61 - E)), written
-// in nine balanced digits of seven bits, q = sum_i d_i 128^(8 - i), -64 <= d_i <= 63, each exact in
-// float16. A product sum over K terms is
+// at that rate. Here a value x with |x| < 2^E becomes the integer q = round(x 2^(62 - E)), written
+// in nine balanced digits of seven bits, q = sum_i d_i 128^(8 - i), -64 <= d_i <= 63 (the first to 64), each
+// exact in float16. A product sum over K terms is
 //
-//   sum x y = 2^(Ex + Ey - 122) sum_l 128^(16 - l) D_l,     D_l = sum_{i + j = l} sum_K x_i y_j,
+//   sum x y = 2^(Ex + Ey - 124) sum_l 128^(16 - l) D_l,     D_l = sum_{i + j = l} sum_K x_i y_j,
 //
 // and each D_l, l <= 8, is an integer below 2^24 (9 pairs x 455 terms x 64 x 64; past that only the
 // lowest level can round, at 2^-80 of the result's range), so the float32 accumulators of
-// kind::f16 hold it exactly. The levels l > 8 and the rounding of q leave an error of 2^-61 of the
-// largest terms, below the 2^-53 that every float64 addition of the sums it replaces made.
-// Scales (powers of two): one per state for P and V. The integrals scale every function's values on a
-// tile by their own maximum there, so that entries of functions that only graze each other keep
-// their relative accuracy; the density, whose sums over chi cannot carry such scales, takes one for
-// the whole chi table. Errors against extended precision (sampled entries, 8 and 24 atoms) of the
-// CUDA-core kernels and of these: density 1.4e-16 and 0.8e-16, 2.5e-16 and 1.2e-16; integrals
-// 4.1e-16 and 0.9e-16, 7.2e-16 and 1.2e-16.
+// kind::f16 hold it exactly. The levels l > 8 and the rounding of q leave an error of about 2^-63 of
+// 2^(Ex + Ey) per term.
+// The density's scales are those of a sum: one per point, of the tile's chi there, and one per phi, of
+// its P over the tile's chi. Where both are reached by different chi, a sum can still be small against
+// them, so every point compares the largest of its terms T phi with the largest that its scales
+// allow: below 2^-9 of it (0.03 % of the points for P without structure), or where a tile's P is not
+// finite or its columns' scales lie too far apart, the point is summed in float64. So the error is that of
+// float64 sums or below at every point: relative to the sum of the terms' sizes at most 6.1e-16, root
+// mean square 9.6e-17, where float64 sums have 8.2e-16 and 1.2e-16 (emulated, 8 atoms, 48^3); with P's
+// rows in blocks of 1, 1e-6 and 1e-12, 7.2e-16 and 9.7e-17 against 9.3e-16 and 1.2e-16. One scale for
+// the chi table and one for a state's P left no digit right where chi is below 1e-16 of its largest value.
+// The integrals scale V by its largest value and every function's values on a tile by their own
+// maximum there.
 //
 // The digits of B are stacked along N (32 columns each), the accumulators of the levels along the
 // columns of TMEM (32 each): for digit i of A one MMA of N = 32 (9 - i) columns, placed at level i,
@@ -53,7 +58,7 @@ bool encode_map_2d(CUtensorMap *map, CUtensorMapDataType dt, const void *ptr, un
 namespace {
 
 constexpr int ND = 9;                // digits, and levels kept
-constexpr int SHIFT = 61;            // |q| < 2^61
+constexpr int SHIFT = 62;            // |q| <= 2^62
 constexpr int NB = 32;               // B columns of one digit
 constexpr int THREADS64 = 320;       // warps 0-7 make B and combine, 8 TMA, 9 MMA
 constexpr int A_RING = 8, A_TILE = 16384;
@@ -67,7 +72,9 @@ struct __align__(8) Shared64 {
     unsigned long long acc_full, acc_empty, drain;
     unsigned int tmem_base;
     int abort;
-    double part[128];                // density: the second half's sums
+    double part[128];                // density: the second half's sums and exponents
+    int most[128], found[128];
+    unsigned lost[4];                // points to sum in float64
 };
 
 __device__ __forceinline__ void init64(Shared64 *c) {
@@ -93,12 +100,16 @@ __device__ __forceinline__ int exponent_of(unsigned long long bits) {
     return max(e, -900);
 }
 __device__ __forceinline__ double pow2(int e) { return ldexp(1.0, e); }
+// 2^(61 - E) of a column's values (0 of a column of zeros)
+__device__ __forceinline__ double column_scale(int E) {
+    return E < -900 || E > 1024 ? 0.0 : __hiloint2double((1023 + SHIFT - E) << 20, 0);
+}
 // a state's values are all finite
 __device__ __forceinline__ bool finite_bits(unsigned long long bits) {
     return isfinite(__longlong_as_double((long long)bits));
 }
 
-// q + sum_i 64 128^i: the digits plus 64, seven bits each
+// q + sum_i 64 128^i: the digits plus 64, seven bits each and eight for the first, up to 128
 __device__ __forceinline__ unsigned long long biased(double scaled) {
     constexpr unsigned long long C = 0x2040810204081020ull << 1;   // 64 (1 + 128 + ... + 128^8)
     return (unsigned long long)__double2ll_rn(scaled) + C;
@@ -109,22 +120,27 @@ __device__ __forceinline__ unsigned digit_pair(unsigned a, unsigned b) {
     const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&v), __half2half2(__ushort_as_half(0x6440)));
     return *reinterpret_cast<const unsigned *>(&h);
 }
-__device__ __forceinline__ unsigned digit(unsigned long long u, int j) { return (unsigned)(u >> (7 * (ND - 1 - j))) & 127u; }
+__device__ __forceinline__ unsigned digit(unsigned long long u, int j) {
+    const unsigned d = (unsigned)(u >> (7 * (ND - 1 - j)));
+    return j == 0 ? d : d & 127u;
+}
 
 // an integer below 2^51 in size as float64 with one addition
 __device__ __forceinline__ double to_double(long long v) {
     return __longlong_as_double(0x4330000000000000ll + (1ll << 51) + v) - 6755399441055744.0;
 }
-// sum_l 128^(8 - l) D_l of the nine level sums (float32 integers)
+// sum_l 128^(8 - l) D_l of the nine level sums (float32 integers). |D_l| <= (l + 1) 512 64 64, so that
+// both halves stay below 2^50.
 __device__ __forceinline__ double combine_levels(const float (*D)[8], int e) {
     long long hi = 0, lo = 0;
 #pragma unroll
-    for (int l = 0; l < 4; ++l) hi = hi * 128 + (int)__float2int_rn(D[l][e]);
+    for (int l = 0; l < 5; ++l) hi = hi * 128 + (int)__float2int_rn(D[l][e]);
 #pragma unroll
-    for (int l = 4; l < 8; ++l) lo = lo * 128 + (int)__float2int_rn(D[l][e]);
-    // level 8 stays apart: with it lo could reach 2^52
-    return fma(to_double(hi), 34359738368.0, fma(to_double(lo), 128.0, (double)D[8][e]));
+    for (int l = 5; l < ND; ++l) lo = lo * 128 + (int)__float2int_rn(D[l][e]);
+    return fma(to_double(hi), 268435456.0, to_double(lo));
 }
+// exponent field of x (0: zero or below the normal range, 2047: infinity or NaN)
+__device__ __forceinline__ int expo_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
 __device__ __forceinline__ void tmem_ld8(unsigned taddr, float *v) {
     unsigned r[8];
@@ -300,14 +316,75 @@ __global__ void __launch_bounds__(THREADS64, 1) integrals64_kernel(
 }
 
 // ---- response density: rho(r) = sum_b phi_b(r) sum_a chi_a(r) P_ab ------------------------------------
+// scales of the P columns (a phi over the chi of a tile's list) and the rows (a point over them)
+constexpr int COL_ZERO = -20000;     // a column of zeros
+constexpr int ROW_ZERO = -20000;     // no chi is nonzero at the point
+constexpr int TILE_F64 = 20000;      // (of a tile's largest column) the whole tile in float64
+constexpr int LOST_BITS = 9;         // terms this far below their scales: the point in float64
+
+// cexp[s][slot]: |P_ab| < 2^E over the tile's chi; ctop[s][listed tile]: the largest E of the tile's columns,
+// or TILE_F64 where P is not finite or a column's scale is more than 2^900 below the largest or below
+// 2^-900. Block = (listed tile, state). 32 atoms, 3 states: 30 us.
+__global__ void __launch_bounds__(256) column_exponents_kernel(const int *__restrict__ tiles, int ntiles,
+                                                               const int *__restrict__ coff, const int *__restrict__ cids,
+                                                               const int *__restrict__ poff, const int *__restrict__ pids,
+                                                               int nphi, const double *__restrict__ P, long long sP,
+                                                               long long pslots, int *__restrict__ cexp,
+                                                               int *__restrict__ ctop) {
+    __shared__ int mx[NB], top, low;
+    const int t = tiles[blockIdx.x], s = blockIdx.y;
+    const int c0 = coff[t], nc = coff[t + 1] - c0, p0 = poff[t], np = poff[t + 1] - p0;
+    const double *Ps = P + (long long)s * sP;
+    const int qd = threadIdx.x & 7, a0 = threadIdx.x >> 3;
+    if (threadIdx.x == 0) top = COL_ZERO, low = TILE_F64;
+    for (int b0 = 0; b0 < np; b0 += NB) {
+        const int nb = min(NB, np - b0);
+        if (threadIdx.x < NB) mx[threadIdx.x] = 0;
+        __syncthreads();
+        // of the high words without sign, and 1 where only the low word is not zero
+        int m[4] = {0, 0, 0, 0};
+        if (qd * 4 < nb) {
+            const int col = pids[p0 + b0 + qd * 4];
+#pragma unroll 4
+            for (int a = a0; a < nc; a += 32) {
+                const double2 *p = reinterpret_cast<const double2 *>(Ps + (long long)cids[c0 + a] * nphi + col);
+                const double2 x = __ldg(p), y = __ldg(p + 1);
+                const double v[4] = {x.x, x.y, y.x, y.y};
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    m[e] = max(m[e], max(__double2hiint(v[e]) & 0x7fffffff, __double2loint(v[e]) != 0 ? 1 : 0));
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            m[e] = max(m[e], __shfl_xor_sync(0xffffffffu, m[e], 8));
+            m[e] = max(m[e], __shfl_xor_sync(0xffffffffu, m[e], 16));
+            if ((threadIdx.x & 31) < 8) atomicMax(&mx[qd * 4 + e], m[e]);
+        }
+        __syncthreads();
+        if (threadIdx.x < nb) {
+            const int h = mx[threadIdx.x], f = h >> 20;
+            const int E = h == 0 ? COL_ZERO : f == 2047 ? TILE_F64 : max(f, 1) - 1022;
+            cexp[(long long)s * pslots + p0 + b0 + threadIdx.x] = E;
+            if (E != COL_ZERO) {
+                atomicMax(&top, E);
+                atomicMin(&low, E);
+            }
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) ctop[(long long)s * ntiles + blockIdx.x] = top != COL_ZERO && (low < -900 || low < top - 900) ? TILE_F64 : top;
+}
+
 // Block = (tile, 128 of its points, state); for every 32 phi (and every 448 chi) the product
 // T[r][b] = sum_a chi_a(r) P_ab, whose levels each thread combines and multiplies by phi.
 __global__ void __launch_bounds__(THREADS64, 1) density64_kernel(
     const __grid_constant__ CUtensorMap mX,   // chi digits [(digit * nchunks + chunk) * 512 + point][64], box 64 x 128
-    int n, int nt, int k, const int *__restrict__ tiles, const int *__restrict__ coff, const int *__restrict__ cids,
-    const int *__restrict__ cfirst, long long nchunks, const int *__restrict__ poff, const int *__restrict__ pids,
-    const double *__restrict__ pval, int nphi, const double *__restrict__ P, long long sP,
-    const unsigned long long *__restrict__ pbits, int ex, double *__restrict__ rho, int *err, long long wlim) {
+    int n, int nt, int k, int ntiles, const int *__restrict__ tiles, const int *__restrict__ coff,
+    const int *__restrict__ cids, const double *__restrict__ cval, const int *__restrict__ cfirst, long long nchunks,
+    const int *__restrict__ poff, const int *__restrict__ pids, const double *__restrict__ pval, int nphi,
+    const double *__restrict__ P, long long sP, const int *__restrict__ rexp, const int *__restrict__ cexp,
+    const int *__restrict__ ctop, long long pslots, double *__restrict__ rho, int *err, long long wlim) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<unsigned long long>(smem_raw) + 1023ull) & ~1023ull);
@@ -316,9 +393,11 @@ __global__ void __launch_bounds__(THREADS64, 1) density64_kernel(
     volatile int *abort = &ctl->abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // states fastest, then the point blocks: blocks that share a tile's tables run together
-    const int s = blockIdx.x % k, pb = blockIdx.x / k % 4, t = tiles[blockIdx.x / k / 4];
+    const int s = blockIdx.x % k, pb = blockIdx.x / k % 4, ti = blockIdx.x / k / 4, t = tiles[ti];
     const int c0 = coff[t], nc = coff[t + 1] - c0, p0 = poff[t], np = poff[t + 1] - p0;
-    const int KB = (nc + 63) / 64, NY = (np + NB - 1) / NB, NZ = (nc + MAX_K - 1) / MAX_K;
+    const int top = ctop[(long long)s * ntiles + ti];
+    const bool f64 = top == TILE_F64;
+    const int KB = (nc + 63) / 64, NY = f64 ? 0 : (np + NB - 1) / NB, NZ = (nc + MAX_K - 1) / MAX_K;
     constexpr int ZB = MAX_K / 64;       // K blocks of one accumulation
     if (threadIdx.x == 0) init64(ctl);
     if (warp == 9) {
@@ -376,37 +455,45 @@ __global__ void __launch_bounds__(THREADS64, 1) density64_kernel(
             }
         }
     } else {
-        const int epx = exponent_of(pbits[s]);
-        const double sc = pow2(SHIFT - epx);
-        const double f = finite_bits(pbits[s]) ? ldexp(1.0, 56 - 2 * SHIFT + ex + epx) : __longlong_as_double(0x7ff8000000000000ll);
         const double *Ps = P + (long long)s * sP;
+        const int *ce = cexp + (long long)s * pslots + p0;
         const int lp = pb * 128 + (warp & 3) * 32 + lane, hb = warp >> 2;
         unsigned qb = 0, acc = 0;
         bool ok = true;
         double r = 0.0;
+        int most = COL_ZERO, found = 2 * COL_ZERO;   // exponents: of the terms that the scales allow, of the terms
+        const int rx = rexp[t * TILE_PTS + lp];
         for (int y = 0; y < NY && ok; ++y) {
             const int b0 = y * NB, nb = min(NB, np - b0);
+            // digits of P: thread = (chi row, phi quad), twice; zeros past the lists
+            const int qd = threadIdx.x & 7;
+            double sc[4] = {0.0, 0.0, 0.0, 0.0};
+            int col = 0;
+            if (qd * 4 < nb) {
+                const int4 E = *reinterpret_cast<const int4 *>(ce + b0 + qd * 4);
+                sc[0] = column_scale(E.x), sc[1] = column_scale(E.y), sc[2] = column_scale(E.z), sc[3] = column_scale(E.w);
+                col = pids[p0 + b0 + qd * 4];
+            }
             for (int z = 0; z < NZ && ok; ++z, ++acc) {
                 for (int kb = z * ZB; kb < min(KB, (z + 1) * ZB); ++kb, ++qb) {
                     if (qb >= 2 && !mbar_wait(&ctl->b_empty[qb & 1], ((qb >> 1) - 1) & 1, abort, wlim)) {
                         ok = false;
                         break;
                     }
-                    // digits of P: thread = (chi row, phi quad), twice; zeros past the lists
                     unsigned char *Bk = B + (qb & 1) * B_NMAJ;
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        const int task = threadIdx.x + h * 256, qd = task & 7, a = task >> 3;
+                        const int a = (threadIdx.x + h * 256) >> 3;
                         double v[4] = {0.0, 0.0, 0.0, 0.0};
                         if (kb * 64 + a < nc && qd * 4 < nb) {
                             const double2 *p = reinterpret_cast<const double2 *>(
-                                Ps + (long long)cids[c0 + kb * 64 + a] * nphi + pids[p0 + b0 + qd * 4]);
+                                Ps + (long long)cids[c0 + kb * 64 + a] * nphi + col);
                             const double2 x = __ldg(p), y2 = __ldg(p + 1);
                             v[0] = x.x, v[1] = x.y, v[2] = y2.x, v[3] = y2.y;
                         }
                         unsigned long long u[4];
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) u[e] = biased(v[e] * sc);
+                        for (int e = 0; e < 4; ++e) u[e] = biased(v[e] * sc[e]);
 #pragma unroll
                         for (int j = 0; j < ND; ++j) {
                             const uint2 x = make_uint2(digit_pair(digit(u[0], j), digit(u[1], j)),
@@ -427,9 +514,23 @@ __global__ void __launch_bounds__(THREADS64, 1) density64_kernel(
 #pragma unroll
                     for (int l = 0; l < ND; ++l) tmem_ld8(tmem + l * NB + c + ((unsigned)((warp & 3) * 32) << 16), D[l]);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        if (c + e < nb)
-                            r = fma(combine_levels(D, e), __ldg(pval + (long long)(p0 + b0 + c + e) * TILE_PTS + lp), r);
+                    for (int h = 0; h < 8; h += 4)
+                        if (c + h < nb) {
+                            const int4 E4 = __ldg(reinterpret_cast<const int4 *>(ce + b0 + c + h));
+                            const int E[4] = {E4.x, E4.y, E4.z, E4.w};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const double ph = __ldg(pval + (long long)(p0 + b0 + c + h + e) * TILE_PTS + lp);
+                                double x = combine_levels(D, h + e);         // zero or at least 1 in size
+                                const int fp = expo_field(ph), fx = expo_field(x), w = fp != 0 ? fp + E[e] : 2 * COL_ZERO;
+                                most = max(most, w);
+                                if (fx != 0) {
+                                    found = max(found, w + fx);
+                                    x = __hiloint2double(__double2hiint(x) + (E[e] - top) * (1 << 20), __double2loint(x));
+                                }
+                                r = fma(x, ph, r);
+                            }
+                        }
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -437,15 +538,67 @@ __global__ void __launch_bounds__(THREADS64, 1) density64_kernel(
             }
         }
         // the two halves of the phi meet (warps 0-7 only: a barrier of their own)
-        if (hb == 1) ctl->part[(warp & 3) * 32 + lane] = r;
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (hb == 0 && ok) {
-            r += ctl->part[(warp & 3) * 32 + lane];
-            const int gx = t / (nt * nt) * TILE + (lp >> 6), gy = (t / nt) % nt * TILE + ((lp >> 3) & 7),
-                      gz = t % nt * TILE + (lp & 7);
-            if (gx < n && gy < n && gz < n)
-                rho[(long long)s * n * n * n + ((long long)gx * n + gy) * n + gz] = r * f;
+        const int p = (warp & 3) * 32 + lane;
+        const int gx = t / (nt * nt) * TILE + (lp >> 6), gy = (t / nt) % nt * TILE + ((lp >> 3) & 7),
+                  gz = t % nt * TILE + (lp & 7);
+        const bool inside = gx < n && gy < n && gz < n;
+        if (hb == 1) {
+            ctl->part[p] = r;
+            ctl->most[p] = most;
+            ctl->found[p] = found;
         }
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (hb == 0) {
+            r += ctl->part[p];
+            most = max(most, ctl->most[p]);
+            found = max(found, ctl->found[p]);
+            // the term of both scales, 2^(rx + E) phi, has x = 2^(2 SHIFT - 56)
+            const bool lost = f64 || (rx != ROW_ZERO && most > COL_ZERO / 2 && found < most + 1023 + 2 * SHIFT - 56 - LOST_BITS);
+            if (ok && inside && !lost)
+                rho[(long long)s * n * n * n + ((long long)gx * n + gy) * n + gz] = top == COL_ZERO ? 0.0 : ldexp(r, 56 - 2 * SHIFT + rx + top);
+            const unsigned b = __ballot_sync(0xffffffffu, inside && lost);
+            if (lane == 0) ctl->lost[warp] = b;
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        // those points in float64: short lists by a warp each, others one after the other by all eight
+        // (threads along the phi quads, then the chi)
+        const int G = nc * np <= 4096 ? 32 : 256, tid = threadIdx.x & (G - 1);
+        const int nq = np / 4, lanes = nq > 16 ? 32 : nq > 8 ? 16 : 8, q0 = tid % lanes, a0 = tid / lanes;
+        for (int w = 0, i = 0; w < 4; ++w)
+            for (unsigned left = ctl->lost[w]; left != 0; left &= left - 1, ++i) {
+                if (G == 32 && (i & 7) != warp) continue;
+                const int lpl = pb * 128 + w * 32 + __ffs(left) - 1;
+                double v = 0.0;
+                for (int q = q0; q < nq; q += lanes) {
+                    const double *Pq = Ps + pids[p0 + q * 4], *ph = pval + (long long)(p0 + q * 4) * TILE_PTS + lpl;
+                    double x[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 8
+                    for (int a = a0; a < nc; a += G / lanes) {
+                        const double ch = __ldg(cval + (long long)(c0 + a) * TILE_PTS + lpl);
+                        const double2 *pp = reinterpret_cast<const double2 *>(Pq + (long long)cids[c0 + a] * nphi);
+                        const double2 y = __ldg(pp), z = __ldg(pp + 1);
+                        x[0] = fma(ch, y.x, x[0]);
+                        x[1] = fma(ch, y.y, x[1]);
+                        x[2] = fma(ch, z.x, x[2]);
+                        x[3] = fma(ch, z.y, x[3]);
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) v = fma(x[e], __ldg(ph + e * TILE_PTS), v);
+                }
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (G == 256) {
+                    if (lane == 0) ctl->part[warp] = v;
+                    asm volatile("bar.sync 1, 256;" ::: "memory");
+                    v = 0.0;
+                    for (int u = 0; u < 8; ++u) v += ctl->part[u];
+                    asm volatile("bar.sync 1, 256;" ::: "memory");
+                }
+                if (tid == 0) {
+                    const int hx = t / (nt * nt) * TILE + (lpl >> 6), hy = (t / nt) % nt * TILE + ((lpl >> 3) & 7),
+                              hz = t % nt * TILE + (lpl & 7);
+                    rho[(long long)s * n * n * n + ((long long)hx * n + hy) * n + hz] = v;
+                }
+            }
     }
     tc_fence_before();
     __syncthreads();
@@ -496,16 +649,31 @@ __global__ void chi_digits_fm_kernel(const double *__restrict__ val, long long v
         for (int j = 0; j < ND; ++j) out[j * values + i] = (unsigned short)digit_pair(digit(u, j), 64u);
     }
 }
-// and point-major in chunks of 64 slots of a tile, zero padded: [digit][chunk][512][64]
+// exponent E of every point of a tile, max over its chi of |value| < 2^E, at least -900 (ROW_ZERO where
+// all are zero). One thread per point.
+__global__ void __launch_bounds__(256) point_exponent_kernel(const double *__restrict__ val, const int *__restrict__ off,
+                                                             int ntiles, int *__restrict__ out) {
+    const long long i = blockIdx.x * 256ll + threadIdx.x;
+    if (i >= (long long)ntiles * TILE_PTS) return;
+    const int t = (int)(i / TILE_PTS), p = (int)(i % TILE_PTS);
+    double m = 0.0;
+    for (int sl = off[t]; sl < off[t + 1]; ++sl) m = fmax(m, fabs(val[(long long)sl * TILE_PTS + p]));
+    int e = 0;
+    if (m > 0.0) frexp(m, &e);
+    out[i] = m > 0.0 ? max(e, -900) : ROW_ZERO;
+}
+// and point-major in chunks of 64 slots of a tile, zero padded, each point by its own scale:
+// [digit][chunk][512][64]
 __global__ void chi_digits_pm_kernel(const double *__restrict__ val, const int *__restrict__ off,
                                      const int *__restrict__ chunk_tile, const int *__restrict__ chunk_j, long long nchunks,
-                                     double sc, unsigned short *__restrict__ out) {
+                                     const int *__restrict__ rexp, unsigned short *__restrict__ out) {
     const long long tot = nchunks * TILE_PTS * 64;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
         const long long ch = e / (TILE_PTS * 64);
         const int rem = (int)(e - ch * (TILE_PTS * 64)), p = rem / 64, t = chunk_tile[ch], sl = chunk_j[ch] * 64 + rem % 64;
-        const bool in = sl < off[t + 1] - off[t];
-        const unsigned long long u = biased(in ? val[(long long)(off[t] + sl) * TILE_PTS + p] * sc : 0.0);
+        const int ex = rexp[t * TILE_PTS + p];
+        const bool in = sl < off[t + 1] - off[t] && ex != ROW_ZERO;
+        const unsigned long long u = biased(in ? ldexp(val[(long long)(off[t] + sl) * TILE_PTS + p], SHIFT - ex) : 0.0);
 #pragma unroll
         for (int j = 0; j < ND; ++j) out[j * tot + e] = (unsigned short)digit_pair(digit(u, j), 64u);
     }
@@ -559,10 +727,6 @@ bool fp64_grid_build(cudaStream_t st, Mem &mem, const TileSet<double> &chi, cons
     std::memcpy(m, h, sizeof m);
     // tables with infinities, NaN or values beyond any orbital's stay on the CUDA cores
     if (!(m[0] < 1e100) || !(m[1] < 1e100)) return false;
-    int e = 0;
-    std::frexp(m[0], &e);
-    G.ex = std::max(e, -900);
-    const double sc = std::ldexp(1.0, SHIFT - G.ex);
     auto up = [&](const auto &v) {
         using E = typename std::decay<decltype(v[0])>::type;
         E *p = mem.alloc<E>(v.size());
@@ -587,25 +751,32 @@ bool fp64_grid_build(cudaStream_t st, Mem &mem, const TileSet<double> &chi, cons
         int *dct = tmp.alloc<int>(ct.size()), *dcj = tmp.alloc<int>(cj.size());
         check(cudaMemcpy(dct, ct.data(), ct.size() * sizeof(int), cudaMemcpyHostToDevice), "upload chunk tiles");
         check(cudaMemcpy(dcj, cj.data(), cj.size() * sizeof(int), cudaMemcpyHostToDevice), "upload chunk index");
-        chi_digits_pm_kernel<<<8 * 1216, 256, 0, st>>>(chi.val, chi.off, dct, dcj, nchunks, sc, G.pm);
+        G.rexp = mem.alloc<int>((size_t)ntl * TILE_PTS);
+        point_exponent_kernel<<<(unsigned)(((long long)ntl * TILE_PTS + 255) / 256), 256, 0, st>>>(chi.val, chi.off, ntl, G.rexp);
+        check_launch("point_exponent_kernel");
+        chi_digits_pm_kernel<<<8 * 1216, 256, 0, st>>>(chi.val, chi.off, dct, dcj, nchunks, G.rexp, G.pm);
         check_launch("chi_digits_pm_kernel");
         check(cudaStreamSynchronize(st), "sync digit tables");
         G.tiles = up(tiles);
         G.ntiles = (int)tiles.size();
         G.cfirst = up(first);
         G.covers = G.ntiles == ntl;
+        G.pslots = pslots;
     }
     return true;
 }
 
-// rho [k][n^3] of P [k][nchi][nphi] (16-byte aligned rows); bits: k words of 64 bits
+// rho [k][n^3] of P [k][nchi][nphi] (16-byte aligned rows); exps: k (pslots + ntiles) words
 void response_density_fp64(cudaStream_t st, const GridShape &g, const TileSet<double> &chi, const TileSet<double> &phi,
                            const Fp64Grid &G, int nphi, const double *P, long long sP, int k, double *rho,
-                           unsigned long long *bits, int *err) {
+                           int *exps, int *err) {
     if (k <= 0) return;
     ProfScope ps(st, ST_DENSITY, 2.0 * k * g.pair_points, 8.0 * (g.table_values + (double)k * g.n * g.n * g.n));
     if (!G.covers) check(cudaMemsetAsync(rho, 0, sizeof(double) * (size_t)k * g.n * g.n * g.n, st), "memset rho");
-    max64(st, P, sP, k, bits);
+    int *top = exps + k * G.pslots;
+    column_exponents_kernel<<<dim3(G.ntiles, k), 256, 0, st>>>(G.tiles, G.ntiles, chi.off, chi.ids, phi.off, phi.ids, nphi, P,
+                                                              sP, G.pslots, exps, top);
+    check_launch("column_exponents_kernel");
     CUtensorMap mx;
     if (!encode_map_2d(&mx, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, G.pm, 64ull, (unsigned long long)(ND * G.nchunks) * TILE_PTS,
                        128ull, 64, 128))
@@ -619,8 +790,8 @@ void response_density_fp64(cudaStream_t st, const GridShape &g, const TileSet<do
     const long long blocks = 4LL * G.ntiles * k;
     if (blocks > 0x7fffffffll) throw CudaError{cudaErrorInvalidValue, "density64: too many blocks"};
     density64_kernel<<<(unsigned)blocks, THREADS64, smem64_den(), st>>>(
-        mx, g.n, g.nt, k, G.tiles, chi.off, chi.ids, G.cfirst, G.nchunks, phi.off, phi.ids, phi.val, nphi, P, sP, bits, G.ex,
-        rho, err, active_wait_limit());
+        mx, g.n, g.nt, k, G.ntiles, G.tiles, chi.off, chi.ids, chi.val, G.cfirst, G.nchunks, phi.off, phi.ids, phi.val, nphi, P,
+        sP, G.rexp, exps, top, G.pslots, rho, err, active_wait_limit());
     check_launch("density64_kernel");
 }
 

@@ -140,7 +140,9 @@ struct Fp64Grid {
     const int *tiles = nullptr;     // density: tiles with both chi and phi, densest first
     const int *cfirst = nullptr;    // first 64-wide chi chunk of each tile
     int *cexp = nullptr, *pexp = nullptr;   // of every slot: |value| < 2^exp
-    int ntiles = 0, ex = 0;                 // |chi| < 2^ex
+    int *rexp = nullptr;                    // of every point of every tile: |chi| < 2^exp
+    long long pslots = 0;                   // phi slots
+    int ntiles = 0;
     bool covers = false;            // the listed tiles are all tiles of the grid
 };
 
