@@ -131,8 +131,11 @@ typedef struct {
 
 typedef struct {
     int32_t precision;        /* TDDFT_FP64: all arithmetic in float64, the grid contractions by
-                                 exact splitting of float64 values on the tensor cores (their
-                                 rounding error is that of float64 sums or below).
+                                 exact splitting of float64 values on the tensor cores. The
+                                 density's error is that of float64 sums or below at every
+                                 point; the integrals' is that of float64 sums of the tiles'
+                                 largest |chi| times largest |V phi|: relative to these, not to
+                                 an entry that is far smaller.
                                  TDDFT_MIXED: matrices, grids and FFTs in float32; traces,
                                  line search, Gram-Schmidt, eigenvalues in float64 */
     int32_t mode;             /* TDDFT_MODE_FULL (Eq. operator_RPA); TDDFT_MODE_TDA (B = 0:

@@ -275,7 +275,6 @@ struct Impl {
     // float64 contexts: grid contractions by exact splitting on the tensor cores
     Fp64Grid g64;
     bool int64_tc = false, dens64_tc = false;
-    unsigned long long *bits64 = nullptr;
     int *exps64 = nullptr;
     IItem *int_items = nullptr;
     int nint_items = 0, int_pch = 48;
@@ -517,7 +516,7 @@ void response_density_fp64(cudaStream_t st, const GridShape &g, const TileSet<do
                            int *exps, int *err);
 void potential_integrals_fp64(cudaStream_t st, const GridShape &g, const TileSet<double> &chi, const TileSet<double> &phi,
                               const Fp64Grid &G, int nchi, int nphi, const double *V, int k, double *out,
-                              unsigned long long *bits, int *err);
+                              int *err);
 int noalloc_max_states();
 void response_density_tc_noalloc(cudaStream_t st, const GridShape &g, const TileSet<float> &chi,
                                  const TileSet<float> &phi, const unsigned short *chi_pm, int CK, int NPmax,
@@ -837,7 +836,6 @@ void ensure_workspace(tddft_ctx *c, Impl<T> &I, int states) {
         (size_t)std::max({states * len, states * n3, states * c->nnz_abi()}));
     I.tc_bits = I.wmem.template alloc<unsigned>((size_t)states);
     I.tc_scale = I.wmem.template alloc<float>((size_t)2 * states);
-    I.bits64 = I.wmem.template alloc<unsigned long long>((size_t)states);
     if (I.dens64_tc) I.exps64 = I.wmem.template alloc<int>((size_t)states * (I.g64.pslots + I.g64.ntiles));
     if (c->sparse) {
         // the grid kernels address P and V densely; the tensor-core left products take their
@@ -910,7 +908,7 @@ void integrals(tddft_ctx *c, Impl<T> &I, int ns) {
     }
     if constexpr (sizeof(T) == 8) {
         if (I.int64_tc) {
-            potential_integrals_fp64(c->st, c->grid(), I.chi, I.phi, I.g64, c->nc, c->nv, I.V, ns, out, I.bits64,
+            potential_integrals_fp64(c->st, c->grid(), I.chi, I.phi, I.g64, c->nc, c->nv, I.V, ns, out,
                                      tc_error_word());
             done = true;
         }

@@ -22,8 +22,13 @@
 // mean square 9.6e-17, where float64 sums have 8.2e-16 and 1.2e-16 (emulated, 8 atoms, 48^3); with P's
 // rows in blocks of 1, 1e-6 and 1e-12, 7.2e-16 and 9.7e-17 against 9.3e-16 and 1.2e-16. One scale for
 // the chi table and one for a state's P left no digit right where chi is below 1e-16 of its largest value.
-// The integrals scale V by its largest value and every function's values on a tile by their own
-// maximum there.
+// The integrals' scales are chi's and (V phi)'s largest values on the tile, each function its own. An
+// entry's error is about 2^-63 of the sum over tiles of 512 times their product, below that of a float64
+// sum wherever the entry's terms come within 2^-10 of it; entries of functions that only graze each
+// other have the same absolute error and fewer digits than a float64 sum would give them. A tile whose
+// V is not finite is summed in float64. Largest error of small-8's entries, of the largest entry: V
+// without structure 3.3e-16, float64 sums 6.4e-16; V a Gaussian of 1 A, 3.6e-16 and 7.5e-16 (with one
+// scale for all of V 6e-11).
 //
 // The digits of B are stacked along N (32 columns each), the accumulators of the levels along the
 // columns of TMEM (32 each): for digit i of A one MMA of N = 32 (9 - i) columns, placed at level i,
@@ -35,8 +40,8 @@
 // warp 9 issues the MMAs of this one, then combine the levels in integers and float64. Every wait is
 // bounded.
 // Measured (GB300, stage, CUDA events, CUDA-core kernel and this): 8 atoms, 48^3, 1 state: density 0.57
-// and 0.10 ms, integrals 1.05 and 0.08; 32 atoms with 4 + 9 functions, 90^3, 3 states: density 19.3 and
-// 1.09 ms, integrals 21.2 and 0.91. Bound by the issue and shared-memory reads of the MMAs (A is read
+// and 0.08 ms, integrals 1.05 and 0.07; 32 atoms with 4 + 9 functions, 90^3, 3 states: density 19.3 and
+// 0.98 ms, integrals 21.2 and 0.85. Bound by the issue and shared-memory reads of the MMAs (A is read
 // once per digit: 45 digit products in 10 MMAs) and, in small systems, by a block's start and end.
 #include "tc_common.cuh"
 #include "tddft_internal.h"
@@ -75,6 +80,7 @@ struct __align__(8) Shared64 {
     double part[128];                // density: the second half's sums and exponents
     int most[128], found[128];
     unsigned lost[4];                // points to sum in float64
+    int vmax[8], down[NB];           // integrals: V's exponents by warp, the columns' scales
 };
 
 __device__ __forceinline__ void init64(Shared64 *c) {
@@ -93,20 +99,9 @@ __device__ __forceinline__ void init64(Shared64 *c) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-// exponent E with max < 2^E from the bits of max |x| (clamped so that 2^(61 - E) is finite)
-__device__ __forceinline__ int exponent_of(unsigned long long bits) {
-    int e = 0;
-    frexp(__longlong_as_double((long long)bits), &e);
-    return max(e, -900);
-}
-__device__ __forceinline__ double pow2(int e) { return ldexp(1.0, e); }
-// 2^(61 - E) of a column's values (0 of a column of zeros)
+// 2^(62 - E) of a column's values (0 of a column of zeros)
 __device__ __forceinline__ double column_scale(int E) {
     return E < -900 || E > 1024 ? 0.0 : __hiloint2double((1023 + SHIFT - E) << 20, 0);
-}
-// a state's values are all finite
-__device__ __forceinline__ bool finite_bits(unsigned long long bits) {
-    return isfinite(__longlong_as_double((long long)bits));
 }
 
 // q + sum_i 64 128^i: the digits plus 64, seven bits each and eight for the first, up to 128
@@ -138,6 +133,12 @@ __device__ __forceinline__ double combine_levels(const float (*D)[8], int e) {
 #pragma unroll
     for (int l = 5; l < ND; ++l) lo = lo * 128 + (int)__float2int_rn(D[l][e]);
     return fma(to_double(hi), 268435456.0, to_double(lo));
+}
+// E with |x| < 2^E of one value: VAL_ZERO of zero, VAL_BAD of infinity and NaN
+constexpr int VAL_ZERO = -8192, VAL_BAD = 8191;
+__device__ __forceinline__ int value_exponent(double x) {
+    const int h = __double2hiint(x) & 0x7fffffff, f = h >> 20;
+    return (h | __double2loint(x)) == 0 ? VAL_ZERO : f == 2047 ? VAL_BAD : max(f, 1) - 1022;
 }
 // exponent field of x (0: zero or below the normal range, 2047: infinity or NaN)
 __device__ __forceinline__ int expo_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
@@ -181,15 +182,16 @@ __device__ __forceinline__ bool mma_block(Shared64 *ctl, volatile int *abort, un
 __global__ void __launch_bounds__(THREADS64, 1) integrals64_kernel(
     const __grid_constant__ CUtensorMap mX,   // chi digits [digit * slots + slot][512], box 64 x 128
     int n, int nt, int k, const IItem *__restrict__ items, long long slots, const int *__restrict__ cids,
-    const int *__restrict__ pids, const double *__restrict__ pval, const int *__restrict__ cexp,
-    const int *__restrict__ pexp, int nchi, int nphi, const double *__restrict__ V,
-    const unsigned long long *__restrict__ vbits, double dV, double *__restrict__ out, int *err, long long wlim) {
+    const double *__restrict__ cval, const int *__restrict__ pids, const double *__restrict__ pval,
+    const int *__restrict__ cexp, const short *__restrict__ pexp, int nchi, int nphi, const double *__restrict__ V, double dV,
+    double *__restrict__ out, int *err, long long wlim) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<unsigned long long>(smem_raw) + 1023ull) & ~1023ull);
     unsigned char *A = base, *B = base + A_RING * A_TILE;
     double *Vt = reinterpret_cast<double *>(B + 2 * B_KMAJ);
-    Shared64 *ctl = reinterpret_cast<Shared64 *>(Vt + TILE_PTS);
+    short *Ve = reinterpret_cast<short *>(Vt + TILE_PTS);
+    Shared64 *ctl = reinterpret_cast<Shared64 *>(Ve + TILE_PTS);
     volatile int *abort = &ctl->abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int s = blockIdx.x % k;
@@ -200,14 +202,6 @@ __global__ void __launch_bounds__(THREADS64, 1) integrals64_kernel(
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
                      "r"(512));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-    // V on the tile, scaled so that the products with scaled phi become q
-    const int ev = exponent_of(vbits[s]);
-    const double vs = pow2(SHIFT - ev);
-    const int tx = d.t / (nt * nt), ty = (d.t / nt) % nt, tz = d.t % nt;
-    for (int lp = threadIdx.x; lp < TILE_PTS; lp += THREADS64) {
-        const int gx = tx * TILE + (lp >> 6), gy = ty * TILE + ((lp >> 3) & 7), gz = tz * TILE + (lp & 7);
-        Vt[lp] = (gx < n && gy < n && gz < n) ? V[(long long)s * n3 + ((long long)gx * n + gy) * n + gz] * vs : 0.0;
     }
     tc_fence_before();
     __syncthreads();
@@ -249,11 +243,58 @@ __global__ void __launch_bounds__(THREADS64, 1) integrals64_kernel(
             }
         }
     } else {
-        // digits of V phi: thread = (phi b, octet o of the K block's points)
+        // V on the tile and its exponents, then V scaled by the largest (as it is where it is not finite)
+        const int tx = d.t / (nt * nt), ty = (d.t / nt) % nt, tz = d.t % nt;
+        double vr[2];
+        int etv = VAL_ZERO;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int lp = threadIdx.x + h * 256;
+            const int gx = tx * TILE + (lp >> 6), gy = ty * TILE + ((lp >> 3) & 7), gz = tz * TILE + (lp & 7);
+            vr[h] = (gx < n && gy < n && gz < n) ? V[(long long)s * n3 + ((long long)gx * n + gy) * n + gz] : 0.0;
+            const int E = value_exponent(vr[h]);
+            Ve[lp] = (short)E;
+            etv = max(etv, E);
+        }
+        etv = __reduce_max_sync(0xffffffffu, etv);
+        if (lane == 0) ctl->vmax[warp] = etv;
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+#pragma unroll
+        for (int i = 0; i < 8; ++i) etv = max(etv, ctl->vmax[i]);
+        const bool bad = etv == VAL_BAD;
+        etv = etv == VAL_ZERO || bad ? 0 : max(etv, -900);
+        const double vs = __hiloint2double((1023 + SHIFT - etv) << 20, 0);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) Vt[threadIdx.x + h * 256] = bad ? vr[h] : vr[h] * vs;
+        // digits of V phi: thread = (phi b, octet o of the K block's points). phi takes the exponent of the
+        // scale 2^E of its column of products without V's: phi 2^-down, |V phi| < 2^(etv + down)
         const int o = threadIdx.x & 7, b = threadIdx.x >> 3;
         bool ok = true;
-        // phi / 2^E of its slot: the exponent field takes -E (|phi| < 2^E, so no overflow; zero stays zero)
-        const int down = b < d.np ? pexp[d.p0 + b] : 0;
+        int down;
+        {
+            unsigned m = 0xc000c000u, pm = 0xe000e000u;       // pairs of exponents: V phi, phi
+            const uint4 *pe = reinterpret_cast<const uint4 *>(pexp + (long long)(d.p0 + b) * TILE_PTS + o * 8);
+            const uint4 *ve = reinterpret_cast<const uint4 *>(Ve + o * 8);
+            if (b < d.np)
+#pragma unroll
+                for (int kb = 0; kb < KB; ++kb) {
+                    const uint4 x = __ldg(pe + kb * 8), y = ve[kb * 8];
+                    m = __vmaxs2(m, __vmaxs2(__vmaxs2(__vadd2(x.x, y.x), __vadd2(x.y, y.y)),
+                                             __vmaxs2(__vadd2(x.z, y.z), __vadd2(x.w, y.w))));
+                    pm = __vmaxs2(pm, __vmaxs2(__vmaxs2(x.x, x.y), __vmaxs2(x.z, x.w)));
+                }
+#pragma unroll
+            for (int i = 1; i < 8; i *= 2) {
+                m = __vmaxs2(m, __shfl_xor_sync(0xffffffffu, m, i));
+                pm = __vmaxs2(pm, __shfl_xor_sync(0xffffffffu, pm, i));
+            }
+            const int mw = max((int)(short)(m & 0xffffu), (int)(short)(m >> 16));
+            const int mp = max((int)(short)(pm & 0xffffu), (int)(short)(pm >> 16));
+            // 2^900 at most above phi's largest value, so that no phi leaves the range
+            down = mw < VAL_ZERO / 2 || bad ? 0 : max(max(mw - etv, mp - 900), -1000);
+            if (o == 0) ctl->down[b] = down;
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");
         auto scaled = [&](double x) {
             const int hi = __double2hiint(x), ef = (hi >> 20) & 0x7ff;
             return ef != 0 && ef > down ? __hiloint2double(hi - down * (1 << 20), __double2loint(x)) : 0.0;
@@ -264,7 +305,8 @@ __global__ void __launch_bounds__(THREADS64, 1) integrals64_kernel(
             const double2 *vv = reinterpret_cast<const double2 *>(Vt + kb * 64 + o * 8);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const double2 p = b < d.np ? __ldg(pp + e) : make_double2(0.0, 0.0), v = vv[e];
+                const double2 p = b < d.np && !bad ? __ldg(pp + e) : make_double2(0.0, 0.0);
+                const double2 v = bad ? make_double2(0.0, 0.0) : vv[e];
                 u[2 * e] = biased(scaled(p.x) * v.x);
                 u[2 * e + 1] = biased(scaled(p.y) * v.y);
             }
@@ -288,23 +330,32 @@ __global__ void __launch_bounds__(THREADS64, 1) integrals64_kernel(
         }
         ok = ok && mbar_wait(&ctl->acc_full, 0, abort, wlim) && !*abort;
         tc_fence_after();
-        // rows of chi over warps 0-3 and 4-7, the phi halves between the two groups. x w is
-        // 2^(56 - (61 - ec) - (61 - ep - ev)) times the combined levels
+        // rows of chi over warps 0-3 and 4-7, the phi halves between the two groups
         const int a = (warp & 3) * 32 + lane;
-        const double f = finite_bits(vbits[s]) ? ldexp(dV, 56 - 2 * SHIFT + ev + (a < d.nc ? cexp[d.c0 + a] : 0))
-                                               : __longlong_as_double(0x7ff8000000000000ll);
+        const int ea = 56 - 2 * SHIFT + etv + (a < d.nc ? cexp[d.c0 + a] : 0);
         double *o_row = out + (long long)s * nchi * nphi + (a < d.nc ? (long long)cids[d.c0 + a] * nphi : 0);
         for (int c = (warp >> 2) * 16; c < (warp >> 2) * 16 + 16 && c < d.np; c += 8) {
             float D[ND][8];
 #pragma unroll
             for (int l = 0; l < ND; ++l) tmem_ld8(tmem + l * NB + c + ((unsigned)((warp & 3) * 32) << 16), D[l]);
-            if (!ok || a >= d.nc) continue;
+            if (!ok || a >= d.nc || bad) continue;
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-                if (c + e < d.np)
-                    atomicAdd(o_row + pids[d.p0 + c + e], f * __hiloint2double((1023 + pexp[d.p0 + c + e]) << 20, 0) *
-                                                              combine_levels(D, e));
+                if (c + e < d.np) {
+                    double x = combine_levels(D, e);
+                    const int f = expo_field(x), up = ea + ctl->down[c + e];
+                    if (f != 0) x = f + up > 0 ? __hiloint2double(__double2hiint(x) + up * (1 << 20), __double2loint(x)) : ldexp(x, up);
+                    atomicAdd(o_row + pids[d.p0 + c + e], dV * x);
+                }
         }
+        // V not finite on the tile: the sums in float64
+        if (ok && bad && a < d.nc)
+            for (int c = (warp >> 2) * 16; c < (warp >> 2) * 16 + 16 && c < d.np; ++c) {
+                const double *x = cval + (long long)(d.c0 + a) * TILE_PTS, *y = pval + (long long)(d.p0 + c) * TILE_PTS;
+                double v = 0.0;
+                for (int i = 0; i < TILE_PTS; ++i) v = fma(__ldg(x + i), __ldg(y + i) * Vt[i], v);
+                atomicAdd(o_row + pids[d.p0 + c], dV * v);
+            }
     }
     tc_fence_before();
     __syncthreads();
@@ -324,7 +375,7 @@ constexpr int LOST_BITS = 9;         // terms this far below their scales: the p
 
 // cexp[s][slot]: |P_ab| < 2^E over the tile's chi; ctop[s][listed tile]: the largest E of the tile's columns,
 // or TILE_F64 where P is not finite or a column's scale is more than 2^900 below the largest or below
-// 2^-900. Block = (listed tile, state). 32 atoms, 3 states: 30 us.
+// 2^-900. Block = (listed tile, state). 32 atoms, 3 states: 17 us.
 __global__ void __launch_bounds__(256) column_exponents_kernel(const int *__restrict__ tiles, int ntiles,
                                                                const int *__restrict__ coff, const int *__restrict__ cids,
                                                                const int *__restrict__ poff, const int *__restrict__ pids,
@@ -640,6 +691,11 @@ __global__ void __launch_bounds__(256) slot_exponent_kernel(const double *__rest
     if ((threadIdx.x & 31) == 0) out[sl] = max(e, -900);
 }
 
+__global__ void value_exponents_kernel(const double *__restrict__ val, long long values, short *__restrict__ out) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < values; i += (long long)gridDim.x * blockDim.x)
+        out[i] = (short)value_exponent(val[i]);
+}
+
 // digit tables of chi: function-major [digit][slot][512], each slot by its own scale
 __global__ void chi_digits_fm_kernel(const double *__restrict__ val, long long values, const int *__restrict__ cexp,
                                      unsigned short *__restrict__ out) {
@@ -679,7 +735,7 @@ __global__ void chi_digits_pm_kernel(const double *__restrict__ val, const int *
     }
 }
 
-size_t smem64_int() { return 1024 + A_RING * A_TILE + 2 * B_KMAJ + TILE_PTS * sizeof(double) + sizeof(Shared64); }
+size_t smem64_int() { return 1024 + A_RING * A_TILE + 2 * B_KMAJ + TILE_PTS * (sizeof(double) + sizeof(short)) + sizeof(Shared64); }
 size_t smem64_den() { return 1024 + A_RING * A_TILE + 2 * B_NMAJ + sizeof(Shared64); }
 
 void max64(cudaStream_t st, const double *x, long long len, int rows, unsigned long long *bits) {
@@ -736,10 +792,11 @@ bool fp64_grid_build(cudaStream_t st, Mem &mem, const TileSet<double> &chi, cons
     G.slots = slots;
     G.fm = mem.alloc<unsigned short>((size_t)ND * values);
     G.cexp = mem.alloc<int>(slots);
-    G.pexp = mem.alloc<int>(pslots);
+    G.pexp = mem.alloc<short>((size_t)pslots * TILE_PTS);
     slot_exponent_kernel<<<(unsigned)((slots + 7) / 8), 256, 0, st>>>(chi.val, slots, G.cexp);
-    slot_exponent_kernel<<<(unsigned)((pslots + 7) / 8), 256, 0, st>>>(phi.val, pslots, G.pexp);
     check_launch("slot_exponent_kernel");
+    value_exponents_kernel<<<8 * 152, 256, 0, st>>>(phi.val, pslots * TILE_PTS, G.pexp);
+    check_launch("value_exponents_kernel");
     chi_digits_fm_kernel<<<8 * 1216, 256, 0, st>>>(chi.val, values, G.cexp, G.fm);
     check_launch("chi_digits_fm_kernel");
     G.items = up(items);
@@ -795,15 +852,14 @@ void response_density_fp64(cudaStream_t st, const GridShape &g, const TileSet<do
     check_launch("density64_kernel");
 }
 
-// out [k][nchi][nphi] of V [k][n^3]; bits: k words of 64 bits
+// out [k][nchi][nphi] of V [k][n^3]
 void potential_integrals_fp64(cudaStream_t st, const GridShape &g, const TileSet<double> &chi, const TileSet<double> &phi,
                               const Fp64Grid &G, int nchi, int nphi, const double *V, int k, double *out,
-                              unsigned long long *bits, int *err) {
+                              int *err) {
     if (k <= 0) return;
     ProfScope ps(st, ST_INTEGRALS, 2.0 * k * g.pair_points,
                  8.0 * (g.table_values + (double)k * g.n * g.n * g.n + (double)k * nchi * nphi));
     check(cudaMemsetAsync(out, 0, sizeof(double) * (size_t)k * nchi * nphi, st), "memset(integrals)");
-    max64(st, V, (long long)g.n * g.n * g.n, k, bits);
     CUtensorMap mx;
     if (!encode_map_2d(&mx, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, G.fm, (unsigned long long)TILE_PTS,
                        (unsigned long long)(ND * G.slots), (unsigned long long)TILE_PTS * 2, 64, 128))
@@ -817,7 +873,7 @@ void potential_integrals_fp64(cudaStream_t st, const GridShape &g, const TileSet
     const long long blocks = G.nitems * k;
     if (blocks > 0x7fffffffll) throw CudaError{cudaErrorInvalidValue, "integrals64: too many blocks"};
     integrals64_kernel<<<(unsigned)blocks, THREADS64, smem64_int(), st>>>(
-        mx, g.n, g.nt, k, G.items, G.slots, chi.ids, phi.ids, phi.val, G.cexp, G.pexp, nchi, nphi, V, bits, g.dV, out, err,
+        mx, g.n, g.nt, k, G.items, G.slots, chi.ids, chi.val, phi.ids, phi.val, G.cexp, G.pexp, nchi, nphi, V, g.dV, out, err,
         active_wait_limit());
     check_launch("integrals64_kernel");
 }

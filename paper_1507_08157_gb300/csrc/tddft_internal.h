@@ -139,7 +139,8 @@ struct Fp64Grid {
     const IItem *items = nullptr;   // integrals: at most 128 chi and 32 phi of a tile
     const int *tiles = nullptr;     // density: tiles with both chi and phi, densest first
     const int *cfirst = nullptr;    // first 64-wide chi chunk of each tile
-    int *cexp = nullptr, *pexp = nullptr;   // of every slot: |value| < 2^exp
+    int *cexp = nullptr;                    // of every chi slot: |value| < 2^exp
+    short *pexp = nullptr;                  // of every phi value
     int *rexp = nullptr;                    // of every point of every tile: |chi| < 2^exp
     long long pslots = 0;                   // phi slots
     int ntiles = 0;

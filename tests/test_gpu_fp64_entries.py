@@ -103,3 +103,71 @@ def test_density_of_a_bad_kernel_entry_is_bad_where_it_reaches(tddft, spread9, b
     for q in range(3):
         keep = ~reach if q == 1 else np.ones_like(reach)
         assert np.max(np.abs(rho[q] - ref[q])[keep]) <= tol * np.max(np.abs(ref[q])), q
+
+
+def _potentials(s, kind):
+    rng = np.random.default_rng(6)
+    V = rng.standard_normal((2, s.n, s.n, s.n))
+    if kind == "peak":
+        V[0, s.n // 2, s.n // 2, s.n // 2] = 1e12
+        V[1, 3, 4, 5] = -1e30
+    elif kind == "gaussian":
+        x = (np.arange(s.n) - s.n / 2) * s.h
+        V[:] = np.exp(-0.25 * sum(np.meshgrid(x ** 2, x ** 2, x ** 2, indexing="ij")))
+    elif kind == "spread":
+        V *= 10.0 ** rng.uniform(-12, 0, V.shape)
+    elif kind == "zeros":
+        V[0, : s.n // 2] = 0.0
+        V[1] = 0.0
+    return V
+
+
+def _tile_scales(s, V):
+    """Sum over tiles of max |chi_a| max |V phi_b|, [a, b]."""
+    nt = -(-s.n // 8)
+
+    def tops(full):
+        pad = np.zeros((full.shape[0],) + (nt * 8,) * 3)
+        pad[:, : s.n, : s.n, : s.n] = np.abs(full)
+        return pad.reshape(-1, nt, 8, nt, 8, nt, 8).max(axis=(2, 4, 6)).reshape(full.shape[0], -1)
+
+    return tops(ogrid.full_grid(s.chi, s.n)) @ tops(ogrid.full_grid(s.phi, s.n) * V).T
+
+
+@pytest.mark.parametrize("radius", [2.5, 6.0])
+@pytest.mark.parametrize("kind", ["plain", "peak", "gaussian", "spread", "zeros"])
+def test_integrals_keep_their_tiles_accuracy(tddft, kind, radius):
+    """Bound per entry: 2^-47 of the tiles' scales (per product 2^-60 for the digit products left out and
+    2^-62 for the digits' rounding, of scales at most 8 times the largest values, 512 of them) and, of the
+    sum of the terms' sizes, the rounding of float64 sums of at most 45^3 terms added in quadrature,
+    8 sqrt(45^3) 2^-53 < 1e-12."""
+    s = sy.generate(sy.Recipe(natoms=9, cell_ang=14.0, ngrid=45, nchi=9, radius_ang=radius, seed=57))
+    chi, phi, achi, aphi = _sets(s)
+    V = _potentials(s, kind)
+    out = tddft.Context(s, precision="fp64", precond="none").potential_integrals(V)
+    ref = ogrid.potential_integrals(chi, phi, V, s.dV)
+    size = ogrid.potential_integrals(achi, aphi, np.abs(V), s.dV)
+    for q in range(2):
+        assert np.all(np.abs(out[q] - ref[q]) <= 2.0 ** -47 * s.dV * _tile_scales(s, V[q]) + 1e-12 * size[q] + 1e-300), q
+        assert np.max(np.abs(out[q] - ref[q])) <= 1e-13 * np.max(size[q]), q
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-12), ("mixed", 2e-3)])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_integrals_of_a_bad_potential_are_bad_where_it_reaches(tddft, spread9, bad, precision, tol):
+    s = spread9
+    chi, phi, _, _ = _sets(s)
+    V = np.random.default_rng(8).standard_normal((3, s.n, s.n, s.n))
+    ref = ogrid.potential_integrals(chi, phi, V, s.dV)
+    i = 9
+    p = tuple((s.phi.box[i, :3] + s.phi.box[i, 3:] // 2) % s.n)     # the centre of an atom's functions
+    V[1][p] = bad
+    out = tddft.Context(s, precision=precision, precond="none").potential_integrals(V)
+    t = tuple(x // 8 for x in p)
+    reach = np.outer(*[[_tiles_of(s, f, j)[t] for j in range(f.nfun)] for f in (s.chi, s.phi)])
+    assert 0 < reach.sum() < reach.size
+    hit = np.outer(np.abs(ogrid.values_at(chi, p)) > 0, np.abs(ogrid.values_at(phi, p)) > 0)
+    assert hit.any() and not np.any(np.isfinite(out[1][hit])) and np.all(reach[hit])
+    for q in range(3):
+        keep = ~reach if q == 1 else np.ones_like(reach)
+        assert np.max(np.abs(out[q] - ref[q])[keep]) <= tol * np.max(np.abs(ref[q])), q
