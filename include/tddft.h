@@ -315,6 +315,9 @@ tddft_status tddft_response_density_noalloc(tddft_ctx *ctx, int32_t k, const flo
  * sign-flipped and Gram-Schmidt orthonormalised in the metric of Eq. ortho, then f is applied.
  * Errors: INVALID, BREAKDOWN (dependent start vectors), NOMEM, CUDA. */
 tddft_status tddft_state_create(tddft_ctx *ctx, int32_t k, const double *Y0, tddft_state **out);
+/* The context keeps the device memory of its last destroyed state for its next one (at most 4 GiB over
+ * all contexts of the process). It is freed with the context, and by any allocation of the library
+ * that would fail without it. */
 void tddft_state_destroy(tddft_state *st);
 
 /* One preconditioned CG iteration (Sec. III C): Q_ij, multi-state gradient, preconditioner

@@ -338,16 +338,7 @@ class SlabPool {
             }
         }
         drop();
-        void *p = nullptr;
-        cudaError_t e = cudaMalloc(&p, bytes);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            if (release_spare_slabs()) e = cudaMalloc(&p, bytes);
-        }
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            throw std::bad_alloc();
-        }
+        void *p = device_alloc<char>(bytes);
         *got = bytes;
         return p;
     }
@@ -824,6 +815,7 @@ void ensure_workspace(tddft_ctx *c, Impl<T> &I, int states) {
     if (states <= I.cap) return;
     check(ctx_sync(c), "sync before workspace");
     I.wmem.release();
+    I.cap = 0;            // until every buffer is there
     const long long len = c->len(), n3 = c->n3();
     I.rho = I.wmem.template alloc<T>((size_t)states * n3);
     I.V = I.wmem.template alloc<T>((size_t)states * n3);
@@ -1235,17 +1227,18 @@ void set_density_units(Impl<float> &I, int cch, int pch) {
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work[a] > work[b]; });
     std::vector<DItem> sorted(items.size());
     for (size_t i = 0; i < order.size(); ++i) sorted[i] = items[order[i]];
-    I.umem_dens.release();
-    L.nitems = (int)sorted.size();
-    L.covers = live == ntl;
-    DUnit *du = I.umem_dens.alloc<DUnit>(us.size());
-    DItem *di = I.umem_dens.alloc<DItem>(sorted.size());
+    Mem m;                // the old lists stay until the new ones are there
+    DUnit *du = m.alloc<DUnit>(us.size());
+    DItem *di = m.alloc<DItem>(sorted.size());
     if (!us.empty()) {
         check(cudaMemcpy(du, us.data(), us.size() * sizeof(DUnit), cudaMemcpyHostToDevice), "upload density units");
         check(cudaMemcpy(di, sorted.data(), sorted.size() * sizeof(DItem), cudaMemcpyHostToDevice), "upload density items");
     }
+    std::swap(I.umem_dens.ptrs, m.ptrs);
     L.units = du;
     L.items = di;
+    L.nitems = (int)sorted.size();
+    L.covers = live == ntl;
 }
 
 // the integrals' items: each tile in chunks of 128 chi with all its phi, which the kernel takes in
@@ -1262,11 +1255,12 @@ void set_integrals_items(Impl<float> &I, int pch) {
             items.push_back(IItem{t, coff[t] + cc, std::min(128, nct - cc), poff[t], npt});
     }
     std::stable_sort(items.begin(), items.end(), [](const IItem &a, const IItem &b) { return a.np > b.np; });
-    I.umem_int.release();
-    I.int_items = I.umem_int.alloc<IItem>(items.size());
+    Mem m;
+    IItem *d = m.alloc<IItem>(items.size());
     if (!items.empty())
-        check(cudaMemcpy(I.int_items, items.data(), items.size() * sizeof(IItem), cudaMemcpyHostToDevice),
-              "upload integrals items");
+        check(cudaMemcpy(d, items.data(), items.size() * sizeof(IItem), cudaMemcpyHostToDevice), "upload integrals items");
+    std::swap(I.umem_int.ptrs, m.ptrs);
+    I.int_items = d;
     I.nint_items = (int)items.size();
     I.int_pch = pch;
 }
@@ -1292,15 +1286,14 @@ bool set_integrals_units(Impl<float> &I, int cch, int pch) {
     const int NPi = std::max(16, (maxnp + 15) / 16 * 16);
     if (integrals_tc_group(NPi, 1, maxnc) < 1) return false;
     std::vector<VTile> all;
-    for (int q = 0; q < 3; ++q) {
-        I.int_count[q] = (int)by[q].size();
-        all.insert(all.end(), by[q].begin(), by[q].end());
-    }
-    I.umem_iu.release();
-    I.int_units = I.umem_iu.alloc<VTile>(std::max<size_t>(1, all.size()));
+    for (int q = 0; q < 3; ++q) all.insert(all.end(), by[q].begin(), by[q].end());
+    Mem m;
+    VTile *d = m.alloc<VTile>(all.size());
     if (!all.empty())
-        check(cudaMemcpy(I.int_units, all.data(), all.size() * sizeof(VTile), cudaMemcpyHostToDevice),
-              "upload integrals units");
+        check(cudaMemcpy(d, all.data(), all.size() * sizeof(VTile), cudaMemcpyHostToDevice), "upload integrals units");
+    std::swap(I.umem_iu.ptrs, m.ptrs);
+    I.int_units = d;
+    for (int q = 0; q < 3; ++q) I.int_count[q] = (int)by[q].size();
     I.maxc = maxnc;
     I.NPint = NPi;
     return true;
@@ -1988,7 +1981,8 @@ void ensure_learned(tddft_ctx *c, Impl<T> &I, int k) {
     const int na = c->natoms;
     if (!I.lfc) {
         const int nb = 2 * c->nca * c->nva, nf = 2 * c->nca * c->nca + 2 * c->nva * c->nva + 1;
-        I.lfc = I.lmemf.template alloc<float>((size_t)na * 2 * c->nca * c->nca);
+        I.lmemf.release();       // of an attempt that failed
+        float *lfc = I.lmemf.template alloc<float>((size_t)na * 2 * c->nca * c->nca);
         I.lfv = I.lmemf.template alloc<float>((size_t)na * 2 * c->nva * c->nva);
         I.ldist = I.lmemf.template alloc<float>((size_t)na * na);
         I.lF = I.lmemf.template alloc<float>((size_t)na * na * nf);
@@ -1996,15 +1990,17 @@ void ensure_learned(tddft_ctx *c, Impl<T> &I, int k) {
         check(cudaMemcpyAsync(I.ldist, c->adist.data(), (size_t)na * na * sizeof(float), cudaMemcpyHostToDevice,
                               c->st),
               "upload atom distances");
-        learned_fixed_features<T>(c->st, I.Mc, I.Sc, c->nc, c->nca, na, I.lfc);
+        learned_fixed_features<T>(c->st, I.Mc, I.Sc, c->nc, c->nca, na, lfc);
         learned_fixed_features<T>(c->st, I.Mv, I.Sv, c->nv, c->nva, na, I.lfv);
-        learned_feature_rows(c->st, I.lfc, I.lfv, I.ldist, na, c->nca, c->nva, I.lF);
+        learned_feature_rows(c->st, lfc, I.lfv, I.ldist, na, c->nca, c->nva, I.lF);
         check(ctx_sync(c), "sync learned features");
+        I.lfc = lfc;
     }
     const long long rows = (long long)k * na * na;
     if (rows <= I.lrows) return;
     check(ctx_sync(c), "sync before learned buffers");
     I.lmemr.release();
+    I.lrows = 0;
     I.ls = I.lmemr.template alloc<float>((size_t)rows);
     I.lrows = rows;
 }

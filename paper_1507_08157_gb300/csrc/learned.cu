@@ -346,6 +346,7 @@ void ensure_rows(tddft_mlp *m, long long rows) {
     if (rows <= B.rows) return;
     check(cudaDeviceSynchronize(), "sync before model buffers");
     B.mem.release();
+    B.rows = 0;           // until every buffer is there
     const int ld = m->nb + m->nf;
     B.H1 = B.mem.alloc<float>((size_t)rows * m->w);
     B.H2 = B.mem.alloc<float>((size_t)rows * m->w);

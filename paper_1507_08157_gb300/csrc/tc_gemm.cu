@@ -833,19 +833,6 @@ __global__ void transpose_split_kernel(const float *__restrict__ in, int rows, i
 // scratch for the split operands, one buffer per stream (grown on demand, never shrunk): work on
 // one stream runs in order, so its products may share a buffer, while products on different
 // streams (the contexts of a batch) run concurrently and must not
-struct Scratch {
-    float *p = nullptr;
-    size_t cap = 0;
-    float *get(size_t n) {
-        if (n > cap) {
-            if (p) cudaFree(p);   // synchronises the device: earlier users of the buffer are done
-            p = nullptr;
-            check(cudaMalloc(&p, n * sizeof(float)), "cudaMalloc tc scratch");
-            cap = n;
-        }
-        return p;
-    }
-};
 std::mutex g_scratch_mu;
 std::vector<std::pair<cudaStream_t, Scratch *>> g_scratch;
 Scratch &scratch(cudaStream_t st) {
@@ -894,8 +881,13 @@ bool const_split(cudaStream_t st, const float *p, bool trans, int rows, int K, i
         }
     SplitCopy c{trans, rows, K, ld, nullptr, nullptr, (K + 3) / 4 * 4};
     const size_t n = (size_t)rows * c.kp;
-    check(cudaMalloc(&c.hi, n * sizeof(float)), "cudaMalloc constant split");
-    if (!raw) check(cudaMalloc(&c.lo, n * sizeof(float)), "cudaMalloc constant split");
+    c.hi = device_alloc<float>(n);
+    if (!raw) try {
+            c.lo = device_alloc<float>(n);
+        } catch (...) {
+            cudaFree(c.hi);
+            throw;
+        }
     if (!trans) {
         split_kernel<<<grid1((long long)n), 256, 0, st>>>(p, rows, K, ld, 0, c.hi, c.lo, c.kp, 0, 1);
     } else {

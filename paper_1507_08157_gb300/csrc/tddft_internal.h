@@ -1,6 +1,8 @@
 // Internal declarations shared by the translation units of libtddft.
 #pragma once
 
+#include "device_memory.h"
+
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -16,34 +18,6 @@ constexpr int TILE_PTS = TILE * TILE * TILE;
 struct CudaError {
     cudaError_t code;
     std::string where;
-};
-
-// owning list of device allocations (freed on release or destruction)
-bool release_spare_slabs();   // frees the memory that contexts keep of destroyed states; true if there was any
-
-struct Mem {
-    std::vector<void *> ptrs;
-    template <typename T>
-    T *alloc(size_t n) {
-        void *p = nullptr;
-        if (n == 0) n = 1;
-        cudaError_t e = cudaMalloc(&p, n * sizeof(T));
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            if (release_spare_slabs()) e = cudaMalloc(&p, n * sizeof(T));
-        }
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            throw std::bad_alloc();
-        }
-        ptrs.push_back(p);
-        return static_cast<T *>(p);
-    }
-    void release() {
-        for (void *p : ptrs) cudaFree(p);
-        ptrs.clear();
-    }
-    ~Mem() { release(); }
 };
 
 void check(cudaError_t e, const char *where);   // throws CudaError on failure
