@@ -135,7 +135,10 @@ typedef struct {
                                  density's error is that of float64 sums or below at every
                                  point; the integrals' is that of float64 sums of the tiles'
                                  largest |chi| times largest |V phi|: relative to these, not to
-                                 an entry that is far smaller.
+                                 an entry that is far smaller. Its tables take 36 bytes per
+                                 tabulated chi value (and padding) beside the 8 of the value;
+                                 where they would take more than half of the free memory, the
+                                 contractions run on the CUDA cores.
                                  TDDFT_MIXED: matrices, grids and FFTs in float32; traces,
                                  line search, Gram-Schmidt, eigenvalues in float64 */
     int32_t mode;             /* TDDFT_MODE_FULL (Eq. operator_RPA); TDDFT_MODE_TDA (B = 0:

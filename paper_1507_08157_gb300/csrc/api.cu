@@ -1442,7 +1442,7 @@ void build_impl(tddft_ctx *c, const tddft_system *s, const tddft_sparse_system *
             check(cudaMemcpy(I->poff_h.data(), I->phi.off, (ntl + 1) * sizeof(int), cudaMemcpyDeviceToHost), "D2H off");
             I->quads_ok = c->nv % 4 == 0 && phi_lists_in_quads(*I);
             I->int64_tc = fp64_grid_build(st, I->mem, I->chi, I->phi, I->coff_h, I->poff_h, I->quads_ok, I->g64);
-            I->dens64_tc = I->int64_tc && I->quads_ok;
+            I->dens64_tc = I->int64_tc && I->g64.pm;
         }
     }
     double pp = 0.0, tv = 0.0;

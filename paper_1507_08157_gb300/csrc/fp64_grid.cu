@@ -748,10 +748,13 @@ void max64(cudaStream_t st, const double *x, long long len, int rows, unsigned l
 
 }  // namespace
 
-// Digit tables and lists of a context: coff, poff, pids on the host as on the device. False (and
-// nothing made) when a tile's TMA rows would not fit 31 bits.
-bool fp64_grid_build(cudaStream_t st, Mem &mem, const TileSet<double> &chi, const TileSet<double> &phi,
-                     const std::vector<int> &coff, const std::vector<int> &poff, bool quads, Fp64Grid &G) {
+// Digit tables and lists of a context: coff, poff on the host as on the device. False (and nothing made)
+// when a tile's TMA rows would not fit 31 bits, a table holds values beyond any orbital's, or the tables
+// would take more than half of the free memory: the contractions then run on the CUDA cores, as
+// they did where only the float64 tables fit. G.pm is null where the density's do not fit beside
+// the integrals'.
+bool fp64_grid_build(cudaStream_t st, Mem &out, const TileSet<double> &chi, const TileSet<double> &phi,
+                     const std::vector<int> &coff, const std::vector<int> &poff, bool quads, Fp64Grid &result) try {
     const int ntl = chi.ntiles;
     const long long slots = coff[ntl], values = slots * TILE_PTS;
     std::vector<int> tiles, first(ntl + 1, 0), ct, cj;
@@ -773,6 +776,18 @@ bool fp64_grid_build(cudaStream_t st, Mem &mem, const TileSet<double> &chi, cons
                (long long)(coff[b + 1] - coff[b]) * (poff[b + 1] - poff[b]);
     });
     const long long pslots = poff[ntl];
+    // 18 bytes per chi value function-major, as many and the padding point-major, 2 per phi value
+    const size_t fm_bytes = (size_t)ND * values * 2 + (size_t)pslots * TILE_PTS * 2;
+    const size_t pm_bytes = quads ? (size_t)ND * nchunks * TILE_PTS * 64 * 2 + (size_t)ntl * TILE_PTS * 4 : 0;
+    size_t room = 0, total = 0;
+    if (cudaMemGetInfo(&room, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (fm_bytes > room / 2) return false;
+    const bool make_pm = quads && fm_bytes + pm_bytes <= room / 2;
+    Mem mem;
+    Fp64Grid G;
     unsigned long long *bits = mem.alloc<unsigned long long>(2), h[2];
     max64(st, chi.val, values, 1, bits);
     max64(st, phi.val, pslots * TILE_PTS, 1, bits + 1);
@@ -801,7 +816,7 @@ bool fp64_grid_build(cudaStream_t st, Mem &mem, const TileSet<double> &chi, cons
     check_launch("chi_digits_fm_kernel");
     G.items = up(items);
     G.nitems = (long long)items.size();
-    if (quads) {
+    if (make_pm) {
         G.nchunks = nchunks;
         G.pm = mem.alloc<unsigned short>((size_t)ND * nchunks * TILE_PTS * 64);
         Mem tmp;
@@ -820,7 +835,12 @@ bool fp64_grid_build(cudaStream_t st, Mem &mem, const TileSet<double> &chi, cons
         G.covers = G.ntiles == ntl;
         G.pslots = pslots;
     }
+    out.ptrs.insert(out.ptrs.end(), mem.ptrs.begin(), mem.ptrs.end());
+    mem.ptrs.clear();
+    result = G;
     return true;
+} catch (const std::bad_alloc &) {
+    return false;
 }
 
 // rho [k][n^3] of P [k][nchi][nphi] (16-byte aligned rows); exps: k (pslots + ntiles) words

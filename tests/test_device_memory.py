@@ -72,3 +72,42 @@ def test_sources_allocate_through_the_helper():
         text = open(os.path.join(CSRC, f)).read()
         calls = text.count("cudaMalloc(")
         assert calls == (2 if f == "device_memory.h" else 1 if f == "tc_gemm.cu" else 0), f
+
+
+BUILD = """
+#include "tddft_internal.h"
+#include <cstdio>
+namespace tddft {
+bool fp64_grid_build(cudaStream_t st, Mem &mem, const TileSet<double> &chi, const TileSet<double> &phi,
+                     const std::vector<int> &coff, const std::vector<int> &poff, bool quads, Fp64Grid &G);
+}
+extern "C" {                       // for Mem's inline parts here; the library has its own runtime
+cudaError_t cudaFree(void *) { return cudaSuccess; }
+cudaError_t cudaMalloc(void **, size_t) { return cudaErrorMemoryAllocation; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+}
+int main() {
+    using namespace tddft;
+    TileSet<double> chi{}, phi{};
+    chi.ntiles = phi.ntiles = 1;
+    Mem mem;
+    Fp64Grid G;
+    const bool made = fp64_grid_build(nullptr, mem, chi, phi, {0, 8}, {0, 4}, true, G);
+    return made || !mem.ptrs.empty() || G.fm || G.pm;
+}
+"""
+
+
+def test_float64_digit_tables_that_do_not_fit_leave_the_other_kernels(tmp_path):
+    # without a device every allocation fails: no tables, and no error that would refuse the context
+    gxx, inc = shutil.which("g++"), "/usr/local/cuda/include"
+    if not gxx or not os.path.isdir(inc):
+        pytest.skip("no g++ or CUDA headers")
+    from paper_1507_08157_gb300 import build
+    lib = build.build()
+    (tmp_path / "build.cpp").write_text(BUILD)
+    exe = str(tmp_path / "build")
+    subprocess.run([gxx, "-std=c++17", "-I", inc, "-I", CSRC, str(tmp_path / "build.cpp"), lib, "-o", exe], check=True)
+    env = dict(os.environ, CUDA_VISIBLE_DEVICES="", LD_LIBRARY_PATH=os.path.dirname(lib))
+    res = subprocess.run([exe], capture_output=True, text=True, env=env)
+    assert res.returncode == 0, (res.returncode, res.stderr)
