@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(BT_THREADS, 1) bsr_tc_kernel(
                 for (int q = 0; q < nsl; ++q, ++it) {
                     const int s = (int)(it % BT_STAGES);
                     const unsigned par = (unsigned)((it / BT_STAGES) & 1);
-                    if (!mbar_wait(&ctl->full[s], par, abort, wlim)) {
+                    if (!mbar_wait_warp(&ctl->full[s], par, abort, wlim)) {
                         go = false;
                         break;
                     }
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(BT_THREADS, 1) bsr_tc_kernel(
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++tcount) {
             const int oi = t % nout, b = t / nout, o = out[oi];
             const int buf = tcount & 1, use = tcount >> 1;
-            if (!mbar_wait(&ctl->acc_full[buf], (unsigned)(use & 1), abort, wlim)) break;
+            if (!mbar_wait_warp(&ctl->acc_full[buf], (unsigned)(use & 1), abort, wlim)) break;
             tc_fence_after();
             float *Cb = C + (long long)b * sC + (long long)o * CB_SIZE + (long long)(warp * 32) * CB_C;
             const float *mb = mask ? mask + (long long)o * CB_SIZE + (long long)(warp * 32) * CB_C : nullptr;

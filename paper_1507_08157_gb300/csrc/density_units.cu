@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(DU_THREADS, 1) density_units_kernel(
                                 const uint2 y1 = (id >= 0 && r1 >= 0) ? __ldg(Pl + (r1 + id)) : make_uint2(0u, 0u);
                                 v[j] = make_uint4(y0.x, y0.y, y1.x, y1.y);
                             }
-                            if (buse > 0) ok = mbar_wait(&ctl->b_empty[bi], (buse - 1) & 1, abort, wlim);
+                            if (buse > 0) ok = mbar_wait_warp(&ctl->b_empty[bi], (buse - 1) & 1, abort, wlim);
                             if (ok)
 #pragma unroll
                                 for (int j = 0; j < 8; ++j)
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(DU_THREADS, 1) density_units_kernel(
                                 const int row = __shfl_sync(0xffffffffu, qr, h * 8 + j);
                                 v[j] = (id >= 0 && row >= 0) ? __ldg(Ps + (row + id)) : make_uint4(0u, 0u, 0u, 0u);
                             }
-                            if (h == 0 && buse > 0 && !mbar_wait(&ctl->b_empty[bi], (buse - 1) & 1, abort, wlim)) {
+                            if (h == 0 && buse > 0 && !mbar_wait_warp(&ctl->b_empty[bi], (buse - 1) & 1, abort, wlim)) {
                                 ok = false;
                                 break;
                             }
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(DU_THREADS, 1) density_units_kernel(
                         t1 = *o1 * scale[s1];
                     }
                     const float inv0 = scale[k + s0], inv1 = scale[k + s1];
-                    ok = mbar_wait(&ctl->acc_full[grp], uses & 1, abort, wlim) && !*abort;
+                    ok = __all_sync(0xffffffffu, mbar_wait(&ctl->acc_full[grp], uses & 1, abort, wlim) && !*abort);
                     ++uses;
                     tc_fence_after();
                     if (!ok) break;

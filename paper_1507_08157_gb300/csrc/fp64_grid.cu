@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(THREADS64, 1) integrals64_kernel(
                 u[2 * e] = biased(scaled(p.x) * v.x);
                 u[2 * e + 1] = biased(scaled(p.y) * v.y);
             }
-            if (kb >= 2 && !mbar_wait(&ctl->b_empty[kb & 1], ((kb >> 1) - 1) & 1, abort, wlim)) {
+            if (kb >= 2 && !mbar_wait_warp(&ctl->b_empty[kb & 1], ((kb >> 1) - 1) & 1, abort, wlim)) {
                 ok = false;
                 break;
             }
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(THREADS64, 1) integrals64_kernel(
             __syncwarp();
             if (lane == 0) mbar_arrive(&ctl->b_full[kb & 1]);
         }
-        ok = ok && mbar_wait(&ctl->acc_full, 0, abort, wlim) && !*abort;
+        ok = ok && __all_sync(0xffffffffu, mbar_wait(&ctl->acc_full, 0, abort, wlim) && !*abort);
         tc_fence_after();
         // rows of chi over warps 0-3 and 4-7, the phi halves between the two groups
         const int a = (warp & 3) * 32 + lane;
@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(THREADS64, 1) density64_kernel(
             }
             for (int z = 0; z < NZ && ok; ++z, ++acc) {
                 for (int kb = z * ZB; kb < min(KB, (z + 1) * ZB); ++kb, ++qb) {
-                    if (qb >= 2 && !mbar_wait(&ctl->b_empty[qb & 1], ((qb >> 1) - 1) & 1, abort, wlim)) {
+                    if (qb >= 2 && !mbar_wait_warp(&ctl->b_empty[qb & 1], ((qb >> 1) - 1) & 1, abort, wlim)) {
                         ok = false;
                         break;
                     }
@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(THREADS64, 1) density64_kernel(
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&ctl->b_full[qb & 1]);
                 }
-                ok = ok && mbar_wait(&ctl->acc_full, acc & 1, abort, wlim) && !*abort;
+                ok = ok && __all_sync(0xffffffffu, mbar_wait(&ctl->acc_full, acc & 1, abort, wlim) && !*abort);
                 tc_fence_after();
                 if (!ok) break;
                 for (int c = hb * 16; c < hb * 16 + 16 && c < nb; c += 8) {

@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(DENS_THREADS, 1) density_tc_kernel(
         const int send = aligned ? (eg ? gs : gsplit) : (eg ? 0 : gs);
         for (int pb = 0; pb < TILE_PTS / 128; ++pb) {
             const int acc = pb & 1;
-            const bool ok = mbar_wait(&ctl->acc_full[acc], (pb >> 1) & 1, abort, wlim) && !*abort;
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(&ctl->acc_full[acc], (pb >> 1) & 1, abort, wlim) && !*abort);
             tc_fence_after();
             const int lp = pb * 128 + quarter * 32 + lane;
             float r[16];
@@ -636,7 +636,7 @@ __global__ void __launch_bounds__(192, 3) integrals_tc_kernel(
         // then the epilogue
         for (int kb = 0; kb < KS; ++kb) {
             const int st = kb & 1, use = kb >> 1;
-            if (!mbar_wait(&ctl->x_full[st], use & 1, abort, wlim)) break;
+            if (!mbar_wait_warp(&ctl->x_full[st], use & 1, abort, wlim)) break;
             unsigned char *W = Ws + (size_t)st * NB * 128;
             for (int idx = threadIdx.x; idx < np * 8; idx += 128) {
                 const int row = idx >> 3, c8 = idx & 7;
@@ -655,7 +655,7 @@ __global__ void __launch_bounds__(192, 3) integrals_tc_kernel(
             fence_async_smem();
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&ctl->w_ready[st])) : "memory");
         }
-        const bool ok = mbar_wait(&ctl->acc_done, 0, abort, wlim) && !*abort;
+        const bool ok = __all_sync(0xffffffffu, mbar_wait(&ctl->acc_done, 0, abort, wlim) && !*abort);
         tc_fence_after();
         const float f = dV / vs;
         for (int mb = 0; mb < MB; ++mb) {

@@ -200,8 +200,7 @@ __global__ void __launch_bounds__(IU_THREADS, 1) integrals_units_kernel(
         // producer of slice `warp`: lane = octet of points (lane & 7) and phi rows (lane >> 3) + 4 i
         const int o = lane & 7, r = lane >> 3;
         unsigned j = 0;
-        bool ok = true;
-        for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x) {
+        for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
             const IItem d = list[it / groups];
             const int mp = (d.np + pch - 1) / pch;
             int q0, q1;
@@ -209,7 +208,7 @@ __global__ void __launch_bounds__(IU_THREADS, 1) integrals_units_kernel(
             const int gx = d.t / (nt * nt) * TILE + warp, gy = (d.t / nt) % nt * TILE + o, gz = d.t % nt * TILE;
             const bool row_in = gx < n && gy < n;
             const float *vp = V + ((long long)gx * n + gy) * n + gz;
-            for (int y = 0; y < mp && ok; ++y) {
+            for (int y = 0; y < mp; ++y) {
                 int b0, nb;
                 phi_chunk(d.np, mp, y, b0, nb);
                 const int NB = (nb + 15) / 16 * 16;
@@ -230,10 +229,9 @@ __global__ void __launch_bounds__(IU_THREADS, 1) integrals_units_kernel(
                     const float c0 = v_scale(bits[s0]), c1 = v_scale(bits[s1]);
 #pragma unroll
                     for (int e = 0; e < 8; ++e) v0[e] *= c0, v1[e] *= c1;
-                    if (j > 0 && !mbar_wait(&ctl->w_empty[warp], (j - 1) & 1, abort, wlim)) {
-                        ok = false;
-                        break;
-                    }
+                    // after an abort the warp walks on to the end without waiting: its stores stay inside the
+                    // stage, and nothing reads them (leaving the loop by a vote of the lanes took 4 % of the kernel)
+                    if (j > 0) mbar_wait(&ctl->w_empty[warp], (j - 1) & 1, abort, wlim);
                     unsigned char *w = W + warp * W_STAGE;
 #pragma unroll
                     for (int i = 0; i < IU_PHI / 4; ++i) {
@@ -279,7 +277,7 @@ __global__ void __launch_bounds__(IU_THREADS, 1) integrals_units_kernel(
                 for (int q = q0; q < q1; ++q, ++j) {
                     if ((j & 1) != grp) continue;
                     const unsigned acc = j & 3;
-                    ok = mbar_wait(&ctl->acc_full[acc], (j >> 2) & 1, abort, wlim) && !*abort;
+                    ok = __all_sync(0xffffffffu, mbar_wait(&ctl->acc_full[acc], (j >> 2) & 1, abort, wlim) && !*abort);
                     tc_fence_after();
                     if (!ok) break;
                     const unsigned ta = tmem + acc * 128 + ((unsigned)((warp & 3) * 32) << 16);

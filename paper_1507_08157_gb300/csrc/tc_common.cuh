@@ -53,6 +53,13 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long *b, unsigned parity
     return true;
 }
 
+// The same for the lanes of a converged warp, which then meet at warp-wide instructions: the whole warp
+// goes on or none of it, though lanes may read the clock and the abort word at different times.
+__device__ __forceinline__ bool mbar_wait_warp(unsigned long long *b, unsigned parity, volatile int *abort,
+                                               long long limit) {
+    return __all_sync(0xffffffffu, mbar_wait(b, parity, abort, limit));
+}
+
 // teardown after an abort: wait, again bounded, for the phase `parity` of b to complete whatever
 // the abort flag says, so that a copy or an MMA this thread started lands before the block exits
 __device__ __forceinline__ void mbar_drain(unsigned long long *b, unsigned parity, long long limit) {

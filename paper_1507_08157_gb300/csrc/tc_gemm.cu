@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(
                 for (int kb = 0; kb < nk; ++kb, ++it) {
                     const int s = (int)(it % S);
                     const unsigned par = (unsigned)((it / S) & 1);
-                    if (!mbar_wait(&ctl->full[s], par, abort, wlim)) {
+                    if (!mbar_wait_warp(&ctl->full[s], par, abort, wlim)) {
                         go = false;
                         break;
                     }
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(
         int tcount = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++tcount) {
             const int buf = tcount & 1, use = tcount >> 1;
-            if (!mbar_wait(&ctl->acc_full[buf], (unsigned)(use & 1), abort, wlim)) break;
+            if (!mbar_wait_warp(&ctl->acc_full[buf], (unsigned)(use & 1), abort, wlim)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int n0 = (t % tn) * TN, m0 = ((t / tn) % tm) * TBM, b = t / (tn * tm);
             float *Cb = C + (long long)b * sC;
@@ -390,13 +390,13 @@ __global__ void __launch_bounds__(XGEMM_THREADS, 1) tc_gemm_x_kernel(
         for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++tcount) {
             const int buf = tcount & 1, use = tcount >> 1;
             // the whole warp goes on or none of it
-            if (!__all_sync(0xffffffffu, mbar_wait(&ctl->acc_empty[buf], (unsigned)((use & 1) ^ 1), abort, wlim))) break;
+            if (!mbar_wait_warp(&ctl->acc_empty[buf], (unsigned)((use & 1) ^ 1), abort, wlim)) break;
             const unsigned acc_t = tmem + (unsigned)(buf * ACC);
             for (int kb = 0; kb < nk; ++kb, ++it) {
                 const int s = (int)(it % XS);
                 // (one term: W is used as it landed)
-                ok = __all_sync(0xffffffffu, (SPLIT || mbar_wait(&ctl->full[s], (unsigned)((it / XS) & 1), abort, wlim)) &&
-                                                 mbar_wait(&ctl->ready[s], (unsigned)((it / XS) & 1), abort, wlim));
+                ok = (SPLIT || mbar_wait_warp(&ctl->full[s], (unsigned)((it / XS) & 1), abort, wlim)) &&
+                     mbar_wait_warp(&ctl->ready[s], (unsigned)((it / XS) & 1), abort, wlim);
                 if (!ok) break;
                 tc_fence_after();
                 if (elect_one()) {
@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(XGEMM_THREADS, 1) tc_gemm_x_kernel(
                 if ((int)(it & 1) != group) continue;
                 const int s = (int)(it % XS);
                 // the stores into TMEM are for the whole warp: it goes on or none of it
-                go = __all_sync(0xffffffffu, mbar_wait(&ctl->full[s], (unsigned)((it / XS) & 1), abort, wlim));
+                go = mbar_wait_warp(&ctl->full[s], (unsigned)((it / XS) & 1), abort, wlim);
                 if (!go) break;
                 unsigned char *st = tiles + (size_t)s * X_STAGE_BYTES;
                 tc_fence_after();      // the stage's last MMAs are done: their completion came before the load
@@ -497,8 +497,7 @@ __global__ void __launch_bounds__(XGEMM_THREADS, 1) tc_gemm_x_kernel(
         int tcount = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++tcount) {
             const int buf = tcount & 1, use = tcount >> 1;
-            const bool full = mbar_wait(&ctl->acc_full[buf], (unsigned)(use & 1), abort, wlim);
-            if (!__all_sync(0xffffffffu, full)) break;
+            if (!mbar_wait_warp(&ctl->acc_full[buf], (unsigned)(use & 1), abort, wlim)) break;
             tc_fence_after();
             int l0, c0, b;
             tile(t, l0, c0, b);
