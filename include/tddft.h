@@ -266,7 +266,8 @@ tddft_status tddft_fxc(tddft_ctx *ctx, double *fxc);
  *     most chi_chunk x phi_chunk functions of a tile (kind 1; chi 128 or 256, phi 32 or 64);
  *   potential_integrals: chunks of at most 128 chi x phi_chunk (32, 48) where every tile's phi
  *     list is whole aligned quads, else units of at most chi_chunk (128, 256, 384) x phi_chunk
- *     (32, 64, 128).
+ *     (32, 64, 128). With k = 1 and such lists also units of 256 or 384 chi: the choice between
+ *     the two is kept for calls of one state, the chunks only where they won.
  * Each candidate runs once to warm up and three times timed with CUDA events on the context's
  * stream (ms = the mean). The fastest of each stage is installed and kept by the context for all
  * later calls (chosen = 1). out receives up to cap entries, count the number of candidates.

@@ -2984,7 +2984,10 @@ tddft_status tddft_autotune(tddft_ctx *c, int32_t k, tddft_tuning_entry *out, in
             const int cuts[][2] = {{384, 128}, {256, 128}, {128, 128}, {384, 64}, {256, 64}, {128, 64}, {384, 32}};
             int best = -1;
             double best_ms = 1e300;
+            const int items_pch = I.int_pch;
             if (I.int_quads) {
+                // the items themselves, also of one state (which may be routed to the units)
+                if (k == 1) I.int_single = false;
                 for (const int pch : {48, 32}) {
                     set_integrals_items(I, pch);
                     add("potential_integrals", 1, 128, pch, time_it([&]() { integrals(c, I, k); }));
@@ -2994,8 +2997,12 @@ tddft_status tddft_autotune(tddft_ctx *c, int32_t k, tddft_tuning_entry *out, in
                     }
                 }
             }
+            // units: for lists that are not whole quads, and for one state (wider than the items' 128 chi, so
+            // that a row says which kernel it is)
             for (const auto &cut : cuts) {
-                if (I.int_quads || !set_integrals_units(I, cut[0], cut[1])) continue;
+                if (I.int_quads && (k > 1 || cut[0] == 128)) continue;
+                if (!set_integrals_units(I, cut[0], cut[1])) continue;
+                if (I.int_quads) I.int_single = true;
                 add("potential_integrals", 1, cut[0], cut[1], time_it([&]() { integrals(c, I, k); }));
                 if (rows.back().ms < best_ms) {
                     best_ms = rows.back().ms;
@@ -3004,8 +3011,10 @@ tddft_status tddft_autotune(tddft_ctx *c, int32_t k, tddft_tuning_entry *out, in
             }
             if (best >= 0) {
                 rows[best].chosen = 1;
-                if (I.int_quads) set_integrals_items(I, rows[best].phi_chunk);
-                else set_integrals_units(I, rows[best].chi_chunk, rows[best].phi_chunk);
+                const bool items = I.int_quads && rows[best].chi_chunk == 128;
+                if (I.int_quads) set_integrals_items(I, items ? rows[best].phi_chunk : items_pch);
+                if (!items) set_integrals_units(I, rows[best].chi_chunk, rows[best].phi_chunk);
+                if (I.int_quads && k == 1) I.int_single = !items;
             }
         }
         check_tc_error(c);
