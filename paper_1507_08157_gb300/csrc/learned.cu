@@ -79,28 +79,42 @@ __global__ void row_weights_kernel(const float *__restrict__ s, long long per, f
 
 // Column sums out[j] = sum_r D[r][j], the bias gradients. Bound by reading D once (67 MB for the
 // last layer at 16384 rows, 10 us at the HBM rate); one thread per column walking all rows kept 8
-// blocks busy and took 5.5 ms for the
-// three layers, this 0.1 ms. Blocks of 128 columns x 4 row phases over row
-// slices; each thread keeps a compensated float32 pair (Knuth's two-sum: the pair carries 48
-// bits, where float64 adds, scarce on this part, would bound the loop), the phases and slices are
-// added in float64 in a fixed order.
+// blocks busy and took 5.5 ms for the three layers, this 0.1 ms. Blocks of 128 columns x 4 row phases
+// over row slices; each thread keeps an unevaluated sum of three float32 (Knuth's two-sum twice: more
+// than the 53 bits of a float64 sum, whose adds, scarce on this part, would bound the loop) and falls back
+// on float64 where float32 overflows on the way; the phases and slices are added in float64 in a
+// fixed order.
 constexpr int CS_COLS = 128, CS_PH = 4;
 __global__ void __launch_bounds__(CS_COLS * CS_PH) colsum_part_kernel(const float *__restrict__ D, long long n, int w,
                                                                       long long per, double *__restrict__ part) {
     __shared__ double red[CS_PH][CS_COLS];
     const int j = blockIdx.x * CS_COLS + threadIdx.x;
     const long long r0 = blockIdx.y * per, r1 = r0 + per < n ? r0 + per : n;
-    float s = 0.0f, c = 0.0f;
-    if (j < w) {
-#pragma unroll 8
-        for (long long r = r0 + threadIdx.y; r < r1; r += CS_PH) {
-            const float x = D[r * w + j];
-            const float t = s + x, z = t - s;
-            c += (s - (t - z)) + (x - z);
-            s = t;
-        }
+    // a + b -> a, its rounding error returned
+    auto two_sum = [](float &a, float b) {
+        const float t = a + b, z = t - a, e = (a - (t - z)) + (b - z);
+        a = t;
+        return e;
+    };
+    float s = 0.0f, c = 0.0f, e = 0.0f;
+    const int step = CS_PH * w;
+    const float *const first = D + (r0 + threadIdx.y) * w + j, *p = first;
+    const int rows = j < w ? (int)((r1 - r0 - threadIdx.y + CS_PH - 1) / CS_PH) : 0;
+    int left = rows;
+    for (; left >= 8; left -= 8, p += 8 * step) {
+        float x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = p[u * step];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) e += two_sum(c, two_sum(s, x[u]));
     }
-    red[threadIdx.y][threadIdx.x] = isfinite(s) ? (double)s + (double)c : (double)s;   // inf: its error term is NaN
+    for (; left > 0; --left, p += step) e += two_sum(c, two_sum(s, *p));
+    double sum = (double)s + ((double)c + (double)e);
+    if (!isfinite(s)) {
+        sum = 0.0;
+        for (int r = 0; r < rows; ++r) sum += (double)first[(long long)r * step];
+    }
+    red[threadIdx.y][threadIdx.x] = sum;
     __syncthreads();
     if (threadIdx.y == 0 && j < w) {
         double v = 0.0;
@@ -108,11 +122,19 @@ __global__ void __launch_bounds__(CS_COLS * CS_PH) colsum_part_kernel(const floa
         part[(long long)blockIdx.y * w + j] = v;
     }
 }
-__global__ void colsum_final_kernel(const double *__restrict__ part, int slices, int w, float *__restrict__ out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= w) return;
+// 32 columns a block, the slices over eight warps (in one thread per column the float64 adds followed one
+// another: 5.9 and 2 us)
+__global__ void __launch_bounds__(256) colsum_final_kernel(const double *__restrict__ part, int slices, int w,
+                                                           float *__restrict__ out) {
+    __shared__ double red[8][33];
+    const int j = blockIdx.x * 32 + threadIdx.x;
     double s = 0.0;
-    for (int q = 0; q < slices; ++q) s += part[(long long)q * w + j];
+    if (j < w)
+        for (int q = threadIdx.y; q < slices; q += 8) s += part[(long long)q * w + j];
+    red[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y != 0 || j >= w) return;
+    for (int q = 1; q < 8; ++q) s += red[q][threadIdx.x];
     out[j] = (float)s;
 }
 
@@ -366,15 +388,15 @@ void ensure_rows(tddft_mlp *m, long long rows) {
 }
 
 // out = column sums of D [n][w]; scratch (gram_scratch_doubles(64, 32) doubles) holds the slices' sums.
-// At least 64 rows per thread so that the partial sums stay a small part of the reads.
+// At least 32 rows per thread so that the partial sums stay a small part of the reads.
 void colsum(cudaStream_t st, const float *D, long long n, int w, float *out, double *scratch) {
     const long long fit = gram_scratch_doubles(64, 32) / w;
-    const long long slices = std::max<long long>(1, std::min({(n + 64 * CS_PH - 1) / (64 * CS_PH), fit, 512LL}));
+    const long long slices = std::max<long long>(1, std::min({(n + 32 * CS_PH - 1) / (32 * CS_PH), fit, 512LL}));
     const long long per = (n + slices - 1) / slices;
     const int used = (int)((n + per - 1) / per);
     colsum_part_kernel<<<dim3((w + CS_COLS - 1) / CS_COLS, used), dim3(CS_COLS, CS_PH), 0, st>>>(D, n, w, per, scratch);
     check_launch("colsum_part");
-    colsum_final_kernel<<<(w + 127) / 128, 128, 0, st>>>(scratch, used, w, out);
+    colsum_final_kernel<<<(w + 31) / 32, dim3(32, 8), 0, st>>>(scratch, used, w, out);
     check_launch("colsum_final");
 }
 
