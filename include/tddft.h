@@ -263,7 +263,9 @@ tddft_status tddft_fxc(tddft_ctx *ctx, double *fxc);
  * TDDFT_MIXED context it times, on k trial states of the context's own system (deterministic
  * pseudo-random P and V), every candidate cut of the grid work into tensor-core units:
  *   response_density: the per-tile kernels (kind 0, when every tile fits them) and units of at
- *     most chi_chunk x phi_chunk functions of a tile (kind 1; chi 128 or 256, phi 32 or 64);
+ *     most chi_chunk x phi_chunk functions of a tile (kind 1; chi 128 or 256, phi 32 or 64). With
+ *     k = 1 on lists past the per-tile kernels' also 320 x 128, which streams chi: that choice is
+ *     kept for calls of one state, the others only where they won;
  *   potential_integrals: chunks of at most 128 chi x phi_chunk (32, 48) where every tile's phi
  *     list is whole aligned quads, else units of at most chi_chunk (128, 256, 384) x phi_chunk
  *     (32, 64, 128). With k = 1 and such lists also units of 256 or 384 chi: the choice between

@@ -259,8 +259,12 @@ struct Impl {
     unsigned short *chi_pmc = nullptr, *phi_pmc = nullptr;
     long long nchunks_chi = 0;
     DUnitList dunits;
+    // one state on the chi streaming kernel (lists past the per-tile kernels'), its units
+    bool dens_single = false;
+    const DUnit *sunits = nullptr;
+    int nsunits = 0;
     std::vector<int> coff_h, poff_h, cfirst_h, pfirst_h;    // host tile offsets, first chunks
-    Mem umem_dens, umem_int, umem_iu;              // unit lists (replaced when the autotuner recuts)
+    Mem umem_dens, umem_ds, umem_int, umem_iu;     // unit lists (replaced when the autotuner recuts)
     unsigned short *P16 = nullptr;        // float16 copy of P for the units' gather (workspace)
     int CK = 0, NPmax = 0, nslots_chi = 0, nslots_phi = 0, maxc = 0;
     int NPint = 0;            // phi rows of the integrals' B stage (the largest unit's phi, to 16)
@@ -496,6 +500,10 @@ void response_density_units(cudaStream_t st, const GridShape &g, const TileSet<f
                             const unsigned short *chi_pmc, long long nchunks_chi, const unsigned short *phi_pmc,
                             const DUnitList &ul, int nchi, int nphi, const float *P, long long sP, int k, float *rho,
                             unsigned short *P16, unsigned *bits, float *scale, int *err);
+void response_density_stream(cudaStream_t st, const GridShape &g, const TileSet<float> &chi, const TileSet<float> &phi,
+                             const unsigned short *chi_pmc, long long nchunks_chi, const unsigned short *phi_pmc,
+                             const DUnit *units, int nunits, int nphi, const float *P, long long sP, int k, float *rho,
+                             unsigned *bits, int *err);
 void potential_integrals_units(cudaStream_t st, const GridShape &g, const TileSet<float> &chi, const TileSet<float> &phi,
                                const unsigned short *chi_fm16, int nslots, const unsigned short *phi_fm16,
                                const IItem *list, int nlist, int pch, int nchi, int nphi, const float *V, int k,
@@ -853,6 +861,11 @@ void density(tddft_ctx *c, Impl<T> &I, const T *P, int ns) {
         P = I.dense;
     }
     if constexpr (sizeof(T) == 4) {
+        if (I.dens_units && ns == 1 && I.dens_single) {
+            response_density_stream(c->st, c->grid(), I.chi, I.phi, I.chi_pmc, I.nchunks_chi, I.phi_pmc, I.sunits, I.nsunits,
+                                    c->nv, P, (long long)c->nc * c->nv, ns, I.rho, I.tc_bits, tc_error_word());
+            return;
+        }
         if (I.dens_units) {
             response_density_units(c->st, c->grid(), I.chi, I.phi, I.chi_pmc, I.nchunks_chi, I.phi_pmc, I.dunits, c->nc,
                                    c->nv, P, (long long)c->nc * c->nv, ns, I.rho, I.P16, I.tc_bits, I.tc_scale,
@@ -1235,10 +1248,31 @@ void set_density_units(Impl<float> &I, int cch, int pch) {
         check(cudaMemcpy(di, sorted.data(), sorted.size() * sizeof(DItem), cudaMemcpyHostToDevice), "upload density items");
     }
     std::swap(I.umem_dens.ptrs, m.ptrs);
+    L.cut[0] = cch;
+    L.cut[1] = pch;
     L.units = du;
     L.items = di;
     L.nitems = (int)sorted.size();
     L.covers = live == ntl;
+}
+
+// the streaming density's units: at most 320 chi and 128 phi of a tile
+void set_density_stream(Impl<float> &I) {
+    if (I.sunits) return;
+    const std::vector<int> &coff = I.coff_h, &poff = I.poff_h;
+    std::vector<DUnit> us;
+    for (int t = 0; t < I.chi.ntiles; ++t) {
+        const int nct = coff[t + 1] - coff[t], npt = poff[t + 1] - poff[t];
+        for (int cc = 0; cc < nct; cc += 320)
+            for (int pc = 0; pc < npt; pc += 128)
+                us.push_back(DUnit{t, coff[t] + cc, std::min(320, nct - cc), poff[t] + pc, std::min(128, npt - pc),
+                                   I.cfirst_h[t] + cc / 64, I.pfirst_h[t] + pc / 32, 0});
+    }
+    DUnit *d = I.umem_ds.alloc<DUnit>(us.size());
+    if (!us.empty())
+        check(cudaMemcpy(d, us.data(), us.size() * sizeof(DUnit), cudaMemcpyHostToDevice), "upload density stream units");
+    I.sunits = d;
+    I.nsunits = (int)us.size();
 }
 
 // the integrals' items: each tile in chunks of 128 chi with all its phi, which the kernel takes in
@@ -1389,6 +1423,11 @@ void build_impl(tddft_ctx *c, const tddft_system *s, const tddft_sparse_system *
                 if (!per_tile && !(nu && nu[0] == '1') && c->nv % 4 == 0 && build_density_chunks(c, *I)) {
                     set_density_units(*I, 256, 64);
                     I->dens_units = true;
+                    // figures in density_units.cu
+                    if (I->dunits.adds) {
+                        set_density_stream(*I);
+                        I->dens_single = true;
+                    }
                 }
             }
             // integrals: units of at most 384 chi and 128 phi slots of one tile (a denser tile is
@@ -2949,6 +2988,7 @@ tddft_status tddft_autotune(tddft_ctx *c, int32_t k, tddft_tuning_entry *out, in
         // response density: the per-tile kernels (when every tile fits them) and units of each cut
         {
             const bool units_possible = c->nv % 4 == 0 && build_density_chunks(c, I);
+            const int dens_cut[2] = {I.dunits.cut[0], I.dunits.cut[1]};
             int best = -1;
             double best_ms = 1e300;
             if (I.grid_tc) {
@@ -2959,6 +2999,7 @@ tddft_status tddft_autotune(tddft_ctx *c, int32_t k, tddft_tuning_entry *out, in
             }
             if (units_possible) {
                 const int cuts[][2] = {{256, 64}, {128, 64}, {256, 32}, {128, 32}};
+                if (k == 1) I.dens_single = false;      // the units themselves first
                 for (const auto &cut : cuts) {
                     set_density_units(I, cut[0], cut[1]);
                     I.dens_units = true;
@@ -2969,10 +3010,23 @@ tddft_status tddft_autotune(tddft_ctx *c, int32_t k, tddft_tuning_entry *out, in
                     }
                 }
             }
+            // for one state of lists past the per-tile kernels' also the streaming kernel, in its only cut
+            const bool stream = units_possible && k == 1 && I.dunits.adds;
+            if (stream) {
+                set_density_stream(I);
+                I.dens_single = true;
+                add("response_density", 1, 320, 128, time_it([&]() { density(c, I, I.bufP, k); }));
+                if (rows.back().ms < best_ms) {
+                    best_ms = rows.back().ms;
+                    best = (int)rows.size() - 1;
+                }
+            }
             if (best >= 0) {
                 rows[best].chosen = 1;
                 if (rows[best].kind == 1) {
-                    set_density_units(I, rows[best].chi_chunk, rows[best].phi_chunk);
+                    const bool single = rows[best].chi_chunk == 320;
+                    if (k == 1) I.dens_single = single;
+                    set_density_units(I, single ? dens_cut[0] : rows[best].chi_chunk, single ? dens_cut[1] : rows[best].phi_chunk);
                     I.dens_units = true;
                 } else {
                     I.dens_units = false;

@@ -33,8 +33,7 @@
 // atoms): 5400 MMAs, 9900 warp loads of the gather and 710 accumulators per SM share 1.1 M cycles,
 // and the epilogue's path per accumulator (TMEM loads and dependent multiply-adds) is the longest.
 // A state without a partner takes half a pair's gather, MMAs and epilogue (three states of the 200
-// atoms 0.43 and 0.36 ms). One state alone uses each 128 KB of chi once and waits for it: there the
-// chi streaming kernel was faster on dense clusters (200 atoms 0.21 and 0.23, 140 atoms 0.25 and 0.21).
+// atoms 0.43 and 0.36 ms). One state of a dense cluster takes the streaming kernel at the end.
 #include "tc_common.cuh"
 #include "tddft_internal.h"
 
@@ -496,6 +495,251 @@ __global__ void __launch_bounds__(256) pack_quads_kernel(const float *__restrict
     }
 }
 
+// ---- one state on dense tiles ---------------------------------------------------------------------------
+// The kernel above keeps chi for all states, so that one state alone waits for each 128 KB of it. Where
+// lists are long (no tile's chi fit one of its accumulations) one state is faster with chi streamed:
+// units of at most 5 x 64 chi and 4 x 32 phi of a tile, each adding its part to rho with float32
+// reductions. Persistent, one block per SM over (unit, state): warp 4 brings 128 points x 64 chi at a
+// time by TMA through a ring, warp 5 issues the MMAs (M = 128 points, N = 128 phi, K = the unit's chi),
+// warps 6-7 and 12-15 gather the next item's float32 P (scaled to float16) into the other B buffer, and
+// two groups of four warps multiply their accumulator by phi. Every wait is bounded.
+// Measured (entry point with its conversions, one state, the kernel above and this): clusters at 0.1
+// atoms per A^3 with 4 + 4 functions, 200 atoms 295 and 264 us, 150 atoms 164 and 146, 110 atoms with 4 + 9 172 and 155. Not
+// so on the shorter lists of 140 atoms in the chromophore's cell (269 and 314), nor with two states.
+constexpr int DS_THREADS = 512, DS_GATHER = 192, DS_STAGES = 4;
+constexpr int DS_KB = 5, DS_NB = 128;      // chi blocks of 64 and phi of a unit
+struct __align__(8) DsShared {
+    unsigned long long a_full[DS_STAGES], a_empty[DS_STAGES];
+    unsigned long long acc_full[2], acc_empty[2];
+    unsigned long long b_full[2], b_free[2];
+    unsigned long long drain;
+    unsigned int tmem_base;
+    int abort;
+};
+
+__global__ void __launch_bounds__(DS_THREADS, 1) density_stream_kernel(
+    const __grid_constant__ CUtensorMap mX,   // [chi chunk * 512 + point][64] f16, box 64 x 128
+    int n, int nt, int k, const DUnit *__restrict__ units, int nitems, const int *__restrict__ cids,
+    const int *__restrict__ pids, int nphi, const unsigned short *__restrict__ phi_pmc,
+    const float *__restrict__ P, long long sP, const unsigned *__restrict__ bits, float *__restrict__ rho,
+    int *err, long long wlim) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *base = reinterpret_cast<unsigned char *>(
+        (reinterpret_cast<unsigned long long>(smem_raw) + 1023ull) & ~1023ull);
+    constexpr int NB = DS_NB;
+    unsigned char *A = base;                                      // ring [STAGES][128 x 128 B]
+    unsigned char *Bb = base + DS_STAGES * 16384;              // [2][DS_KB][NB x 128 B]
+    constexpr size_t bsize = (size_t)DS_KB * NB * 128;
+    DsShared *ctl = reinterpret_cast<DsShared *>(Bb + 2 * bsize);
+    volatile int *abort = &ctl->abort;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long n3 = (long long)n * n * n;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < DS_STAGES; ++i) {
+            mbar_init(&ctl->a_full[i], 1);
+            mbar_init(&ctl->a_empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&ctl->acc_full[i], 1);
+            mbar_init(&ctl->acc_empty[i], 128);
+            mbar_init(&ctl->b_full[i], DS_GATHER);
+            mbar_init(&ctl->b_free[i], 1);
+        }
+        mbar_init(&ctl->drain, 1);
+        ctl->abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 5) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
+                     "r"(256));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const unsigned tmem = ctl->tmem_base;
+
+    if (warp == 4) {
+        if (lane == 0) {
+            long long q = 0;
+            for (int it = blockIdx.x; it < nitems && !*abort; it += gridDim.x) {
+                const DUnit u = units[it / k];
+                const int KB = (u.nc + 63) / 64;
+                for (int pb = 0; pb < TILE_PTS / 128; ++pb)
+                    for (int kb = 0; kb < KB; ++kb, ++q) {
+                        const int st = (int)(q % DS_STAGES);
+                        const long long use = q / DS_STAGES;
+                        if (use > 0 && !mbar_wait(&ctl->a_empty[st], (unsigned)((use - 1) & 1), abort, wlim)) break;
+                        mbar_expect_tx(&ctl->a_full[st], 16384);
+                        tma_load_2d(A + st * 16384, &mX, &ctl->a_full[st], 0, (u.cch + kb) * TILE_PTS + pb * 128);
+                    }
+            }
+            if (*abort)
+                for (long long j = q > DS_STAGES ? q - DS_STAGES : 0; j < q; ++j)
+                    mbar_drain(&ctl->a_full[j % DS_STAGES], (unsigned)((j / DS_STAGES) & 1), wlim);
+        }
+    } else if (warp == 5) {
+        if (lane == 0) {
+            const unsigned idesc = idesc_f16(128, NB);
+            long long q = 0, pbg = 0;
+            int j = 0;
+            bool ok = true;
+            for (int it = blockIdx.x; it < nitems && ok; it += gridDim.x, ++j) {
+                const DUnit u = units[it / k];
+                const int KB = (u.nc + 63) / 64;
+                const int buf = j & 1;
+                if (!mbar_wait(&ctl->b_full[buf], (unsigned)((j >> 1) & 1), abort, wlim)) break;
+                tc_fence_after();
+                const unsigned char *B = Bb + buf * bsize;
+                for (int pb = 0; pb < TILE_PTS / 128 && ok; ++pb, ++pbg) {
+                    const int acc = (int)(pbg & 1);
+                    const long long ause = pbg >> 1;
+                    if (ause > 0 && !mbar_wait(&ctl->acc_empty[acc], (unsigned)((ause - 1) & 1), abort, wlim)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    for (int kb = 0; kb < KB; ++kb, ++q) {
+                        const int st = (int)(q % DS_STAGES);
+                        if (!mbar_wait(&ctl->a_full[st], (unsigned)((q / DS_STAGES) & 1), abort, wlim)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const unsigned a = smem_u32(A + st * 16384), bb = smem_u32(B + (size_t)kb * NB * 128);
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk)
+                            mma_f16(tmem + acc * 128, smem_desc(a + kk * 32), smem_desc(bb + kk * 32), idesc,
+                                    (kb > 0 || kk > 0) ? 1u : 0u);
+                        mma_commit(&ctl->a_empty[st]);
+                    }
+                    if (!ok) break;
+                    mma_commit(&ctl->acc_full[acc]);
+                }
+                if (!ok) break;
+                mma_commit(&ctl->b_free[buf]);
+            }
+            if (*abort) {
+                mma_commit(&ctl->drain);
+                mbar_drain(&ctl->drain, 0, wlim);
+            }
+        }
+    } else if ((warp >= 6 && warp < 8) || warp >= 12) {
+        // the P block of each item (rows = the unit's phi, K = its chi) by phi quads, zeros past
+        // the unit's counts (every row and K column of the buffer is written)
+        const int rank = (warp < 8 ? warp - 6 : warp - 10) * 32 + lane;   // warps 6, 7, 12-15: 0 .. 191
+        int j = 0;
+        for (int it = blockIdx.x; it < nitems; it += gridDim.x, ++j) {
+            const DUnit u = units[it / k];
+            const int s = it % k;
+            const int KB = (u.nc + 63) / 64;
+            const int buf = j & 1;
+            if (j >= 2 && !mbar_wait_warp(&ctl->b_free[buf], (unsigned)(((j >> 1) - 1) & 1), abort, wlim)) break;
+            unsigned char *B = Bb + buf * bsize;
+            const float sc = state_scale(bits[s]);
+            const float *Ps = P + (long long)s * sP;
+            constexpr int nq = NB / 4;
+            const int total = nq * KB * 8;
+            for (int i0 = rank; i0 < total; i0 += 2 * DS_GATHER) {
+                float4 v[2][8];
+#pragma unroll
+                for (int uu = 0; uu < 2; ++uu) {
+                    const int idx = i0 + uu * DS_GATHER;
+                    const int qd = idx % nq, ch = idx / nq;
+                    const bool live = idx < total && qd * 4 < u.np;
+                    const float *Pq = Ps + (live ? pids[u.p0 + qd * 4] : 0);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int a = (ch >> 3) * 64 + (ch & 7) * 8 + e;
+                        v[uu][e] = (live && a < u.nc)
+                                       ? __ldg(reinterpret_cast<const float4 *>(Pq + (long long)cids[u.c0 + a] * nphi))
+                                       : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    }
+                }
+#pragma unroll
+                for (int uu = 0; uu < 2; ++uu) {
+                    const int idx = i0 + uu * DS_GATHER;
+                    if (idx >= total) continue;
+                    const int qd = idx % nq, ch = idx / nq;
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        unsigned short h[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const float x = r == 0 ? v[uu][e].x : r == 1 ? v[uu][e].y : r == 2 ? v[uu][e].z : v[uu][e].w;
+                            h[e] = __half_as_ushort(__float2half_rn(x * sc));
+                        }
+                        uint4 qv;
+                        qv.x = h[0] | ((unsigned)h[1] << 16);
+                        qv.y = h[2] | ((unsigned)h[3] << 16);
+                        qv.z = h[4] | ((unsigned)h[5] << 16);
+                        qv.w = h[6] | ((unsigned)h[7] << 16);
+                        *reinterpret_cast<uint4 *>(B + (size_t)(ch >> 3) * NB * 128 + sw128_offset(qd * 4 + r, ch & 7)) = qv;
+                    }
+                }
+            }
+            fence_async_smem();
+            mbar_arrive(&ctl->b_full[buf]);
+        }
+    } else {
+        // epilogue groups: warps 0-3 accumulator 0 (even point blocks), warps 8-11 accumulator 1
+        const int eg = warp < 4 ? 0 : 1, quarter = warp & 3;
+        long long ause = 0;
+        for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+            const DUnit u = units[it / k];
+            const int s = it % k;
+            const int tx = u.t / (nt * nt), ty = (u.t / nt) % nt, tz = u.t % nt;
+            const float inv = 1.0f / state_scale(bits[s]);
+            bool stop = false;
+            for (int pb = eg; pb < TILE_PTS / 128; pb += 2, ++ause) {
+                const bool ok = __all_sync(0xffffffffu, mbar_wait(&ctl->acc_full[eg], (unsigned)(ause & 1), abort, wlim) && !*abort);
+                tc_fence_after();
+                const int lp = pb * 128 + quarter * 32 + lane;
+                float r = 0.0f;
+                if (ok) {
+                    for (int c = 0; c < u.np; c += 32) {
+                        const uint4 *q = reinterpret_cast<const uint4 *>(
+                            phi_pmc + ((long long)(u.pch + c / 32) * TILE_PTS + lp) * 32);
+                        uint4 ph[4];
+#pragma unroll
+                        for (int w = 0; w < 4; ++w) ph[w] = __ldg(q + w);
+                        float v[32];
+                        tmem_ld32(tmem + eg * 128 + ((unsigned)(quarter * 32) << 16) + (unsigned)c, v);
+#pragma unroll
+                        for (int w = 0; w < 4; ++w) {
+                            const __half2 *hh = reinterpret_cast<const __half2 *>(&ph[w]);
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const float2 f2 = __half22float2(hh[e]);
+                                r = fmaf(v[8 * w + 2 * e], f2.x, r);
+                                r = fmaf(v[8 * w + 2 * e + 1], f2.y, r);
+                            }
+                        }
+                    }
+                }
+                tc_fence_before();
+                mbar_arrive(&ctl->acc_empty[eg]);
+                if (!ok) {
+                    stop = true;
+                    break;
+                }
+                const int gx = tx * TILE + (lp >> 6), gy = ty * TILE + ((lp >> 3) & 7), gz = tz * TILE + (lp & 7);
+                if (gx < n && gy < n && gz < n)
+                    atomicAdd(rho + (long long)s * n3 + ((long long)gx * n + gy) * n + gz, r * inv);
+            }
+            if (stop) break;
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 5) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256));
+    }
+    if (threadIdx.x == 0 && ctl->abort) atomicExch(err, 1);
+}
+size_t density_stream_smem() { return 1024 + (size_t)DS_STAGES * 16384 + 2 * (size_t)DS_KB * DS_NB * 128 + sizeof(DsShared); }
+
 size_t density_units_smem() { return 1024 + A_BYTES + (size_t)DU_STAGES * B_STAGE + sizeof(DuShared); }
 
 }  // namespace
@@ -549,6 +793,41 @@ void response_density_units(cudaStream_t st, const GridShape &g, const TileSet<f
         reinterpret_cast<const uint4 *>(P16), s16, phi_pmc, phi.val, scale, rho, ul.chunked ? 1 : 0, ul.adds ? 1 : 0, err,
         active_wait_limit());
     check_launch("density_units_kernel");
+}
+
+// rho [k][n^3] of P [k][nchi][nphi] by the streaming kernel (P rows 16-byte aligned); units: at most 320 chi
+// and 128 phi of a tile each; bits: k words.
+void response_density_stream(cudaStream_t st, const GridShape &g, const TileSet<float> &chi, const TileSet<float> &phi,
+                             const unsigned short *chi_pmc, long long nchunks_chi, const unsigned short *phi_pmc,
+                             const DUnit *units, int nunits, int nphi, const float *P, long long sP, int k, float *rho,
+                             unsigned *bits, int *err) {
+    if (k <= 0) return;
+    ProfScope ps(st, ST_DENSITY, 2.0 * k * g.pair_points, 2.0 * g.table_values + 4.0 * k * g.n * g.n * g.n);
+    check(cudaMemsetAsync(rho, 0, sizeof(float) * (size_t)k * g.n * g.n * g.n, st), "memset rho");
+    const long long nitems = (long long)nunits * k;
+    if (nitems == 0) return;
+    if (nitems > (1LL << 31) - 1) throw CudaError{cudaErrorInvalidValue, "density stream: too many items"};
+    check(cudaMemsetAsync(bits, 0, sizeof(unsigned) * k, st), "memset maxabs");
+    const int per = std::max(8, 1216 / k);
+    max_bits_kernel<<<dim3((unsigned)std::min<long long>(per, (sP + 2047) / 2048), k), 256, 0, st>>>(P, sP, bits);
+    check_launch("max_bits_kernel");
+    CUtensorMap mx;
+    if (!encode_map_2d(&mx, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, chi_pmc, 64ull, (unsigned long long)nchunks_chi * TILE_PTS,
+                       128ull, 64, 128))
+        throw CudaError{cudaErrorInvalidValue, "cuTensorMapEncodeTiled (density stream)"};
+    static const bool attr = [&]() {
+        check(cudaFuncSetAttribute(density_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)density_stream_smem()),
+              "attr density_stream");
+        return true;
+    }();
+    (void)attr;
+    int dev = 0, sms = 0;
+    check(cudaGetDevice(&dev), "cudaGetDevice");
+    check(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
+    density_stream_kernel<<<(int)std::min<long long>(sms, nitems), DS_THREADS, density_stream_smem(), st>>>(
+        mx, g.n, g.nt, k, units, (int)nitems, chi.ids, phi.ids, nphi, phi_pmc, P, sP, bits, rho, err, active_wait_limit());
+    check_launch("density_stream_kernel");
 }
 
 }  // namespace tddft

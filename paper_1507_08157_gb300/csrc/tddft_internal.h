@@ -94,6 +94,7 @@ struct DUnitList {
     const DItem *items = nullptr;
     const DUnit *units = nullptr;
     int nitems = 0;
+    int cut[2] = {256, 64};   // most chi of an item, phi of a unit
     bool covers = false;      // every tile of the grid has both chi and phi
     bool phi32 = false;       // phi in float32 instead of float16 (at most 32 per unit)
     bool adds = false;        // units add to rho (float32 reductions, in their order) instead of carrying a sum
