@@ -269,22 +269,23 @@ __global__ void __launch_bounds__(DU_THREADS, 1) density_units_kernel(
 #pragma unroll
                                 for (int j = 0; j < 8; ++j)
                                     if (2 * j < nq) *reinterpret_cast<uint4 *>(b + ((j << 4) ^ x)) = v[j];
-                        } else
-                        for (int h = 0; h * 8 < nq; ++h) {
-                            uint4 v[8];
+                        } else {
+                            for (int h = 0; h * 8 < nq; ++h) {
+                                uint4 v[8];
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                const int row = __shfl_sync(0xffffffffu, qr, h * 8 + j);
-                                v[j] = (id >= 0 && row >= 0) ? __ldg(Ps + (row + id)) : make_uint4(0u, 0u, 0u, 0u);
-                            }
-                            if (h == 0 && buse > 0 && !mbar_wait_warp(&ctl->b_empty[bi], (buse - 1) & 1, abort, wlim)) {
-                                ok = false;
-                                break;
-                            }
+                                for (int j = 0; j < 8; ++j) {
+                                    const int row = __shfl_sync(0xffffffffu, qr, h * 8 + j);
+                                    v[j] = (id >= 0 && row >= 0) ? __ldg(Ps + (row + id)) : make_uint4(0u, 0u, 0u, 0u);
+                                }
+                                if (h == 0 && buse > 0 && !mbar_wait_warp(&ctl->b_empty[bi], (buse - 1) & 1, abort, wlim)) {
+                                    ok = false;
+                                    break;
+                                }
 #pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                if (h * 8 + j < nq)
-                                    *reinterpret_cast<uint4 *>(b + h * (B_STAGE / 2) + ((j << 4) ^ x)) = v[j];
+                                for (int j = 0; j < 8; ++j)
+                                    if (h * 8 + j < nq)
+                                        *reinterpret_cast<uint4 *>(b + h * (B_STAGE / 2) + ((j << 4) ^ x)) = v[j];
+                            }
                         }
                         if (!ok) break;
                         fence_async_smem();
@@ -504,8 +505,9 @@ __global__ void __launch_bounds__(256) pack_quads_kernel(const float *__restrict
 // warps 6-7 and 12-15 gather the next item's float32 P (scaled to float16) into the other B buffer, and
 // two groups of four warps multiply their accumulator by phi. Every wait is bounded.
 // Measured (entry point with its conversions, one state, the kernel above and this): clusters at 0.1
-// atoms per A^3 with 4 + 4 functions, 200 atoms 295 and 264 us, 150 atoms 164 and 146, 110 atoms with 4 + 9 172 and 155. Not
-// so on the shorter lists of 140 atoms in the chromophore's cell (269 and 314), nor with two states.
+// atoms per A^3 with 4 + 4 functions, 200 atoms 295 and 264 us, 150 atoms 164 and 146; 110 atoms with 4 + 9
+// 172 and 155. With five states of 200 atoms the kernel above is the faster (0.88 and 0.59 ms). Lists that
+// fit the per-tile kernels keep the items (no line between the two was looked for among them).
 constexpr int DS_THREADS = 512, DS_GATHER = 192, DS_STAGES = 4;
 constexpr int DS_KB = 5, DS_NB = 128;      // chi blocks of 64 and phi of a unit
 struct __align__(8) DsShared {

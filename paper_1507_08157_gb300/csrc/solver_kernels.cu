@@ -1429,11 +1429,12 @@ void gram_blocks(cudaStream_t st, int k, int njob, const GramBlock<T> *job, int 
     // float64 rows of at most 8192 elements: a warp walks 256 elements a step, so its share stays short
     // of the row kernel's (1024 elements: 180 us and 6 us for 16 pairs; 8192 elements, 64 pairs: the
     // warps read the rows about as fast as the row kernel's few blocks)
-    if (sizeof(T) == 8 && len <= 8192) {
-        gram_short_kernel<T><<<(js.pairs + 3) / 4, 128, 0, st>>>(js, len);
-        check_launch("gram_short_kernel");
-        return;
-    }
+    if constexpr (sizeof(T) == 8)
+        if (len <= 8192) {
+            gram_short_kernel<T><<<(js.pairs + 3) / 4, 128, 0, st>>>(js, len);
+            check_launch("gram_short_kernel");
+            return;
+        }
     const int ny = most * k;
     auto grid_of = [&](int q) { return ((k + q - 1) / q) * ((ny + q - 1) / q); };
     if (vec && k + ny <= 256 * GMAXT / 16 && grid_of(4) <= 128) {
@@ -1634,18 +1635,22 @@ template <typename T>
 bool cg_reduced(cudaStream_t st, int rc, int rv, const T *Mc, const T *Mv, const T *r, T *z, int nb, double tol, int maxit,
                 int *iters) {
     const size_t sm = sizeof(T) * ((size_t)rc * rc + (size_t)rv * rv + 4 * (size_t)rc * rv);
-    if (sizeof(T) != 8 || nb < 1 || (long long)rc * rv * (rc + rv) > 131072 || sm > 200 * 1024) return false;
-    ProfScope ps(st, ST_SMALL, 0.0, 0.0);
-    static const bool attr = []() {   // once per process, thread-safe
-        check(cudaFuncSetAttribute(cg_reduced_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024),
-              "attr cg_reduced");
+    if (nb < 1 || (long long)rc * rv * (rc + rv) > 131072 || sm > 200 * 1024) return false;
+    if constexpr (sizeof(T) == 8) {
+        ProfScope ps(st, ST_SMALL, 0.0, 0.0);
+        static const bool attr = []() {   // once per process, thread-safe
+            check(cudaFuncSetAttribute(cg_reduced_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024),
+                  "attr cg_reduced");
+            return true;
+        }();
+        (void)attr;
+        check(cudaMemsetAsync(iters, 0, sizeof(int), st), "memset cg iterations");
+        cg_reduced_kernel<T><<<nb, std::min(CG_THREADS, (rc * rv + 127) / 128 * 128), sm, st>>>(rc, rv, Mc, Mv, r, z, tol, maxit,
+                                                                                             iters);
+        check_launch("cg_reduced_kernel");
         return true;
-    }();
-    (void)attr;
-    check(cudaMemsetAsync(iters, 0, sizeof(int), st), "memset cg iterations");
-    cg_reduced_kernel<T><<<nb, std::min(CG_THREADS, (rc * rv + 127) / 128 * 128), sm, st>>>(rc, rv, Mc, Mv, r, z, tol, maxit, iters);
-    check_launch("cg_reduced_kernel");
-    return true;
+    }
+    return false;
 }
 template bool cg_reduced<float>(cudaStream_t, int, int, const float *, const float *, const float *, float *, int, double,
                                 int, int *);

@@ -88,10 +88,10 @@ __device__ __forceinline__ unsigned long long smem_desc(unsigned saddr) {
     return d;
 }
 
-// For an M/N-major operand: rows of 64 elements (128 bytes) along M/N, one row per K, 8-K groups 1024 B
-// apart, the leading byte offset the distance of consecutive blocks of 64 along M/N.
-// the low words of the two descriptors vary with the address alone, so that an issuing thread forms
-// a descriptor with one add: start address in 16-byte units, plus the block distance for M/N-major
+// Low words of the descriptors of K-major and M/N-major operands (desc_lo, desc_lo_mn): they alone vary with
+// the address, so that an issuing thread forms a descriptor with one add. M/N-major: rows of 64
+// elements (128 bytes) along M/N, one row per K, 8-K groups 1024 B apart, the leading byte offset the
+// distance of consecutive blocks of 64 along M/N.
 __device__ __forceinline__ unsigned desc_lo(unsigned saddr) { return ((saddr & 0x3FFFF) >> 4) | (1u << 16); }
 __device__ __forceinline__ unsigned desc_lo_mn(unsigned saddr, unsigned blocks) {
     return ((saddr & 0x3FFFF) >> 4) | ((blocks >> 4) << 16);
