@@ -25,8 +25,9 @@
 // that streams.
 // Measured (GB300, whole stage, CUDA events, before and after): 140 atoms, 4 + 9 functions each, 135^3,
 // 10 states 1.68 and 0.77 ms, 7 states 1.20 and 0.64; 200 atoms, 180^3, 4 states 3.58 and 1.70; 20
-// atoms, 90^3, 2 states 0.044 and 0.037. Bound by the issue and shared-memory reads of the MMAs (X is
-// read once per pair of states) and the output's reductions (2 GB in 16-byte pieces at 140 atoms).
+// atoms, 90^3, 2 states 0.044 and 0.037. At 140 atoms no unit is at its limit: tensor pipe 26 % (N = 96),
+// L1 and shared memory 43 % (X is read once per pair of states), L2's reductions 15 % (1.28 GB in 16-byte
+// pieces), issue slots 46 %; the warps wait for loads, out of TMEM above all.
 #include "tc_common.cuh"
 #include "tddft_internal.h"
 
