@@ -20,7 +20,9 @@
 // finite or its columns' scales lie too far apart, the point is summed in float64. So the error is that of
 // float64 sums or below at every point: relative to the sum of the terms' sizes at most 6.1e-16, root
 // mean square 9.6e-17, where float64 sums have 8.2e-16 and 1.2e-16 (emulated, 8 atoms, 48^3); with P's
-// rows in blocks of 1, 1e-6 and 1e-12, 7.2e-16 and 9.7e-17 against 9.3e-16 and 1.2e-16. One scale for
+// rows in blocks of 1, 1e-6 and 1e-12, 7.2e-16 and 9.7e-17 against 9.3e-16 and 1.2e-16. (Entry point, 32
+// atoms and 3 states: P without structure or decaying with distance 1.05 and 1.07 ms, such rows, where
+// 40 % of the points are summed again, 7.5; CUDA cores 17.2 to 18.0.) One scale for
 // the chi table and one for a state's P left no digit right where chi is below 1e-16 of its largest value.
 // The integrals' scales are chi's and (V phi)'s largest values on the tile, each function its own. An
 // entry's error is about 2^-63 of the sum over tiles of 512 times their product, below that of a float64
