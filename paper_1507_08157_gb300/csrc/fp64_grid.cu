@@ -28,7 +28,7 @@
 // entry's error is about 2^-63 of the sum over tiles of 512 times their product, below that of a float64
 // sum wherever the entry's terms come within 2^-10 of it; entries of functions that only graze each
 // other have the same absolute error and fewer digits than a float64 sum would give them. A tile whose
-// V is not finite is summed in float64. Largest error of small-8's entries, of the largest entry: V
+// V is not finite is summed in float64. Largest error of small-8's entries, of the largest entry (emulated): V
 // without structure 3.3e-16, float64 sums 6.4e-16; V a Gaussian of 1 A, 3.6e-16 and 7.5e-16 (with one
 // scale for all of V 6e-11).
 //
